@@ -399,6 +399,14 @@ int64_t ebic_bitmap_bytes(int64_t rows, int32_t cols) {
 
 }  // extern "C"
 
+int64_t bitmap_stride(int64_t rows, int32_t cols) {
+  const int64_t w = round_up(rows, 128) / 32;
+  if (!code_bytes_for(cols)) return w;
+  for (int64_t line = 32; line >= 8; line /= 2)
+    if (round_up(w, line) - w <= w / 16) return round_up(w, line);
+  return w;
+}
+
 void ctx_release_buffers(ebic_ctx *ctx) {
   gen_state_free(ctx->gen);
   ctx->gen = nullptr;
@@ -410,7 +418,7 @@ void ctx_release_buffers(ebic_ctx *ctx) {
   ctx->pair_cnt_ok = false;
   ctx->codes_ready = false;
   ctx->tuned = false;
-  ctx->R = ctx->R_pad = ctx->Wst = 0;
+  ctx->R = ctx->R_pad = ctx->Wst = ctx->Gst = 0;
   ctx->C = 0;
 }
 
@@ -424,16 +432,16 @@ constexpr int64_t kLoadSegments = 4;
 int load_matrix_segmented(ebic_ctx *ctx, const float *x, int64_t rows, int32_t cols,
                           int64_t R_pad) {
   const bool bitmap = ctx->tuned_mode == EBIC_MODE_BITMAP;
-  const int64_t C = cols, Wst = R_pad / 32;
-  const int cb = code_bytes_for(cols), nb = code_plane_bits(cols);
+  const int64_t C = cols, Gst = bitmap_stride(rows, cols);
+  const int cb = code_bytes_for(cols);
   const int64_t S = code_stride_for(rows, cb);
   cudaStream_t s = ctx->stream;
   EBIC_CHECK_CUDA(ctx, ctx->stage_x.ensure((size_t)rows * C * sizeof(float), s));
   EBIC_CHECK_CUDA(ctx, ctx->codes.ensure((size_t)C * S * cb, s));
-  EBIC_CHECK_CUDA(ctx, ctx->planes.ensure((size_t)C * code_plane_stride(nb) * Wst * 4, s));
   EBIC_CHECK_CUDA(ctx, cudaMemsetAsync(ctx->codes.p, 0, (size_t)C * S * cb, s));
   if (bitmap) {
-    EBIC_CHECK_CUDA(ctx, ctx->bitmap.ensure((size_t)ebic_bitmap_bytes(rows, cols), s));
+    EBIC_CHECK_CUDA(ctx, ctx->planes.ensure((size_t)code_plane_words(cols, Gst) * 4, s));
+    EBIC_CHECK_CUDA(ctx, ctx->bitmap.ensure((size_t)(C * C * Gst) * 4, s));
     EBIC_CHECK_CUDA(ctx, prepare_bitmap_eval());
     const size_t nc = (size_t)C * C * sizeof(unsigned long long);
     EBIC_CHECK_CUDA(ctx, ctx->pair_cnt.ensure(nc, s));
@@ -467,15 +475,21 @@ int load_matrix_segmented(ebic_ctx *ctx, const float *x, int64_t rows, int32_t c
     EBIC_CHECK_CUDA(ctx, launch_upload_rows(stage, rows, cols, R_pad, ctx->keys.as<uint32_t>(),
                                             ctx->d_err.as<int32_t>(), r0, r1, s));
     EBIC_CHECK_CUDA(ctx, launch_rank_codes_rows(ctx->keys.as<uint32_t>(), R_pad, cols,
-                                                ctx->codes.p, cb, S, ctx->planes.as<uint32_t>(),
-                                                Wst, ctx->num_sms, r0, r1, s));
+                                                ctx->codes.p, cb, S, ctx->num_sms, r0, r1, s));
     prof_count(ctx, -1, 1);
     prof_count(ctx, EBIC_KERNEL_RANK_CODES, 1);
+    if (bitmap) {  // (a segment is a multiple of 2,048 rows: whole chunks of planes)
+      EBIC_CHECK_CUDA(ctx, launch_code_planes(ctx->codes.p, cb, S, cols, Gst,
+                                              ctx->planes.as<uint32_t>(), s, r0 / 2048,
+                                              r1 < R_pad ? r1 / 2048 : -1));
+      prof_count(ctx, -1, 1);
+    }
   }
   if (bitmap) {
-    EBIC_CHECK_CUDA(ctx, launch_build_bitmap_planes(ctx->planes.as<uint32_t>(), nb, cols, Wst,
+    EBIC_CHECK_CUDA(ctx, launch_build_bitmap_planes(ctx->planes.as<uint32_t>(), cols, Gst,
                                                     ctx->bitmap.as<uint32_t>(),
-                                                    ctx->pair_cnt.as<unsigned long long>(), s));
+                                                    ctx->pair_cnt.as<unsigned long long>(),
+                                                    ctx->num_sms, s));
     prof_count(ctx, EBIC_KERNEL_BITMAP_BUILD, 1);
   }
   int32_t herr = 0;
@@ -486,11 +500,11 @@ int load_matrix_segmented(ebic_ctx *ctx, const float *x, int64_t rows, int32_t c
   ctx->R = rows;
   ctx->C = cols;
   ctx->R_pad = R_pad;
-  ctx->Wst = Wst;
+  ctx->Wst = R_pad / 32;
+  ctx->Gst = Gst;
   direct_tma_prepare(&ctx->dtma, ctx->keys.as<uint32_t>(), R_pad, cols);
   ctx->code_bytes = cb;
   ctx->code_stride = S;
-  ctx->plane_bits = nb;
   ctx->codes_ready = true;
   ctx->bitmap_ok = bitmap;
   ctx->pair_cnt_ok = bitmap;
@@ -556,6 +570,7 @@ int ebic_load_matrix(ebic_ctx *ctx, const float *x, int64_t rows, int32_t cols, 
   ctx->C = cols;
   ctx->R_pad = R_pad;
   ctx->Wst = R_pad / 32;
+  ctx->Gst = bitmap_stride(rows, cols);
   direct_tma_prepare(&ctx->dtma, ctx->keys.as<uint32_t>(), R_pad, cols);
   // per-row rank codes for the direct form (C <= 1,024), built on the direct form's first use
   ctx->code_bytes = code_bytes_for(cols);
@@ -572,7 +587,7 @@ int ebic_build_bitmap(ebic_ctx *ctx) {
   if (ctx->bitmap_ok) return EBIC_OK;
   DeviceGuard g(ctx->device);
   const size_t bytes = (size_t)ebic_bitmap_bytes(ctx->R, ctx->C);
-  EBIC_CHECK_CUDA(ctx, ctx->bitmap.ensure(bytes, ctx->stream));
+  EBIC_CHECK_CUDA(ctx, ctx->bitmap.ensure((size_t)ctx->C * ctx->C * ctx->Gst * 4, ctx->stream));
   EBIC_CHECK_CUDA(ctx, prepare_bitmap_eval());
   // With rank codes (C <= 1,024) the words come from the codes' bit planes, else from the keys.
   if (ctx->code_bytes) EBIC_TRY(ensure_codes(ctx));
@@ -581,14 +596,20 @@ int ebic_build_bitmap(ebic_ctx *ctx) {
     const size_t nc = (size_t)ctx->C * ctx->C * sizeof(unsigned long long);
     EBIC_CHECK_CUDA(ctx, ctx->pair_cnt.ensure(nc, ctx->stream));
     EBIC_CHECK_CUDA(ctx, cudaMemsetAsync(ctx->pair_cnt.p, 0, nc, ctx->stream));
+    EBIC_CHECK_CUDA(ctx, ctx->planes.ensure((size_t)code_plane_words(ctx->C, ctx->Gst) * 4,
+                                            ctx->stream));
   }
-  cudaEvent_t ev = prof_begin(ctx);
-  if (ctx->code_bytes)
-    EBIC_CHECK_CUDA(ctx, launch_build_bitmap_planes(ctx->planes.as<uint32_t>(), ctx->plane_bits,
-                                                    ctx->C, ctx->Wst, ctx->bitmap.as<uint32_t>(),
+  cudaEvent_t ev = prof_begin(ctx);  // (the planes and the words)
+  if (ctx->code_bytes) {
+    EBIC_CHECK_CUDA(ctx, launch_code_planes(ctx->codes.p, ctx->code_bytes, ctx->code_stride,
+                                            ctx->C, ctx->Gst, ctx->planes.as<uint32_t>(),
+                                            ctx->stream));
+    prof_count(ctx, -1, 1);
+    EBIC_CHECK_CUDA(ctx, launch_build_bitmap_planes(ctx->planes.as<uint32_t>(), ctx->C, ctx->Gst,
+                                                    ctx->bitmap.as<uint32_t>(),
                                                     ctx->pair_cnt.as<unsigned long long>(),
-                                                    ctx->stream));
-  else
+                                                    ctx->num_sms, ctx->stream));
+  } else
     EBIC_CHECK_CUDA(ctx, launch_build_bitmap(ctx->keys.as<uint32_t>(), ctx->R_pad, ctx->C,
                                              ctx->Wst, ctx->bitmap.as<uint32_t>(), ctx->stream));
   prof_end(ctx, ev, EBIC_KERNEL_BITMAP_BUILD, (double)bytes,
@@ -610,8 +631,15 @@ int ebic_copy_bitmap(ebic_ctx *ctx, uint32_t *out, int64_t n_words) {
   if (!out || n_words < need) return ebic_fail(ctx, EBIC_EINVAL, "output too small");
   DeviceGuard g(ctx->device);
   EBIC_TRY(check_device_ptr(ctx, out, "out"));
-  EBIC_CHECK_CUDA(ctx, cudaMemcpyAsync(out, ctx->bitmap.p, (size_t)need * 4, cudaMemcpyDefault,
-                                       ctx->stream));
+  if (ctx->Gst == ctx->Wst) {
+    EBIC_CHECK_CUDA(ctx, cudaMemcpyAsync(out, ctx->bitmap.p, (size_t)need * 4, cudaMemcpyDefault,
+                                         ctx->stream));
+  } else {  // (the stored rows are padded)
+    EBIC_CHECK_CUDA(ctx, cudaMemcpy2DAsync(out, (size_t)ctx->Wst * 4, ctx->bitmap.p,
+                                           (size_t)ctx->Gst * 4, (size_t)ctx->Wst * 4,
+                                           (size_t)ctx->C * ctx->C, cudaMemcpyDefault,
+                                           ctx->stream));
+  }
   EBIC_CHECK_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
   return EBIC_OK;
 }
@@ -725,20 +753,14 @@ int ebic_eval_population(ebic_ctx *ctx, const int32_t *col_idx, const int32_t *o
 int ensure_codes(ebic_ctx *ctx) {
   if (!ctx->code_bytes || ctx->codes_ready) return EBIC_OK;
   const int64_t S = ctx->code_stride, C = ctx->C;
-  ctx->plane_bits = code_plane_bits(ctx->C);
   EBIC_CHECK_CUDA(ctx, ctx->codes.ensure((size_t)C * S * ctx->code_bytes, ctx->stream));
-  EBIC_CHECK_CUDA(ctx, ctx->planes.ensure(
-                           (size_t)C * code_plane_stride(ctx->plane_bits) * ctx->Wst * 4,
-                           ctx->stream));
   cudaEvent_t ev = prof_begin(ctx);
   EBIC_CHECK_CUDA(ctx, launch_rank_codes(ctx->keys.as<uint32_t>(), ctx->R_pad, ctx->C,
-                                         ctx->codes.p, ctx->code_bytes, S,
-                                         ctx->planes.as<uint32_t>(), ctx->Wst, ctx->num_sms,
+                                         ctx->codes.p, ctx->code_bytes, S, ctx->num_sms,
                                          ctx->stream));
-  // algorithmic bytes: keys read, codes and planes written
+  // algorithmic bytes: keys read, codes written
   prof_end(ctx, ev, EBIC_KERNEL_RANK_CODES,
-           (double)C * ctx->R_pad * 4.0 + (double)C * S * ctx->code_bytes +
-               (double)C * ctx->plane_bits * ctx->Wst * 4.0,
+           (double)C * ctx->R_pad * 4.0 + (double)C * S * ctx->code_bytes,
            (double)C * ctx->R_pad, (double)ctx->R_pad);
   prof_count(ctx, EBIC_KERNEL_RANK_CODES, 1);
   if (ctx->prof) {  // (later work on the stream is ordered after the build anyway)
@@ -765,7 +787,7 @@ EvalArgs eval_args_for(const ebic_ctx *ctx) {
   a.bitmap = ctx->bitmap_ok ? ctx->bitmap.as<uint32_t>() : nullptr;
   a.R = ctx->R;
   a.R_pad = ctx->R_pad;
-  a.Wst = ctx->Wst;
+  a.Wst = ctx->Gst;
   a.C = ctx->C;
   a.err = ctx->d_kerr.as<int32_t>();
   a.dtma = ctx->dtma.ok ? &ctx->dtma : nullptr;
@@ -778,7 +800,7 @@ EvalArgs eval_args_for(const ebic_ctx *ctx) {
 }
 
 int64_t eval_passes(const ebic_ctx *ctx, int mode) {
-  if (mode == EBIC_MODE_BITMAP) return (ctx->Wst + 127) / 128;
+  if (mode == EBIC_MODE_BITMAP) return (ctx->Gst + 127) / 128;
   if (ctx->codes_ready) return ctx->code_stride / code_rows_per_pass(ctx->code_bytes);
   return ctx->R_pad / 128;
 }

@@ -52,10 +52,7 @@ __device__ __forceinline__ void wait_prior_grid() {
 // found by a branchless binary search (equal keys get equal codes, as the definition requires).
 // A block owns 16 consecutive rows: their keys are staged column by column with coalesced loads
 // in a shared [C][17] tile, each row's codes replace its keys in the tile, and the tile is
-// written out column by column (codes [C][S]) together with the codes' bit planes: plane p of
-// column c, word w has bit j = bit p of code(32 w + j, c), the operand of the pair-bitmap build
-// (matrix.cu), stored [C][Wst][NBP] (a word's nb planes together, NBP = nb rounded up to a
-// multiple of 4, so that they load as 16-byte vectors); a block fills one half of each word.
+// written out column by column (codes [C][S]).
 constexpr int kRankRows = 16;                 // rows per block tile
 constexpr int kTileStride = kRankRows + 1;    // tile entries per column (bank spread)
 
@@ -136,20 +133,17 @@ __device__ __forceinline__ int count_below(const uint32_t *srt, uint32_t q) {
 }
 
 // T: code type (uint8_t for C <= 128, uint16_t for C <= 1,024); EPL: keys per lane
-// (32 * EPL >= C).  planes may be null (no bit planes wanted); nb planes per column.
+// (32 * EPL >= C).
 template <typename T, int EPL>
 __global__ void __launch_bounds__(kThreads, 2)
     k_rank_codes(const uint32_t *__restrict__ keys, int64_t R_pad, int32_t C, int64_t S,
-                 T *__restrict__ codes, uint32_t *__restrict__ planes, int64_t Wst, int nb,
-                 int64_t t_begin, int64_t t_end) {
+                 T *__restrict__ codes, int64_t t_begin, int64_t t_end) {
   constexpr int N = 32 * EPL;
   constexpr int kSorted = N + N / 32;  // words of one warp's sorted buffer
   extern __shared__ __align__(16) uint32_t s_rank[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t *srt = s_rank + warp * kSorted;
   uint32_t *tile = s_rank + kWarps * kSorted;  // [C][kTileStride]: keys, then codes in place
-  uint16_t *planes16 = reinterpret_cast<uint16_t *>(planes);
-  const int nbp = (nb + 3) & ~3;  // planes per (column, word) in the layout
   // (tiles [t_begin, t_end) of the R_pad / kRankRows)
   for (int64_t t = t_begin + blockIdx.x; t < t_end; t += gridDim.x) {
     const int64_t r0 = t * kRankRows;
@@ -181,25 +175,113 @@ __global__ void __launch_bounds__(kThreads, 2)
       const int c = i / kRankRows, rho = i % kRankRows;
       codes[(int64_t)c * S + r0 + rho] = (T)tile[c * kTileStride + rho];
     }
-    if (planes) {
-      // two columns per warp step: lanes 0-15 hold column c's 16 rows, lanes 16-31 column c + 1's
-      const int64_t w = r0 / 32, half = (r0 / kRankRows) & 1;
-      const int sub = lane >> 4;
-      for (int c2 = 2 * warp; c2 < C; c2 += 2 * kWarps) {
-        const int c = c2 + sub;
-        const uint32_t code = c < C ? tile[c * kTileStride + (lane & 15)] : 0u;
-        uint32_t mine = 0;
-        for (int p = 0; p < nb; ++p) {
-          const uint32_t bits = __ballot_sync(kFull, (code >> p) & 1u);
-          if ((lane & 15) == p) mine = sub ? (bits >> 16) : (bits & 0xFFFFu);
-        }
-        const int p = lane & 15;
-        if (p < nb && c < C)
-          planes16[2 * (((int64_t)c * Wst + w) * nbp + p) + half] = (uint16_t)mine;
-      }
-    }
     __syncthreads();  // the tile is read before the next rows overwrite it
   }
+}
+
+// ------------------------------------------------------------------------------- bit planes
+//
+// Bit planes of the codes, the operand of the pair-bitmap build (matrix.cu): plane p of column c,
+// word w has bit j = bit p of code(32 w + j, c).  Stored [C][chunks][NB][64]: a chunk is 64 words
+// (2,048 rows) of a column, its planes one after the other, so that a column's chunk is one
+// contiguous span for the build and every access of a warp is a whole 128- or 256-byte line.
+// Words past the code rows S are zero.
+// A lane owns one word: it loads its 32 rows' codes (contiguous bytes of the code column) and
+// transposes the bits in its registers, rows against planes, by 4 (16-bit codes) or 3 (8-bit
+// codes) rounds of masked exchanges between registers.  Nothing crosses lanes.  The ballot form
+// this replaced (inside the rank-code kernel, ten ballots and selects per column and 32 rows, and
+// 16-bit stores) was more than a fifth of that kernel's instructions.
+// Bound: HBM (reads the codes, writes the planes).
+
+// One exchange: bits of `a` under ~m stay, those under m go to b's lower half shifted by K, and
+// back (the 2 x 2 block transposition of a bit matrix).
+template <int K>
+__host__ __device__ __forceinline__ void swap_bits(uint32_t &a, uint32_t &b, uint32_t m) {
+  // m: the low K bits of every 2 K-bit field
+  const uint32_t na = (a & m) | ((b & m) << K);
+  const uint32_t nb = ((a >> K) & m) | (b & ~m);
+  a = na;
+  b = nb;
+}
+
+// 16-bit codes: v[q] holds rows 2 q and 2 q + 1; afterwards v[p] is plane p's word.
+__host__ __device__ __forceinline__ void transpose_codes16(uint32_t (&v)[16]) {
+  uint32_t r[16];
+  // r[i]: row i in the low half, row i + 16 in the high half
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    const uint32_t lo = v[i / 2], hi = v[i / 2 + 8];
+    r[i] = (i & 1) ? ((lo >> 16) | (hi & 0xFFFF0000u)) : ((lo & 0xFFFFu) | (hi << 16));
+  }
+  // the two 16 x 16 bit matrices (low and high halves) transposed together
+#pragma unroll
+  for (int i = 0; i < 8; ++i) swap_bits<8>(r[i], r[i + 8], 0x00FF00FFu);
+#pragma unroll
+  for (int i = 0; i < 16; ++i)
+    if (!(i & 4)) swap_bits<4>(r[i], r[i + 4], 0x0F0F0F0Fu);
+#pragma unroll
+  for (int i = 0; i < 16; ++i)
+    if (!(i & 2)) swap_bits<2>(r[i], r[i + 2], 0x33333333u);
+#pragma unroll
+  for (int i = 0; i < 16; i += 2) swap_bits<1>(r[i], r[i + 1], 0x55555555u);
+#pragma unroll
+  for (int i = 0; i < 16; ++i) v[i] = r[i];
+}
+
+// 8-bit codes: v[q] holds rows 4 q .. 4 q + 3; afterwards v[p] is plane p's word.
+__host__ __device__ __forceinline__ void transpose_codes8(uint32_t (&v)[8]) {
+  uint32_t r[8];
+  // r[i]: rows i, i + 8, i + 16, i + 24 in its four bytes
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int s = 8 * (i & 3), q = i / 4;
+    r[i] = ((v[q] >> s) & 0xFFu) | (((v[q + 2] >> s) & 0xFFu) << 8) |
+           (((v[q + 4] >> s) & 0xFFu) << 16) | (((v[q + 6] >> s) & 0xFFu) << 24);
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) swap_bits<4>(r[i], r[i + 4], 0x0F0F0F0Fu);
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    if (!(i & 2)) swap_bits<2>(r[i], r[i + 2], 0x33333333u);
+#pragma unroll
+  for (int i = 0; i < 8; i += 2) swap_bits<1>(r[i], r[i + 1], 0x55555555u);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = r[i];
+}
+
+// One warp per (column, half chunk of 32 words), columns outermost; chunks [ch0, ch1).
+template <int W, int NB>
+__global__ void __launch_bounds__(kThreads) k_code_planes(const uint8_t *__restrict__ codes,
+                                                          int64_t S, int32_t C, int64_t chunks,
+                                                          int64_t ch0, int64_t ch1,
+                                                          uint32_t *__restrict__ planes) {
+  const int lane = threadIdx.x & 31;
+  const int64_t halves = 2 * (ch1 - ch0);
+  const int64_t id = (int64_t)blockIdx.x * kWarps + (threadIdx.x >> 5);
+  const int64_t c = id / halves, h = id - c * halves;
+  if (c >= C) return;  // (whole warps)
+  const int64_t ch = ch0 + (h >> 1);
+  const int in = (int)(h & 1) * 32 + lane;  // word within the chunk
+  const int64_t row = (ch * 64 + in) * 32;
+  constexpr int NV = 8 * W;  // registers of 32 codes
+  uint32_t v[NV];
+  const uint4 *src = reinterpret_cast<const uint4 *>(codes + (c * S + row) * W);
+  const bool on = row < S;  // (S is a multiple of 256)
+#pragma unroll
+  for (int q = 0; q < NV / 4; ++q) {
+    const uint4 x = on ? __ldg(src + q) : make_uint4(0u, 0u, 0u, 0u);
+    v[4 * q] = x.x;
+    v[4 * q + 1] = x.y;
+    v[4 * q + 2] = x.z;
+    v[4 * q + 3] = x.w;
+  }
+  if constexpr (W == 2)
+    transpose_codes16(v);
+  else
+    transpose_codes8(v);
+  uint32_t *dst = planes + (c * chunks + ch) * (int64_t)(NB * 64) + in;
+#pragma unroll
+  for (int p = 0; p < NB; ++p) dst[p * 64] = v[p];
 }
 
 // ------------------------------------------------------------------------------- evaluation
@@ -382,14 +464,48 @@ int code_plane_bits(int32_t C) {
   return nb;
 }
 
-int code_plane_stride(int nb) { return (nb + 3) & ~3; }
+int64_t code_plane_chunks(int64_t Wst) { return (Wst + 63) / 64; }
+
+int64_t code_plane_words(int32_t C, int64_t Wst) {
+  return (int64_t)C * code_plane_chunks(Wst) * code_plane_bits(C) * 64;
+}
+
+cudaError_t launch_code_planes(const void *codes, int code_bytes, int64_t S, int32_t C,
+                               int64_t Wst, uint32_t *planes, cudaStream_t s, int64_t ch0,
+                               int64_t ch1) {
+  const int64_t chunks = code_plane_chunks(Wst);
+  if (ch1 < 0 || ch1 > chunks) ch1 = chunks;
+  if (C < 2 || C > 1024 || code_bytes != (C <= 128 ? 1 : 2) || ch0 < 0 || ch0 >= ch1)
+    return cudaErrorInvalidValue;
+  const int64_t warps = (int64_t)C * 2 * (ch1 - ch0);
+  const unsigned grid = (unsigned)((warps + kWarps - 1) / kWarps);
+  const uint8_t *cd = static_cast<const uint8_t *>(codes);
+#define EBIC_PLANES(W, NB)                                                               \
+  case NB:                                                                               \
+    k_code_planes<W, NB><<<grid, kThreads, 0, s>>>(cd, S, C, chunks, ch0, ch1, planes); \
+    break
+  switch (code_plane_bits(C)) {
+    EBIC_PLANES(1, 1);
+    EBIC_PLANES(1, 2);
+    EBIC_PLANES(1, 3);
+    EBIC_PLANES(1, 4);
+    EBIC_PLANES(1, 5);
+    EBIC_PLANES(1, 6);
+    EBIC_PLANES(1, 7);
+    EBIC_PLANES(2, 8);
+    EBIC_PLANES(2, 9);
+    EBIC_PLANES(2, 10);
+    default: return cudaErrorInvalidValue;
+  }
+#undef EBIC_PLANES
+  return cudaGetLastError();
+}
 
 namespace {
 
 template <typename T, int EPL>
 cudaError_t launch_rank_epl(const uint32_t *keys, int64_t R_pad, int32_t C, T *codes, int64_t S,
-                            uint32_t *planes, int64_t Wst, int nb, int num_sms, cudaStream_t s,
-                            int64_t r_begin, int64_t r_end) {
+                            int num_sms, cudaStream_t s, int64_t r_begin, int64_t r_end) {
   constexpr int N = 32 * EPL;
   const size_t smem = (size_t)kWarps * (N + N / 32) * 4 + (size_t)C * kTileStride * 4;
   // one fixed limit for every context (no call lowers another's), set once per device
@@ -414,23 +530,22 @@ cudaError_t launch_rank_epl(const uint32_t *keys, int64_t R_pad, int32_t C, T *c
   const int64_t t_begin = r_begin / kRankRows, t_end = r_end / kRankRows;
   const int64_t grid = std::min<int64_t>(
       t_end - t_begin, (int64_t)num_sms * blocks_per_sm(k_rank_codes<T, EPL>, smem));
-  k_rank_codes<T, EPL><<<(unsigned)grid, kThreads, smem, s>>>(keys, R_pad, C, S, codes, planes,
-                                                                Wst, nb, t_begin, t_end);
+  k_rank_codes<T, EPL><<<(unsigned)grid, kThreads, smem, s>>>(keys, R_pad, C, S, codes,
+                                                                t_begin, t_end);
   return cudaGetLastError();
 }
 
 }  // namespace
 
 cudaError_t launch_rank_codes_rows(const uint32_t *keys, int64_t R_pad, int32_t C, void *codes,
-                                   int code_bytes, int64_t S, uint32_t *planes, int64_t Wst,
-                                   int num_sms, int64_t r_begin, int64_t r_end, cudaStream_t s) {
+                                   int code_bytes, int64_t S, int num_sms, int64_t r_begin,
+                                   int64_t r_end, cudaStream_t s) {
   if (C > 1024 || code_bytes != (C <= 128 ? 1 : 2)) return cudaErrorInvalidValue;
   if (r_begin < 0 || r_begin % kRankRows || r_end > R_pad || r_end % kRankRows ||
       r_end <= r_begin)
     return cudaErrorInvalidValue;
-  const int nb = code_plane_bits(C);
 #define EBIC_RANK(T, EPL, cd) \
-  launch_rank_epl<T, EPL>(keys, R_pad, C, cd, S, planes, Wst, nb, num_sms, s, r_begin, r_end)
+  launch_rank_epl<T, EPL>(keys, R_pad, C, cd, S, num_sms, s, r_begin, r_end)
   if (code_bytes == 1) {
     uint8_t *cd = static_cast<uint8_t *>(codes);
     return C <= 32 ? EBIC_RANK(uint8_t, 1, cd) : C <= 64 ? EBIC_RANK(uint8_t, 2, cd)
@@ -443,13 +558,11 @@ cudaError_t launch_rank_codes_rows(const uint32_t *keys, int64_t R_pad, int32_t 
 }
 
 cudaError_t launch_rank_codes(const uint32_t *keys, int64_t R_pad, int32_t C, void *codes,
-                              int code_bytes, int64_t S, uint32_t *planes, int64_t Wst,
-                              int num_sms, cudaStream_t s) {
+                              int code_bytes, int64_t S, int num_sms, cudaStream_t s) {
   // (the rows of the code columns past R_pad, up to S, stay zero)
   cudaError_t e = cudaMemsetAsync(codes, 0, (size_t)C * S * code_bytes, s);
   if (e != cudaSuccess) return e;
-  return launch_rank_codes_rows(keys, R_pad, C, codes, code_bytes, S, planes, Wst, num_sms, 0,
-                                R_pad, s);
+  return launch_rank_codes_rows(keys, R_pad, C, codes, code_bytes, S, num_sms, 0, R_pad, s);
 }
 
 cudaError_t launch_eval_codes(const EvalArgs &a0, const PopView &pv, int num_sms, cudaStream_t s,

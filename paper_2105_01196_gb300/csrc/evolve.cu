@@ -1815,7 +1815,7 @@ GenArgs gen_args(ebic_ctx *ctx, GenState *g) {
   if (g->fuse_np > 0) {
     ga.bitmap = ctx->bitmap.as<uint32_t>();
     ga.pair_cnt = ctx->pair_cnt_ok ? ctx->pair_cnt.as<unsigned long long>() : nullptr;
-    ga.Wst = ctx->Wst;
+    ga.Wst = ctx->Gst;
     ga.R = ctx->R;
     ga.neg = p.neg_trends;
     ga.ns = p.non_strict;

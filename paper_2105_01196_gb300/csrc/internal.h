@@ -101,7 +101,7 @@ struct PopView {
 struct EvalArgs {
   const uint32_t *keys;    // [C][R_pad] order keys
   const uint32_t *bitmap;  // [C][C][Wst] pair words (bitmap path)
-  int64_t R, R_pad, Wst;   // rows, padded rows, words per column pair (R_pad / 32)
+  int64_t R, R_pad, Wst;   // rows, padded rows, words per stored pair row (ebic_ctx::Gst)
   int32_t C;
   int32_t neg, rnum, rden, min_rows, col_cap;
   int32_t non_strict, last_kept;  // pair-test variants (trend.cuh)
@@ -136,22 +136,26 @@ struct EvalArgs {
 };
 
 // Per-row rank codes (codes.cu): code width for C columns (1 for C <= 128, 2 for C <= 1024,
-// else 0 = none), rows per pass of the code kernel, padded rows per code column, the number of
-// bit planes of the codes (bits of C - 1) and their stride (planes stored per column and word: nb
-// rounded up to a multiple of 4), the rank kernel (zero-fills the padding; writes the bit planes
-// [C][Wst][stride] too when `planes` is not null) and the direct evaluation over codes.
+// else 0 = none), rows per pass of the code kernel, padded rows per code column, the rank kernel
+// (zero-fills the padding), and the direct evaluation over codes.  The codes' bit planes (bits of
+// C - 1 per column) are the pair-bitmap build's operand, [C][chunks][bits][64] words:
+// code_plane_words in all, by chunks of 64 words of a column's rows (launch_code_planes: chunks
+// [ch0, ch1) only, ch1 < 0: to the end).
 int code_bytes_for(int32_t C);
 int64_t code_rows_per_pass(int code_bytes);
 int64_t code_stride_for(int64_t R, int code_bytes);
 int code_plane_bits(int32_t C);
-int code_plane_stride(int nb);
+int64_t code_plane_chunks(int64_t Wst);
+int64_t code_plane_words(int32_t C, int64_t Wst);
 cudaError_t launch_rank_codes(const uint32_t *keys, int64_t R_pad, int32_t C, void *codes,
-                              int code_bytes, int64_t S, uint32_t *planes, int64_t Wst,
-                              int num_sms, cudaStream_t s);
+                              int code_bytes, int64_t S, int num_sms, cudaStream_t s);
 // The rows [r_begin, r_end) only (multiples of 16), codes not cleared beforehand.
 cudaError_t launch_rank_codes_rows(const uint32_t *keys, int64_t R_pad, int32_t C, void *codes,
-                                   int code_bytes, int64_t S, uint32_t *planes, int64_t Wst,
-                                   int num_sms, int64_t r_begin, int64_t r_end, cudaStream_t s);
+                                   int code_bytes, int64_t S, int num_sms, int64_t r_begin,
+                                   int64_t r_end, cudaStream_t s);
+cudaError_t launch_code_planes(const void *codes, int code_bytes, int64_t S, int32_t C,
+                               int64_t Wst, uint32_t *planes, cudaStream_t s, int64_t ch0 = 0,
+                               int64_t ch1 = -1);
 cudaError_t launch_eval_codes(const EvalArgs &a, const PopView &pv, int num_sms, cudaStream_t s,
                               bool pdl);
 
@@ -192,7 +196,8 @@ struct ebic_ctx {
   std::string err;
 
   // matrix
-  int64_t R = 0, R_pad = 0, Wst = 0;
+  int64_t R = 0, R_pad = 0, Wst = 0;  // (Wst = R_pad / 32: words of a pair row)
+  int64_t Gst = 0;                    // words a pair row takes in the bitmap (bitmap_stride)
   int32_t C = 0;
   bool have_matrix = false;
   DevBuf keys, bitmap, stage_x;
@@ -210,13 +215,11 @@ struct ebic_ctx {
   DirectTma dtma;
   DevBuf d_kerr;
 
-  // per-row rank codes of the loaded matrix (code_bytes 0: none) and their bit planes
-  // [C][Wst][code_plane_stride(plane_bits)] (the pair-bitmap build's operand), built together
-  // on first use
+  // per-row rank codes of the loaded matrix (code_bytes 0: none), built on first use, and their
+  // bit planes (the pair-bitmap build's operand), built with the bitmap
   DevBuf codes, planes;
   int code_bytes = 0;
   int64_t code_stride = 0;
-  int plane_bits = 0;
   bool codes_ready = false;
 
   // autotuner decisions for the loaded matrix (tune.cu)
@@ -281,6 +284,14 @@ int stage_population(ebic_ctx *ctx, const int32_t *col_idx, const int32_t *offse
 int ebic_check_eval_params(ebic_ctx *ctx, const ebic_params *p);
 int ebic_check_run_params(ebic_ctx *ctx, const ebic_params *p);
 
+// Words a pair row of a rows x cols matrix takes in the stored bitmap: its R_pad / 32 words, padded
+// with zero words to a whole 128-byte line (32 words), or 64 or 32 bytes, where that adds at most
+// 1/16.  Without it, every second pair row of 60,000 rows (7,504 bytes) starts in the middle of a
+// 32-byte sector: the build's stores alone took 1.73 ms at 60,000 x 1,000 against 1.25 ms padded
+// (1.32 ms padded to sectors only), and the evaluations' reads touch a line more per piece.
+// Above 1,024 columns (the build from the keys) rows are not padded.
+int64_t bitmap_stride(int64_t rows, int32_t cols);
+
 // matrix.cu
 cudaError_t launch_upload(const float *x, int64_t R, int32_t C, int64_t R_pad, int32_t layout,
                           uint32_t *keys, int32_t *err, cudaStream_t s);
@@ -290,14 +301,12 @@ cudaError_t launch_upload_rows(const float *x, int64_t R, int32_t C, int64_t R_p
                                cudaStream_t s);
 cudaError_t launch_build_bitmap(const uint32_t *keys, int64_t R_pad, int32_t C, int64_t Wst,
                                 uint32_t *bitmap, cudaStream_t s);
-// The same bitmap from the bit planes of the rank codes (nb planes per column, nb <= 10); with
-// cnt (C * C, zeroed beforehand) also the pair rows' popcounts: for a < b, cnt[a * C + b] =
-// popcount(G[a][b]) | popcount(G[b][a]) << 32.
-// chunk0 / chunk1: only the 32-word row chunks [chunk0, chunk1) (chunk1 < 0: to the end).
-cudaError_t launch_build_bitmap_planes(const uint32_t *planes, int nb, int32_t C, int64_t Wst,
-                                       uint32_t *bitmap, unsigned long long *cnt,
-                                       cudaStream_t s, int64_t chunk0 = 0,
-                                       int64_t chunk1 = -1);
+// The same bitmap from the bit planes of the rank codes (launch_code_planes), with cnt (C * C,
+// zeroed beforehand) the pair rows' popcounts: for a < b, cnt[a * C + b] = popcount(G[a][b]) |
+// popcount(G[b][a]) << 32.
+cudaError_t launch_build_bitmap_planes(const uint32_t *planes, int32_t C, int64_t Wst,
+                                       uint32_t *bitmap, unsigned long long *cnt, int num_sms,
+                                       cudaStream_t s);
 
 // eval.cu
 cudaError_t launch_validate_csr(const int32_t *cols, const int32_t *off, int32_t n, int32_t C,

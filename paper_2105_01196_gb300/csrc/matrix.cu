@@ -176,19 +176,24 @@ __global__ void __launch_bounds__(kBW * 32, 4) k_build_bitmap(const uint32_t *__
 // gt = [code_b > code_a] = G[a][b] and lt = [code_a > code_b] = G[b][a] in every bit: a higher
 // differing bit overrides the lower ones, equal bits keep them.  Ties and pad rows (code 0
 // everywhere) set neither.
-// A warp owns four a-columns (their planes in registers) and one 32-word chunk of rows (a word
-// per lane, so every store is one coalesced 128-byte row piece), and walks b over a piece of at
-// most kPiece columns after its own; the b planes of a block's eight warps come through L1.
-// The b-range of an a-block is cut into pieces so that every block has about the same work
-// (the first a-blocks pair with many more columns than the last ones).  The row chunk is the
-// fastest block index, so the blocks resident together write adjacent 128-byte pieces of the
-// same pair rows, which L2 then merges into whole sectors before they reach DRAM.  Piece p of
-// a-block g starts at column 32 (g + 4 p); the pieces run in the order of that start (then of
-// g), so the blocks in flight together read the same b planes, which stay in L2 between them.
-constexpr int kPA = 4;       // a-columns per warp
-constexpr int kPiece = 128;  // b-columns per block (at most)
-constexpr int kMaxABlocks = 32;  // a-blocks of 32 columns: C <= 1,024
-constexpr int kMaxPieces = kMaxABlocks * (1024 / kPiece);
+// A warp owns two a-columns (their planes in registers) and one chunk of 64 words of rows (two
+// words per lane, so every store is one coalesced 256-byte row piece), and walks b over a piece
+// of consecutive columns after its own; the block's eight warps share the staged b planes.
+// The row chunk is the fastest block index, so the blocks resident together write adjacent
+// 256-byte pieces of the same pair rows, which L2 then merges into whole sectors before they
+// reach DRAM.  The b-range of an a-block is cut into pieces of 16 << shift columns, so that the
+// launch has enough blocks of about the same work to fill the GPU evenly (the first a-blocks
+// pair with many more columns than the last ones): see launch_build_bitmap_planes.  The pieces
+// run in the order of their first column (then of the a-block), so the blocks in flight together
+// read the same b planes, which stay in L2 between them.
+constexpr int kPA = 2;            // a-columns per warp
+constexpr int kBuildWarps = 8;    // warps per block
+constexpr int kABlock = kBuildWarps * kPA;  // a-columns per block
+constexpr int kMaxPieceShift = 3;  // pieces of 16, 32, 64 or 128 columns
+constexpr int kMaxABlocks = 1024 / kABlock;  // C <= 1,024
+// pieces of 16 columns over every a-block of 16: 64 - g for a-block g
+static_assert(kABlock == 16, "the piece count below");
+constexpr int kMaxPieces = kMaxABlocks * (kMaxABlocks + 1) / 2;
 
 struct PieceTable {
   uint16_t item[kMaxPieces];  // piece y of the launch: a-block << 8 | piece within the a-block
@@ -201,19 +206,20 @@ __device__ __forceinline__ uint32_t lop3(uint32_t a, uint32_t b, uint32_t c) {
   return d;
 }
 
-template <int NB>
-__device__ __forceinline__ void plane_compare(const uint32_t (&A)[NB], const uint32_t (&B)[NB],
-                                              uint32_t &gt, uint32_t &lt) {
-  gt = 0u;
-  lt = 0u;
-#pragma unroll
-  for (int p = 0; p < NB; ++p) {
-    gt = lop3<0x8E>(A[p], B[p], gt);  // (B & ~A) | (~(A ^ B) & gt)
-    lt = lop3<0xB2>(A[p], B[p], lt);  // (A & ~B) | (~(A ^ B) & lt)
-  }
+// The lowest plane, and one further plane's step, for both directions of a pair in the two words
+// of a lane.
+__device__ __forceinline__ void plane_first(uint2 A, uint2 B, uint2 &gt, uint2 &lt) {
+  gt = make_uint2(B.x & ~A.x, B.y & ~A.y);
+  lt = make_uint2(A.x & ~B.x, A.y & ~B.y);
+}
+__device__ __forceinline__ void plane_step(uint2 A, uint2 B, uint2 &gt, uint2 &lt) {
+  gt.x = lop3<0x8E>(A.x, B.x, gt.x);  // (B & ~A) | (~(A ^ B) & gt)
+  gt.y = lop3<0x8E>(A.y, B.y, gt.y);
+  lt.x = lop3<0xB2>(A.x, B.x, lt.x);  // (A & ~B) | (~(A ^ B) & lt)
+  lt.y = lop3<0xB2>(A.y, B.y, lt.y);
 }
 
-constexpr int kBB = 16;  // b-columns per staged batch (48 KB of static shared memory at NB = 10)
+constexpr int kBB = 8;  // b-columns per staged batch (40 KB of static shared memory at NB = 10)
 
 __device__ __forceinline__ void cp_async16_bm(void *smem, const void *gmem) {
   const unsigned saddr = (unsigned)__cvta_generic_to_shared(smem);
@@ -229,77 +235,98 @@ __device__ __forceinline__ void cp_wait_bm() {
 
 // The b planes of a block's piece are staged in shared memory, kBB columns at a time and
 // double-buffered (cp.async by the whole block; the next batch is in flight while the current
-// one is compared), so the eight warps share one copy and read it with constant offsets.  The
-// planes are stored [C][Wst][NBP] (NBP = NB rounded up to 4): a column's chunk of 32 words is
-// one contiguous span, copied as is, and each lane reads its word's planes as NBP / 4 16-byte
-// vectors (lanes 48 or 16 bytes apart: no bank conflicts; 32 bytes apart at NBP = 8: two-way).
+// one is compared), so the eight warps share one copy.  A column's chunk is one contiguous span
+// [NB][64] of the planes, copied as is; a lane reads the two words of a plane as one 8-byte load
+// (a warp's loads are one 256-byte line: no bank conflicts).
+// Two words per lane and two a-columns give eight independent comparator chains per b column
+// within 80 registers (24 warps per SM), and everything a pair costs besides its comparators
+// (addresses, stores, the warp sum of its counts) comes once per 64 words.
 // The pair counts are accumulated too (cnt, zeroed beforehand): for a < b, cnt[a * C + b] holds
 // the rows of G[a][b] (its popcount) in its low 32 bits and those of G[b][a] in its high 32
-// bits.  Each warp adds its 32 words' counts of a pair by one warp sum (the two directions'
-// counts packed in 16-bit halves, at most 1,024 each) and one 64-bit atomic.
-// In the last row chunk, lanes past Wst hold zero planes for a (not loaded) and for b (their
-// staged words are zeroed once and never copied): every such row compares equal, so their words
-// are zero (and not stored) and add nothing to the sums.
+// bits.  Each warp adds its 64 words' counts of a pair by one warp sum (the two directions'
+// counts packed in 16-bit halves, at most 2,048 each); lane j keeps the sums of the j-th of 32
+// consecutive b columns, so that the atomics (64-bit) go out 32 at a time.
+// What bounds it: the ALU pipe (40 lop3 of about 54 ALU instructions per pair and 64 words; the
+// pipe is about 80% busy, the stores alone would take 1.25 ms at 60,000 x 1,000).  Measured with
+// the planes' transposition, before (one word per lane, four a-columns per warp, planes written
+// by the rank kernel) and now: 60,000 x 1,000 2.00 -> 1.65 ms, 33,333 x 777 685 -> 576 us,
+// 20,000 x 500 185 -> 140 us, 10,000 x 100 44 -> 14 us.  Without the counts it takes 1.36 ms; four
+// blocks per SM (64 registers, spills) 1.87 ms, four a-columns per warp (128 registers, two
+// blocks) 1.83 ms, the b loop unrolled 2 or 4 times 1.71-1.73 ms.
+// In the last chunk, words past Wst have zero planes in every column: they compare equal, so
+// their words are zero (and not stored) and add nothing to the sums.
 template <int NB>
-__global__ void __launch_bounds__(256, 2) k_build_bitmap_planes(const uint32_t *__restrict__ planes,
+__global__ void __launch_bounds__(kBuildWarps * 32, 3) k_build_bitmap_planes(const uint32_t *__restrict__ planes,
                                                              int32_t C, int64_t Wst,
+                                                             int64_t chunks, int shift,
                                                              PieceTable tab,
                                                              uint32_t *__restrict__ G,
-                                                             unsigned long long *__restrict__ cnt,
-                                                             int64_t chunk0) {
-  constexpr int NBP = (NB + 3) & ~3;
-  __shared__ __align__(16) uint32_t s_b[2][kBB][32][NBP];
+                                                             unsigned long long *__restrict__ cnt) {
+  constexpr int kSpan = NB * 64;  // words of a column's chunk
+  __shared__ __align__(16) uint32_t s_b[2][kBB][kSpan];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   // this block's a-block and piece (blockIdx.x is the row chunk: the blocks running together
   // write neighbouring pieces of the same pair rows)
   const int item = tab.item[blockIdx.y];
   const int ablk = item >> 8, piece = item & 0xFF;
-  const int64_t w0 = (chunk0 + (int64_t)blockIdx.x) * 32, w = w0 + lane;
+  const int64_t ch = blockIdx.x;
+  const int64_t w = ch * 64 + 2 * lane;  // the lane's words w, w + 1 (Wst is even: both or none)
   const bool w_ok = w < Wst;
-  const int a0 = (ablk * 8 + warp) * kPA;
-  const int b_lo = ablk * 8 * kPA + piece * kPiece;  // the piece's b-range
-  const int b_hi = min(C, b_lo + kPiece);
-  const int b_first = max(b_lo, ablk * 8 * kPA + kPA);  // the first b any warp of the block needs
-  uint32_t A[kPA][NB];
+  const int a0 = ablk * kABlock + warp * kPA;
+  const int b_lo = ablk * kABlock + (piece << (shift + 4));  // the piece's b-range
+  const int b_hi = min(C, b_lo + (16 << shift));
+  const int b_first = max(b_lo, ablk * kABlock + kPA);  // the first b any warp of the block needs
+  const int64_t cstride = chunks * kSpan;               // words between columns of the planes
+  const uint32_t *pl = planes + ch * kSpan;             // column c's chunk at pl + c * cstride
+  auto issue = [&](int t, int nbb) {  // batch t: columns b_first + t kBB + bb, bb < nbb
+    const int bs = b_first + t * kBB;
+    for (int j = threadIdx.x; j < nbb * (kSpan / 4); j += kBuildWarps * 32) {
+      const int bb = j / (kSpan / 4), part = j - bb * (kSpan / 4);
+      cp_async16_bm(&s_b[t & 1][bb][part * 4], pl + (int64_t)(bs + bb) * cstride + part * 4);
+    }
+    cp_commit_bm();
+  };
+  const int n_b = b_hi - b_first;  // (<= 0: no b beyond the block's columns in this piece)
+  const int n_batches = n_b > 0 ? (n_b + kBB - 1) / kBB : 0;
+  if (n_batches > 0) issue(0, min(kBB, n_b));
+  uint2 A[kPA][NB];
 #pragma unroll
   for (int i = 0; i < kPA; ++i) {
-    const bool on = a0 + i < C && w_ok;
-    const uint4 *src = reinterpret_cast<const uint4 *>(planes + ((int64_t)(a0 + i) * Wst + w) * NBP);
+    const uint2 *src = reinterpret_cast<const uint2 *>(pl + (int64_t)(a0 + i) * cstride) + lane;
 #pragma unroll
-    for (int q = 0; q < NBP / 4; ++q) {
-      const uint4 v = on ? __ldg(src + q) : make_uint4(0u, 0u, 0u, 0u);
-      const uint32_t e[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-        if (4 * q + k < NB) A[i][4 * q + k] = e[k];
-    }
+    for (int p = 0; p < NB; ++p) A[i][p] = a0 + i < C ? __ldg(src + 32 * p) : make_uint2(0u, 0u);
   }
   const int64_t row = (int64_t)C * Wst;  // words between G[a][.] and G[a + 1][.]
-  // this warp's 32 words' counts of G[a][b] (gt) and G[b][a] (lt), packed, summed over the lanes
-  auto warp_counts = [&](uint32_t gt, uint32_t lt) -> unsigned {
-    return __reduce_add_sync(0xFFFFFFFFu, (unsigned)__popc(gt) + ((unsigned)__popc(lt) << 16));
+  // this warp's 64 words' counts of G[a][b] (gt) and G[b][a] (lt), packed, summed over the lanes
+  auto warp_counts = [&](uint2 gt, uint2 lt) -> unsigned {
+    return __reduce_add_sync(0xFFFFFFFFu,
+                             (unsigned)(__popc(gt.x) + __popc(gt.y)) +
+                                 ((unsigned)(__popc(lt.x) + __popc(lt.y)) << 16));
   };
   auto add_counts = [&](int a, int b, unsigned n) {  // (a < b)
     if (n)
       atomicAdd(cnt + (int64_t)a * C + b,
                 (unsigned long long)(n & 0xFFFFu) | ((unsigned long long)(n >> 16) << 32));
   };
+  auto store = [&](uint32_t *p, uint2 v) { __stcs(reinterpret_cast<uint2 *>(p), v); };
   if (piece == 0 && a0 < C) {
     // the diagonal words, and the pairs among the warp's own columns
 #pragma unroll
     for (int i = 0; i < kPA; ++i) {
       const int a = a0 + i;
       if (a >= C) break;
-      if (w_ok) G[(int64_t)a * row + (int64_t)a * Wst + w] = 0u;
+      if (w_ok) store(G + (int64_t)a * row + (int64_t)a * Wst + w, make_uint2(0u, 0u));
 #pragma unroll
       for (int i2 = i + 1; i2 < kPA; ++i2) {
         const int b = a0 + i2;
         if (b < C) {
-          uint32_t gt, lt;
-          plane_compare<NB>(A[i], A[i2], gt, lt);
+          uint2 gt, lt;
+          plane_first(A[i][0], A[i2][0], gt, lt);
+#pragma unroll
+          for (int p = 1; p < NB; ++p) plane_step(A[i][p], A[i2][p], gt, lt);
           if (w_ok) {
-            __stcs(G + (int64_t)a * row + (int64_t)b * Wst + w, gt);
-            __stcs(G + (int64_t)b * row + (int64_t)a * Wst + w, lt);
+            store(G + (int64_t)a * row + (int64_t)b * Wst + w, gt);
+            store(G + (int64_t)b * row + (int64_t)a * Wst + w, lt);
           }
           const unsigned n = warp_counts(gt, lt);
           if (lane == 0) add_counts(a, b, n);
@@ -307,35 +334,17 @@ __global__ void __launch_bounds__(256, 2) k_build_bitmap_planes(const uint32_t *
       }
     }
   }
-  if (b_first >= b_hi) return;  // (the whole block: no b beyond its columns in this piece)
-  // staging: batch t holds b = b_first + t kBB + bb; copy j of a batch is 16-byte part j % span
-  // of column bb = j / span (span: the chunk's words x NBP / 4; Wst % 4 == 0)
-  const int n_batches = (b_hi - b_first + kBB - 1) / kBB;
-  const int valid = (int)(Wst - w0 >= 32 ? 32 : Wst - w0);  // words of this chunk
-  const int span = valid * NBP / 4;
-  if (valid < 32) {  // the tail lanes' staged words, in both buffers
-    for (int j = threadIdx.x; j < 2 * kBB * (32 - valid) * NBP; j += blockDim.x) {
-      const int k = j % NBP, l = valid + (j / NBP) % (32 - valid), bb = j / (NBP * (32 - valid));
-      (&s_b[0][0][0][0])[((int64_t)bb * 32 + l) * NBP + k] = 0u;
-    }
-  }
-  auto issue = [&](int t) {
-    const int bs = b_first + t * kBB, nbb = min(kBB, b_hi - bs);
-    for (int j = threadIdx.x; j < nbb * span; j += blockDim.x) {
-      const int bb = j / span, part = j - bb * span;
-      cp_async16_bm(&s_b[t & 1][bb][0][0] + part * 4,
-                    planes + ((int64_t)(bs + bb) * Wst + w0) * NBP + part * 4);
-    }
-    cp_commit_bm();
-  };
   // G[a][b] at a * row + b * Wst, G[b][a] at b * row + a * Wst; (a + i)'s words sit i rows (or
-  // i * Wst words) past a's: 32-bit offsets from two pointers
+  // i * Wst words) past a's: 32-bit offsets from two pointers (32-bit offsets for the b columns
+  // too, from pointers set once per batch, made the build 5% slower)
   const uint32_t row32 = (uint32_t)row, wst32 = (uint32_t)Wst;  // (checked at launch)
   const bool active = a0 < C;  // (the whole warp; lanes past Wst store nothing)
-  issue(0);
+  unsigned sum[kPA];
+#pragma unroll
+  for (int i = 0; i < kPA; ++i) sum[i] = 0u;
   for (int t = 0; t < n_batches; ++t) {
     if (t + 1 < n_batches) {
-      issue(t + 1);
+      issue(t + 1, min(kBB, n_b - (t + 1) * kBB));
       cp_wait_bm<1>();
     } else {
       cp_wait_bm<0>();
@@ -346,40 +355,38 @@ __global__ void __launch_bounds__(256, 2) k_build_bitmap_planes(const uint32_t *
     if (active && bb0 < nbb) {
       uint32_t *g_ab = G + (int64_t)a0 * row + (int64_t)(bs + bb0) * Wst + w;
       uint32_t *g_ba = G + (int64_t)(bs + bb0) * row + (int64_t)a0 * Wst + w;
-      // (b columns are independent: unrolled, their comparator chains interleave; the build at
-      // 60,000 x 1,000 took 2.00 ms unrolled 4 times, 2.21-2.22 ms 1 or 2 times, 2.21 ms 8 times,
-      // 2.17 ms 16 times; with a test of b against the warp's columns inside the loop, a select of
-      // the tail lanes' counts and the counts optional, 2.33 ms rolled and 2.18 ms at best)
-#pragma unroll 4
+#pragma unroll 1
       for (int bb = bb0; bb < nbb; ++bb) {
-        uint32_t B[NB];
+        const uint2 *sb = reinterpret_cast<const uint2 *>(&s_b[t & 1][bb][0]) + lane;
+        uint2 gt[kPA], lt[kPA];
 #pragma unroll
-        for (int q = 0; q < NBP / 4; ++q) {
-          const uint4 v = *reinterpret_cast<const uint4 *>(&s_b[t & 1][bb][lane][4 * q]);
-          const uint32_t e[4] = {v.x, v.y, v.z, v.w};
+        for (int i = 0; i < kPA; ++i) plane_first(A[i][0], sb[0], gt[i], lt[i]);
 #pragma unroll
-          for (int k = 0; k < 4; ++k)
-            if (4 * q + k < NB) B[4 * q + k] = e[k];
+        for (int p = 1; p < NB; ++p) {
+          const uint2 B = sb[32 * p];
+#pragma unroll
+          for (int i = 0; i < kPA; ++i) plane_step(A[i][p], B, gt[i], lt[i]);
         }
-        unsigned n[kPA];
+        const bool mine = lane == ((t * kBB + bb) & 31);
 #pragma unroll
         for (int i = 0; i < kPA; ++i) {
-          uint32_t gt, lt;
-          plane_compare<NB>(A[i], B, gt, lt);
           if (w_ok) {
-            __stcs(g_ab + (uint32_t)i * row32, gt);
-            __stcs(g_ba + (uint32_t)i * wst32, lt);
+            store(g_ab + (uint32_t)i * row32, gt[i]);
+            store(g_ba + (uint32_t)i * wst32, lt[i]);
           }
-          n[i] = warp_counts(gt, lt);
-        }
-        if (lane < kPA) {  // lane i adds pair (a0 + i, b)'s counts
-          unsigned mine = n[0];
-#pragma unroll
-          for (int i = 1; i < kPA; ++i) mine = lane == i ? n[i] : mine;
-          add_counts(a0 + lane, bs + bb, mine);
+          const unsigned n = warp_counts(gt[i], lt[i]);
+          sum[i] = mine ? n : sum[i];
         }
         g_ab += Wst;
         g_ba += row;
+      }
+    }
+    if (active && ((t & 3) == 3 || t + 1 == n_batches)) {  // 32 columns' counts, or the last ones
+      const int b = b_first + (t & ~3) * kBB + lane;
+#pragma unroll
+      for (int i = 0; i < kPA; ++i) {
+        if (b < b_hi) add_counts(a0 + i, b, sum[i]);  // (0 where b is not after the columns)
+        sum[i] = 0u;
       }
     }
     __syncthreads();  // every warp is done with this buffer before batch t + 2 refills it
@@ -429,51 +436,56 @@ cudaError_t launch_build_bitmap(const uint32_t *keys, int64_t R_pad, int32_t C, 
   return cudaGetLastError();
 }
 
-cudaError_t launch_build_bitmap_planes(const uint32_t *planes, int nb, int32_t C, int64_t Wst,
-                                       uint32_t *bitmap, unsigned long long *cnt,
-                                       cudaStream_t s, int64_t chunk0, int64_t chunk1) {
-  const int64_t n_all = (Wst + 31) / 32;
-  if (chunk1 < 0 || chunk1 > n_all) chunk1 = n_all;
-  if (chunk0 < 0 || chunk0 >= chunk1) return chunk0 == chunk1 ? cudaSuccess : cudaErrorInvalidValue;
-  const int64_t n_chunks = chunk1 - chunk0;
-  const int n_ablk = (C + 8 * kPA - 1) / (8 * kPA);
+cudaError_t launch_build_bitmap_planes(const uint32_t *planes, int32_t C, int64_t Wst,
+                                       uint32_t *bitmap, unsigned long long *cnt, int num_sms,
+                                       cudaStream_t s) {
+  const int64_t chunks = code_plane_chunks(Wst);
+  const int n_ablk = (C + kABlock - 1) / kABlock;
   if (!cnt) return cudaErrorInvalidValue;  // (the pair counts are always accumulated)
-  // (the kernel offsets rows of the bitmap by up to 3 * C * Wst words in 32 bits)
-  if (n_ablk > kMaxABlocks || n_chunks > 0x7FFFFFFF || 4 * (int64_t)C * Wst > 0xFFFFFFFFll)
+  // (the kernel offsets rows of the bitmap by up to C * Wst words in 32 bits)
+  if (C < 2 || n_ablk > kMaxABlocks || chunks > 0x7FFFFFFF ||
+      4 * (int64_t)C * Wst > (1ll << 32))
     return cudaErrorInvalidValue;
-  // every (a-block g, piece p) with b in [32 g, C), in the order of the piece's first column
-  // 32 (g + 4 p), then of g
+  // every (a-block g, piece p) with b in [16 g, C), in the order of the piece's first column
+  // 16 g + len p, then of g.  The longest piece that still gives kWaves blocks per resident block
+  // (three per SM), so that the last wave and the uneven first pieces are a small part of the launch
+  // (8 waves against 24 and 60: 576, 599 and 598 us at 33,333 x 777; 1.64, 1.65 and 1.68 ms at
+  // 60,000 x 1,000; with pieces of 128 columns always, a 10,000 x 100 matrix had 40 blocks)
+  constexpr int64_t kWaves = 8;
   PieceTable tab{};
-  int total = 0;
-  const int k_max = (C + 8 * kPA - 1) / (8 * kPA);
-  for (int k = 0; k < k_max; ++k)
-    for (int g = k % 4; g <= k && g < n_ablk; g += 4) {
-      const int piece = (k - g) / 4;  // (starts at column 32 k < C)
-      tab.item[total++] = (uint16_t)(g << 8 | piece);
-    }
-  const dim3 grid((unsigned)n_chunks, (unsigned)total), block(256);  // (total <= 32 * 8 pieces)
-  switch (nb) {
-    case 1: k_build_bitmap_planes<1><<<grid, block, 0, s>>>(planes, C, Wst, tab, bitmap, cnt, chunk0);
-      break;
-    case 2: k_build_bitmap_planes<2><<<grid, block, 0, s>>>(planes, C, Wst, tab, bitmap, cnt, chunk0);
-      break;
-    case 3: k_build_bitmap_planes<3><<<grid, block, 0, s>>>(planes, C, Wst, tab, bitmap, cnt, chunk0);
-      break;
-    case 4: k_build_bitmap_planes<4><<<grid, block, 0, s>>>(planes, C, Wst, tab, bitmap, cnt, chunk0);
-      break;
-    case 5: k_build_bitmap_planes<5><<<grid, block, 0, s>>>(planes, C, Wst, tab, bitmap, cnt, chunk0);
-      break;
-    case 6: k_build_bitmap_planes<6><<<grid, block, 0, s>>>(planes, C, Wst, tab, bitmap, cnt, chunk0);
-      break;
-    case 7: k_build_bitmap_planes<7><<<grid, block, 0, s>>>(planes, C, Wst, tab, bitmap, cnt, chunk0);
-      break;
-    case 8: k_build_bitmap_planes<8><<<grid, block, 0, s>>>(planes, C, Wst, tab, bitmap, cnt, chunk0);
-      break;
-    case 9: k_build_bitmap_planes<9><<<grid, block, 0, s>>>(planes, C, Wst, tab, bitmap, cnt, chunk0);
-      break;
-    case 10: k_build_bitmap_planes<10><<<grid, block, 0, s>>>(planes, C, Wst, tab, bitmap, cnt, chunk0);
-      break;
+  int total = 0, shift = kMaxPieceShift;
+  for (;; --shift) {
+    const int len = 16 << shift;
+    total = 0;
+    for (int g = 0; g < n_ablk; ++g) total += (C - g * kABlock + len - 1) / len;
+    if (shift == 0 || chunks * total >= kWaves * 3 * num_sms) break;
+  }
+  const int len = 16 << shift;
+  int at = 0;
+  for (int start = 0; start < C; start += std::min(len, kABlock))
+    for (int g = 0; g < n_ablk && g * kABlock <= start; ++g)
+      if ((start - g * kABlock) % len == 0)
+        tab.item[at++] = (uint16_t)(g << 8 | (start - g * kABlock) / len);
+  if (at != total) return cudaErrorInvalidValue;
+  const dim3 grid((unsigned)chunks, (unsigned)total), block(kBuildWarps * 32);
+#define EBIC_BUILD(NB)                                                                        \
+  case NB:                                                                                    \
+    k_build_bitmap_planes<NB><<<grid, block, 0, s>>>(planes, C, Wst, chunks, shift, tab, bitmap, \
+                                                     cnt);                                    \
+    break
+  switch (code_plane_bits(C)) {
+    EBIC_BUILD(1);
+    EBIC_BUILD(2);
+    EBIC_BUILD(3);
+    EBIC_BUILD(4);
+    EBIC_BUILD(5);
+    EBIC_BUILD(6);
+    EBIC_BUILD(7);
+    EBIC_BUILD(8);
+    EBIC_BUILD(9);
+    EBIC_BUILD(10);
     default: return cudaErrorInvalidValue;
   }
+#undef EBIC_BUILD
   return cudaGetLastError();
 }
