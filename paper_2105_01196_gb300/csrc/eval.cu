@@ -20,6 +20,7 @@
 #include <mutex>
 #include <type_traits>
 
+#include "csr.cuh"
 #include "internal.h"
 #include "tables.cuh"
 #include "items.cuh"
@@ -55,31 +56,14 @@ __device__ __forceinline__ uint4 ldg4(const uint32_t *p) {
 
 // ------------------------------------------------------------------------------- validation
 
-// One warp per individual: lane k holds columns k and k + 32 (sentinels that no column and no
-// other lane's sentinel equals past the length); a column out of range, a repeated column, a
-// start below 0 or a length outside [2, 64] sets bit 2 of *err.
+// One warp per individual; a bad one (csr_bad) sets bit 2 of *err.
 __global__ void k_validate_csr(const int32_t *__restrict__ cols, const int32_t *__restrict__ off,
                                int32_t n, int32_t C, int32_t *__restrict__ err) {
   const int lane = threadIdx.x & 31;
   const int64_t i = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (i >= n) return;  // (whole warps)
-  const int s = off[i], e = off[i + 1];
-  const int L = e - s;
-  bool bad = (s < 0) || L < 2 || L > EBIC_MAX_LEN;  // (warp-uniform)
-  if (!bad) {
-    const bool in0 = lane < L, in1 = lane + 32 < L;
-    const int c0 = in0 ? cols[s + lane] : -1 - lane;
-    const int c1 = in1 ? cols[s + 32 + lane] : -33 - lane;
-    // (every lane takes part in each collective: none sits in a short-circuited operand)
-    const unsigned m0 = __match_any_sync(kFull, c0), m1 = __match_any_sync(kFull, c1);
-    bad = (in0 && (c0 < 0 || c0 >= C)) || (in1 && (c1 < 0 || c1 >= C));
-    bad = bad || __popc(m0) > 1 || __popc(m1) > 1;
-    for (int j = 0; j < 32; ++j) {
-      const int b = __shfl_sync(kFull, c0, j);
-      bad = bad || c1 == b;
-    }
-  }
-  if (__any_sync(kFull, bad) && lane == 0) atomicOr(err, 2);
+  int c0, c1;
+  if (csr_bad(cols, off[i], off[i + 1], C, lane, &c0, &c1) && lane == 0) atomicOr(err, 2);
 }
 
 // ------------------------------------------------------------------------------- direct form

@@ -5,9 +5,15 @@
 // allocation fails or fragments the pool; and latency-critical callers, for whom cudaFree's
 // device-wide synchronisation and the allocator's unbounded latency are not acceptable.  This
 // entry point takes every input and output from the caller, and keeps its scratch (per-individual
-// count accumulators, the work-queue counter and an error word) in one file-scope
-// `static __device__` array of fixed size, which every GPU that loads the library holds until
-// the process exits.
+// count accumulators and an error word) in one file-scope `static __device__` array of fixed size,
+// which every GPU that loads the library holds until the process exits.
+//
+// A call is three launches and one synchronisation: k_na_prepare checks the matrix and the
+// population and clears the accumulators, k_na_eval counts, k_na_finish writes the outputs.  The
+// later two find the error word set and do nothing when the check failed; the host reads it at
+// the end.  (With the result of the check read back before the evaluation, clears as separate
+// operations, and the evaluation one row per lane from a queue of items on one counter, a call
+// took 329 us at 10,000 x 100, 800 individuals: 214 us of it in the evaluation.)
 //
 // Host code cannot name that array's device address directly: in host code its name stands for
 // a host-side shadow.  The address is therefore fetched once per device with
@@ -20,8 +26,10 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <mutex>
 
+#include "csr.cuh"
 #include "internal.h"
 #include "trend.cuh"
 
@@ -34,8 +42,8 @@ constexpr int kMaxDevices = 64;
 
 struct NoAllocScratch {
   int32_t counts[3 * EBIC_NOALLOC_MAX_IND];  // rows_pos | rows_neg | rows_any accumulators
-  int32_t work;                              // work-queue counter
-  int32_t err;                               // 1: non-finite matrix value, 2: bad chromosome
+  int32_t reserved;
+  int32_t err;  // 1: non-finite matrix value, 2: bad chromosome; 0 between calls
 };
 
 static __device__ __align__(256) NoAllocScratch g_noalloc_scratch;
@@ -47,51 +55,74 @@ __device__ __forceinline__ int threshold(int L, int num, int den) {
   return (num * (L - 1) + den - 1) / den;
 }
 
-// Checks the matrix for NaN/Inf and the population for invalid chromosomes.
-__global__ void k_na_validate(const float *__restrict__ x, int64_t total,
-                              const int32_t *__restrict__ cols, const int32_t *__restrict__ off,
-                              int32_t n, int32_t C, NoAllocScratch *sc) {
-  bool bad_x = false;
-  const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t q = tid; q < total; q += stride) {
-    const uint32_t u = __float_as_uint(__ldg(x + q));
-    bad_x |= (u & 0x7F800000u) == 0x7F800000u;
-  }
-  if (__any_sync(kFull, bad_x) && (threadIdx.x & 31) == 0) atomicOr(&sc->err, 1);
-  for (int64_t i = tid; i < n; i += stride) {
-    const int s = off[i], L = off[i + 1] - s;
-    bool bad = s < 0 || L < 2 || L > EBIC_MAX_LEN;
-    for (int k = 0; k < L && !bad; ++k) {
-      const int c = cols[s + k];
-      if (c < 0 || c >= C) bad = true;
-      for (int j = 0; j < k && !bad; ++j)
-        if (cols[s + j] == c) bad = true;
-    }
-    if (bad) atomicOr(&sc->err, 2);
-  }
+// Waits for the preceding kernel of a programmatic launch (no-op otherwise).
+__device__ __forceinline__ void wait_prior_grid() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-// Direct float32 comparisons (-0 equals +0; no FTZ in this file's compilation), one row per
-// lane, warps pulling (individual, segment of 32-row passes) items from sc->work.  NS / LK are
-// the pair-test variants of trend.cuh.
-template <bool NEG, bool NS, bool LK>
-__global__ void __launch_bounds__(kNaThreads) k_na_eval(const float *__restrict__ x, int64_t R,
-                                                        const int32_t *__restrict__ cols,
-                                                        const int32_t *__restrict__ off,
-                                                        int32_t n, int32_t n_seg,
-                                                        int32_t seg_passes, int32_t rnum,
-                                                        int32_t rden, NoAllocScratch *sc) {
+__device__ __forceinline__ bool not_finite(uint32_t u) { return (u & 0x7F800000u) == 0x7F800000u; }
+
+// Checks the population (a warp per individual) and the matrix for NaN/Inf (16-byte loads from
+// the first 16-byte boundary on, any alignment of x), and clears the accumulators.
+// Bound: HBM (one read of x).
+__global__ void __launch_bounds__(kNaThreads) k_na_prepare(const float *__restrict__ x,
+                                                           int64_t total,
+                                                           const int32_t *__restrict__ cols,
+                                                           const int32_t *__restrict__ off,
+                                                           int32_t n, int32_t C,
+                                                           NoAllocScratch *sc) {
+  const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  const int lane = threadIdx.x & 31;
+  for (int64_t q = tid; q < 3 * (int64_t)n; q += stride) sc->counts[q] = 0;
+  bool bad = false;
+  for (int64_t i = tid >> 5; i < n; i += stride >> 5) {  // (whole warps)
+    int c0, c1;
+    bad |= csr_bad(cols, off[i], off[i + 1], C, lane, &c0, &c1);
+  }
+  const uint32_t *u = reinterpret_cast<const uint32_t *>(x);
+  int64_t head = (int64_t)((16 - (reinterpret_cast<uintptr_t>(x) & 15)) & 15) / 4;
+  if (head > total) head = total;
+  const int64_t vecs = (total - head) / 4;
+  const uint4 *v = reinterpret_cast<const uint4 *>(u + head);
+  bool bad_x = false;
+#pragma unroll 4
+  for (int64_t q = tid; q < vecs; q += stride) {
+    const uint4 w = __ldg(v + q);
+    bad_x |= not_finite(w.x) || not_finite(w.y) || not_finite(w.z) || not_finite(w.w);
+  }
+  // the up to three values on either side of the 16-byte pieces
+  const int64_t tail0 = head + 4 * vecs;
+  if (tid < head) bad_x |= not_finite(__ldg(u + tid));
+  if (tid < total - tail0) bad_x |= not_finite(__ldg(u + tail0 + tid));
+  const unsigned e = (__any_sync(kFull, bad_x) ? 1u : 0u) | (__any_sync(kFull, bad) ? 2u : 0u);
+  if (e && lane == 0) atomicOr(&sc->err, (int)e);
+}
+
+// Direct float32 comparisons (-0 equals +0; no FTZ in this file's compilation).  An item is an
+// individual and a segment of 128-row passes, segment-major, taken by the warps in turn; a lane
+// counts four rows of a pass: consecutive ones by one 16-byte load per column where every column
+// starts on a 16-byte boundary (VEC: x aligned, R a multiple of 4), else rows 32 apart by four
+// 4-byte loads (coalesced whatever the alignment).  NS / LK are the pair-test variants of
+// trend.cuh.  Bound: L2 (4 bytes per row and pair, about 8 TB/s): 43 us at 10,000 x 100, 800
+// individuals of 2-20 columns (214 us with a row per lane and the items of 32-row passes taken
+// from one counter), 0.96 ms at 30,000 x 300, 4,000 individuals of 2-40 (1.04 ms with three items
+// per warp instead of six, 1.22 ms with one).
+template <bool NEG, bool NS, bool LK, bool VEC>
+__global__ void __launch_bounds__(kNaThreads, 4) k_na_eval(const float *__restrict__ x, int64_t R,
+                                                           const int32_t *__restrict__ cols,
+                                                           const int32_t *__restrict__ off,
+                                                           int32_t n, int32_t n_seg,
+                                                           int32_t seg_passes, int32_t rnum,
+                                                           int32_t rden, NoAllocScratch *sc) {
   __shared__ int64_t s_base[kNaWarps][EBIC_MAX_LEN];
+  wait_prior_grid();
+  if (sc->err) return;  // (a bad population is never indexed with)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t passes_total = (R + 31) / 32;
-  const int32_t n_items = n * n_seg;
-  for (;;) {
-    int q = 0;
-    if (lane == 0) q = atomicAdd(&sc->work, 1);
-    q = __shfl_sync(kFull, q, 0);
-    if (q >= n_items) break;
-    const int i = q / n_seg, seg = q - i * n_seg;
+  const int64_t passes_total = (R + 127) / 128;
+  const int64_t n_items = (int64_t)n * n_seg, W = (int64_t)gridDim.x * kNaWarps;
+  for (int64_t q = (int64_t)blockIdx.x * kNaWarps + warp; q < n_items; q += W) {
+    const int seg = (int)(q / n), i = (int)(q - (int64_t)seg * n);
     const int st = off[i], L = off[i + 1] - st;
     __syncwarp();
     for (int k = lane; k < L; k += 32) s_base[warp][k] = (int64_t)cols[st + k] * R;
@@ -101,12 +132,38 @@ __global__ void __launch_bounds__(kNaThreads) k_na_eval(const float *__restrict_
     const int64_t p1 = min(p0 + seg_passes, passes_total);
     int cp = 0, cn = 0, ca = 0;
     for (int64_t pass = p0; pass < p1; ++pass) {
-      const int64_t r = pass * 32 + lane;
-      if (r < R) {
-        RowTrend<float, NEG, NS, LK> tr;
-        tr.start(__ldg(x + s_base[warp][0] + r));
-        for (int k = 1; k < L; ++k) tr.step(__ldg(x + s_base[warp][k] + r));
-        const bool po = tr.inc >= t, ne = NEG && tr.dec >= t;
+      const int64_t r0 = pass * 128 + (VEC ? 4 * lane : lane);
+      const int step = VEC ? 1 : 32;  // the lane's rows: r0 + j * step
+      // column k's four values (0 past the last row)
+      auto load = [&](int k, float (&v)[4]) {
+        const float *p = x + s_base[warp][k] + r0;
+        if (VEC) {
+          const float4 f = r0 < R ? __ldg(reinterpret_cast<const float4 *>(p))
+                                  : make_float4(0.f, 0.f, 0.f, 0.f);
+          v[0] = f.x;
+          v[1] = f.y;
+          v[2] = f.z;
+          v[3] = f.w;
+        } else {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) v[j] = r0 + 32 * j < R ? __ldg(p + 32 * j) : 0.f;
+        }
+      };
+      RowTrend<float, NEG, NS, LK> tr[4];
+      float v[4];
+      load(0, v);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) tr[j].start(v[j]);
+#pragma unroll 4
+      for (int k = 1; k < L; ++k) {
+        load(k, v);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) tr[j].step(v[j]);
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const bool valid = r0 + j * step < R;
+        const bool po = valid && tr[j].inc >= t, ne = valid && NEG && tr[j].dec >= t;
         cp += po;
         cn += ne;
         ca += po || ne;
@@ -126,8 +183,9 @@ __global__ void __launch_bounds__(kNaThreads) k_na_eval(const float *__restrict_
 __global__ void k_na_finish(const int32_t *__restrict__ off, int32_t n, int32_t min_rows,
                             int32_t col_cap, const NoAllocScratch *sc, int32_t *rows_pos,
                             int32_t *rows_neg, int32_t *rows_any, uint64_t *fitness) {
+  wait_prior_grid();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
+  if (i >= n || sc->err) return;
   const int rp = sc->counts[i], rn = sc->counts[n + i], ra = sc->counts[2 * n + i];
   if (rows_pos) rows_pos[i] = rp;
   if (rows_neg) rows_neg[i] = rn;
@@ -141,11 +199,32 @@ __global__ void k_na_finish(const int32_t *__restrict__ off, int32_t n, int32_t 
 
 using NaKernel = void (*)(const float *, int64_t, const int32_t *, const int32_t *, int32_t,
                           int32_t, int32_t, int32_t, int32_t, NoAllocScratch *);
-// Indexed by neg_trends * 4 + non_strict * 2 + last_kept.
-const NaKernel kNaEval[8] = {k_na_eval<false, false, false>, k_na_eval<false, false, true>,
-                             k_na_eval<false, true, false>,  k_na_eval<false, true, true>,
-                             k_na_eval<true, false, false>,  k_na_eval<true, false, true>,
-                             k_na_eval<true, true, false>,   k_na_eval<true, true, true>};
+// Indexed by neg_trends * 8 + non_strict * 4 + last_kept * 2 + aligned.
+#define EBIC_NA(NEG, NS) \
+  k_na_eval<NEG, NS, false, false>, k_na_eval<NEG, NS, false, true>, \
+      k_na_eval<NEG, NS, true, false>, k_na_eval<NEG, NS, true, true>
+const NaKernel kNaEval[16] = {EBIC_NA(false, false), EBIC_NA(false, true), EBIC_NA(true, false),
+                              EBIC_NA(true, true)};
+#undef EBIC_NA
+
+// Launches `kern` so that it may be scheduled while the previous kernel of the stream drains (it
+// waits for that kernel's results before it reads them).
+template <class... Args>
+cudaError_t launch_next(void (*kern)(Args...), unsigned grid, unsigned block, cudaStream_t s,
+                        Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
+int g_num_sms[kMaxDevices] = {};  // set with the scratch address
 
 // Set-up for `device`, done once: with the device current, fetch the device address of the
 // scratch array and query every kernel of this file, so that the module (array and code) is in
@@ -160,9 +239,11 @@ cudaError_t scratch_for_device(int device, NoAllocScratch **out) {
     void *ptr = nullptr;
     e = cudaGetSymbolAddress(&ptr, g_noalloc_scratch);
     cudaFuncAttributes fa;
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_na_validate);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_na_prepare);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_na_finish);
-    for (int k = 0; k < 8 && e == cudaSuccess; ++k) e = cudaFuncGetAttributes(&fa, kNaEval[k]);
+    for (int k = 0; k < 16 && e == cudaSuccess; ++k) e = cudaFuncGetAttributes(&fa, kNaEval[k]);
+    if (e == cudaSuccess)
+      e = cudaDeviceGetAttribute(&g_num_sms[device], cudaDevAttrMultiProcessorCount, device);
     if (prev >= 0 && prev != device) cudaSetDevice(prev);
     if (e != cudaSuccess) return e;
     g_scratch_addr[device] = static_cast<NoAllocScratch *>(ptr);
@@ -244,54 +325,48 @@ extern "C" int ebic_eval_population_noalloc(const float *x, int64_t rows, int32_
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   int status = EBIC_OK;
   do {
-    // The array keeps the previous call's contents: clear the accumulators this call uses, the
-    // work counter and the error word.
-    if ((e = cudaMemsetAsync(sc->counts, 0, (size_t)3 * n_ind * sizeof(int32_t), s)) != cudaSuccess)
-      break;
-    if ((e = cudaMemsetAsync(&sc->work, 0, 2 * sizeof(int32_t), s)) != cudaSuccess) break;
-    k_na_validate<<<1024, 256, 0, s>>>(x, rows * (int64_t)cols, col_idx, offsets, n_ind, cols,
-                                       sc);
+    const int64_t num_sms = g_num_sms[device], total = rows * (int64_t)cols;
+    const int64_t pre = std::max((total / 16 + kNaThreads - 1) / kNaThreads,
+                                 (int64_t)(n_ind + kNaWarps - 1) / kNaWarps);
+    k_na_prepare<<<(unsigned)std::min<int64_t>(pre, 8 * num_sms), kNaThreads, 0, s>>>(
+        x, total, col_idx, offsets, n_ind, cols, sc);
     if ((e = cudaGetLastError()) != cudaSuccess) break;
+    // Segments: about six items per resident warp (four blocks per SM), so that the uneven
+    // lengths even out without a queue.
+    const int64_t passes_total = (rows + 127) / 128;
+    int64_t seg = ((int64_t)n_ind * passes_total) / (6 * 4 * num_sms * kNaWarps);
+    if (seg < 1) seg = 1;
+    if (seg > passes_total) seg = passes_total;
+    int64_t n_seg = (passes_total + seg - 1) / seg;
+    const int64_t grid =
+        std::min<int64_t>(((int64_t)n_ind * n_seg + kNaWarps - 1) / kNaWarps, 4 * num_sms);
+    const int aligned = rows % 4 == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0;
+    const NaKernel kern = kNaEval[(p->neg_trends ? 8 : 0) + (p->non_strict ? 4 : 0) +
+                                  (p->last_kept ? 2 : 0) + aligned];
+    if ((e = launch_next(kern, (unsigned)grid, kNaThreads, s, x, rows, col_idx, offsets, n_ind,
+                         (int32_t)n_seg, (int32_t)seg, p->ratio_num, p->ratio_den, sc)) !=
+        cudaSuccess)
+      break;
+    if ((e = launch_next(k_na_finish, (unsigned)((n_ind + 255) / 256), 256u, s, offsets, n_ind,
+                         p->min_rows, p->col_cap, (const NoAllocScratch *)sc, rows_pos, rows_neg,
+                         rows_any, fitness)) != cudaSuccess)
+      break;
     int32_t herr = 0;
     if ((e = cudaMemcpyAsync(&herr, &sc->err, sizeof(herr), cudaMemcpyDeviceToHost, s)) !=
         cudaSuccess)
       break;
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) break;
-    if (herr & 1) {
-      status = fail(msg, msg_len, EBIC_ENAN, "matrix holds NaN or Inf");
-      break;
+    if (herr) {  // (the word is 0 between calls)
+      if ((e = cudaMemsetAsync(&sc->err, 0, sizeof(herr), s)) != cudaSuccess) break;
+      if ((e = cudaStreamSynchronize(s)) != cudaSuccess) break;
+      status = (herr & 1) ? fail(msg, msg_len, EBIC_ENAN, "matrix holds NaN or Inf")
+                          : fail(msg, msg_len, EBIC_EINVAL, "invalid chromosome in the population");
     }
-    if (herr & 2) {
-      status = fail(msg, msg_len, EBIC_EINVAL, "invalid chromosome in the population");
-      break;
-    }
-    int num_sms = 0;
-    if ((e = cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, device)) !=
-        cudaSuccess)
-      break;
-    const int64_t passes_total = (rows + 31) / 32;
-    int64_t seg = ((int64_t)n_ind * passes_total) / ((int64_t)8 * num_sms * kNaWarps * 2);
-    if (seg < 1) seg = 1;
-    if (seg > passes_total) seg = passes_total;
-    int64_t n_seg = (passes_total + seg - 1) / seg;
-    while ((int64_t)n_ind * n_seg > (1LL << 30)) {
-      seg *= 2;
-      n_seg = (passes_total + seg - 1) / seg;
-    }
-    int64_t grid = ((int64_t)n_ind * n_seg + kNaWarps - 1) / kNaWarps;
-    if (grid > (int64_t)num_sms * 2) grid = (int64_t)num_sms * 2;
-    const NaKernel kern =
-        kNaEval[(p->neg_trends ? 4 : 0) + (p->non_strict ? 2 : 0) + (p->last_kept ? 1 : 0)];
-    kern<<<(unsigned)grid, kNaThreads, 0, s>>>(x, rows, col_idx, offsets, n_ind, (int32_t)n_seg,
-                                               (int32_t)seg, p->ratio_num, p->ratio_den, sc);
-    if ((e = cudaGetLastError()) != cudaSuccess) break;
-    k_na_finish<<<(n_ind + 255) / 256, 256, 0, s>>>(offsets, n_ind, p->min_rows, p->col_cap, sc,
-                                                    rows_pos, rows_neg, rows_any, fitness);
-    if ((e = cudaGetLastError()) != cudaSuccess) break;
-    e = cudaStreamSynchronize(s);
   } while (false);
   if (prev >= 0 && prev != device) cudaSetDevice(prev);
   if (e != cudaSuccess) {
+    cudaGetLastError();
+    cudaMemsetAsync(&sc->err, 0, sizeof(int32_t), s);  // (whatever stopped the call)
     cudaGetLastError();
     char buf[256];
     snprintf(buf, sizeof(buf), "CUDA error: %s", cudaGetErrorString(e));

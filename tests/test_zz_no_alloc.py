@@ -206,3 +206,32 @@ def test_noalloc_binding_checks_arguments_without_converting(ebic):
         with pytest.raises(ebic.EbicError) as e:
             ebic.ebic_eval_population_noalloc(params=p, **kw)
         assert e.value.code == ebic.EBIC_EINVAL, list(change)
+
+
+@pytest.mark.parametrize("R,C,offset", [(1, 2, 0), (3, 5, 0), (127, 3, 1), (128, 4, 2), (130, 7, 3),
+                                        (4096, 33, 0), (4100, 9, 1), (5001, 20, 0)])
+def test_noalloc_any_alignment_and_row_count(ebic, R, C, offset):
+    """Row counts around the 128-row passes and multiples of 4, and matrices that start 0 to 3 floats
+    past a 16-byte boundary (16-byte loads, or 4-byte ones where a column is not aligned): equal
+    to the oracle in every pair-test variant; a NaN in the first or last value is found."""
+    torch = pytest.importorskip("torch")
+    dev = torch.device("cuda:0")
+    x, ci, off = make_inputs(R + C, R, C, 37)
+    store = torch.zeros(R * C + 4, dtype=torch.float32, device=dev)
+    x_cm = store[offset:offset + R * C].reshape(C, R)
+    x_cm.copy_(torch.from_numpy(np.ascontiguousarray(x.T)))
+    ci_d, off_d = torch.from_numpy(ci).to(dev), torch.from_numpy(off).to(dev)
+    for neg, num, den, ns, lk in VARIANTS:
+        p = ebic.Params.make(neg_trends=neg, ratio_num=num, ratio_den=den, min_rows=0,
+                             non_strict=ns, last_kept=lk)
+        op = OParams(neg_trends=neg, ratio_num=num, ratio_den=den, min_rows=0, col_cap=p.col_cap,
+                     non_strict=ns, last_kept=lk)
+        outs = _outs(torch, 37, dev)
+        ebic.ebic_eval_population_noalloc(x_cm, ci_d, off_d, p, *outs)
+        assert _same([o.cpu().numpy() for o in outs], ocounts.eval_population(x, ci, off, op))
+    for at in (0, R * C - 1):
+        y = x_cm.clone()
+        y.view(-1)[at] = float("nan")
+        with pytest.raises(ebic.EbicError) as e:
+            ebic.ebic_eval_population_noalloc(y, ci_d, off_d, p, *outs)
+        assert e.value.code == ebic.EBIC_ENAN
