@@ -4,8 +4,10 @@
 #include <string.h>
 
 #include <algorithm>
+#include <map>
 #include <mutex>
 #include <new>
+#include <tuple>
 
 #include "internal.h"
 
@@ -68,6 +70,27 @@ cudaMemPool_t library_pool() {
   return pools[dev];
 }
 
+int resident_blocks(const void *kernel, int threads, size_t smem) {
+  static std::mutex mu;
+  static std::map<std::tuple<int, const void *, int, size_t>, int> known;
+  int dev = 0, nb = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) cudaGetLastError();
+  const auto key = std::make_tuple(dev, kernel, threads, smem);
+  std::lock_guard<std::mutex> lock(mu);
+  const auto it = known.find(key);
+  if (it != known.end()) return it->second;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, threads, smem) != cudaSuccess) {
+    cudaGetLastError();
+    return 1;
+  }
+  nb = std::max(nb, 1);
+  try {
+    known[key] = nb;
+  } catch (...) {  // (asked again next time)
+  }
+  return nb;
+}
+
 int ebic_fail(ebic_ctx *ctx, int code, const std::string &msg) {
   if (ctx) ctx->err = msg;
   return code;
@@ -89,6 +112,55 @@ bool ebic_is_device_ptr(const void *p) {
     return false;
   }
   return attr.type == cudaMemoryTypeDevice || attr.type == cudaMemoryTypeManaged;
+}
+
+// The context's pinned block (see ebic_ctx::pin).  Pinning host memory takes a few hundred
+// microseconds, so blocks of closed contexts are kept for the next ones, up to kPinKeep of them.
+constexpr size_t kPinStatus = 256, kPinIn = 256 << 10, kPinOut = 256 << 10;
+constexpr size_t kPinKeep = 8;
+static std::mutex g_pin_mu;
+static unsigned char *g_pin_free[kPinKeep];
+static size_t g_pin_n = 0;
+
+static unsigned char *take_pin() {
+  {
+    std::lock_guard<std::mutex> lock(g_pin_mu);
+    if (g_pin_n) return g_pin_free[--g_pin_n];
+  }
+  void *p = nullptr;
+  if (cudaHostAlloc(&p, kPinStatus + kPinIn + kPinOut,
+                    cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  return static_cast<unsigned char *>(p);
+}
+
+static void give_pin(unsigned char *p) {  // (no work of the context is left that uses it)
+  if (!p) return;
+  {
+    std::lock_guard<std::mutex> lock(g_pin_mu);
+    if (g_pin_n < kPinKeep) {
+      g_pin_free[g_pin_n++] = p;
+      return;
+    }
+  }
+  cudaFreeHost(p);
+}
+
+// Whether p is memory of the device (as ebic_is_device_ptr); EBIC_EINVAL when it is another
+// device's.  One query for both.
+static int classify_ptr(ebic_ctx *ctx, const void *p, const char *name, bool *is_device) {
+  *is_device = false;
+  cudaPointerAttributes attr;
+  if (cudaPointerGetAttributes(&attr, p) != cudaSuccess) {
+    cudaGetLastError();
+    return EBIC_OK;
+  }
+  if (attr.type == cudaMemoryTypeDevice && attr.device != ctx->device)
+    return ebic_fail(ctx, EBIC_EINVAL, std::string(name) + " is memory of another device");
+  *is_device = attr.type == cudaMemoryTypeDevice || attr.type == cudaMemoryTypeManaged;
+  return EBIC_OK;
 }
 
 static int check_device_ptr(ebic_ctx *ctx, const void *p, const char *name) {
@@ -362,7 +434,10 @@ int ebic_create(ebic_ctx **out, int32_t device, void *cuda_stream) {
   if (ctx->d_err.ensure(64, ctx->stream) != cudaSuccess ||
       ctx->d_work.ensure(64, ctx->stream) != cudaSuccess ||
       ctx->d_kerr.ensure(64, ctx->stream) != cudaSuccess ||
-      cudaMemset(ctx->d_kerr.p, 0, 64) != cudaSuccess) {
+      cudaMemset(ctx->d_kerr.p, 0, 64) != cudaSuccess ||
+      cudaMemset(ctx->d_work.p, 0, 64) != cudaSuccess ||
+      !(ctx->pin = take_pin())) {
+    cudaGetLastError();
     ebic_destroy(ctx);
     return EBIC_ENOMEM;
   }
@@ -381,6 +456,7 @@ int ebic_destroy(ebic_ctx *ctx) {
                     &ctx->ev_cols, &ctx->ev_off, &ctx->ev_out, &ctx->ev_fit, &ctx->d_kerr,
                     &ctx->codes, &ctx->planes, &ctx->pair_cnt};
   for (DevBuf *b : bufs) b->release();
+  give_pin(ctx->pin);
   prof_collect(ctx);
   for (cudaEvent_t e : ctx->ev_pool) cudaEventDestroy(e);
   for (cudaEvent_t e : ctx->seg_ev) cudaEventDestroy(e);
@@ -658,6 +734,48 @@ int ebic_copy_pair_counts(ebic_ctx *ctx, uint64_t *out, int64_t n) {
   return EBIC_OK;
 }
 
+// The plain form: a launch per individual, which needs the offsets on the host.
+static int eval_population_plain(ebic_ctx *ctx, const int32_t *col_idx, const int32_t *offsets,
+                                 int32_t n_ind, EvalArgs &a, void *const outs[4]) {
+  cudaStream_t s = ctx->stream;
+  StagedPop sp;
+  EBIC_TRY(stage_population(ctx, col_idx, offsets, n_ind, true, &sp));
+  PopView pv{};
+  pv.cols = sp.d_cols;
+  pv.off = sp.d_off;
+  pv.n = n_ind;
+  EBIC_CHECK_CUDA(ctx, cudaMemsetAsync(a.rows_pos, 0, (size_t)n_ind * 3 * 4, s));
+  cudaEvent_t ev = prof_begin(ctx);
+  for (int32_t i = 0; i < n_ind; ++i)
+    EBIC_CHECK_CUDA(ctx, launch_eval_plain(a, sp.d_cols + sp.h_off[i],
+                                           sp.h_off[i + 1] - sp.h_off[i], i, s));
+  prof_end(ctx, ev, EBIC_KERNEL_EVAL, (double)sp.total * (double)ctx->R_pad * 4.0,
+           (double)(sp.total - n_ind) * (double)ctx->R * (a.neg ? 2.0 : 1.0),
+           (double)n_ind * (double)ctx->R);
+  prof_count(ctx, EBIC_KERNEL_EVAL, n_ind);
+  EBIC_CHECK_CUDA(ctx, launch_fitness(a, pv, s));
+  prof_count(ctx, -1, 1);
+  for (int k = 0; k < 3; ++k)
+    if (outs[k])
+      EBIC_CHECK_CUDA(ctx, cudaMemcpyAsync(outs[k], a.rows_pos + (size_t)k * n_ind,
+                                           (size_t)n_ind * 4, cudaMemcpyDefault, s));
+  if (outs[3])
+    EBIC_CHECK_CUDA(ctx, cudaMemcpyAsync(outs[3], a.fitness, (size_t)n_ind * 8,
+                                         cudaMemcpyDefault, s));
+  EBIC_CHECK_CUDA(ctx, cudaStreamSynchronize(s));
+  prof_collect(ctx);
+  return EBIC_OK;
+}
+
+// One evaluation is three launches (check and clears, evaluation, fitness and outputs) and one
+// synchronisation; the evaluation and the output do nothing when the check failed.  Only where
+// AUTO's choice of the form depends on the mean length of a device population is there a second
+// synchronisation, after the check.  A small host population goes through the context's pinned
+// block, which the first launch reads and the last one writes, instead of through copies.
+// (With separate clears, copies and two to three synchronisations, a call took about 90 us more
+// than its kernels: 64 individuals on 200 x 20 from host arrays 110 us, now 31; 800 on
+// 10,000 x 100 112 and 57 us; 4,096 on 20,000 x 500 by the bitmap 199 and 122 us; 512 on
+// 5,001 x 1,500 125 and 62 us.)
 int ebic_eval_population(ebic_ctx *ctx, const int32_t *col_idx, const int32_t *offsets,
                          int32_t n_ind, const ebic_params *p, int32_t *rows_pos,
                          int32_t *rows_neg, int32_t *rows_any, uint64_t *fitness) {
@@ -668,84 +786,171 @@ int ebic_eval_population(ebic_ctx *ctx, const int32_t *col_idx, const int32_t *o
   if (n_ind == 0) return EBIC_OK;
   if (!col_idx || !offsets) return ebic_fail(ctx, EBIC_EINVAL, "col_idx/offsets NULL");
   DeviceGuard g(ctx->device);
-  EBIC_TRY(check_device_ptr(ctx, col_idx, "col_idx"));
-  EBIC_TRY(check_device_ptr(ctx, offsets, "offsets"));
+  bool dev_cols, dev_off, dev_out[4] = {};
+  EBIC_TRY(classify_ptr(ctx, col_idx, "col_idx", &dev_cols));
+  EBIC_TRY(classify_ptr(ctx, offsets, "offsets", &dev_off));
   void *outs[4] = {rows_pos, rows_neg, rows_any, fitness};
-  for (void *o : outs)
-    if (o) EBIC_TRY(check_device_ptr(ctx, o, "output"));
+  for (int k = 0; k < 4; ++k)
+    if (outs[k]) EBIC_TRY(classify_ptr(ctx, outs[k], "output", &dev_out[k]));
+  if (dev_cols != dev_off)
+    return ebic_fail(ctx, EBIC_EINVAL, "col_idx and offsets must both be host or both device");
   cudaStream_t s = ctx->stream;
-  StagedPop sp;
-  EBIC_TRY(stage_population(ctx, col_idx, offsets, n_ind, p->mode == EBIC_MODE_PLAIN, &sp));
-  const int32_t *d_cols = sp.d_cols, *d_off = sp.d_off;
-  const std::vector<int32_t> &h_off = sp.h_off;
-  const double mean_len = sp.mean_len;
-  const int64_t total = sp.total;
-
-  int mode = choose_mode(ctx, p->mode, n_ind, mean_len, 1, p->last_kept);
-  if (mode == EBIC_MODE_BITMAP && !ctx->bitmap_ok) EBIC_TRY(ebic_build_bitmap(ctx));
-  if (direct_form_used(ctx, mode, p)) EBIC_TRY(ensure_codes(ctx));
-
-  EBIC_CHECK_CUDA(ctx, ctx->ev_out.ensure((size_t)n_ind * 3 * sizeof(int32_t), ctx->stream));
-  EBIC_CHECK_CUDA(ctx, ctx->ev_fit.ensure((size_t)n_ind * sizeof(uint64_t), ctx->stream));
-  EvalArgs a = eval_args_for(ctx);
-  a.neg = p->neg_trends;
-  a.non_strict = p->non_strict;
-  a.last_kept = p->last_kept;
-  a.rnum = p->ratio_num;
-  a.rden = p->ratio_den;
-  a.min_rows = p->min_rows;
-  a.col_cap = p->col_cap;
-  a.rows_pos = ctx->ev_out.as<int32_t>();
-  a.rows_neg = a.rows_pos + n_ind;
-  a.rows_any = a.rows_neg + n_ind;
-  a.fitness = ctx->ev_fit.as<uint64_t>();
-  a.work = ctx->d_work.as<int32_t>();
-  a.seg_passes = ctx->tuned ? (mode == EBIC_MODE_BITMAP ? ctx->seg_bitmap
-                                                      : (mode == EBIC_MODE_DIRECT ? ctx->seg_direct : 0))
-                            : 0;
-  a.ipw = p->ipw > 0 ? p->ipw : (ctx->tuned && mode == EBIC_MODE_BITMAP ? ctx->ipw_bitmap : 1);
-  PopView pv{};
-  pv.cols = d_cols;
-  pv.off = d_off;
-  pv.n = n_ind;
-
-  const double pairs = (double)(total - n_ind), nd = a.neg ? 2.0 : 1.0;
-  const double ev_bytes = eval_bytes(ctx, mode, total, n_ind, a.neg);
-  const double ev_ops = pairs * (double)ctx->R * nd, ev_units = (double)n_ind * (double)ctx->R;
-  if (mode == EBIC_MODE_PLAIN) {
-    EBIC_CHECK_CUDA(ctx, cudaMemsetAsync(a.rows_pos, 0, (size_t)n_ind * 3 * 4, s));
-    cudaEvent_t ev = prof_begin(ctx);
-    for (int32_t i = 0; i < n_ind; ++i)
-      EBIC_CHECK_CUDA(ctx, launch_eval_plain(a, d_cols + h_off[i], h_off[i + 1] - h_off[i], i, s));
-    prof_end(ctx, ev, EBIC_KERNEL_EVAL, (double)total * (double)ctx->R_pad * 4.0, ev_ops,
-             ev_units);
-    prof_count(ctx, EBIC_KERNEL_EVAL, n_ind);
-    EBIC_CHECK_CUDA(ctx, launch_fitness(a, pv, s));
-    prof_count(ctx, -1, 1);
-  } else {
-    cudaEvent_t e0 = prof_event(ctx), e1 = prof_event(ctx);
-    EBIC_CHECK_CUDA(ctx, launch_eval(mode, a, pv, ctx->num_sms, s, e0, e1));
-    prof_push(ctx, e0, e1, EBIC_KERNEL_EVAL, ev_bytes, ev_ops, ev_units);
+  const size_t n = (size_t)n_ind;
+  EBIC_CHECK_CUDA(ctx, ctx->ev_out.ensure(n * 3 * sizeof(int32_t), s));
+  EBIC_CHECK_CUDA(ctx, ctx->ev_fit.ensure(n * sizeof(uint64_t), s));
+  int32_t *counts = ctx->ev_out.as<int32_t>(), *sw = ctx->d_work.as<int32_t>();
+  EvalArgs a{};
+  auto set_args = [&]() {  // (the matrix's fields change with what is built)
+    a = eval_args_for(ctx);
+    a.neg = p->neg_trends;
+    a.non_strict = p->non_strict;
+    a.last_kept = p->last_kept;
+    a.rnum = p->ratio_num;
+    a.rden = p->ratio_den;
+    a.min_rows = p->min_rows;
+    a.col_cap = p->col_cap;
+    a.rows_pos = counts;
+    a.rows_neg = counts + n;
+    a.rows_any = counts + 2 * n;
+    a.fitness = ctx->ev_fit.as<uint64_t>();
+    a.work = sw + kSweepWork;
+  };
+  if (p->mode == EBIC_MODE_PLAIN) {
+    set_args();
+    return eval_population_plain(ctx, col_idx, offsets, n_ind, a, outs);
+  }
+  volatile int32_t *status = reinterpret_cast<volatile int32_t *>(ctx->pin);
+  int32_t *status_d = reinterpret_cast<int32_t *>(ctx->pin);
+  unsigned char *pin_in = ctx->pin + kPinStatus, *pin_out = pin_in + kPinIn;
+  const int32_t *src_cols = col_idx, *src_off = offsets;  // what the first launch reads
+  const int32_t *d_cols = col_idx, *d_off = offsets;      // what the evaluation reads
+  int32_t *copy_cols = nullptr, *copy_off = nullptr;
+  int64_t total = 0;
+  bool known = false;
+  if (!dev_cols) {
+    // the offsets are checked here (they size the copy), the columns by the first launch
+    for (int32_t i = 0; i < n_ind; ++i) {
+      const int64_t L = (int64_t)offsets[i + 1] - offsets[i];
+      if (offsets[i] < 0 || L < 2 || L > EBIC_MAX_LEN)
+        return ebic_fail(ctx, EBIC_EINVAL, "individual " + std::to_string(i) +
+                                               ": length must be in [2, 64]");
+    }
+    total = (int64_t)offsets[n_ind] - offsets[0];
+    known = true;
+    const size_t nc = (size_t)offsets[n_ind] * 4, no = (n + 1) * 4;
+    EBIC_CHECK_CUDA(ctx, ctx->ev_cols.ensure(nc + 16, s));
+    EBIC_CHECK_CUDA(ctx, ctx->ev_off.ensure(no, s));
+    d_cols = ctx->ev_cols.as<int32_t>();
+    d_off = ctx->ev_off.as<int32_t>();
+    if (nc + no <= kPinIn) {
+      memcpy(pin_in, offsets, no);
+      memcpy(pin_in + no, col_idx, nc);
+      src_off = reinterpret_cast<const int32_t *>(pin_in);
+      src_cols = reinterpret_cast<const int32_t *>(pin_in + no);
+      copy_cols = ctx->ev_cols.as<int32_t>();
+      copy_off = ctx->ev_off.as<int32_t>();
+    } else {
+      EBIC_CHECK_CUDA(ctx, cudaMemcpyAsync(ctx->ev_cols.p, col_idx, nc, cudaMemcpyHostToDevice, s));
+      EBIC_CHECK_CUDA(ctx, cudaMemcpyAsync(ctx->ev_off.p, offsets, no, cudaMemcpyHostToDevice, s));
+      src_cols = d_cols;
+      src_off = d_off;
+    }
+  }
+  const bool wait_len =
+      !known && mode_needs_mean_len(ctx, p->mode, n_ind, 1, p->last_kept);
+  // (the algorithmic work, for the kernel statistics, needs the total too)
+  const bool want_ends = !known && (wait_len || ctx->prof);
+  status[4] = 0;
+  EBIC_CHECK_CUDA(ctx, launch_sweep_prepare(src_cols, src_off, n_ind, ctx->C, counts, sw,
+                                            copy_cols, copy_off,
+                                            want_ends ? status_d + 2 : nullptr, s));
+  prof_count(ctx, -1, 1);
+  if (want_ends) {
+    EBIC_CHECK_CUDA(ctx, cudaStreamSynchronize(s));
+    if (status[4]) {
+      EBIC_CHECK_CUDA(ctx, cudaMemsetAsync(sw, 0, 64, s));
+      EBIC_CHECK_CUDA(ctx, cudaStreamSynchronize(s));
+      return ebic_fail(ctx, EBIC_EINVAL, "invalid chromosome in the population");
+    }
+    total = (int64_t)status[3] - status[2];
+    known = true;
+  }
+  const double mean_len = known ? (double)total / n_ind : 2.0;  // (2: any length will do)
+  const int mode = choose_mode(ctx, p->mode, n_ind, mean_len, 1, p->last_kept);
+  // from here on a failure leaves the check's word to be cleared
+  auto evaluate = [&]() -> int {
+    if (mode == EBIC_MODE_BITMAP && !ctx->bitmap_ok) EBIC_TRY(ebic_build_bitmap(ctx));
+    if (direct_form_used(ctx, mode, p)) EBIC_TRY(ensure_codes(ctx));
+    set_args();
+    a.seg_passes =
+        ctx->tuned ? (mode == EBIC_MODE_BITMAP ? ctx->seg_bitmap
+                                               : (mode == EBIC_MODE_DIRECT ? ctx->seg_direct : 0))
+                   : 0;
+    a.ipw = p->ipw > 0 ? p->ipw : (ctx->tuned && mode == EBIC_MODE_BITMAP ? ctx->ipw_bitmap : 1);
+    PopView pv{};
+    pv.cols = d_cols;
+    pv.off = d_off;
+    pv.n = n_ind;
+    pv.stop = sw + kSweepErr;
+    const double pairs = (double)(total - n_ind), nd = a.neg ? 2.0 : 1.0;
+    cudaEvent_t e0 = prof_begin(ctx);
+    EBIC_CHECK_CUDA(ctx, launch_eval_kernel(mode, a, pv, ctx->num_sms, s, true));
+    prof_end(ctx, e0, EBIC_KERNEL_EVAL, eval_bytes(ctx, mode, total, n_ind, a.neg),
+             pairs * (double)ctx->R * nd, (double)n_ind * (double)ctx->R);
     prof_count(ctx, EBIC_KERNEL_EVAL, 1);
+    // device outputs are written in place; host outputs come through the pinned block, or from
+    // the device buffers by copies once the call is known to be good
+    SweepOut o{};
+    bool copy_out = false;
+    const bool fits = n * 20 <= kPinOut;
+    for (int k = 0; k < 3; ++k) {
+      if (!outs[k]) continue;
+      if (dev_out[k])
+        o.rows[k] = static_cast<int32_t *>(outs[k]);
+      else if (fits)
+        o.rows[k] = reinterpret_cast<int32_t *>(pin_out + n * 8) + k * n;
+      else
+        copy_out = true;
+    }
+    if (fitness) {
+      copy_out |= !dev_out[3] && !fits;
+      o.fitness = dev_out[3] ? fitness
+                  : fits     ? reinterpret_cast<uint64_t *>(pin_out)
+                             : ctx->ev_fit.as<uint64_t>();
+    }
+    EBIC_CHECK_CUDA(ctx, launch_sweep_finish(a, pv, sw, o, status_d, s));
     prof_count(ctx, -1, 1);
+    EBIC_CHECK_CUDA(ctx, cudaStreamSynchronize(s));
+    prof_collect(ctx);
+    if (status[0]) return ebic_fail(ctx, EBIC_EINVAL, "invalid chromosome in the population");
+    for (int k = 0; k < 3; ++k)
+      if (outs[k] && !dev_out[k] && fits)
+        memcpy(outs[k], pin_out + n * 8 + (size_t)k * n * 4, n * 4);
+    if (fitness && !dev_out[3] && fits) memcpy(fitness, pin_out, n * 8);
+    if (copy_out) {
+      for (int k = 0; k < 3; ++k)
+        if (outs[k] && !dev_out[k])
+          EBIC_CHECK_CUDA(ctx, cudaMemcpyAsync(outs[k], counts + (size_t)k * n, n * 4,
+                                               cudaMemcpyDeviceToHost, s));
+      if (fitness && !dev_out[3])
+        EBIC_CHECK_CUDA(ctx, cudaMemcpyAsync(fitness, ctx->ev_fit.p, n * 8,
+                                             cudaMemcpyDeviceToHost, s));
+      EBIC_CHECK_CUDA(ctx, cudaStreamSynchronize(s));
+    }
+    if (status[1]) {
+      cudaMemset(ctx->d_kerr.p, 0, 4);
+      return ebic_fail(ctx, EBIC_ETIMEOUT, "a bounded device wait expired in the evaluation");
+    }
+    return EBIC_OK;
+  };
+  status[0] = status[1] = 0;
+  const int st = evaluate();
+  if (st != EBIC_OK) {  // (a call that stopped half way may leave the words set)
+    cudaMemsetAsync(sw, 0, 64, s);
+    cudaStreamSynchronize(s);
+    cudaGetLastError();
   }
-  int32_t *dsts[3] = {rows_pos, rows_neg, rows_any};
-  for (int k = 0; k < 3; ++k)
-    if (dsts[k])
-      EBIC_CHECK_CUDA(ctx, cudaMemcpyAsync(dsts[k], a.rows_pos + (size_t)k * n_ind,
-                                           (size_t)n_ind * 4, cudaMemcpyDefault, s));
-  if (fitness)
-    EBIC_CHECK_CUDA(ctx, cudaMemcpyAsync(fitness, a.fitness, (size_t)n_ind * 8,
-                                         cudaMemcpyDefault, s));
-  int32_t kerr = 0;
-  EBIC_CHECK_CUDA(ctx, cudaMemcpyAsync(&kerr, ctx->d_kerr.p, 4, cudaMemcpyDeviceToHost, s));
-  EBIC_CHECK_CUDA(ctx, cudaStreamSynchronize(s));
-  prof_collect(ctx);
-  if (kerr) {
-    cudaMemset(ctx->d_kerr.p, 0, 4);
-    return ebic_fail(ctx, EBIC_ETIMEOUT, "a bounded device wait expired in the evaluation");
-  }
-  return EBIC_OK;
+  return st;
 }
 
 }  // extern "C"
@@ -825,15 +1030,25 @@ int choose_mode(const ebic_ctx *ctx, int requested, int64_t n_ind, double mean_l
   if (ctx->tuned) return ctx->tuned_mode;
   if (ctx->bitmap_ok) return EBIC_MODE_BITMAP;
   const double Wst = (double)ctx->Wst, C = (double)ctx->C;
+  if (!cost_model_prefers_bitmap((double)ctx->R_pad, C, ctx->code_bytes, (double)n_ind, mean_len,
+                                 (double)expected_sweeps))
+    return EBIC_MODE_DIRECT;
+  // (the query of the free memory is slow: only where a bitmap is wanted)
   const double bitmap_bytes = C * C * Wst * 4.0;
   size_t free_b = 0, total_b = 0;
   if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
     cudaGetLastError();
     free_b = 0;
   }
-  if (bitmap_bytes > 0.5 * (double)free_b) return EBIC_MODE_DIRECT;
-  return cost_model_prefers_bitmap((double)ctx->R_pad, C, ctx->code_bytes, (double)n_ind,
-                                   mean_len, (double)expected_sweeps)
-             ? EBIC_MODE_BITMAP
-             : EBIC_MODE_DIRECT;
+  return bitmap_bytes > 0.5 * (double)free_b ? EBIC_MODE_DIRECT : EBIC_MODE_BITMAP;
+}
+
+bool mode_needs_mean_len(const ebic_ctx *ctx, int requested, int64_t n_ind, int expected_sweeps,
+                         int last_kept) {
+  if (requested != EBIC_MODE_AUTO || last_kept || ctx->tuned || ctx->bitmap_ok) return false;
+  auto prefers = [&](double mean_len) {
+    return cost_model_prefers_bitmap((double)ctx->R_pad, (double)ctx->C, ctx->code_bytes,
+                                     (double)n_ind, mean_len, (double)expected_sweeps);
+  };
+  return prefers(2.0) != prefers((double)std::min<int32_t>(EBIC_MAX_LEN, ctx->C));
 }

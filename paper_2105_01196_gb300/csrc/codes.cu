@@ -422,16 +422,6 @@ __global__ void __launch_bounds__(kThreads, 4) k_eval_codes(EvalArgs a, PopView 
   }
 }
 
-template <class K>
-int blocks_per_sm(K kern, size_t smem) {
-  int nb = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, kThreads, smem) != cudaSuccess) {
-    cudaGetLastError();
-    nb = 1;
-  }
-  return nb < 1 ? 1 : nb;
-}
-
 template <class... Args>
 cudaError_t launch_pdl_opt(void (*kern)(Args...), dim3 grid, dim3 block, cudaStream_t s,
                            bool pdl, Args... args) {
@@ -529,7 +519,7 @@ cudaError_t launch_rank_epl(const uint32_t *keys, int64_t R_pad, int32_t C, T *c
   }
   const int64_t t_begin = r_begin / kRankRows, t_end = r_end / kRankRows;
   const int64_t grid = std::min<int64_t>(
-      t_end - t_begin, (int64_t)num_sms * blocks_per_sm(k_rank_codes<T, EPL>, smem));
+      t_end - t_begin, (int64_t)num_sms * resident_blocks((const void *)k_rank_codes<T, EPL>, kThreads, smem));
   k_rank_codes<T, EPL><<<(unsigned)grid, kThreads, smem, s>>>(keys, R_pad, C, S, codes,
                                                                 t_begin, t_end);
   return cudaGetLastError();
@@ -583,7 +573,7 @@ cudaError_t launch_eval_codes(const EvalArgs &a0, const PopView &pv, int num_sms
       k_eval_codes<2, true, true, false>,   k_eval_codes<2, true, true, true>};
   const Kernel kern = table[(W == 2 ? 8 : 0) + (a.neg ? 4 : 0) + (a.non_strict ? 2 : 0) +
                             (a.last_kept ? 1 : 0)];
-  const int bps = blocks_per_sm(kern, 0);
+  const int bps = resident_blocks((const void *)kern, kThreads, 0);
   const int64_t warps = (int64_t)num_sms * bps * kWarps;
   // Segments: the autotuner's size when it set one, else enough work items for ~8 per
   // resident warp; at most 2^30 items in total.

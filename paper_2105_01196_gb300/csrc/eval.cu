@@ -66,6 +66,80 @@ __global__ void k_validate_csr(const int32_t *__restrict__ cols, const int32_t *
   if (csr_bad(cols, off[i], off[i + 1], C, lane, &c0, &c1) && lane == 0) atomicOr(err, 2);
 }
 
+// The first launch of a population evaluation: checks the population (a warp per individual; a bad
+// one sets sw[kSweepErr], and the evaluation and the output then do nothing), clears the count
+// accumulators and the work counter, and copies a population read from pinned host memory to the
+// device (dcols, doff; null when it is on the device already).  ends (pinned host memory, or
+// null) receives the first and the last offset, and 1 in its third word for a bad population.
+// It stands for a check and four clears as separate operations, each of which cost a launch.
+__global__ void __launch_bounds__(kThreads) k_sweep_prepare(const int32_t *__restrict__ cols,
+                                                            const int32_t *__restrict__ off,
+                                                            int32_t n, int32_t C,
+                                                            int32_t *__restrict__ counts,
+                                                            int32_t *__restrict__ sw,
+                                                            int32_t *__restrict__ dcols,
+                                                            int32_t *__restrict__ doff,
+                                                            int32_t *__restrict__ ends) {
+  const int lane = threadIdx.x & 31;
+  const int64_t i = (int64_t)blockIdx.x * kWarps + (threadIdx.x >> 5);
+  if (i == 0 && lane == 0) {
+    sw[kSweepWork] = 0;
+    if (ends) {
+      ends[0] = off[0];
+      ends[1] = off[n];
+    }
+  }
+  if (i >= n) return;  // (whole warps)
+  if (lane < 3) counts[(int64_t)lane * n + i] = 0;
+  const int s = off[i], e = off[i + 1];
+  int c0, c1;
+  const bool bad = csr_bad(cols, s, e, C, lane, &c0, &c1);
+  if (bad && lane == 0) {
+    atomicOr(sw + kSweepErr, 2);
+    if (ends) ends[2] = 1;
+  }
+  if (dcols && !bad) {
+    if (lane < e - s) dcols[s + lane] = c0;
+    if (lane + 32 < e - s) dcols[s + 32 + lane] = c1;
+    if (lane == 0) {
+      doff[i] = s;
+      if (i == n - 1) doff[n] = e;
+    }
+  }
+}
+
+// The last launch of a population evaluation: fitness, the outputs (caller's device memory, pinned
+// host memory, or the accumulators themselves; null: not wanted), and from the last block to
+// finish the state of the call (status, pinned host memory: the error word of the check, the
+// kernels' error word), with the words reset for the next call.
+__global__ void k_sweep_finish(EvalArgs a, PopView pv, int32_t *__restrict__ sw, SweepOut o,
+                               int32_t *status) {
+  wait_prior_grid();
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int err = sw[kSweepErr];
+  if (i < pv.n && !err) {
+    const int rp = a.rows_pos[i], rn = a.rows_neg[i], ra = a.rows_any[i];
+    if (o.rows[0]) o.rows[0][i] = rp;
+    if (o.rows[1]) o.rows[1][i] = rn;
+    if (o.rows[2]) o.rows[2][i] = ra;
+    if (o.fitness) {
+      const int L = pv_len(pv, i);
+      const int sh = L < a.col_cap ? L : a.col_cap;
+      o.fitness[i] = ra < a.min_rows ? 0ull : ((uint64_t)ra << sh);
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();  // (this block has read the error word)
+    if (atomicAdd(sw + kSweepDone, 1) == (int)gridDim.x - 1) {
+      status[0] = err;
+      status[1] = *a.err;
+      sw[kSweepErr] = 0;
+      sw[kSweepDone] = 0;
+    }
+  }
+}
+
 // ------------------------------------------------------------------------------- direct form
 
 // NS / LK: the pair-test variants of trend.cuh (ties count for both directions / compare with
@@ -357,6 +431,7 @@ __device__ __forceinline__ void bitmap_staged_items(const EvalArgs &a, const Pop
       if (pv.off) {
         myst = pv.off[i];
         myL = pv.off[i + 1] - myst;
+        if (items::stopped(pv)) myL = 0;  // (a bad population's columns are not read)
       } else {
         myst = i * pv.stride;
         myL = pv.len[i];
@@ -838,27 +913,12 @@ __global__ void k_fitness(EvalArgs a, PopView pv) {
   a.fitness[i] = (dead || ra < a.min_rows) ? 0ull : ((uint64_t)ra << sh);
 }
 
-int blocks_per_sm_for(const void *kernel, size_t smem) {
-  int nb = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, kThreads, smem) != cudaSuccess) {
-    cudaGetLastError();
-    nb = 1;
-  }
-  return nb < 1 ? 1 : nb;
-}
-
 }  // namespace
 
 cudaError_t launch_validate_csr(const int32_t *cols, const int32_t *off, int32_t n, int32_t C,
                                 int32_t *err, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   k_validate_csr<<<(unsigned)((n + 7) / 8), 256, 0, s>>>(cols, off, n, C, err);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_fitness(const EvalArgs &a, const PopView &pv, cudaStream_t s) {
-  if (pv.n <= 0 || !a.fitness) return cudaSuccess;
-  k_fitness<<<(pv.n + 255) / 256, 256, 0, s>>>(a, pv);
   return cudaGetLastError();
 }
 
@@ -882,6 +942,26 @@ cudaError_t launch_maybe_pdl(void (*kern)(Args...), dim3 grid, dim3 block, size_
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
+cudaError_t launch_sweep_prepare(const int32_t *cols, const int32_t *off, int32_t n, int32_t C,
+                                 int32_t *counts, int32_t *sw, int32_t *dcols, int32_t *doff,
+                                 int32_t *ends, cudaStream_t s) {
+  k_sweep_prepare<<<(unsigned)(((int64_t)n + kWarps - 1) / kWarps), kThreads, 0, s>>>(
+      cols, off, n, C, counts, sw, dcols, doff, ends);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_sweep_finish(const EvalArgs &a, const PopView &pv, int32_t *sw,
+                                const SweepOut &o, int32_t *status, cudaStream_t s) {
+  return launch_maybe_pdl(k_sweep_finish, dim3((unsigned)((pv.n + 255) / 256)), dim3(256), 0, s,
+                          true, a, pv, sw, o, status);
+}
+
+cudaError_t launch_fitness(const EvalArgs &a, const PopView &pv, cudaStream_t s) {
+  if (pv.n <= 0 || !a.fitness) return cudaSuccess;
+  k_fitness<<<(pv.n + 255) / 256, 256, 0, s>>>(a, pv);
+  return cudaGetLastError();
 }
 
 using EvalKernel = void (*)(EvalArgs, PopView);
@@ -952,7 +1032,7 @@ cudaError_t launch_eval_kernel(int mode, const EvalArgs &a0, const PopView &pv, 
     const cudaError_t e = prepare_bitmap_eval();
     if (e != cudaSuccess) return e;
   }
-  const int bps = blocks_per_sm_for((const void *)kern, smem);
+  const int bps = resident_blocks((const void *)kern, kThreads, smem);
   const int64_t warps = (int64_t)num_sms * bps * kWarps;
   const int64_t n_grp = ((int64_t)pv.n + a.ipw - 1) / a.ipw;
   // Segments: the autotuner's size when it set one, else enough work items for ~8 per

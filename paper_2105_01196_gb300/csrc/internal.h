@@ -97,6 +97,17 @@ struct PopView {
   const int32_t *list_n;
 };
 
+// Words of a context's evaluation state on the device (ebic_ctx::d_work): the evaluation kernels'
+// work counter, and for ebic_eval_population the error word of the population check (0 between
+// calls) and the number of finished blocks of the last launch (0 between calls).
+enum { kSweepWork = 0, kSweepErr = 1, kSweepDone = 2 };
+
+// Where the outputs of a population evaluation go (null: not wanted).
+struct SweepOut {
+  int32_t *rows[3];
+  uint64_t *fitness;
+};
+
 // Matrix geometry and the outputs of one evaluation sweep.
 struct EvalArgs {
   const uint32_t *keys;    // [C][R_pad] order keys
@@ -210,6 +221,9 @@ struct ebic_ctx {
 
   // scratch for single evaluations
   DevBuf d_err, d_work, ev_cols, ev_off, ev_out, ev_fit;
+  // pinned host memory the device reads and writes: the state of a call (kPinStatus words), then
+  // kPinIn bytes of a small host population and kPinOut bytes of its results (abi.cu)
+  unsigned char *pin = nullptr;
 
   // staged direct form of the loaded matrix, and the kernels' error word
   DirectTma dtma;
@@ -311,6 +325,12 @@ cudaError_t launch_build_bitmap_planes(const uint32_t *planes, int32_t C, int64_
 // eval.cu
 cudaError_t launch_validate_csr(const int32_t *cols, const int32_t *off, int32_t n, int32_t C,
                                 int32_t *err, cudaStream_t s);
+// The first and the last launch of ebic_eval_population (sw: ebic_ctx::d_work, see kSweepErr).
+cudaError_t launch_sweep_prepare(const int32_t *cols, const int32_t *off, int32_t n, int32_t C,
+                                 int32_t *counts, int32_t *sw, int32_t *dcols, int32_t *doff,
+                                 int32_t *ends, cudaStream_t s);
+cudaError_t launch_sweep_finish(const EvalArgs &a, const PopView &pv, int32_t *sw,
+                                const SweepOut &o, int32_t *status, cudaStream_t s);
 // Zeroes the outputs and the work counter, evaluates, writes fitness.  When ev0/ev1 are not
 // null they are recorded on `s` immediately before and after the evaluation kernel.
 cudaError_t launch_eval(int mode, const EvalArgs &a, const PopView &pv, int num_sms,
@@ -325,11 +345,18 @@ cudaError_t launch_eval_plain(const EvalArgs &a, const int32_t *d_cols, int32_t 
 cudaError_t launch_eval_kernel(int mode, const EvalArgs &a, const PopView &pv, int num_sms,
                                cudaStream_t s, bool pdl = false);
 cudaError_t launch_fitness(const EvalArgs &a, const PopView &pv, cudaStream_t s);
+// Blocks of `threads` threads and `smem` bytes of dynamic shared memory of `kernel` that one SM of
+// the current device holds at once (at least 1), asked of the runtime once per kernel and size.
+int resident_blocks(const void *kernel, int threads, size_t smem);
 // Raises the bitmap kernels' dynamic shared-memory limit on the current device (once per device;
 // done before any graph capture, with the bitmap's build).
 cudaError_t prepare_bitmap_eval();
 int choose_mode(const ebic_ctx *ctx, int requested, int64_t n_ind, double mean_len,
                 int expected_sweeps, int last_kept);
+// Whether choose_mode gives the same answer whatever the mean length (its cost model is linear in
+// it, so the two ends of the range tell).
+bool mode_needs_mean_len(const ebic_ctx *ctx, int requested, int64_t n_ind, int expected_sweeps,
+                         int last_kept);
 // The cost model behind AUTO without tuning (and the job server's footprint): whether building
 // the pair bitmap and running `sweeps` bitmap sweeps is expected to beat `sweeps` direct sweeps.
 // Costs are in units of about 1.3 ns on GB300, measured per unit on the tie-heavy workload

@@ -88,8 +88,8 @@ __device__ __forceinline__ int count(const PopView &pv) {
 // Slot of the launch's individual i.
 __device__ __forceinline__ int slot(const PopView &pv, int i) { return pv.list ? pv.list[i] : i; }
 
-// Whether the run has stopped (the flag is read beside an item's first loads, and tested before
-// the item's first store).
+// Whether the run has stopped, or the caller's population is bad (the flag is read beside an item's
+// first loads, and tested before the item's first store).
 __device__ __forceinline__ bool stopped(const PopView &pv) { return pv.stop && *pv.stop; }
 
 struct Meta {
@@ -106,6 +106,7 @@ __device__ __forceinline__ Meta load_meta(const PopView &pv, int i, int lane) {
   if (pv.off) {
     m.st = pv.off[i];
     m.L = pv.off[i + 1] - m.st;
+    if (stopped(pv)) m.L = 0;  // (a bad population's columns are not read)
   } else {
     m.st = i * pv.stride;
     m.L = pv.len[i];
