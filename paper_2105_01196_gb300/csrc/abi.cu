@@ -432,6 +432,7 @@ int ebic_create(ebic_ctx **out, int32_t device, void *cuda_stream) {
     ctx->own_stream = true;
   }
   if (ctx->d_err.ensure(64, ctx->stream) != cudaSuccess ||
+      ctx->d_ties.ensure(64, ctx->stream) != cudaSuccess ||
       ctx->d_work.ensure(64, ctx->stream) != cudaSuccess ||
       ctx->d_kerr.ensure(64, ctx->stream) != cudaSuccess ||
       cudaMemset(ctx->d_kerr.p, 0, 64) != cudaSuccess ||
@@ -454,7 +455,7 @@ int ebic_destroy(ebic_ctx *ctx) {
   ctx->gen = nullptr;
   DevBuf *bufs[] = {&ctx->keys, &ctx->bitmap, &ctx->stage_x, &ctx->d_err, &ctx->d_work,
                     &ctx->ev_cols, &ctx->ev_off, &ctx->ev_out, &ctx->ev_fit, &ctx->d_kerr,
-                    &ctx->codes, &ctx->planes, &ctx->pair_cnt};
+                    &ctx->codes, &ctx->planes, &ctx->pair_cnt, &ctx->d_ties};
   for (DevBuf *b : bufs) b->release();
   give_pin(ctx->pin);
   prof_collect(ctx);
@@ -567,6 +568,7 @@ int load_matrix_segmented(ebic_ctx *ctx, const float *x, int64_t rows, int32_t c
                                                     ctx->pair_cnt.as<unsigned long long>(),
                                                     ctx->num_sms, s));
     prof_count(ctx, EBIC_KERNEL_BITMAP_BUILD, 1);
+    ctx->tie_state = -1;
   }
   int32_t herr = 0;
   EBIC_CHECK_CUDA(ctx, cudaMemcpyAsync(&herr, ctx->d_err.p, sizeof(int32_t),
@@ -691,6 +693,7 @@ int ebic_build_bitmap(ebic_ctx *ctx) {
   prof_end(ctx, ev, EBIC_KERNEL_BITMAP_BUILD, (double)bytes,
            (double)ctx->C * ctx->C * (double)ctx->R, 0.0);
   prof_count(ctx, EBIC_KERNEL_BITMAP_BUILD, 1);
+  ctx->tie_state = -1;
   if (ctx->prof) {  // (later work on the stream is ordered after the build anyway)
     EBIC_CHECK_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     prof_collect(ctx);
@@ -880,6 +883,9 @@ int ebic_eval_population(ebic_ctx *ctx, const int32_t *col_idx, const int32_t *o
   // from here on a failure leaves the check's word to be cleared
   auto evaluate = [&]() -> int {
     if (mode == EBIC_MODE_BITMAP && !ctx->bitmap_ok) EBIC_TRY(ebic_build_bitmap(ctx));
+    if (mode == EBIC_MODE_BITMAP && p->neg_trends && p->ratio_num < p->ratio_den &&
+        eval_args_for(ctx).stage_bitmap)
+      EBIC_TRY(ensure_tie_state(ctx));
     if (direct_form_used(ctx, mode, p)) EBIC_TRY(ensure_codes(ctx));
     set_args();
     a.seg_passes =
@@ -955,6 +961,26 @@ int ebic_eval_population(ebic_ctx *ctx, const int32_t *col_idx, const int32_t *o
 
 }  // extern "C"
 
+// Individuals without ties are looked for where at most 1/8 of the column pairs are tied: an
+// individual of np pairs has none with probability (7/8)^np or more, and the look costs every item
+// a round trip to the pair counts.
+int ensure_tie_state(ebic_ctx *ctx) {
+  if (!ctx->bitmap_ok || !ctx->pair_cnt_ok) {
+    ctx->tie_state = 0;
+    return EBIC_OK;
+  }
+  if (ctx->tie_state >= 0) return EBIC_OK;
+  EBIC_CHECK_CUDA(ctx, launch_count_tied(ctx->pair_cnt.as<unsigned long long>(), ctx->C, ctx->R,
+                                         ctx->d_ties.as<int32_t>(), ctx->stream));
+  prof_count(ctx, -1, 1);
+  volatile int32_t *n = reinterpret_cast<volatile int32_t *>(ctx->pin) + 8;
+  EBIC_CHECK_CUDA(ctx, cudaMemcpyAsync(ctx->pin + 32, ctx->d_ties.p, sizeof(int32_t),
+                                       cudaMemcpyDeviceToHost, ctx->stream));
+  EBIC_CHECK_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+  ctx->tie_state = 16 * (int64_t)*n <= (int64_t)ctx->C * (ctx->C - 1);
+  return EBIC_OK;
+}
+
 int ensure_codes(ebic_ctx *ctx) {
   if (!ctx->code_bytes || ctx->codes_ready) return EBIC_OK;
   const int64_t S = ctx->code_stride, C = ctx->C;
@@ -990,6 +1016,8 @@ EvalArgs eval_args_for(const ebic_ctx *ctx) {
   EvalArgs a{};
   a.keys = ctx->keys.as<uint32_t>();
   a.bitmap = ctx->bitmap_ok ? ctx->bitmap.as<uint32_t>() : nullptr;
+  a.pair_cnt = ctx->bitmap_ok && ctx->pair_cnt_ok ? ctx->pair_cnt.as<unsigned long long>() : nullptr;
+  a.tie_free = a.pair_cnt && ctx->tie_state == 1;
   a.R = ctx->R;
   a.R_pad = ctx->R_pad;
   a.Wst = ctx->Gst;

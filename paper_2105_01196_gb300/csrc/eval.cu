@@ -874,6 +874,253 @@ __global__ void __launch_bounds__(kThreads, 2) k_eval_bitmap(EvalArgs a, PopView
   }
 }
 
+// Staged form for matrices with few ties (a.tie_free; both directions; the bitmap exceeds L2).
+// Where no pair of an individual has ties in any row, a pair that does not rise falls, so the
+// falling pairs' words are the complements of the rising ones' and their count is np - inc: the
+// rows of one direction give both, half the bytes and half the counters.  An individual with a
+// tied pair has its rows of the two directions counted one after the other.
+// A unit is up to eight rows of one direction of one pass (512 bytes a row; short exact
+// chromosomes: the next eight rows of the item, whatever their pass), copied by cp.async into a
+// ring of three units per warp; each lane reads back only the bytes it copied (a lane past Wst,
+// which copies nothing, reads what the ring held; its words are masked out of the counts).  An
+// individual of one pair is scored from the pair counts alone.
+constexpr int kUnit = 8;  // rows per unit
+constexpr int kRing = 3;  // units in flight per warp
+constexpr int kRingWords = kRing * kUnit * kPassWords;
+// (the ring, then the word offsets of an individual's rows in each direction)
+constexpr size_t kRingSmem = (size_t)kWarps * (kRingWords * 4 + 2 * EBIC_MAX_LEN * 8);
+
+// Adds eight inputs: four full adders into the ones, two into the twos, one into the fours, a
+// ripple from the eights.
+__device__ __forceinline__ void cnt_add8(Cnt6 &c, uint32_t x0, uint32_t x1, uint32_t x2,
+                                         uint32_t x3, uint32_t x4, uint32_t x5, uint32_t x6,
+                                         uint32_t x7) {
+  const uint32_t tA = maj3(c.b0, x0, x1);
+  c.b0 ^= x0 ^ x1;
+  const uint32_t tB = maj3(c.b0, x2, x3);
+  c.b0 ^= x2 ^ x3;
+  const uint32_t tC = maj3(c.b0, x4, x5);
+  c.b0 ^= x4 ^ x5;
+  const uint32_t tD = maj3(c.b0, x6, x7);
+  c.b0 ^= x6 ^ x7;
+  const uint32_t fA = maj3(c.b1, tA, tB);
+  c.b1 ^= tA ^ tB;
+  const uint32_t fB = maj3(c.b1, tC, tD);
+  c.b1 ^= tC ^ tD;
+  uint32_t k = maj3(c.b2, fA, fB);
+  c.b2 ^= fA ^ fB;
+  uint32_t t = c.b3 & k;
+  c.b3 ^= k;
+  k = t;
+  t = c.b4 & k;
+  c.b4 ^= k;
+  c.b5 ^= t;
+}
+
+template <bool NS>
+__global__ void __launch_bounds__(kThreads, 2) k_eval_bitmap_one(EvalArgs a, PopView pv) {
+  extern __shared__ __align__(128) uint32_t s_ring[];
+  wait_prior_grid();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t *ring = s_ring + warp * kRingWords + lane * 4;  // unit u's row j: + (8 u + j) * 128
+  int64_t *up = reinterpret_cast<int64_t *>(s_ring + kWarps * kRingWords) + warp * 2 * EBIC_MAX_LEN;
+  int64_t *down = up + EBIC_MAX_LEN;
+  const int64_t Wst = a.Wst;
+  const int64_t passes_total = (Wst + kPassWords - 1) / kPassWords;
+  const int32_t n_ind = items::count(pv);
+  const int32_t n_side = items::move_chunks(a), n_all = n_side + n_ind * a.n_seg;
+  const uint4 zero4 = make_uint4(0u, 0u, 0u, 0u);
+  const uint4 ones = make_uint4(kFull, kFull, kFull, kFull);
+  for (int q = items::first(); q < n_all; q = items::next(a.work, lane, q, n_all)) {
+    if (q < n_side) {
+      if (items::stopped(pv)) return;  // a stopped run changes nothing
+      items::move_chunk(a, q, lane);
+      continue;
+    }
+    const int seg = (q - n_side) / n_ind;  // segment-major
+    const int i = items::slot(pv, (q - n_side) - seg * n_ind);
+    const items::Meta m = items::load_meta(pv, i, lane);
+    if (items::stopped(pv)) return;  // (read with the item's loads; before any store)
+    if (m.dead || m.L < 2) continue;
+    const items::Insert ins = items::insert_start(pv, seg, m.h, lane);
+    const int L = m.L, np = L - 1;
+    // lane k: pairs k and 32 + k
+    const int n0 = __shfl_down_sync(kFull, m.c0, 1), n1 = __shfl_down_sync(kFull, m.c1, 1);
+    const int c32 = __shfl_sync(kFull, m.c1, 0);
+    const int d0 = lane < 31 ? n0 : c32, d1 = n1;  // (pair 63 does not exist: L <= 64)
+    bool tied = false;
+    if (lane < np) tied |= pair_has_ties(a.pair_cnt, a.C, m.c0, d0, a.R);
+    if (lane + 32 < np) tied |= pair_has_ties(a.pair_cnt, a.C, m.c1, d1, a.R);
+    __syncwarp();  // (the previous item's reads of the offsets are done)
+    up[lane] = ((int64_t)m.c0 * a.C + d0) * Wst;
+    down[lane] = ((int64_t)d0 * a.C + m.c0) * Wst;
+    up[lane + 32] = ((int64_t)m.c1 * a.C + d1) * Wst;
+    down[lane + 32] = ((int64_t)d1 * a.C + m.c1) * Wst;
+    const bool one = !__any_sync(kFull, tied);
+    if (np == 1) {  // (the pair's counts over every row, from the first segment's item)
+      if (seg == 0 && lane == 0) {
+        int ab, ba;
+        pair_counts(a.pair_cnt, a.C, m.c0, d0, &ab, &ba);
+        const int R = (int)a.R, rp = NS ? R - ba : ab, rn = NS ? R - ab : ba;
+        a.rows_pos[i] = rp;
+        a.rows_neg[i] = rn;
+        a.rows_any[i] = NS ? R : rp + rn;
+      }
+      items::insert_finish(pv, ins, m.h, i);
+      continue;
+    }
+    __syncwarp();
+    const int D = one ? 1 : 2;
+    const bool comp = NS && !one;  // ties hold both ways: complements of the opposite words
+    const int t = threshold(L, a.rnum, a.rden);
+    const int p0 = seg * a.seg_passes;
+    const int p1 = (int)min((int64_t)p0 + a.seg_passes, passes_total);
+    int cp = 0, cn = 0, ca = 0;
+    const int64_t *rows0 = comp ? down : up, *rows1 = comp ? up : down;
+    const uint32_t *Gl = a.bitmap + lane * 4;
+    // one pass's counts from its words of each direction
+    auto finish_pass = [&](int pass, uint4 pos, uint4 neg) {
+      const int64_t w = (int64_t)pass * kPassWords + lane * 4;
+      if ((w + 4) * 32 > a.R) {  // the rows past R (and lanes past Wst) follow no trend
+        const uint4 vm = make_uint4(valid_bits(w, a.R), valid_bits(w + 1, a.R),
+                                    valid_bits(w + 2, a.R), valid_bits(w + 3, a.R));
+        pos = and4(pos, vm);
+        neg = and4(neg, vm);
+      }
+      cp += popc4(pos);
+      cn += popc4(neg);
+      ca += popc4(make_uint4(pos.x | neg.x, pos.y | neg.y, pos.z | neg.z, pos.w | neg.w));
+    };
+    const int T = np * D;
+    if (t == np && T <= kUnit) {
+      // exact and short: the AND of a direction's words, whole passes of T rows per unit
+      const int ppu = kUnit / T, n_units = (p1 - p0 + ppu - 1) / ppu;
+      auto issue = [&](int u) {
+        int64_t w = (int64_t)(p0 + u * ppu) * kPassWords;
+        uint32_t *dst = ring + (u % kRing) * kUnit * kPassWords;
+        const int64_t w_end = min((int64_t)p1 * kPassWords, Wst - lane * 4);
+        for (int pp = 0; pp < ppu; ++pp, w += kPassWords)
+          for (int r = 0; r < T; ++r, dst += kPassWords)
+            if (w < w_end)  // (Wst % 4 == 0: a lane's 4 words all exist or not)
+              cp_async16(dst, Gl + (r < np ? rows0[r] : rows1[r - np]) + w);
+        cp_async_commit();  // (an empty group past the end keeps the waits' count)
+      };
+      // (one copy of each part: the code of the two loops has to stay in the instruction cache)
+#pragma unroll 1
+      for (int u = -kRing; u < n_units; ++u) {
+        if (u >= 0) {
+          cp_async_wait<kRing - 1>();
+          const uint32_t *st = ring + (u % kRing) * kUnit * kPassWords;
+          const int q0 = p0 + u * ppu, q1 = min(p1, q0 + ppu);
+          for (int pass = q0; pass < q1; ++pass) {
+            uint4 ap = ones, an = ones;  // (lanes past Wst are masked out in finish_pass)
+            for (int r = 0; r < np; ++r, st += kPassWords) {
+              uint4 v = *reinterpret_cast<const uint4 *>(st);
+              if (comp) v = not4(v);
+              ap = and4(ap, v);
+              if (one) an = and4(an, not4(v));
+            }
+            if (!one)
+              for (int r = 0; r < np; ++r, st += kPassWords) {
+                uint4 v = *reinterpret_cast<const uint4 *>(st);
+                if (comp) v = not4(v);
+                an = and4(an, v);
+              }
+            finish_pass(pass, ap, an);
+          }
+        }
+        issue(u + kRing);
+      }
+    } else {
+      // counting (an exact test of more rows counts too): a unit is the next eight rows (at
+      // most) of one direction of one pass
+      const int n_units = (p1 - p0) * D * ((np + kUnit - 1) / kUnit);
+      int iq = p0, id = 0, ik = 0;  // next unit to copy: pass, direction, first pair
+      const uint32_t *src = Gl + (int64_t)p0 * kPassWords;
+      int cq = p0, cd = 0, ck = 0;  // next unit to count
+      Cnt6 P[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) cnt_zero(P[j]);
+      uint4 pos = zero4;
+#pragma unroll 1
+      for (int u = -kRing; u < n_units; ++u) {
+        if (u >= 0) {
+          cp_async_wait<kRing - 1>();
+          const uint32_t *st = ring + (u % kRing) * kUnit * kPassWords;
+          uint4 v[kUnit];
+#pragma unroll
+          for (int j = 0; j < kUnit; ++j) {
+            v[j] = zero4;
+            if (ck + j < np) {
+              v[j] = *reinterpret_cast<const uint4 *>(st + j * kPassWords);
+              if (comp) v[j] = not4(v[j]);
+            }
+          }
+#define EBIC_ADD8(W, f)                                                                        \
+  cnt_add8(P[W], v[0].f, v[1].f, v[2].f, v[3].f, v[4].f, v[5].f, v[6].f, v[7].f)
+          EBIC_ADD8(0, x);
+          EBIC_ADD8(1, y);
+          EBIC_ADD8(2, z);
+          EBIC_ADD8(3, w);
+#undef EBIC_ADD8
+          ck += kUnit;
+          if (ck >= np) {  // the direction is complete
+            ck = 0;
+            uint4 ge = make_uint4(cnt_ge(P[0], t), cnt_ge(P[1], t), cnt_ge(P[2], t),
+                                  cnt_ge(P[3], t));
+            if (D == 2 && cd == 0) {
+              pos = ge;
+              cd = 1;
+            } else {
+              if (one) {  // np - inc >= t: not inc >= np - t + 1
+                const int tn = np - t + 1;
+                pos = ge;
+                ge = not4(make_uint4(cnt_ge(P[0], tn), cnt_ge(P[1], tn), cnt_ge(P[2], tn),
+                                     cnt_ge(P[3], tn)));
+              }
+              finish_pass(cq, pos, ge);
+              cd = 0;
+              ++cq;
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) cnt_zero(P[j]);
+          }
+        }
+        // unit u + kRing's copies into the slot just counted
+        if (iq < p1) {
+          uint32_t *dst = ring + ((u + kRing) % kRing) * kUnit * kPassWords;
+          const int64_t *rw = (id ? rows1 : rows0) + ik;
+          if ((int64_t)iq * kPassWords + lane * 4 < Wst) {
+#pragma unroll
+            for (int j = 0; j < kUnit; ++j)
+              if (ik + j < np) cp_async16(dst + j * kPassWords, src + rw[j]);
+          }
+          ik += kUnit;
+          if (ik >= np) {
+            ik = 0;
+            if (++id == D) {
+              id = 0;
+              ++iq;
+              src += kPassWords;
+            }
+          }
+        }
+        cp_async_commit();  // (an empty group past the end keeps the waits' count)
+      }
+    }
+    cp_async_wait<0>();  // (the empty groups; nothing of this item is in flight any more)
+    items::insert_finish(pv, ins, m.h, i);
+    cp = __reduce_add_sync(kFull, cp);
+    cn = __reduce_add_sync(kFull, cn);
+    ca = __reduce_add_sync(kFull, ca);
+    if (lane == 0) {
+      if (cp) atomicAdd(a.rows_pos + i, cp);
+      if (cn) atomicAdd(a.rows_neg + i, cn);
+      if (ca) atomicAdd(a.rows_any + i, ca);
+    }
+  }
+}
+
 // ------------------------------------------------------------------------------- plain form
 
 // One launch per individual; one row per thread; block counts by __syncthreads_count and one
@@ -998,6 +1245,10 @@ cudaError_t prepare_bitmap_eval() {
   std::lock_guard<std::mutex> lock(mu);
   if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
   if (attr_set[dev]) return cudaSuccess;
+  for (const EvalKernel k : {k_eval_bitmap_one<false>, k_eval_bitmap_one<true>})
+    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)kRingSmem)) != cudaSuccess)
+      return e;
   for (int k = 0; k < 8; ++k)
     if ((e = cudaFuncSetAttribute(bitmap_kernel(k & 2, k & 1, true, k & 4),
                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1025,9 +1276,16 @@ cudaError_t launch_eval_kernel(int mode, const EvalArgs &a0, const PopView &pv, 
   const bool stage = bitmap && a.stage_bitmap && a.rnum < a.rden;  // (ratio 1: all exact)
   // Individuals per work item: groups (ipw > 1) are a form of the staged kernel.
   a.ipw = stage ? std::max(1, std::min(a0.ipw, kMaxIpw)) : 1;
-  const EvalKernel kern = bitmap ? bitmap_kernel(a.neg, a.non_strict, stage, a.ipw > 1)
-                                 : direct_kernel(a.neg, a.non_strict, a.last_kept);
-  const size_t smem = stage ? kBitmapSmem : 0;
+  // One direction's words for both where the matrix has few ties (a.tie_free: see
+  // k_eval_bitmap_one); with ties, both directions' words beside each other, which then keep HBM
+  // busy with 16 warps per SM (a kernel counting the directions in turn took 0.67 ms at
+  // 60,000 x 1,000, against 0.55 ms).
+  const bool one = stage && a.neg && a.tie_free && a.pair_cnt && a.ipw == 1;
+  const EvalKernel kern =
+      one ? (a.non_strict ? k_eval_bitmap_one<true> : k_eval_bitmap_one<false>)
+      : bitmap ? bitmap_kernel(a.neg, a.non_strict, stage, a.ipw > 1)
+               : direct_kernel(a.neg, a.non_strict, a.last_kept);
+  const size_t smem = one ? kRingSmem : (stage ? kBitmapSmem : 0);
   if (stage) {
     const cudaError_t e = prepare_bitmap_eval();
     if (e != cudaSuccess) return e;
@@ -1036,8 +1294,11 @@ cudaError_t launch_eval_kernel(int mode, const EvalArgs &a0, const PopView &pv, 
   const int64_t warps = (int64_t)num_sms * bps * kWarps;
   const int64_t n_grp = ((int64_t)pv.n + a.ipw - 1) / a.ipw;
   // Segments: the autotuner's size when it set one, else enough work items for ~8 per
-  // resident warp; at most 2^30 items in total.
-  int64_t seg = a0.seg_passes > 0 ? a0.seg_passes : (n_grp * passes_total) / (8 * warps);
+  // resident warp (4 in the one-direction form, whose items are half as long: 4,096 individuals
+  // of 2-20 columns on 20,001 x 500 took 32 us against 44 us with 8, 8,192 of 2-3 columns on
+  // 60,000 x 1,000 37 against 47 us); at most 2^30 items in total.
+  int64_t seg = a0.seg_passes > 0 ? a0.seg_passes
+                                  : (n_grp * passes_total) / ((one ? 4 : 8) * warps);
   if (seg < 1) seg = 1;
   if (seg > passes_total) seg = passes_total;
   int64_t n_seg = (passes_total + seg - 1) / seg;

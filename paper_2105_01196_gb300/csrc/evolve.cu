@@ -33,6 +33,7 @@
 
 #include "internal.h"
 #include "tables.cuh"
+#include "trend.cuh"
 
 namespace {
 
@@ -103,6 +104,7 @@ struct GenArgs {
   const unsigned long long *pair_cnt;
   int64_t Wst, R;
   int32_t neg, ns, rnum, rden, fuse_np;
+  int32_t tie_free;  // look for children whose pairs have no ties (pair_cnt not null)
   int32_t *todo;
 };
 
@@ -576,12 +578,12 @@ __device__ __forceinline__ bool fuse_child(const GenArgs &ga, int L) {
 
 // The counts of one pass (lane's 4 words w .. w + 3; act: they exist) from the ANDs of its pair
 // rows in each direction.
-__device__ __forceinline__ void fuse_pass_counts(const GenArgs &ga, bool neg, bool ns, bool act,
+__device__ __forceinline__ void fuse_pass_counts(const GenArgs &ga, bool neg, bool mask, bool act,
                                                  int64_t w, uint4 ap, uint4 an, int &cp, int &cn,
                                                  int &ca) {
   const uint4 zero4 = make_uint4(0u, 0u, 0u, 0u);
   uint4 pos = act ? ap : zero4, ng = (neg && act) ? an : zero4;
-  if (ns && act) {  // (pad rows hold complemented zeros)
+  if (mask && act && (w + 4) * 32 > ga.R) {  // (pad rows hold complemented zeros)
     const uint4 vm = make_uint4(fuse_valid(w, ga.R), fuse_valid(w + 1, ga.R),
                                 fuse_valid(w + 2, ga.R), fuse_valid(w + 3, ga.R));
     pos = fuse_and(pos, vm);
@@ -597,12 +599,14 @@ __device__ __forceinline__ void fuse_pass_counts(const GenArgs &ga, bool neg, bo
 // words of pass 0; unit u of a pass is pair u / 2's positive (even u) or negative row with
 // negative trends, else pair u's row).  NG groups are in flight: 2 in the warp's own region, 4
 // with a second region (stage2) borrowed from a warp of the block that has no slot left.
-template <int UPP, int NG>
+// ONE: a pass's rows are the pairs' positive rows only, and the negative direction's words are
+// their complements (no ties in any of the pairs).
+template <int UPP, int NG, bool ONE>
 __device__ void w_eval_exact_small(const GenArgs &ga, const uint32_t *const (&src)[4],
                                    uint32_t *stage, uint32_t *stage2, int lane, int &cp, int &cn,
                                    int &ca) {
   constexpr int PPG = kFuseGroup / UPP;  // passes per group
-  const bool neg = ga.neg != 0, ns = ga.ns != 0;
+  const bool neg = ga.neg != 0, ns = ga.ns != 0 && !ONE;
   const int64_t Wst = ga.Wst;
   const int passes = (int)((Wst + kFuseWords - 1) / kFuseWords);
   const int n_groups = (passes + PPG - 1) / PPG;
@@ -649,27 +653,34 @@ __device__ void w_eval_exact_small(const GenArgs &ga, const uint32_t *const (&sr
         for (int u = 0; u < UPP; ++u) {
           uint4 v = *reinterpret_cast<const uint4 *>(unit(gi, pp * UPP + u));
           if (ns) v = make_uint4(~v.x, ~v.y, ~v.z, ~v.w);
-          if (neg && (u & 1))
-            an = fuse_and(an, v);
-          else
+          if (ONE) {
             ap = fuse_and(ap, v);
+            an = fuse_and(an, make_uint4(~v.x, ~v.y, ~v.z, ~v.w));
+          } else if (neg && (u & 1)) {
+            an = fuse_and(an, v);
+          } else {
+            ap = fuse_and(ap, v);
+          }
         }
       }
-      if (q < passes) fuse_pass_counts(ga, neg, ns, act, w, ap, an, cp, cn, ca);
+      if (q < passes) fuse_pass_counts(ga, neg, ns || ONE, act, w, ap, an, cp, cn, ca);
     }
     if (gi + NG < n_groups) issue(gi + NG);
   }
 }
 
 // Row counts (positive trend, negative trend, either) of the exact test of c[0 .. L-1] (L >= 2),
-// in every lane.  stage: the warp's kFuseSlots * kFuseWords words of shared memory (16-byte
+// in every lane.  ONE: with negative trends, no pair of the child has ties, and the positive rows
+// give both directions.  stage: the warp's kFuseSlots * kFuseWords words of shared memory (16-byte
 // aligned), free for this call; stage2: a second such region (borrowed), or null.  Only passes of
 // at most kFuseGroup pair rows use the second region.
-__device__ void w_eval_exact(const GenArgs &ga, const int32_t *c, int L, uint32_t *stage,
-                             uint32_t *stage2, int lane, int &rp, int &rn, int &ra) {
+template <bool ONE>
+__device__ void w_eval_exact(const GenArgs &ga, const int32_t *c, int L, uint32_t *stage, uint32_t *stage2, int lane, int &rp, int &rn,
+                             int &ra) {
   const int np = L - 1;
-  const bool neg = ga.neg != 0, ns = ga.ns != 0;
-  const int upp = neg ? 2 * np : np;  // units per pass: pair j's positive (then negative) row
+  const bool neg = ga.neg != 0, two = neg && !ONE;  // (two: both directions' rows are read)
+  const bool ns = ga.ns != 0 && !ONE;
+  const int upp = two ? 2 * np : np;  // units per pass: pair j's positive (then negative) row
   const int64_t Wst = ga.Wst;
   if (upp <= kFuseGroup) {
     // every lane: the addresses of the pass's rows (pairs 0 .. np-1 <= 3: columns c[0 .. 4])
@@ -677,8 +688,8 @@ __device__ void w_eval_exact(const GenArgs &ga, const int32_t *c, int L, uint32_
     const uint32_t *src[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      const int j = neg ? (u >> 1) : u;
-      const bool nd = neg && (u & 1);
+      const int j = two ? (u >> 1) : u;
+      const bool nd = two && (u & 1);
       const int jj = j < np ? j : 0;  // (rows past upp are never read)
       const uint32_t a = (uint32_t)c[jj], b = (uint32_t)c[jj + 1];
       const uint32_t row = (ns != nd) ? b * C + a : a * C + b;
@@ -688,17 +699,17 @@ __device__ void w_eval_exact(const GenArgs &ga, const int32_t *c, int L, uint32_
     __syncwarp();  // every lane's earlier use of the region is done
     if (stage2) {
       switch (upp) {
-        case 1: w_eval_exact_small<1, 4>(ga, src, stage, stage2, lane, cp, cn, ca); break;
-        case 2: w_eval_exact_small<2, 4>(ga, src, stage, stage2, lane, cp, cn, ca); break;
-        case 3: w_eval_exact_small<3, 4>(ga, src, stage, stage2, lane, cp, cn, ca); break;
-        default: w_eval_exact_small<4, 4>(ga, src, stage, stage2, lane, cp, cn, ca); break;
+        case 1: w_eval_exact_small<1, 4, ONE>(ga, src, stage, stage2, lane, cp, cn, ca); break;
+        case 2: w_eval_exact_small<2, 4, ONE>(ga, src, stage, stage2, lane, cp, cn, ca); break;
+        case 3: w_eval_exact_small<3, 4, ONE>(ga, src, stage, stage2, lane, cp, cn, ca); break;
+        default: w_eval_exact_small<4, 4, ONE>(ga, src, stage, stage2, lane, cp, cn, ca); break;
       }
     } else {
       switch (upp) {
-        case 1: w_eval_exact_small<1, 2>(ga, src, stage, stage, lane, cp, cn, ca); break;
-        case 2: w_eval_exact_small<2, 2>(ga, src, stage, stage, lane, cp, cn, ca); break;
-        case 3: w_eval_exact_small<3, 2>(ga, src, stage, stage, lane, cp, cn, ca); break;
-        default: w_eval_exact_small<4, 2>(ga, src, stage, stage, lane, cp, cn, ca); break;
+        case 1: w_eval_exact_small<1, 2, ONE>(ga, src, stage, stage, lane, cp, cn, ca); break;
+        case 2: w_eval_exact_small<2, 2, ONE>(ga, src, stage, stage, lane, cp, cn, ca); break;
+        case 3: w_eval_exact_small<3, 2, ONE>(ga, src, stage, stage, lane, cp, cn, ca); break;
+        default: w_eval_exact_small<4, 2, ONE>(ga, src, stage, stage, lane, cp, cn, ca); break;
       }
     }
     rp = __reduce_add_sync(kFull, cp);
@@ -725,8 +736,8 @@ __device__ void w_eval_exact(const GenArgs &ga, const int32_t *c, int L, uint32_
 #pragma unroll
     for (int k = 0; k < kFuseGroup; ++k) {
       if (iq < passes) {
-        const int j = neg ? (ir >> 1) : ir, h = j >> 5;  // (the same in every lane)
-        const bool nd = neg && (ir & 1);
+        const int j = two ? (ir >> 1) : ir, h = j >> 5;  // (the same in every lane)
+        const bool nd = two && (ir & 1);
         const uint32_t row =
             __shfl_sync(kFull, h ? (nd ? row_n[1] : row_p[1]) : (nd ? row_n[0] : row_p[0]),
                         j & 31);
@@ -742,7 +753,7 @@ __device__ void w_eval_exact(const GenArgs &ga, const int32_t *c, int L, uint32_
     }
     fuse_commit();
   };
-  const uint4 ones = make_uint4(kFull, kFull, kFull, kFull), zero4 = make_uint4(0u, 0u, 0u, 0u);
+  const uint4 ones = make_uint4(kFull, kFull, kFull, kFull);
   uint4 ap = ones, an = ones;
   int cq = 0, cr = 0, cp = 0, cn = 0, ca = 0;
   __syncwarp();  // every lane's earlier use of the region is done
@@ -762,22 +773,17 @@ __device__ void w_eval_exact(const GenArgs &ga, const int32_t *c, int L, uint32_
           uint4 v = *reinterpret_cast<const uint4 *>(
               stage + ((gi & 1) * kFuseGroup + k) * kFuseWords + lane * 4);
           if (ns) v = make_uint4(~v.x, ~v.y, ~v.z, ~v.w);
-          if (neg && (cr & 1))
-            an = fuse_and(an, v);
-          else
+          if (ONE) {
             ap = fuse_and(ap, v);
+            an = fuse_and(an, make_uint4(~v.x, ~v.y, ~v.z, ~v.w));
+          } else if (neg && (cr & 1)) {
+            an = fuse_and(an, v);
+          } else {
+            ap = fuse_and(ap, v);
+          }
         }
         if (++cr == upp) {  // the pass is complete
-          uint4 pos = act ? ap : zero4, ng = (neg && act) ? an : zero4;
-          if (ns && act) {
-            const uint4 vm = make_uint4(fuse_valid(w, ga.R), fuse_valid(w + 1, ga.R),
-                                        fuse_valid(w + 2, ga.R), fuse_valid(w + 3, ga.R));
-            pos = fuse_and(pos, vm);
-            ng = fuse_and(ng, vm);
-          }
-          cp += fuse_popc(pos);
-          cn += fuse_popc(ng);
-          ca += fuse_popc(make_uint4(pos.x | ng.x, pos.y | ng.y, pos.z | ng.z, pos.w | ng.w));
+          fuse_pass_counts(ga, neg, ns || ONE, act, w, ap, an, cp, cn, ca);
           ap = ones;
           an = ones;
           cr = 0;
@@ -807,9 +813,11 @@ static_assert(kEvoScratch % 4 == 0, "scratch rows and staged units start on 16-b
 // counts stored, its key entered in generation g's duplicate table, as the evaluation launch
 // would) or listed for the evaluation launch.  Returns its tabu-flag value: 2 evaluated from the
 // pair words, 3 (a one-pair chromosome) from the pair-count table, 0 listed.
+// TF: the matrix has few tied pairs (ga.tie_free), and children without any are looked for.
 // s_free (k_evolve_seq; null otherwise): bit w set while warp w of the block has no slot left,
 // its region (of kEvolveWarpInts ints from `regions`) then free; a pair-word evaluation borrows
 // one such region for two more copy groups in flight and gives it back at its end.
+template <bool TF>
 __device__ int fuse_or_list(const GenArgs &ga, const int32_t *c, int L, uint64_t h, int s,
                             int par, uint32_t *stage, int lane, int32_t *regions,
                             uint32_t *s_free) {
@@ -853,7 +861,16 @@ __device__ int fuse_or_list(const GenArgs &ga, const int32_t *c, int L, uint64_t
       uint32_t *stage2 =
           lent >= 0 ? reinterpret_cast<uint32_t *>(regions + lent * kEvolveWarpInts + kEvoStage)
                     : nullptr;
-      w_eval_exact(ga, c, L, stage, stage2, lane, rp, rn, ra);
+      // no ties in any pair: the positive rows' words give both directions (np <= 63 pairs)
+      bool tied = !TF;
+      if (TF)
+        for (int k = lane; k < L - 1; k += 32)
+          tied |= pair_has_ties(ga.pair_cnt, ga.C, c[k], c[k + 1], ga.R);
+      // (half the words read: evolve 34 -> 31 us per generation on 20,000 x 500, P = 4,096)
+      if (TF && !__any_sync(kFull, tied))
+        w_eval_exact<true>(ga, c, L, stage, stage2, lane, rp, rn, ra);
+      else
+        w_eval_exact<false>(ga, c, L, stage, stage2, lane, rp, rn, ra);
       if (lent >= 0) {
         __syncwarp();  // (every lane's copies into it have landed and been read)
         if (lane == 0) atomicOr(s_free, 1u << lent);
@@ -918,6 +935,7 @@ size_t evolve_smem(int G, int C) {
 }
 static_assert(kEvolveWarpInts % 4 == 0, "per-warp region must keep 16-byte alignment");
 
+template <bool TF>
 __global__ void __launch_bounds__(kMaxAttemptWarps * 32) k_evolve(GenArgs ga, Buf pb, Buf nb,
                                                                   int par) {
   extern __shared__ __align__(16) int32_t s_evo[];  // kEvolveWarpInts per warp, then usage
@@ -981,7 +999,7 @@ __global__ void __launch_bounds__(kMaxAttemptWarps * 32) k_evolve(GenArgs ga, Bu
   out[lane] = lane < L ? c[lane] : 0;
   out[lane + 32] = lane + 32 < L ? c[lane + 32] : 0;
   const int fused = (!dead && ga.fuse_np > 0)
-                        ? fuse_or_list(ga, c, L, h, s, par,
+                        ? fuse_or_list<TF>(ga, c, L, h, s, par,
                                        reinterpret_cast<uint32_t *>(base + kEvoStage), lane,
                                        nullptr, nullptr)
                         : 0;
@@ -1007,6 +1025,7 @@ __global__ void __launch_bounds__(kMaxAttemptWarps * 32) k_evolve(GenArgs ga, Bu
 // of the column-usage table.
 constexpr int kSeqWarps = 8;
 
+template <bool TF>
 __global__ void __launch_bounds__(kSeqWarps * 32, 4) k_evolve_seq(GenArgs ga, Buf pb, Buf nb,
                                                                int par) {
   extern __shared__ __align__(16) int32_t s_evo[];  // kEvolveWarpInts per warp, then usage
@@ -1061,7 +1080,7 @@ __global__ void __launch_bounds__(kSeqWarps * 32, 4) k_evolve_seq(GenArgs ga, Bu
       out[lane] = lane < L ? c[lane] : 0;
       out[lane + 32] = lane + 32 < L ? c[lane + 32] : 0;
       const int fused = (!dead && ga.fuse_np > 0)
-                            ? fuse_or_list(ga, c, L, h, s, par,
+                            ? fuse_or_list<TF>(ga, c, L, h, s, par,
                                            reinterpret_cast<uint32_t *>(base + kEvoStage), lane,
                                            s_evo, &s_free)
                             : 0;
@@ -1692,6 +1711,7 @@ struct GenState {
   bool reset_pending = false;          // the run state must be cleared before the next run
   const void *graph_buf = nullptr;  // codes or bitmap the captured graphs read (null: keys)
   const void *graph_cnt = nullptr;  // pair-count table the captured graphs read (or null)
+  int graph_tie = -1;               // ebic_ctx::tie_state of the captured graphs
   DevBuf cols[2], len[2], att_hits[2], rows[2], att_dead[2], dead[2], hash[2], fit[2];
   DevBuf dkeys[2], dslot[2];
   DevBuf rows_scr, work, tabu, top, ctl, usage, cand_f, cand_h, cand_s, extract, todo;
@@ -1815,6 +1835,7 @@ GenArgs gen_args(ebic_ctx *ctx, GenState *g) {
   if (g->fuse_np > 0) {
     ga.bitmap = ctx->bitmap.as<uint32_t>();
     ga.pair_cnt = ctx->pair_cnt_ok ? ctx->pair_cnt.as<unsigned long long>() : nullptr;
+    ga.tie_free = ga.pair_cnt && ctx->tie_state == 1;
     ga.Wst = ctx->Gst;
     ga.R = ctx->R;
     ga.neg = p.neg_trends;
@@ -1962,12 +1983,14 @@ cudaError_t launch_generation(ebic_ctx *ctx, GenState *g, int parity, cudaStream
   if (e != cudaSuccess) return e;
   // A block of G attempt warps per slot while every slot's block fits on the GPU at once (the
   // slot's latency is then the launch's); beyond that a warp per slot, attempts in turn.
+  const GenArgs ga = gen_args(ctx, g);
+  const bool tf = ga.fuse_np > 0 && ga.neg && ga.tie_free;
   if ((int64_t)g->P * G <= (int64_t)ctx->num_sms * kEvolveResidentWarps) {
-    e = launch_pdl(k_evolve, dim3((unsigned)g->P), dim3(G * 32), evolve_smem(G, g->C), s,
-                   gen_args(ctx, g), g->buf(parity ^ 1), g->buf(parity), parity);
+    e = launch_pdl(tf ? k_evolve<true> : k_evolve<false>, dim3((unsigned)g->P), dim3(G * 32), evolve_smem(G, g->C), s, ga,
+                   g->buf(parity ^ 1), g->buf(parity), parity);
   } else {
-    e = launch_pdl(k_evolve_seq, dim3((unsigned)g->seq_blocks),
-                   dim3(kSeqWarps * 32), evolve_smem(kSeqWarps, g->C), s, gen_args(ctx, g),
+    e = launch_pdl(tf ? k_evolve_seq<true> : k_evolve_seq<false>, dim3((unsigned)g->seq_blocks),
+                   dim3(kSeqWarps * 32), evolve_smem(kSeqWarps, g->C), s, ga,
                    g->buf(parity ^ 1), g->buf(parity), parity);
   }
   if (e != cudaSuccess) return e;
@@ -2100,14 +2123,15 @@ int gen_create(ebic_ctx *ctx, const ebic_params *p) {
   if (g->top_smem > kFinishSmemMax) return ebic_fail(ctx, EBIC_EINVAL, "top-list workspace too large");
   EBIC_CHECK_CUDA(ctx, cudaFuncSetAttribute(k_finish, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                             (int)kFinishSmemMax));
-  EBIC_CHECK_CUDA(ctx, cudaFuncSetAttribute(k_evolve, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)evolve_smem(kMaxAttemptWarps, kUsageSmemMax)));
-  EBIC_CHECK_CUDA(ctx, cudaFuncSetAttribute(k_evolve_seq,
-                                            cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)evolve_smem(kSeqWarps, kUsageSmemMax)));
+  for (const auto k : {k_evolve<false>, k_evolve<true>})
+    EBIC_CHECK_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)evolve_smem(kMaxAttemptWarps, kUsageSmemMax)));
+  for (const auto k : {k_evolve_seq<false>, k_evolve_seq<true>})
+    EBIC_CHECK_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)evolve_smem(kSeqWarps, kUsageSmemMax)));
   int seq_per_sm = 0;
   EBIC_CHECK_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                           &seq_per_sm, k_evolve_seq, kSeqWarps * 32,
+                           &seq_per_sm, k_evolve_seq<false>, kSeqWarps * 32,
                            evolve_smem(kSeqWarps, ctx->C)));
   g->seq_blocks = (int)std::max<int64_t>(
       1, std::min<int64_t>((g->P + kSeqWarps - 1) / kSeqWarps,
@@ -2190,10 +2214,14 @@ int ensure_eval_ready(ebic_ctx *ctx, GenState *g, const ebic_params *p, int n_ge
                     : (direct && ctx->codes_ready ? ctx->codes.p : nullptr);
   // (and the fusion limit, which the captured evolve launches hold)
   const int fuse = fuse_limit(ctx, mode, p);
-  const void *cnt = fuse > 0 && ctx->pair_cnt_ok ? ctx->pair_cnt.p : nullptr;
+  const void *cnt = mode == EBIC_MODE_BITMAP && ctx->pair_cnt_ok ? ctx->pair_cnt.p : nullptr;
+  if (mode == EBIC_MODE_BITMAP && p->neg_trends &&
+      (fuse > 1 || (p->ratio_num < p->ratio_den && eval_args_for(ctx).stage_bitmap)))
+    EBIC_TRY(ensure_tie_state(ctx));
   if (mode != g->eval_mode || buf != g->graph_buf || fuse != g->fuse_np ||
-      cnt != g->graph_cnt) {
+      cnt != g->graph_cnt || ctx->tie_state != g->graph_tie) {
     g->drop_graphs();
+    g->graph_tie = ctx->tie_state;
     g->graph_buf = buf;
     g->graph_cnt = cnt;
   }

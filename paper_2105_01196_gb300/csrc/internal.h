@@ -112,6 +112,8 @@ struct SweepOut {
 struct EvalArgs {
   const uint32_t *keys;    // [C][R_pad] order keys
   const uint32_t *bitmap;  // [C][C][Wst] pair words (bitmap path)
+  const unsigned long long *pair_cnt;  // [C][C] pair counts (ebic_ctx::pair_cnt), or null
+  int32_t tie_free;        // look for individuals whose pairs have no ties (pair_cnt not null)
   int64_t R, R_pad, Wst;   // rows, padded rows, words per stored pair row (ebic_ctx::Gst)
   int32_t C;
   int32_t neg, rnum, rden, min_rows, col_cap;
@@ -218,6 +220,10 @@ struct ebic_ctx {
   // codes' bit planes (C <= 1,024), else absent
   DevBuf pair_cnt;
   bool pair_cnt_ok = false;
+  // tied column pairs of the bitmap's matrix (d_ties), and what follows: 1 few pairs are tied, so
+  // the evaluations look for individuals without ties; 0 many; -1 not counted yet
+  DevBuf d_ties;
+  int tie_state = -1;
 
   // scratch for single evaluations
   DevBuf d_err, d_work, ev_cols, ev_off, ev_out, ev_fit;
@@ -269,6 +275,9 @@ void prof_collect(ebic_ctx *ctx);
 
 int ebic_fail(ebic_ctx *ctx, int code, const std::string &msg);
 
+// Counts the tied pairs of the bitmap's matrix, once per build (a launch and a synchronisation):
+// called where a form that looks for individuals without ties may run.
+int ensure_tie_state(ebic_ctx *ctx);
 // Builds the rank codes of the loaded matrix if it has some and they are not built yet.
 int ensure_codes(ebic_ctx *ctx);
 // Whether evaluation form `mode` runs the direct kernel (the staged form falls back to it).
@@ -321,6 +330,9 @@ cudaError_t launch_build_bitmap(const uint32_t *keys, int64_t R_pad, int32_t C, 
 cudaError_t launch_build_bitmap_planes(const uint32_t *planes, int32_t C, int64_t Wst,
                                        uint32_t *bitmap, unsigned long long *cnt, int num_sms,
                                        cudaStream_t s);
+// *out (device) = the column pairs with equal values in some row, from the pair counts.
+cudaError_t launch_count_tied(const unsigned long long *cnt, int32_t C, int64_t R, int32_t *out,
+                              cudaStream_t s);
 
 // eval.cu
 cudaError_t launch_validate_csr(const int32_t *cols, const int32_t *off, int32_t n, int32_t C,

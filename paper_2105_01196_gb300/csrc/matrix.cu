@@ -393,7 +393,32 @@ __global__ void __launch_bounds__(kBuildWarps * 32, 3) k_build_bitmap_planes(con
   }
 }
 
+// Pairs of columns with equal values in some row: those whose two counts do not add up to R.
+__global__ void __launch_bounds__(256) k_count_tied(const unsigned long long *__restrict__ cnt,
+                                                    int32_t C, int64_t R, int32_t *out) {
+  int n = 0;
+  for (int64_t q = (int64_t)blockIdx.x * 256 + threadIdx.x; q < (int64_t)C * C;
+       q += (int64_t)gridDim.x * 256) {
+    const int64_t a = q / C, b = q - a * C;
+    if (a < b) {
+      const unsigned long long v = __ldg(cnt + q);
+      n += (int64_t)(uint32_t)v + (int64_t)(v >> 32) != R;
+    }
+  }
+  n = __reduce_add_sync(0xFFFFFFFFu, n);
+  if (n && (threadIdx.x & 31) == 0) atomicAdd(out, n);
+}
+
 }  // namespace
+
+cudaError_t launch_count_tied(const unsigned long long *cnt, int32_t C, int64_t R, int32_t *out,
+                              cudaStream_t s) {
+  const cudaError_t e = cudaMemsetAsync(out, 0, sizeof(int32_t), s);
+  if (e != cudaSuccess) return e;
+  const int64_t blocks = std::min<int64_t>(((int64_t)C * C + 255) / 256, 152 * 8);
+  k_count_tied<<<(unsigned)blocks, 256, 0, s>>>(cnt, C, R, out);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_upload_rows(const float *x, int64_t R, int32_t C, int64_t R_pad,
                                uint32_t *keys, int32_t *err, int64_t r_begin, int64_t r_end,

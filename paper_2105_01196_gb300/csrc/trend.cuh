@@ -11,6 +11,24 @@
 
 #include <stdint.h>
 
+// Whether columns c and d hold equal values in some row, from the pair counts of the bitmap build
+// (cnt[a * C + b], a < b: the rows with b above a and those with a above b, a 32-bit half each):
+// with no ties the two add up to every row.
+__device__ __forceinline__ bool pair_has_ties(const unsigned long long *__restrict__ cnt, int C,
+                                              int c, int d, int64_t R) {
+  const unsigned long long v = __ldg(cnt + (int64_t)min(c, d) * C + max(c, d));
+  return (int64_t)(uint32_t)v + (int64_t)(v >> 32) != R;
+}
+
+// Rows with d above c, and with c above d, from the same counts.
+__device__ __forceinline__ void pair_counts(const unsigned long long *__restrict__ cnt, int C,
+                                            int c, int d, int *up, int *down) {
+  const unsigned long long v = __ldg(cnt + (int64_t)min(c, d) * C + max(c, d));
+  const int lo = (int)(uint32_t)v, hi = (int)(v >> 32);
+  *up = c < d ? lo : hi;
+  *down = c < d ? hi : lo;
+}
+
 template <bool NS, typename T>
 __device__ __forceinline__ bool pair_up(T cur, T ref) {
   return NS ? cur >= ref : cur > ref;

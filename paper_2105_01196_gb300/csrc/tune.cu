@@ -231,7 +231,11 @@ extern "C" int ebic_autotune(ebic_ctx *ctx, const int32_t *col_idx, const int32_
       build_ms = ms;
     }
     a.bitmap = ctx->bitmap.as<uint32_t>();
-    a.stage_bitmap = eval_args_for(ctx).stage_bitmap;  // (the form later runs will use)
+    EBIC_TRY(ensure_tie_state(ctx));
+    const EvalArgs built = eval_args_for(ctx);
+    a.pair_cnt = built.pair_cnt;
+    a.tie_free = built.tie_free;
+    a.stage_bitmap = built.stage_bitmap;  // (the form later runs will use)
     // (individuals per item: the staged form only)
     const int ipw_max = a.stage_bitmap && p->ratio_num < p->ratio_den ? 4 : 1;
     for (int ipw = 1; ipw <= ipw_max; ipw *= 2)
