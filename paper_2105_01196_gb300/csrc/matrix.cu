@@ -54,24 +54,56 @@ __global__ void k_upload_rowmajor(const float *__restrict__ x, int64_t R, int32_
   }
 }
 
-// Column-major x[C][R] -> keys[C][R_pad], one element per thread, grid-stride.
-__global__ void k_upload_colmajor(const float *__restrict__ x, int64_t R, int32_t C,
-                                  int64_t R_pad, uint32_t *__restrict__ keys,
-                                  int32_t *__restrict__ err) {
-  const int64_t total = (int64_t)C * R_pad;
+// Column-major x[C][R] -> keys[C][R_pad]: a block walks 4,096 rows of one column (blockIdx.y, and
+// further columns gridDim.y apart), four rows per thread and step: one 16-byte load where every
+// column starts on a 16-byte boundary (VEC), else four 4-byte loads a warp's width apart; keys are
+// stored the same way.  Bound: HBM.  (One element per thread with its column found by a 64-bit
+// division took 128 us at 33,333 x 777, now 40 us.)
+constexpr int kColRows = 4096;
+
+template <bool VEC>
+__global__ void __launch_bounds__(256) k_upload_colmajor(const float *__restrict__ x, int64_t R,
+                                                         int32_t C, int64_t R_pad,
+                                                         uint32_t *__restrict__ keys,
+                                                         int32_t *__restrict__ err) {
+  const int64_t r_lo = (int64_t)blockIdx.x * kColRows;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   bool bad = false;
-  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < total;
-       q += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t c = q / R_pad, r = q - c * R_pad;
-    uint32_t k = 0u;
-    if (r < R) {
-      const uint32_t u = __float_as_uint(__ldg(x + c * R + r));
-      bad |= not_finite(u);
-      k = order_key(u);
+  for (int64_t c = blockIdx.y; c < C; c += gridDim.y) {
+    const uint32_t *src = reinterpret_cast<const uint32_t *>(x) + c * R;
+    uint32_t *dst = keys + c * R_pad;
+#pragma unroll
+    for (int k = 0; k < kColRows / 1024; ++k) {
+      const int64_t r0 = r_lo + k * 1024 + warp * 128;  // the warp's 128 rows
+      if (VEC) {
+        const int64_t r = r0 + 4 * lane;
+        if (r < R_pad) {  // (R_pad and R are multiples of 4)
+          uint4 v = make_uint4(0u, 0u, 0u, 0u);
+          if (r < R) {
+            v = __ldg(reinterpret_cast<const uint4 *>(src + r));
+            bad |= not_finite(v.x) || not_finite(v.y) || not_finite(v.z) || not_finite(v.w);
+            v = make_uint4(order_key(v.x), order_key(v.y), order_key(v.z), order_key(v.w));
+          }
+          *reinterpret_cast<uint4 *>(dst + r) = v;
+        }
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int64_t r = r0 + 32 * j + lane;
+          if (r < R_pad) {
+            uint32_t key = 0u;
+            if (r < R) {
+              const uint32_t u = __ldg(src + r);
+              bad |= not_finite(u);
+              key = order_key(u);
+            }
+            dst[r] = key;
+          }
+        }
+      }
     }
-    keys[q] = k;
   }
-  if (__any_sync(0xFFFFFFFFu, bad) && (threadIdx.x & 31) == 0) atomicOr(err, 1);
+  if (__any_sync(0xFFFFFFFFu, bad) && lane == 0) atomicOr(err, 1);
 }
 
 // Pair bitmap: G[(a*C + b)*Wst + w] bit j = [key(32w+j, b) > key(32w+j, a)].
@@ -435,10 +467,12 @@ cudaError_t launch_upload(const float *x, int64_t R, int32_t C, int64_t R_pad, i
   if (layout == EBIC_LAYOUT_ROW_MAJOR) {
     return launch_upload_rows(x, R, C, R_pad, keys, err, 0, R_pad, s);
   } else {
-    const int64_t total = (int64_t)C * R_pad;
-    int64_t blocks = (total + 255) / 256;
-    if (blocks > 152 * 32) blocks = 152 * 32;
-    k_upload_colmajor<<<(unsigned)blocks, 256, 0, s>>>(x, R, C, R_pad, keys, err);
+    const dim3 grid((unsigned)((R_pad + kColRows - 1) / kColRows),
+                    (unsigned)std::min<int32_t>(C, 65535));
+    if (R % 4 == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0)
+      k_upload_colmajor<true><<<grid, 256, 0, s>>>(x, R, C, R_pad, keys, err);
+    else
+      k_upload_colmajor<false><<<grid, 256, 0, s>>>(x, R, C, R_pad, keys, err);
   }
   return cudaGetLastError();
 }
