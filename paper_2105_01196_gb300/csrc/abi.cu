@@ -515,7 +515,7 @@ int load_matrix_segmented(ebic_ctx *ctx, const float *x, int64_t rows, int32_t c
   cudaStream_t s = ctx->stream;
   EBIC_CHECK_CUDA(ctx, ctx->stage_x.ensure((size_t)rows * C * sizeof(float), s));
   EBIC_CHECK_CUDA(ctx, ctx->codes.ensure((size_t)C * S * cb, s));
-  EBIC_CHECK_CUDA(ctx, cudaMemsetAsync(ctx->codes.p, 0, (size_t)C * S * cb, s));
+  EBIC_CHECK_CUDA(ctx, launch_clear_code_tail(ctx->codes.p, cb, S, R_pad, cols, s));
   if (bitmap) {
     EBIC_CHECK_CUDA(ctx, ctx->planes.ensure((size_t)code_plane_words(cols, Gst) * 4, s));
     EBIC_CHECK_CUDA(ctx, ctx->bitmap.ensure((size_t)(C * C * Gst) * 4, s));

@@ -50,11 +50,18 @@ __device__ __forceinline__ void wait_prior_grid() {
 // at distance < EPL stay inside a lane; the others pair lanes through one shuffle.  The sorted
 // row goes to shared memory and the rank of each key is the number of sorted keys below it,
 // found by a branchless binary search (equal keys get equal codes, as the definition requires).
-// A block owns 16 consecutive rows: their keys are staged column by column with coalesced loads
-// in a shared [C][17] tile, each row's codes replace its keys in the tile, and the tile is
-// written out column by column (codes [C][S]).
-constexpr int kRankRows = 16;                 // rows per block tile
-constexpr int kTileStride = kRankRows + 1;    // tile entries per column (bank spread)
+// A block owns 8 (up to 128 columns: 16) consecutive rows: their keys are staged column by column
+// in a shared [C][9] (or [C][17]) tile, each row's codes replace its keys in the tile, and the tile
+// is written out column by column (codes [C][S]).  Eight rows leave room for three blocks per SM.
+// What bounds it: shared-memory wavefronts (the searches' bank conflicts, the transpositions) and
+// the ALU pipe, each about half busy with 24 warps per SM.  60,000 x 1,000: 0.69 ms with 16 rows,
+// two blocks and the unrolled shuffle network (1.01 ms with the bit planes), 0.55 ms now;
+// 33,333 x 777 345 -> 270 us, 20,000 x 500 106 -> 89 us.
+// (rows per block tile; tile entries per column, one more for the bank spread)
+template <int EPL>
+constexpr int rank_rows() {
+  return EPL >= 8 ? 8 : 16;
+}
 
 template <int EPL>
 __device__ __forceinline__ void bitonic_sort_row(uint32_t (&v)[EPL], int lane) {
@@ -111,6 +118,88 @@ __device__ __forceinline__ void bitonic_sort_row(uint32_t (&v)[EPL], int lane) {
   }
 }
 
+// The same result for EPL >= 8, in fewer instructions: the cross-lane exchanges of the network
+// above cost a shuffle, a minimum, a maximum and a select per key, where an exchange between two
+// registers of a lane costs a minimum and a maximum for two keys.  So each merge goes through the
+// warp's shared buffer twice: the runs of h lanes are written row by row (row = lane, stride
+// EPL + 1: no bank conflicts), every second run reversed, and read back transposed, thread
+// (blk, jj) = (t / EPL, t % EPL) holding element jj of lanes blk EPL + i in register i.  Lane
+// distances below EPL are then register distances (beyond, with EPL = 8 or 16, shuffles), and the
+// merge ends with the half-cleaners inside a lane after the way back.  The lanes' own keys are
+// sorted first by Batcher's odd-even merge network (191 exchanges for 32 keys).  Loops over the
+// merges are not unrolled: the code of the unrolled network did not fit the instruction cache.
+__device__ __forceinline__ void exchange(uint32_t &a, uint32_t &b) {
+  const uint32_t lo = min(a, b), hi = max(a, b);
+  a = lo;
+  b = hi;
+}
+
+template <int EPL>
+constexpr int sort_buffer_words() {
+  return 32 * (EPL + 1);
+}
+
+template <int EPL>
+__device__ __forceinline__ void merge_sort_row(uint32_t (&v)[EPL], int lane, uint32_t *buf) {
+  constexpr int S = EPL + 1;
+#pragma unroll
+  for (int p = 1; p < EPL; p <<= 1) {
+#pragma unroll
+    for (int k = p; k >= 1; k >>= 1) {
+#pragma unroll
+      for (int j = 0; j < EPL; ++j) {
+        // (lower ends of the exchanges at distance k: j - k mod p in the first k of 2 k)
+        const int r = j - k % p;
+        if (r >= 0 && r % (2 * k) < k && j + k < EPL && j / (2 * p) == (j + k) / (2 * p))
+          exchange(v[j], v[j + k]);
+      }
+    }
+  }
+  const int blk = lane / EPL, jj = lane % EPL;
+#pragma unroll 1
+  for (int h = 1; h < 32; h <<= 1) {
+    // rows out: the second run of each pair reversed (its lanes mirrored, its keys backwards)
+    const bool rev = (lane & h) != 0;
+    uint32_t *out = buf + (rev ? (lane ^ (h - 1)) * S + EPL - 1 : lane * S);
+    const int step = rev ? -1 : 1;
+    __syncwarp();  // (every lane is done with what the buffer held)
+#pragma unroll
+    for (int j = 0; j < EPL; ++j) out[j * step] = v[j];
+    __syncwarp();
+    uint32_t *col = buf + blk * EPL * S + jj;
+#pragma unroll
+    for (int i = 0; i < EPL; ++i) v[i] = col[i * S];
+#pragma unroll
+    for (int d = 16; d >= 1; d >>= 1) {
+      if (h >= d) {  // (uniform)
+        if (d >= EPL) {
+          const bool upper = (lane & d) != 0;
+#pragma unroll
+          for (int i = 0; i < EPL; ++i) {
+            const uint32_t o = __shfl_xor_sync(kFull, v[i], d);
+            v[i] = upper ? max(v[i], o) : min(v[i], o);
+          }
+        } else {
+#pragma unroll
+          for (int i = 0; i < EPL; ++i)
+            if (!(i & d)) exchange(v[i], v[i ^ (d & (EPL - 1))]);
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < EPL; ++i) col[i * S] = v[i];  // (the words this thread read)
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < EPL; ++j) v[j] = buf[lane * S + j];
+#pragma unroll
+    for (int d = EPL / 2; d >= 1; d >>= 1) {
+#pragma unroll
+      for (int j = 0; j < EPL; ++j)
+        if (!(j & d)) exchange(v[j], v[j ^ d]);
+    }
+  }
+}
+
 // Sorted position e sits at e + e / 32 in a warp's shared buffer (one pad word per 32: the
 // stores of positions lane * EPL + j from every lane fall in distinct banks).
 __device__ __forceinline__ int sorted_slot(int e) { return e + (e >> 5); }
@@ -120,26 +209,33 @@ __device__ __forceinline__ int sorted_slot(int e) { return e + (e >> 5); }
 // moves by s + s/32; smaller steps stay inside one 32-block.
 template <int N>
 __device__ __forceinline__ int count_below(const uint32_t *srt, uint32_t q) {
-  const uint32_t *p = srt;
+  int p = 0;
 #pragma unroll
   for (int step = N / 2; step >= 1; step >>= 1) {
     const int d = step >= 32 ? step + step / 32 : step;
     const int t = step >= 32 ? d - 2 : d - 1;
-    if (p[t] < q) p += d;
+    if (srt[p + t] < q) p += d;
   }
-  if (*p < q) ++p;
-  const int pp = (int)(p - srt);
-  return pp - pp / 33;
+  if (srt[p] < q) ++p;
+  return p - p / 33;
+}
+
+template <int EPL>
+constexpr int rank_buffer_words() {
+  return EPL >= 8 && sort_buffer_words<EPL>() > 33 * EPL ? sort_buffer_words<EPL>() : 33 * EPL;
 }
 
 // T: code type (uint8_t for C <= 128, uint16_t for C <= 1,024); EPL: keys per lane
 // (32 * EPL >= C).
 template <typename T, int EPL>
-__global__ void __launch_bounds__(kThreads, 2)
+__global__ void __launch_bounds__(kThreads, EPL >= 32 ? 3 : 2)
     k_rank_codes(const uint32_t *__restrict__ keys, int64_t R_pad, int32_t C, int64_t S,
                  T *__restrict__ codes, int64_t t_begin, int64_t t_end) {
+  constexpr int kRankRows = rank_rows<EPL>(), kTileStride = kRankRows + 1;
+  constexpr int kQuads = kRankRows / 4;
   constexpr int N = 32 * EPL;
-  constexpr int kSorted = N + N / 32;  // words of one warp's sorted buffer
+  // words of one warp's buffer: the sorted row, and before it the sort's transpositions
+  constexpr int kSorted = rank_buffer_words<EPL>();
   extern __shared__ __align__(16) uint32_t s_rank[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t *srt = s_rank + warp * kSorted;
@@ -147,9 +243,16 @@ __global__ void __launch_bounds__(kThreads, 2)
   // (tiles [t_begin, t_end) of the R_pad / kRankRows)
   for (int64_t t = t_begin + blockIdx.x; t < t_end; t += gridDim.x) {
     const int64_t r0 = t * kRankRows;
-    for (int i = threadIdx.x; i < C * kRankRows; i += kThreads) {
-      const int c = i / kRankRows, rho = i % kRankRows;
-      tile[c * kTileStride + rho] = __ldg(keys + (int64_t)c * R_pad + r0 + rho);
+    // keys in: 16-byte pieces of four rows (unrolled twice: more slowed the other phases down)
+#pragma unroll 2
+    for (int i = threadIdx.x; i < C * kQuads; i += kThreads) {
+      const int c = i / kQuads, rho = i % kQuads * 4;
+      const uint4 k = __ldg(reinterpret_cast<const uint4 *>(keys + (int64_t)c * R_pad + r0 + rho));
+      uint32_t *dst = tile + c * kTileStride + rho;
+      dst[0] = k.x;
+      dst[1] = k.y;
+      dst[2] = k.z;
+      dst[3] = k.w;
     }
     __syncthreads();
     for (int rho = warp; rho < kRankRows; rho += kWarps) {
@@ -159,15 +262,25 @@ __global__ void __launch_bounds__(kThreads, 2)
         const int c = j * 32 + lane;  // (any placement of the keys before sorting will do)
         v[j] = c < C ? tile[c * kTileStride + rho] : 0xFFFFFFFFu;
       }
-      bitonic_sort_row<EPL>(v, lane);
-      __syncwarp();  // the previous row's searches are done with the buffer
+      if constexpr (EPL >= 8)
+        merge_sort_row<EPL>(v, lane, srt);
+      else
+        bitonic_sort_row<EPL>(v, lane);
+      __syncwarp();  // the buffer's last reads (the sort's, or the previous row's searches) are done
 #pragma unroll
       for (int j = 0; j < EPL; ++j) srt[sorted_slot(lane * EPL + j)] = v[j];
       __syncwarp();
+      // (eight searches at a time, rolled: the code stays in the instruction cache)
+#pragma unroll 1
+      for (int j0 = 0; j0 < EPL; j0 += (EPL < 8 ? EPL : 8)) {
 #pragma unroll
-      for (int j = 0; j < EPL; ++j) {
-        const int c = j * 32 + lane;  // (this row's slot of column c: only this warp's)
-        if (c < C) tile[c * kTileStride + rho] = (uint32_t)count_below<N>(srt, tile[c * kTileStride + rho]);
+        for (int j = 0; j < (EPL < 8 ? EPL : 8); ++j) {
+          const int c = (j0 + j) * 32 + lane;  // (this row's slot of column c: only this warp's)
+          if (c < C) {
+            uint32_t *slot = tile + c * kTileStride + rho;
+            *slot = (uint32_t)count_below<N>(srt, *slot);
+          }
+        }
       }
     }
     __syncthreads();
@@ -496,10 +609,10 @@ namespace {
 template <typename T, int EPL>
 cudaError_t launch_rank_epl(const uint32_t *keys, int64_t R_pad, int32_t C, T *codes, int64_t S,
                             int num_sms, cudaStream_t s, int64_t r_begin, int64_t r_end) {
-  constexpr int N = 32 * EPL;
-  const size_t smem = (size_t)kWarps * (N + N / 32) * 4 + (size_t)C * kTileStride * 4;
+  constexpr int kRankRows = rank_rows<EPL>(), kTileStride = kRankRows + 1;
+  const size_t smem = (size_t)kWarps * rank_buffer_words<EPL>() * 4 + (size_t)C * kTileStride * 4;
   // one fixed limit for every context (no call lowers another's), set once per device
-  constexpr size_t kLimit = (size_t)kWarps * (1024 + 32) * 4 + (size_t)1024 * kTileStride * 4;
+  constexpr size_t kLimit = (size_t)kWarps * (1024 + 32) * 4 + (size_t)1024 * 17 * 4;
   static_assert(kLimit <= 227 * 1024, "rank-code shared memory");
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -531,7 +644,7 @@ cudaError_t launch_rank_codes_rows(const uint32_t *keys, int64_t R_pad, int32_t 
                                    int code_bytes, int64_t S, int num_sms, int64_t r_begin,
                                    int64_t r_end, cudaStream_t s) {
   if (C > 1024 || code_bytes != (C <= 128 ? 1 : 2)) return cudaErrorInvalidValue;
-  if (r_begin < 0 || r_begin % kRankRows || r_end > R_pad || r_end % kRankRows ||
+  if (r_begin < 0 || r_begin % 16 || r_end > R_pad || r_end % 16 ||
       r_end <= r_begin)
     return cudaErrorInvalidValue;
 #define EBIC_RANK(T, EPL, cd) \
@@ -547,10 +660,18 @@ cudaError_t launch_rank_codes_rows(const uint32_t *keys, int64_t R_pad, int32_t 
 #undef EBIC_RANK
 }
 
+// The rows of the code columns past R_pad, up to S, are zero (the kernel writes the others).
+cudaError_t launch_clear_code_tail(void *codes, int code_bytes, int64_t S, int64_t R_pad,
+                                   int32_t C, cudaStream_t s) {
+  if (S <= R_pad) return cudaSuccess;
+  return cudaMemset2DAsync(static_cast<uint8_t *>(codes) + R_pad * code_bytes,
+                           (size_t)S * code_bytes, 0, (size_t)(S - R_pad) * code_bytes, (size_t)C,
+                           s);
+}
+
 cudaError_t launch_rank_codes(const uint32_t *keys, int64_t R_pad, int32_t C, void *codes,
                               int code_bytes, int64_t S, int num_sms, cudaStream_t s) {
-  // (the rows of the code columns past R_pad, up to S, stay zero)
-  cudaError_t e = cudaMemsetAsync(codes, 0, (size_t)C * S * code_bytes, s);
+  const cudaError_t e = launch_clear_code_tail(codes, code_bytes, S, R_pad, C, s);
   if (e != cudaSuccess) return e;
   return launch_rank_codes_rows(keys, R_pad, C, codes, code_bytes, S, num_sms, 0, R_pad, s);
 }

@@ -162,7 +162,10 @@ int64_t code_plane_chunks(int64_t Wst);
 int64_t code_plane_words(int32_t C, int64_t Wst);
 cudaError_t launch_rank_codes(const uint32_t *keys, int64_t R_pad, int32_t C, void *codes,
                               int code_bytes, int64_t S, int num_sms, cudaStream_t s);
-// The rows [r_begin, r_end) only (multiples of 16), codes not cleared beforehand.
+// The two parts of it: the clearing of the code columns' rows past R_pad, and the rows
+// [r_begin, r_end) only (multiples of 16).
+cudaError_t launch_clear_code_tail(void *codes, int code_bytes, int64_t S, int64_t R_pad,
+                                   int32_t C, cudaStream_t s);
 cudaError_t launch_rank_codes_rows(const uint32_t *keys, int64_t R_pad, int32_t C, void *codes,
                                    int code_bytes, int64_t S, int num_sms, int64_t r_begin,
                                    int64_t r_end, cudaStream_t s);

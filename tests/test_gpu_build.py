@@ -37,3 +37,33 @@ def test_build_at_chunk_and_block_edges(R, C):
         ab, ba = pair_words(x, a, b), pair_words(x, b, a)
         assert np.array_equal(words[a, b, :W], ab) and np.array_equal(words[b, a, :W], ba), (a, b)
         assert int(cnt[a, b]) == popc(ab) | (popc(ba) << 32), (a, b)
+
+
+@pytest.mark.parametrize("C", [2, 31, 33, 65, 128, 129, 255, 257, 511, 513, 777, 1023, 1024])
+@pytest.mark.parametrize("R", [1, 9, 130])
+def test_rank_codes_order_every_pair(R, C):
+    """The rank codes' sort at every lane width (1 to 32 keys per lane, full and partly filled) on
+    rows that are sorted, reversed, constant, two-valued and random, with infinitely close and
+    extreme values: every pair's counts equal the oracle's comparisons (a wrong code shows as a
+    wrong pair)."""
+    from paper_2105_01196_gb300 import ebic
+    g = np.random.default_rng(17 * R + C)
+    x = g.standard_normal((R, C)).astype(np.float32)
+    kinds = [np.sort, lambda v: np.sort(v)[::-1], lambda v: v * 0 + 1,
+             lambda v: np.where(v > 0, np.float32(1), np.float32(-1)), lambda v: v,
+             lambda v: np.nextafter(np.float32(1), np.float32(2)) * (1 + (v > 0) * np.float32(1e-7)),
+             lambda v: v * np.float32(1e37), lambda v: np.round(v * 3) * np.float32(1e-45)]
+    for r in range(R):
+        x[r] = kinds[r % len(kinds)](x[r]).astype(np.float32)
+    x[:, g.random(C) < 0.1] = -0.0
+    cnt = np.zeros(C * C, np.uint64)
+    for layout in (ebic.ROW_MAJOR, ebic.COL_MAJOR):
+        with ebic.Context(0) as ctx:
+            ctx.load_matrix(x if layout == ebic.ROW_MAJOR else np.ascontiguousarray(x.T), layout)
+            ctx.build_bitmap()
+            ctx.copy_pair_counts(cnt)
+        t = cnt.reshape(C, C)
+        for a in g.choice(C, size=min(C, 60), replace=False):
+            up, down = (x > x[:, a:a + 1]).sum(0), (x < x[:, a:a + 1]).sum(0)
+            lo, hi = t[a] & np.uint64(0xFFFFFFFF), t[a] >> np.uint64(32)
+            assert np.array_equal(lo[a + 1:], up[a + 1:]) and np.array_equal(hi[a + 1:], down[a + 1:])
