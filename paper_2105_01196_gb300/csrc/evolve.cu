@@ -32,6 +32,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "items.cuh"
 #include "tables.cuh"
 #include "trend.cuh"
 
@@ -1013,6 +1014,224 @@ __global__ void __launch_bounds__(kMaxAttemptWarps * 32) k_evolve(GenArgs ga, Bu
   }
 }
 
+// The block-per-slot step with the evaluation inside, whatever the child's length: the block's
+// warps, which built the tabu attempts side by side, then count the winning child's rows together
+// (a thread per four words of every pair row, both directions; two words where the test counts,
+// so that the counters of both directions stay within 64 registers and every slot's block is
+// resident at once).  A generation is then two launches instead of three: k_finish takes the
+// evaluation launch's side task (the previous generation's keys into the tabu list).  Elites
+// take their row counts from the list.
+// Bound: latency, the slot's chain of dependent loads (tournament, tabu probe) and then one round
+// trip per four pairs.  10,000 x 100, P = 800: 17.3 us per generation with three launches.
+constexpr int kBlockWarps = 4;        // attempt warps at most
+constexpr int kBlockMaxSteps = 4;     // steps of four words per thread over a pair row, at most
+
+// A 6-bit bit-sliced count of pairs per bit position.
+__device__ __forceinline__ void count_add(uint32_t (&b)[6], uint32_t x) {
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    const uint32_t t = b[k] & x;
+    b[k] ^= x;
+    x = t;
+  }
+}
+
+// Bits whose count is >= t (1 <= t <= 63), most significant bit first.
+__device__ __forceinline__ uint32_t count_ge(const uint32_t (&b)[6], int t) {
+  uint32_t gt = 0u, eq = kFull;
+#pragma unroll
+  for (int k = 5; k >= 0; --k) {
+    if ((t >> k) & 1) {
+      eq &= b[k];
+    } else {
+      gt |= eq & b[k];
+      eq &= ~b[k];
+    }
+  }
+  return gt | eq;
+}
+
+// This thread's share of the row counts of chromosome c[0 .. L-1] (T threads in all).
+__device__ __forceinline__ void block_eval(const GenArgs &ga, const int32_t *c, int L, int tid,
+                                           int T, int &cp, int &cn, int &ca) {
+  const int np = L - 1;
+  const int t = (ga.rnum * np + ga.rden - 1) / ga.rden;
+  const bool neg = ga.neg != 0, ns = ga.ns != 0;
+  const int64_t Wst = ga.Wst;
+  const uint32_t C = (uint32_t)ga.C;
+  // pair k's rows: positive, negative (exchanged and complemented when ties hold both ways)
+  auto row = [&](int k, bool down) -> const uint32_t * {
+    const uint32_t a = (uint32_t)c[k], b = (uint32_t)c[k + 1];
+    return ga.bitmap + (int64_t)(down != ns ? b * C + a : a * C + b) * Wst;
+  };
+  if (t == np) {
+    for (int64_t w = 4 * tid; w < Wst; w += 4 * T) {
+      uint4 ap = make_uint4(kFull, kFull, kFull, kFull), an = ap;
+      for (int k = 0; k < np; k += 4) {
+        uint4 v[4], u[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {  // (past the last pair: that pair again)
+          const int q = min(k + j, np - 1);
+          v[j] = __ldg(reinterpret_cast<const uint4 *>(row(q, false) + w));
+          if (neg) u[j] = __ldg(reinterpret_cast<const uint4 *>(row(q, true) + w));
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          if (ns) v[j] = make_uint4(~v[j].x, ~v[j].y, ~v[j].z, ~v[j].w);
+          ap = fuse_and(ap, v[j]);
+          if (neg) {
+            if (ns) u[j] = make_uint4(~u[j].x, ~u[j].y, ~u[j].z, ~u[j].w);
+            an = fuse_and(an, u[j]);
+          }
+        }
+      }
+      fuse_pass_counts(ga, neg, ns, true, w, ap, an, cp, cn, ca);
+    }
+    return;
+  }
+  for (int64_t w = 2 * tid; w < Wst; w += 2 * T) {
+    uint32_t p0[6] = {}, p1[6] = {}, n0[6] = {}, n1[6] = {};
+    for (int k = 0; k < np; k += 4) {
+      uint2 v[4], u[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        v[j] = u[j] = make_uint2(ns ? kFull : 0u, ns ? kFull : 0u);
+        if (k + j < np) {
+          v[j] = __ldg(reinterpret_cast<const uint2 *>(row(k + j, false) + w));
+          if (neg) u[j] = __ldg(reinterpret_cast<const uint2 *>(row(k + j, true) + w));
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        count_add(p0, ns ? ~v[j].x : v[j].x);
+        count_add(p1, ns ? ~v[j].y : v[j].y);
+        if (neg) {
+          count_add(n0, ns ? ~u[j].x : u[j].x);
+          count_add(n1, ns ? ~u[j].y : u[j].y);
+        }
+      }
+    }
+    uint2 pos = make_uint2(count_ge(p0, t), count_ge(p1, t)), ng = make_uint2(0u, 0u);
+    if (neg) ng = make_uint2(count_ge(n0, t), count_ge(n1, t));
+    if (ns) {
+      const uint32_t m0 = fuse_valid(w, ga.R), m1 = fuse_valid(w + 1, ga.R);
+      pos = make_uint2(pos.x & m0, pos.y & m1);
+      ng = make_uint2(ng.x & m0, ng.y & m1);
+    }
+    cp += __popc(pos.x) + __popc(pos.y);
+    cn += __popc(ng.x) + __popc(ng.y);
+    ca += __popc(pos.x | ng.x) + __popc(pos.y | ng.y);
+  }
+}
+
+__global__ void __launch_bounds__(kBlockWarps * 32, 8) k_evolve_block(GenArgs ga, Buf pb, Buf nb,
+                                                                      int par) {
+  extern __shared__ __align__(16) int32_t s_evo[];  // kEvolveWarpInts per warp, then usage
+  __shared__ int s_ok[kBlockWarps], s_len[kBlockWarps], s_cnt[3];
+  __shared__ uint64_t s_h[kBlockWarps];
+  wait_prior_grid();
+  const int stopped = ga.ctl->stopped, gen = ga.ctl->gen, n_top = ga.ctl->n_top;
+  const int32_t *usage = ga.usage;
+  const int G = blockDim.x >> 5;
+  if (ga.C <= kUsageSmemMax) {
+    int32_t *s_usage = s_evo + G * kEvolveWarpInts;
+    for (int c = threadIdx.x; c < ga.C; c += blockDim.x) s_usage[c] = ga.usage[c];
+    usage = s_usage;
+  }
+  if (stopped) return;
+  if (threadIdx.x < 3) s_cnt[threadIdx.x] = 0;
+  __syncthreads();
+  const int lane = threadIdx.x & 31, a = threadIdx.x >> 5;
+  const int s = blockIdx.x;
+  const int g = gen + 1;
+  int32_t *out = nb.cols + (size_t)s * kS;
+  if (s < min(ga.E, n_top)) {  // elitism: copy top-list entry s with its row counts
+    if (a == 0) {
+      const TopEntry &e = ga.top[s];
+      out[lane] = lane < e.len ? e.cols[lane] : 0;
+      out[lane + 32] = lane + 32 < e.len ? e.cols[lane + 32] : 0;
+      if (lane == 0) {
+        nb.len[s] = e.len;
+        nb.hash[s] = e.h;
+        nb.att_dead[s] = 0;
+        nb.att_hits[s] = 0;
+        ga.rows_scr[s] = e.rp;
+        ga.rows_scr[ga.P + s] = e.rn;
+        ga.rows_scr[2 * ga.P + s] = e.ra;
+        dedup_insert(ga.dkeys[par], ga.dslot[par], ga.dmask, e.h, s);
+      }
+    }
+    return;
+  }
+  int32_t *base = s_evo + a * kEvolveWarpInts;
+  if (a < ga.A) {
+    int L = 0;
+    int32_t *c = base + kEvoChild;
+    w_make_child(ga, pb, g, s, a, c, base + kEvoScratch, base + kEvoA, base + kEvoB, L, lane,
+                 usage);
+    const uint64_t h = chromosome_key(c, L);
+    // lane 0 probes the hashed tabu list, lane 1 generation g-1's live keys
+    const bool hit = (lane == 0 && tabu_contains(ga.tabu, ga.tmask, h)) ||
+                     (lane == 1 && tabu_contains(ga.dkeys[par ^ 1], ga.dmask, h));
+    const bool ok = !__any_sync(kFull, hit);
+    if (lane == 0) {
+      s_ok[a] = ok;
+      s_len[a] = L;
+      s_h[a] = h;
+    }
+  }
+  __syncthreads();
+  int win = -1;  // the lowest attempt that misses the tabu list
+  for (int q = 0; q < ga.A; ++q)
+    if (s_ok[q]) {
+      win = q;
+      break;
+    }
+  const bool dead = win < 0;
+  if (dead) win = ga.A - 1;
+  const int32_t *c = s_evo + win * kEvolveWarpInts + kEvoChild;
+  const int L = s_len[win];
+  const bool table = !dead && L == 2 && ga.pair_cnt != nullptr;
+  if (a == win) {
+    out[lane] = lane < L ? c[lane] : 0;
+    out[lane + 32] = lane + 32 < L ? c[lane + 32] : 0;
+    if (lane == 0) {
+      const uint64_t h = s_h[win];
+      nb.len[s] = L;
+      nb.hash[s] = h;
+      // 1: dead; 2 or 3: live and evaluated here (3: from the pair counts)
+      nb.att_dead[s] = dead ? 1 : (table ? 3 : 2);
+      nb.att_hits[s] = dead ? ga.A : win;
+      if (!dead) dedup_insert(ga.dkeys[par], ga.dslot[par], ga.dmask, h, s);
+    }
+  }
+  if (dead) return;
+  if (table) {  // (as in fuse_or_list)
+    if (a == (win + 1) % G && lane == 0) {
+      int ab, ba;
+      pair_counts(ga.pair_cnt, ga.C, c[0], c[1], &ab, &ba);
+      const int R = (int)ga.R, rp = ga.ns ? R - ba : ab;
+      const int rn = !ga.neg ? 0 : (ga.ns ? R - ab : ba);
+      ga.rows_scr[s] = rp;
+      ga.rows_scr[ga.P + s] = rn;
+      ga.rows_scr[2 * ga.P + s] = ga.ns && ga.neg ? R : rp + rn;
+    }
+    return;
+  }
+  int cp = 0, cn = 0, ca = 0;
+  block_eval(ga, c, L, threadIdx.x, blockDim.x, cp, cn, ca);
+  cp = __reduce_add_sync(kFull, cp);
+  cn = __reduce_add_sync(kFull, cn);
+  ca = __reduce_add_sync(kFull, ca);
+  if (lane == 0) {
+    if (cp) atomicAdd(&s_cnt[0], cp);
+    if (cn) atomicAdd(&s_cnt[1], cn);
+    if (ca) atomicAdd(&s_cnt[2], ca);
+  }
+  __syncthreads();
+  if (threadIdx.x < 3) ga.rows_scr[(size_t)threadIdx.x * ga.P + s] = s_cnt[threadIdx.x];
+}
+
 // The same step for large populations, one warp per slot: a slot's attempts run one after the
 // other in its warp, until one misses the tabu list, which is the retry rule itself (the lowest
 // missing attempt wins; all A hit: the slot is dead with the last attempt's child).  Parallel
@@ -1421,23 +1640,34 @@ __device__ __forceinline__ SlotIn load_slot(const GenArgs &ga, const Buf &nb, in
 
 // Scoring, tabu bookkeeping and the top-list update of generation g (parity par).  Every block
 // scores a share of the slots; the last block to finish then runs the single-block part.
-__global__ void __launch_bounds__(kTopThreads, 1) k_finish(GenArgs ga, Buf nb, int par) {
+// Blocks n_fin and on (the loop without an evaluation launch: mv.mv_table set) do its side task
+// instead: the previous generation's keys join the tabu list, its duplicate table is cleared.
+__global__ void __launch_bounds__(kTopThreads, 1) k_finish(GenArgs ga, Buf nb, int par, int n_fin,
+                                                           EvalArgs mv) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int s_hits, s_live, s_lsum, s_fused, s_flsum, s_table, s_last, s_n, s_cnt, s_stop,
       s_nc;
   GenCtl *ctl = ga.ctl;
   wait_prior_grid();
+  if ((int)blockIdx.x >= n_fin) {
+    if (ctl->stopped) return;
+    const int n = items::move_chunks(mv), step = ((int)gridDim.x - n_fin) * (kTopThreads / 32);
+    for (int m = ((int)blockIdx.x - n_fin) * (kTopThreads / 32) + (threadIdx.x >> 5); m < n;
+         m += step)
+      items::move_chunk(mv, m, threadIdx.x & 31);
+    return;
+  }
   // The counters, the list's last entry and this thread's first slot are loaded in one round,
   // ahead of the stop test (which must still come before any store).
   const int stopped = ctl->stopped, n0 = ctl->n_top, gen0 = ctl->gen;
   const uint64_t last_f = ga.top[ga.K - 1].f, last_h = ga.top[ga.K - 1].h;
-  const int tid = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
+  const int tid = blockIdx.x * blockDim.x + threadIdx.x, stride = n_fin * blockDim.x;
   SlotIn first;
   if (tid < ga.P) first = load_slot(ga, nb, par, tid);
   if (stopped) return;
   // A single block keeps the candidates and counters in shared memory; several blocks use the
   // global arrays and counters and hand over to the last block to finish.
-  const bool single = gridDim.x == 1 && ga.P <= ga.sort_cap;
+  const bool single = n_fin == 1 && ga.P <= ga.sort_cap;
   TopSmem sm;
   const int cw = (ga.C + 31) / 32;
   sm.pool = reinterpret_cast<TopEntry *>(smem);
@@ -1544,7 +1774,7 @@ __global__ void __launch_bounds__(kTopThreads, 1) k_finish(GenArgs ga, Buf nb, i
         atomicAdd(reinterpret_cast<unsigned long long *>(&ctl->flen_cur),
                   (unsigned long long)s_flsum);
       __threadfence();
-      s_last = atomicAdd(&ctl->done, 1) == (int)gridDim.x - 1;
+      s_last = atomicAdd(&ctl->done, 1) == n_fin - 1;
     }
     __syncthreads();
     if (!s_last) return;
@@ -1717,6 +1947,7 @@ struct GenState {
   DevBuf rows_scr, work, tabu, top, ctl, usage, cand_f, cand_h, cand_s, extract, todo;
   uint32_t tcap = 0, dcap = 0, ccap = 0;
   int fuse_np = 0;  // pair limit of the evaluation inside the evolve kernel (0: none)
+  bool block_eval = false;  // k_evolve_block evaluates every child (no evaluation launch)
   int seq_blocks = 1;  // blocks of the persistent k_evolve_seq launch
   int32_t sort_cap = 0;
   int finish_blocks = 1;
@@ -1832,7 +2063,7 @@ GenArgs gen_args(ebic_ctx *ctx, GenState *g) {
   ga.ov_num = p.overlap_num;
   ga.ov_den = p.overlap_den;
   ga.tabu_limit = p.tabu_hit_limit;
-  if (g->fuse_np > 0) {
+  if (g->fuse_np > 0 || g->block_eval) {
     ga.bitmap = ctx->bitmap.as<uint32_t>();
     ga.pair_cnt = ctx->pair_cnt_ok ? ctx->pair_cnt.as<unsigned long long>() : nullptr;
     ga.tie_free = ga.pair_cnt && ctx->tie_state == 1;
@@ -1958,6 +2189,13 @@ cudaError_t find_mark_nodes(cudaGraph_t graph, const cudaEvent_t ev[4], cudaGrap
   return cudaSuccess;
 }
 
+cudaError_t launch_finish(ebic_ctx *ctx, GenState *g, int k, const EvalArgs &mv, cudaStream_t s) {
+  const int chunks = mv.mv_table ? (int)((mv.mv_n + 31) / 32) : 0, per = kTopThreads / 32;
+  const int side = (chunks + per - 1) / per;
+  return launch_pdl(k_finish, dim3((unsigned)(g->finish_blocks + side)), dim3(kTopThreads),
+                    g->top_smem, s, gen_args(ctx, g), g->buf(k), k, g->finish_blocks, mv);
+}
+
 // Scoring kernels shared by initialisation and every generation (buffer k was just built;
 // has_prev: a previous generation sits in buffer k ^ 1).
 cudaError_t launch_scoring(ebic_ctx *ctx, GenState *g, int k, bool has_prev, cudaStream_t s,
@@ -1970,9 +2208,7 @@ cudaError_t launch_scoring(ebic_ctx *ctx, GenState *g, int k, bool has_prev, cud
                               gen_view(g, k, listed), ctx->num_sms, s, true)) != cudaSuccess)
     return e;
   if ((e = mark(s, m, 2)) != cudaSuccess) return e;
-  if ((e = launch_pdl(k_finish, dim3(g->finish_blocks), dim3(kTopThreads), g->top_smem, s,
-                      gen_args(ctx, g), g->buf(k), k)) != cudaSuccess)
-    return e;
+  if ((e = launch_finish(ctx, g, k, EvalArgs{}, s)) != cudaSuccess) return e;
   return mark(s, m, 3);
 }
 
@@ -1984,6 +2220,13 @@ cudaError_t launch_generation(ebic_ctx *ctx, GenState *g, int parity, cudaStream
   // A block of G attempt warps per slot while every slot's block fits on the GPU at once (the
   // slot's latency is then the launch's); beyond that a warp per slot, attempts in turn.
   const GenArgs ga = gen_args(ctx, g);
+  // (while kernel statistics are on, the three launches run apart so that each can be timed)
+  if (g->block_eval && !m) {
+    e = launch_pdl(k_evolve_block, dim3((unsigned)g->P), dim3(G * 32), evolve_smem(G, g->C), s,
+                   ga, g->buf(parity ^ 1), g->buf(parity), parity);
+    if (e != cudaSuccess) return e;
+    return launch_finish(ctx, g, parity, gen_eval_args(ctx, g, parity, true), s);
+  }
   const bool tf = ga.fuse_np > 0 && ga.neg && ga.tie_free;
   if ((int64_t)g->P * G <= (int64_t)ctx->num_sms * kEvolveResidentWarps) {
     e = launch_pdl(tf ? k_evolve<true> : k_evolve<false>, dim3((unsigned)g->P), dim3(G * 32), evolve_smem(G, g->C), s, ga,
@@ -2126,6 +2369,9 @@ int gen_create(ebic_ctx *ctx, const ebic_params *p) {
   for (const auto k : {k_evolve<false>, k_evolve<true>})
     EBIC_CHECK_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)evolve_smem(kMaxAttemptWarps, kUsageSmemMax)));
+  EBIC_CHECK_CUDA(ctx, cudaFuncSetAttribute(k_evolve_block,
+                                            cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            (int)evolve_smem(kBlockWarps, kUsageSmemMax)));
   for (const auto k : {k_evolve_seq<false>, k_evolve_seq<true>})
     EBIC_CHECK_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)evolve_smem(kSeqWarps, kUsageSmemMax)));
@@ -2202,6 +2448,22 @@ int fuse_limit(const ebic_ctx *ctx, int mode, const ebic_params *p) {
   return (int)std::min<int64_t>(EBIC_MAX_LEN - 1, kFuseDefaultUnits / per_pair);
 }
 
+// Whether the loop evaluates every child in k_evolve_block: the bitmap form in the block-per-slot
+// regime (every slot's block resident at once, at most kBlockWarps attempts), no pair limit set
+// (the caller's -1 keeps the evaluation launch), and pair rows short enough that a block's threads
+// cover one in kBlockMaxSteps steps of four words.
+bool block_eval_fits(const ebic_ctx *ctx, int mode, const ebic_params *p, int fuse) {
+  int G = 1;
+  while (G < p->max_attempts) G <<= 1;
+  return mode == EBIC_MODE_BITMAP && fuse == 0 && p->fuse_pairs >= 0 && !p->last_kept &&
+         G <= kBlockWarps &&
+         (int64_t)p->pop_size * G <= (int64_t)ctx->num_sms * kEvolveResidentWarps &&
+         (int64_t)p->pop_size <= (int64_t)ctx->num_sms *
+                                     resident_blocks((const void *)k_evolve_block, G * 32,
+                                                     evolve_smem(G, ctx->C)) &&
+         ctx->Gst <= (int64_t)kBlockMaxSteps * 4 * G * 32;
+}
+
 int ensure_eval_ready(ebic_ctx *ctx, GenState *g, const ebic_params *p, int n_gen) {
   int mode = choose_mode(ctx, p->mode, g->P, 0.5 * (p->init_min_len + p->max_len), n_gen + 1,
                          p->last_kept);
@@ -2214,12 +2476,13 @@ int ensure_eval_ready(ebic_ctx *ctx, GenState *g, const ebic_params *p, int n_ge
                     : (direct && ctx->codes_ready ? ctx->codes.p : nullptr);
   // (and the fusion limit, which the captured evolve launches hold)
   const int fuse = fuse_limit(ctx, mode, p);
+  const bool block = block_eval_fits(ctx, mode, p, fuse);
   const void *cnt = mode == EBIC_MODE_BITMAP && ctx->pair_cnt_ok ? ctx->pair_cnt.p : nullptr;
   if (mode == EBIC_MODE_BITMAP && p->neg_trends &&
       (fuse > 1 || (p->ratio_num < p->ratio_den && eval_args_for(ctx).stage_bitmap)))
     EBIC_TRY(ensure_tie_state(ctx));
   if (mode != g->eval_mode || buf != g->graph_buf || fuse != g->fuse_np ||
-      cnt != g->graph_cnt || ctx->tie_state != g->graph_tie) {
+      cnt != g->graph_cnt || ctx->tie_state != g->graph_tie || block != g->block_eval) {
     g->drop_graphs();
     g->graph_tie = ctx->tie_state;
     g->graph_buf = buf;
@@ -2227,6 +2490,7 @@ int ensure_eval_ready(ebic_ctx *ctx, GenState *g, const ebic_params *p, int n_ge
   }
   g->eval_mode = mode;
   g->fuse_np = fuse;
+  g->block_eval = block;
   return EBIC_OK;
 }
 

@@ -105,7 +105,9 @@ int tune_loop(ebic_ctx *ctx, const ebic_params *p, int gens, int ipw_max, int *b
     ctx->seg_loop = 0;
     ctx->ipw_loop = 1;
     for (int f : kLoopFuseCandidates) {
-      q.fuse_pairs = f;
+      // (none: the library's own form without a limit, as a caller that sets nothing gets it)
+      ctx->fuse_loop = f < 0 ? f : 0;
+      q.fuse_pairs = f < 0 ? 0 : f;
       float ms = 0.f;
       time_loop(&ms);
       if (status != EBIC_OK) break;
@@ -114,7 +116,8 @@ int tune_loop(ebic_ctx *ctx, const ebic_params *p, int gens, int ipw_max, int *b
         best_fuse = f;
       }
     }
-    q.fuse_pairs = best_fuse;
+    ctx->fuse_loop = best_fuse < 0 ? best_fuse : 0;
+    q.fuse_pairs = best_fuse < 0 ? 0 : best_fuse;
   }
   best = DBL_MAX;
   int best_seg = 0, best_ipw = 1;
