@@ -117,6 +117,7 @@ bool ebic_is_device_ptr(const void *p) {
 // The context's pinned block (see ebic_ctx::pin).  Pinning host memory takes a few hundred
 // microseconds, so blocks of closed contexts are kept for the next ones, up to kPinKeep of them.
 constexpr size_t kPinStatus = 256, kPinIn = 256 << 10, kPinOut = 256 << 10;
+static_assert(kPinIn + kPinOut == kPinSpare, "the pinned block's size");
 constexpr size_t kPinKeep = 8;
 static std::mutex g_pin_mu;
 static unsigned char *g_pin_free[kPinKeep];
@@ -311,7 +312,10 @@ int stage_population(ebic_ctx *ctx, const int32_t *col_idx, const int32_t *offse
     int32_t herr = 0;
     EBIC_CHECK_CUDA(ctx, cudaMemcpyAsync(&herr, ctx->d_err.p, 4, cudaMemcpyDeviceToHost, s));
     EBIC_CHECK_CUDA(ctx, cudaStreamSynchronize(s));
-    if (herr) return ebic_fail(ctx, EBIC_EINVAL, "invalid chromosome in the population");
+    if (herr) {
+      EBIC_CHECK_CUDA(ctx, cudaMemsetAsync(ctx->d_err.p, 0, sizeof(int32_t), s));
+      return ebic_fail(ctx, EBIC_EINVAL, "invalid chromosome in the population");
+    }
     if (want_host_offsets) h_off.assign(offsets, offsets + n_ind + 1);
   } else {
     // Device CSR: validate on the device before any kernel indexes the matrix with it.
@@ -330,7 +334,10 @@ int stage_population(ebic_ctx *ctx, const int32_t *col_idx, const int32_t *offse
                                            cudaMemcpyDeviceToHost, s));
     }
     EBIC_CHECK_CUDA(ctx, cudaStreamSynchronize(s));
-    if (herr) return ebic_fail(ctx, EBIC_EINVAL, "invalid chromosome in the population");
+    if (herr) {
+      EBIC_CHECK_CUDA(ctx, cudaMemsetAsync(ctx->d_err.p, 0, sizeof(int32_t), s));
+      return ebic_fail(ctx, EBIC_EINVAL, "invalid chromosome in the population");
+    }
     total = (int64_t)ends[1] - ends[0];
     mean_len = (double)total / n_ind;
   }
@@ -435,8 +442,9 @@ int ebic_create(ebic_ctx **out, int32_t device, void *cuda_stream) {
       ctx->d_ties.ensure(64, ctx->stream) != cudaSuccess ||
       ctx->d_work.ensure(64, ctx->stream) != cudaSuccess ||
       ctx->d_kerr.ensure(64, ctx->stream) != cudaSuccess ||
-      cudaMemset(ctx->d_kerr.p, 0, 64) != cudaSuccess ||
-      cudaMemset(ctx->d_work.p, 0, 64) != cudaSuccess ||
+      cudaMemsetAsync(ctx->d_kerr.p, 0, 64, ctx->stream) != cudaSuccess ||
+      cudaMemsetAsync(ctx->d_work.p, 0, 64, ctx->stream) != cudaSuccess ||
+      cudaMemsetAsync(ctx->d_err.p, 0, 64, ctx->stream) != cudaSuccess ||
       !(ctx->pin = take_pin())) {
     cudaGetLastError();
     ebic_destroy(ctx);
@@ -501,6 +509,18 @@ void ctx_release_buffers(ebic_ctx *ctx) {
 
 namespace {
 
+// Waits for the uploads of a load and reads their error word, which is 0 between calls.
+int read_upload_error(ebic_ctx *ctx) {
+  EBIC_CHECK_CUDA(ctx, cudaMemcpyAsync(ctx->pin, ctx->d_err.p, sizeof(int32_t),
+                                       cudaMemcpyDeviceToHost, ctx->stream));
+  EBIC_CHECK_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+  int32_t herr = 0;
+  memcpy(&herr, ctx->pin, sizeof(herr));
+  if (!herr) return EBIC_OK;
+  EBIC_CHECK_CUDA(ctx, cudaMemsetAsync(ctx->d_err.p, 0, sizeof(int32_t), ctx->stream));
+  return ebic_fail(ctx, EBIC_ENAN, "matrix holds NaN or Inf");
+}
+
 // The segmented load of a row-major host matrix (see ebic_load_matrix): kLoadSegments segments
 // of a multiple of 8,192 rows (whole 1,024-row chunks of the bitmap, whole tiles of every
 // kernel), the last one with the padded tail.
@@ -520,9 +540,7 @@ int load_matrix_segmented(ebic_ctx *ctx, const float *x, int64_t rows, int32_t c
     EBIC_CHECK_CUDA(ctx, ctx->planes.ensure((size_t)code_plane_words(cols, Gst) * 4, s));
     EBIC_CHECK_CUDA(ctx, ctx->bitmap.ensure((size_t)(C * C * Gst) * 4, s));
     EBIC_CHECK_CUDA(ctx, prepare_bitmap_eval());
-    const size_t nc = (size_t)C * C * sizeof(unsigned long long);
-    EBIC_CHECK_CUDA(ctx, ctx->pair_cnt.ensure(nc, s));
-    EBIC_CHECK_CUDA(ctx, cudaMemsetAsync(ctx->pair_cnt.p, 0, nc, s));
+    EBIC_CHECK_CUDA(ctx, ctx->pair_cnt.ensure((size_t)C * C * sizeof(unsigned long long), s));
   }
   if (!ctx->copy_stream)
     EBIC_CHECK_CUDA(ctx, cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking));
@@ -538,7 +556,6 @@ int load_matrix_segmented(ebic_ctx *ctx, const float *x, int64_t rows, int32_t c
   // staging buffer)
   EBIC_CHECK_CUDA(ctx, cudaEventRecord(ctx->seg_ev[n_seg], s));
   EBIC_CHECK_CUDA(ctx, cudaStreamWaitEvent(ctx->copy_stream, ctx->seg_ev[n_seg], 0));
-  EBIC_CHECK_CUDA(ctx, cudaMemsetAsync(ctx->d_err.p, 0, sizeof(int32_t), s));
   float *stage = ctx->stage_x.as<float>();
   for (int64_t i = 0; i < n_seg; ++i) {
     const int64_t r0 = i * seg, r1 = std::min(R_pad, r0 + seg);
@@ -557,8 +574,9 @@ int load_matrix_segmented(ebic_ctx *ctx, const float *x, int64_t rows, int32_t c
     prof_count(ctx, EBIC_KERNEL_RANK_CODES, 1);
     if (bitmap) {  // (a segment is a multiple of 2,048 rows: whole chunks of planes)
       EBIC_CHECK_CUDA(ctx, launch_code_planes(ctx->codes.p, cb, S, cols, Gst,
-                                              ctx->planes.as<uint32_t>(), s, r0 / 2048,
-                                              r1 < R_pad ? r1 / 2048 : -1));
+                                              ctx->planes.as<uint32_t>(),
+                                              i ? nullptr : ctx->pair_cnt.as<unsigned long long>(),
+                                              s, r0 / 2048, r1 < R_pad ? r1 / 2048 : -1));
       prof_count(ctx, -1, 1);
     }
   }
@@ -570,11 +588,7 @@ int load_matrix_segmented(ebic_ctx *ctx, const float *x, int64_t rows, int32_t c
     prof_count(ctx, EBIC_KERNEL_BITMAP_BUILD, 1);
     ctx->tie_state = -1;
   }
-  int32_t herr = 0;
-  EBIC_CHECK_CUDA(ctx, cudaMemcpyAsync(&herr, ctx->d_err.p, sizeof(int32_t),
-                                       cudaMemcpyDeviceToHost, s));
-  EBIC_CHECK_CUDA(ctx, cudaStreamSynchronize(s));
-  if (herr) return ebic_fail(ctx, EBIC_ENAN, "matrix holds NaN or Inf");
+  EBIC_TRY(read_upload_error(ctx));
   ctx->R = rows;
   ctx->C = cols;
   ctx->R_pad = R_pad;
@@ -635,15 +649,10 @@ int ebic_load_matrix(ebic_ctx *ctx, const float *x, int64_t rows, int32_t cols, 
                                          cudaMemcpyHostToDevice, ctx->stream));
     src = ctx->stage_x.as<float>();
   }
-  EBIC_CHECK_CUDA(ctx, cudaMemsetAsync(ctx->d_err.p, 0, sizeof(int32_t), ctx->stream));
   EBIC_CHECK_CUDA(ctx, launch_upload(src, rows, cols, R_pad, layout, ctx->keys.as<uint32_t>(),
                                      ctx->d_err.as<int32_t>(), ctx->stream));
   prof_count(ctx, -1, 1);
-  int32_t herr = 0;
-  EBIC_CHECK_CUDA(ctx, cudaMemcpyAsync(&herr, ctx->d_err.p, sizeof(int32_t),
-                                       cudaMemcpyDeviceToHost, ctx->stream));
-  EBIC_CHECK_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-  if (herr) return ebic_fail(ctx, EBIC_ENAN, "matrix holds NaN or Inf");
+  EBIC_TRY(read_upload_error(ctx));
   ctx->R = rows;
   ctx->C = cols;
   ctx->R_pad = R_pad;
@@ -669,11 +678,10 @@ int ebic_build_bitmap(ebic_ctx *ctx) {
   EBIC_CHECK_CUDA(ctx, prepare_bitmap_eval());
   // With rank codes (C <= 1,024) the words come from the codes' bit planes, else from the keys.
   if (ctx->code_bytes) EBIC_TRY(ensure_codes(ctx));
-  // (and the pair counts, C * C words, accumulated by the same kernel)
+  // (and the pair counts, C * C words, cleared with the planes and accumulated with the words)
   if (ctx->code_bytes) {
     const size_t nc = (size_t)ctx->C * ctx->C * sizeof(unsigned long long);
     EBIC_CHECK_CUDA(ctx, ctx->pair_cnt.ensure(nc, ctx->stream));
-    EBIC_CHECK_CUDA(ctx, cudaMemsetAsync(ctx->pair_cnt.p, 0, nc, ctx->stream));
     EBIC_CHECK_CUDA(ctx, ctx->planes.ensure((size_t)code_plane_words(ctx->C, ctx->Gst) * 4,
                                             ctx->stream));
   }
@@ -681,6 +689,7 @@ int ebic_build_bitmap(ebic_ctx *ctx) {
   if (ctx->code_bytes) {
     EBIC_CHECK_CUDA(ctx, launch_code_planes(ctx->codes.p, ctx->code_bytes, ctx->code_stride,
                                             ctx->C, ctx->Gst, ctx->planes.as<uint32_t>(),
+                                            ctx->pair_cnt.as<unsigned long long>(),
                                             ctx->stream));
     prof_count(ctx, -1, 1);
     EBIC_CHECK_CUDA(ctx, launch_build_bitmap_planes(ctx->planes.as<uint32_t>(), ctx->C, ctx->Gst,

@@ -367,8 +367,13 @@ template <int W, int NB>
 __global__ void __launch_bounds__(kThreads) k_code_planes(const uint8_t *__restrict__ codes,
                                                           int64_t S, int32_t C, int64_t chunks,
                                                           int64_t ch0, int64_t ch1,
-                                                          uint32_t *__restrict__ planes) {
+                                                          uint32_t *__restrict__ planes,
+                                                          unsigned long long *__restrict__ cnt) {
   const int lane = threadIdx.x & 31;
+  if (cnt)  // the pair counts, which the build accumulates, cleared beside
+    for (int64_t q = (int64_t)blockIdx.x * kThreads + threadIdx.x; q < (int64_t)C * C;
+         q += (int64_t)gridDim.x * kThreads)
+      cnt[q] = 0ull;
   const int64_t halves = 2 * (ch1 - ch0);
   const int64_t id = (int64_t)blockIdx.x * kWarps + (threadIdx.x >> 5);
   const int64_t c = id / halves, h = id - c * halves;
@@ -574,8 +579,8 @@ int64_t code_plane_words(int32_t C, int64_t Wst) {
 }
 
 cudaError_t launch_code_planes(const void *codes, int code_bytes, int64_t S, int32_t C,
-                               int64_t Wst, uint32_t *planes, cudaStream_t s, int64_t ch0,
-                               int64_t ch1) {
+                               int64_t Wst, uint32_t *planes, unsigned long long *cnt,
+                               cudaStream_t s, int64_t ch0, int64_t ch1) {
   const int64_t chunks = code_plane_chunks(Wst);
   if (ch1 < 0 || ch1 > chunks) ch1 = chunks;
   if (C < 2 || C > 1024 || code_bytes != (C <= 128 ? 1 : 2) || ch0 < 0 || ch0 >= ch1)
@@ -585,7 +590,7 @@ cudaError_t launch_code_planes(const void *codes, int code_bytes, int64_t S, int
   const uint8_t *cd = static_cast<const uint8_t *>(codes);
 #define EBIC_PLANES(W, NB)                                                               \
   case NB:                                                                               \
-    k_code_planes<W, NB><<<grid, kThreads, 0, s>>>(cd, S, C, chunks, ch0, ch1, planes); \
+    k_code_planes<W, NB><<<grid, kThreads, 0, s>>>(cd, S, C, chunks, ch0, ch1, planes, cnt); \
     break
   switch (code_plane_bits(C)) {
     EBIC_PLANES(1, 1);

@@ -1919,6 +1919,30 @@ __global__ void __launch_bounds__(256) k_extract(const uint32_t *__restrict__ ke
   if (lane == 0) out[(int64_t)e * Wst + w] = m;
 }
 
+// Clears the run state in one launch (segments of 4-byte words, each from a 16-byte boundary) and
+// sets the counters; sixteen separate clears cost a launch each.
+struct ResetSegs {
+  uint32_t *p[14];
+  int64_t words[14];
+};
+
+__global__ void __launch_bounds__(256) k_reset(ResetSegs sg, GenCtl *ctl) {
+  const int64_t tid = (int64_t)blockIdx.x * 256 + threadIdx.x, n = (int64_t)gridDim.x * 256;
+#pragma unroll 1
+  for (int k = 0; k < 14; ++k) {
+    uint4 *v = reinterpret_cast<uint4 *>(sg.p[k]);
+    const int64_t quads = sg.words[k] / 4;
+    for (int64_t q = tid; q < quads; q += n) v[q] = make_uint4(0u, 0u, 0u, 0u);
+    const int64_t tail = 4 * quads + tid;
+    if (tail < sg.words[k]) sg.p[k][tail] = 0u;
+  }
+  if (tid == 0) {
+    GenCtl c{};
+    c.gen = -1;
+    *ctl = c;
+  }
+}
+
 __global__ void k_rehash(const uint64_t *old_keys, uint32_t old_cap, uint64_t *keys,
                          uint32_t mask) {
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -2293,24 +2317,31 @@ namespace {
 // Clears the run state of g (population, duplicate tables, tabu list, top list, column usage,
 // counters) on the context stream; buffers and graphs stay.
 int gen_reset(ebic_ctx *ctx, GenState *g) {
-  const size_t P = (size_t)g->P;
+  const int64_t P = g->P;
+  ResetSegs sg{};
+  int n = 0;
+  int64_t total = 0;
+  auto add = [&](const DevBuf &b, int64_t words) {
+    sg.p[n] = b.as<uint32_t>();
+    sg.words[n++] = words;
+    total += words;
+  };
   for (int k = 0; k < 2; ++k) {
-    EBIC_CHECK_CUDA(ctx, cudaMemsetAsync(g->cols[k].p, 0, P * kS * 4, ctx->stream));
-    EBIC_CHECK_CUDA(ctx, cudaMemsetAsync(g->len[k].p, 0, P * 4, ctx->stream));
-    EBIC_CHECK_CUDA(ctx, cudaMemsetAsync(g->fit[k].p, 0, P * 8, ctx->stream));
-    EBIC_CHECK_CUDA(ctx, cudaMemsetAsync(g->dkeys[k].p, 0, (size_t)g->dcap * 8, ctx->stream));
-    EBIC_CHECK_CUDA(ctx, cudaMemsetAsync(g->dslot[k].p, 0, (size_t)g->dcap * 4, ctx->stream));
+    add(g->cols[k], P * kS);
+    add(g->len[k], P);
+    add(g->fit[k], P * 2);
+    add(g->dkeys[k], (int64_t)g->dcap * 2);
+    add(g->dslot[k], (int64_t)g->dcap);
   }
-  EBIC_CHECK_CUDA(ctx, cudaMemsetAsync(g->rows_scr.p, 0, P * 3 * 4, ctx->stream));
+  add(g->rows_scr, P * 3);
+  add(g->usage, g->C);
+  add(g->top, (int64_t)g->K * (int64_t)sizeof(TopEntry) / 4);
+  add(g->tabu, (int64_t)g->tcap * 2);
   EBIC_CHECK_CUDA(ctx, cudaMemsetAsync(g->work.p, 0, 64, ctx->stream));
-  EBIC_CHECK_CUDA(ctx, cudaMemsetAsync(g->usage.p, 0, (size_t)g->C * 4, ctx->stream));
-  EBIC_CHECK_CUDA(ctx, cudaMemsetAsync(g->top.p, 0, (size_t)g->K * sizeof(TopEntry), ctx->stream));
-  if (g->tcap) EBIC_CHECK_CUDA(ctx, cudaMemsetAsync(g->tabu.p, 0, (size_t)g->tcap * 8, ctx->stream));
-  GenCtl c0{};
-  c0.gen = -1;
-  // (a copy from pageable memory has taken its source before the call returns)
-  EBIC_CHECK_CUDA(ctx, cudaMemcpyAsync(g->ctl.p, &c0, sizeof(c0), cudaMemcpyHostToDevice,
-                                       ctx->stream));
+  const int64_t blocks = std::min<int64_t>((total / 4 + 255) / 256 + 1, (int64_t)ctx->num_sms * 8);
+  k_reset<<<(unsigned)blocks, 256, 0, ctx->stream>>>(sg, g->ctl.as<GenCtl>());
+  EBIC_CHECK_CUDA(ctx, cudaGetLastError());
+  prof_count(ctx, -1, 1);
   g->initialised = false;
   g->reset_pending = false;
   return EBIC_OK;
@@ -2394,10 +2425,16 @@ int gen_create(ebic_ctx *ctx, const ebic_params *p) {
   return gen_reset(ctx, g);
 }
 
+// (through the context's pinned block: a copy to pageable memory is slower)
+constexpr size_t kPinCtl = 64, kPinTop = 256;  // offsets: the counters, and what else is read
+static_assert(kPinCtl + sizeof(GenCtl) <= kPinTop, "the counters' place in the pinned block");
+static_assert(EBIC_MAX_BICLUSTERS * sizeof(TopEntry) <= kPinSpare, "the top list's place");
+
 int read_ctl(ebic_ctx *ctx, GenState *g, GenCtl *out) {
-  EBIC_CHECK_CUDA(ctx, cudaMemcpyAsync(out, g->ctl.p, sizeof(GenCtl), cudaMemcpyDeviceToHost,
-                                       ctx->stream));
+  EBIC_CHECK_CUDA(ctx, cudaMemcpyAsync(ctx->pin + kPinCtl, g->ctl.p, sizeof(GenCtl),
+                                       cudaMemcpyDeviceToHost, ctx->stream));
   EBIC_CHECK_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+  memcpy(out, ctx->pin + kPinCtl, sizeof(GenCtl));
   return EBIC_OK;
 }
 
@@ -2582,7 +2619,8 @@ int ebic_run_generations(ebic_ctx *ctx, const ebic_params *p, int32_t n_gen,
   g->p.fuse_pairs = p->fuse_pairs;
   EBIC_TRY(ensure_eval_ready(ctx, g, p, n_gen));
   GenCtl c{};
-  EBIC_TRY(read_ctl(ctx, g, &c));
+  c.gen = -1;  // (a run that is not initialised: as gen_reset left the counters)
+  if (g->initialised) EBIC_TRY(read_ctl(ctx, g, &c));
   EBIC_TRY(ensure_tabu(ctx, g, c.tabu_count + (int64_t)g->P * ((int64_t)n_gen + 2)));
   cudaStream_t s = ctx->stream;
   const GenCtl c_start = c;
@@ -2598,7 +2636,7 @@ int ebic_run_generations(ebic_ctx *ctx, const ebic_params *p, int32_t n_gen,
     prof_count(ctx, EBIC_KERNEL_FINISH, 1);
     prof_count(ctx, -1, 1);
     g->initialised = true;
-    EBIC_TRY(read_ctl(ctx, g, &c));
+    c.gen = 0;  // (the initial population never ends the run: what is scored next is known)
   }
   if (!c.stopped) {
     for (int i = 0; i < n_gen; ++i) {
@@ -2640,12 +2678,11 @@ int ebic_run_generations(ebic_ctx *ctx, const ebic_params *p, int32_t n_gen,
     }
   }
   // the counters and the kernels' error word, in one synchronisation
+  EBIC_CHECK_CUDA(ctx, cudaMemcpyAsync(ctx->pin + kPinTop, ctx->d_kerr.p, 4,
+                                       cudaMemcpyDeviceToHost, ctx->stream));
+  EBIC_TRY(read_ctl(ctx, g, &c));
   int32_t kerr = 0;
-  EBIC_CHECK_CUDA(ctx, cudaMemcpyAsync(&c, g->ctl.p, sizeof(GenCtl), cudaMemcpyDeviceToHost,
-                                       ctx->stream));
-  EBIC_CHECK_CUDA(ctx, cudaMemcpyAsync(&kerr, ctx->d_kerr.p, 4, cudaMemcpyDeviceToHost,
-                                       ctx->stream));
-  EBIC_CHECK_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+  memcpy(&kerr, ctx->pin + kPinTop, 4);
   if (kerr) {
     cudaMemset(ctx->d_kerr.p, 0, 4);
     return ebic_fail(ctx, EBIC_ETIMEOUT, "a bounded device wait expired in the generation loop");
@@ -2692,33 +2729,37 @@ int ebic_get_toplist(ebic_ctx *ctx, int32_t capacity, int32_t *n_top, int32_t *c
   GenState *g = ctx->gen;
   if (!g || !g->initialised) return ebic_fail(ctx, EBIC_ESTATE, "no run");
   cudaSetDevice(ctx->device);
+  // the counters and the list in one synchronisation
+  EBIC_CHECK_CUDA(ctx, cudaMemcpyAsync(ctx->pin + kPinTop, g->top.p, sizeof(TopEntry) * g->K,
+                                       cudaMemcpyDeviceToHost, ctx->stream));
   GenCtl c{};
   EBIC_TRY(read_ctl(ctx, g, &c));
   if (capacity < c.n_top) return ebic_fail(ctx, EBIC_EINVAL, "capacity below the list size");
-  std::vector<TopEntry> host(c.n_top > 0 ? c.n_top : 1);
-  if (c.n_top > 0)
-    EBIC_CHECK_CUDA(ctx, cudaMemcpy(host.data(), g->top.p, sizeof(TopEntry) * c.n_top,
-                                    cudaMemcpyDeviceToHost));
-  std::vector<int32_t> hc((size_t)c.n_top * kS, 0), hl(c.n_top), hr((size_t)c.n_top * 3);
-  std::vector<uint64_t> hf(c.n_top), hk(c.n_top);
-  for (int e = 0; e < c.n_top; ++e) {
-    for (int k = 0; k < host[e].len; ++k) hc[(size_t)e * kS + k] = host[e].cols[k];
-    hl[e] = host[e].len;
-    hf[e] = host[e].f;
-    hk[e] = host[e].h;
-    hr[e * 3] = host[e].rp;
-    hr[e * 3 + 1] = host[e].rn;
-    hr[e * 3 + 2] = host[e].ra;
+  const TopEntry *top = reinterpret_cast<const TopEntry *>(ctx->pin + kPinTop);
+  const size_t n = (size_t)c.n_top;
+  std::vector<int32_t> hc(n * kS, 0), hl(n), hr(n * 3);
+  std::vector<uint64_t> hf(n), hk(n);
+  for (size_t e = 0; e < n; ++e) {
+    for (int k = 0; k < top[e].len; ++k) hc[e * kS + k] = top[e].cols[k];
+    hl[e] = top[e].len;
+    hf[e] = top[e].f;
+    hk[e] = top[e].h;
+    hr[e * 3] = top[e].rp;
+    hr[e * 3 + 1] = top[e].rn;
+    hr[e * 3 + 2] = top[e].ra;
   }
   if (n_top) *n_top = c.n_top;
-  if (c.n_top > 0) {
-    if (cols) EBIC_CHECK_CUDA(ctx, cudaMemcpy(cols, hc.data(), hc.size() * 4, cudaMemcpyDefault));
-    if (lens) EBIC_CHECK_CUDA(ctx, cudaMemcpy(lens, hl.data(), hl.size() * 4, cudaMemcpyDefault));
-    if (fitness)
-      EBIC_CHECK_CUDA(ctx, cudaMemcpy(fitness, hf.data(), hf.size() * 8, cudaMemcpyDefault));
-    if (keys) EBIC_CHECK_CUDA(ctx, cudaMemcpy(keys, hk.data(), hk.size() * 8, cudaMemcpyDefault));
-    if (rows) EBIC_CHECK_CUDA(ctx, cudaMemcpy(rows, hr.data(), hr.size() * 4, cudaMemcpyDefault));
-  }
+  auto give = [&](void *dst, const void *src, size_t bytes) -> cudaError_t {
+    if (!dst || !bytes) return cudaSuccess;
+    if (ebic_is_device_ptr(dst)) return cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice);
+    memcpy(dst, src, bytes);
+    return cudaSuccess;
+  };
+  EBIC_CHECK_CUDA(ctx, give(cols, hc.data(), hc.size() * 4));
+  EBIC_CHECK_CUDA(ctx, give(lens, hl.data(), hl.size() * 4));
+  EBIC_CHECK_CUDA(ctx, give(fitness, hf.data(), hf.size() * 8));
+  EBIC_CHECK_CUDA(ctx, give(keys, hk.data(), hk.size() * 8));
+  EBIC_CHECK_CUDA(ctx, give(rows, hr.data(), hr.size() * 4));
   return EBIC_OK;
 }
 
@@ -2746,28 +2787,43 @@ int ebic_extract_biclusters(ebic_ctx *ctx, int32_t capacity, uint32_t *rowmask, 
   if (!g || !g->initialised) return ebic_fail(ctx, EBIC_ESTATE, "no run");
   if (!rowmask) return ebic_fail(ctx, EBIC_EINVAL, "rowmask is NULL");
   cudaSetDevice(ctx->device);
-  GenCtl c{};
-  EBIC_TRY(read_ctl(ctx, g, &c));
-  if (capacity < c.n_top) return ebic_fail(ctx, EBIC_EINVAL, "capacity below the list size");
-  const size_t words = (size_t)c.n_top * ctx->Wst;
   const bool dev = ebic_is_device_ptr(rowmask);
-  uint32_t *dst = rowmask;
-  if (!dev) {
-    EBIC_CHECK_CUDA(ctx, g->extract.ensure(words * 4 + 4, ctx->stream));
-    dst = g->extract.as<uint32_t>();
-  }
-  if (words) {
-    const int64_t threads = (int64_t)words * 32;
+  const size_t entry = (size_t)ctx->Wst * 4, all = entry * (size_t)g->K;
+  auto extract = [&](uint32_t *dst, size_t entries) -> cudaError_t {  // (the kernel reads n_top)
+    const int64_t threads = (int64_t)(entries * ctx->Wst) * 32;
     k_extract<<<(unsigned)((threads + 255) / 256), 256, 0, ctx->stream>>>(
         ctx->keys.as<uint32_t>(), ctx->R, ctx->R_pad, ctx->Wst, g->top.as<TopEntry>(),
         g->ctl.as<GenCtl>(), g->p.neg_trends, g->p.ratio_num, g->p.ratio_den, dst);
-    EBIC_CHECK_CUDA(ctx, cudaGetLastError());
     prof_count(ctx, -1, 1);
-    if (!dev)
-      EBIC_CHECK_CUDA(ctx, cudaMemcpyAsync(rowmask, dst, words * 4, cudaMemcpyDeviceToHost,
-                                           ctx->stream));
+    return cudaGetLastError();
+  };
+  GenCtl c{};
+  if (!dev && all <= kPinSpare) {
+    // small masks: extraction of the whole list, its copy and the counters in one synchronisation
+    EBIC_CHECK_CUDA(ctx, g->extract.ensure(all, ctx->stream));
+    EBIC_CHECK_CUDA(ctx, extract(g->extract.as<uint32_t>(), (size_t)g->K));
+    EBIC_CHECK_CUDA(ctx, cudaMemcpyAsync(ctx->pin + kPinTop, g->extract.p, all,
+                                         cudaMemcpyDeviceToHost, ctx->stream));
+    EBIC_TRY(read_ctl(ctx, g, &c));
+    if (capacity < c.n_top) return ebic_fail(ctx, EBIC_EINVAL, "capacity below the list size");
+    memcpy(rowmask, ctx->pin + kPinTop, entry * (size_t)c.n_top);
+  } else {
+    EBIC_TRY(read_ctl(ctx, g, &c));
+    if (capacity < c.n_top) return ebic_fail(ctx, EBIC_EINVAL, "capacity below the list size");
+    const size_t bytes = entry * (size_t)c.n_top;
+    uint32_t *dst = rowmask;
+    if (!dev) {
+      EBIC_CHECK_CUDA(ctx, g->extract.ensure(bytes + 4, ctx->stream));
+      dst = g->extract.as<uint32_t>();
+    }
+    if (bytes) {
+      EBIC_CHECK_CUDA(ctx, extract(dst, (size_t)c.n_top));
+      if (!dev)
+        EBIC_CHECK_CUDA(ctx, cudaMemcpyAsync(rowmask, dst, bytes, cudaMemcpyDeviceToHost,
+                                             ctx->stream));
+    }
+    EBIC_CHECK_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
   }
-  EBIC_CHECK_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
   if (n_out) *n_out = c.n_top;
   return EBIC_OK;
 }
@@ -2871,6 +2927,7 @@ int ebic_load_state(ebic_ctx *ctx, const ebic_params *p, const void *blob, int64
     return ebic_fail(ctx, EBIC_EINVAL, "state blob does not match this matrix and parameters");
   cudaSetDevice(ctx->device);
   EBIC_TRY(gen_create(ctx, p));
+  EBIC_CHECK_CUDA(ctx, cudaStreamSynchronize(ctx->stream));  // (before the copies below)
   GenState *g = ctx->gen;
   if (size < state_fixed_size(g) + h.n_tabu * 8)
     return ebic_fail(ctx, EBIC_EINVAL, "blob truncated");

@@ -153,7 +153,7 @@ struct EvalArgs {
 // (zero-fills the padding), and the direct evaluation over codes.  The codes' bit planes (bits of
 // C - 1 per column) are the pair-bitmap build's operand, [C][chunks][bits][64] words:
 // code_plane_words in all, by chunks of 64 words of a column's rows (launch_code_planes: chunks
-// [ch0, ch1) only, ch1 < 0: to the end).
+// [ch0, ch1) only, ch1 < 0: to the end; it also clears the C * C pair counts cnt when not null).
 int code_bytes_for(int32_t C);
 int64_t code_rows_per_pass(int code_bytes);
 int64_t code_stride_for(int64_t R, int code_bytes);
@@ -170,8 +170,8 @@ cudaError_t launch_rank_codes_rows(const uint32_t *keys, int64_t R_pad, int32_t 
                                    int code_bytes, int64_t S, int num_sms, int64_t r_begin,
                                    int64_t r_end, cudaStream_t s);
 cudaError_t launch_code_planes(const void *codes, int code_bytes, int64_t S, int32_t C,
-                               int64_t Wst, uint32_t *planes, cudaStream_t s, int64_t ch0 = 0,
-                               int64_t ch1 = -1);
+                               int64_t Wst, uint32_t *planes, unsigned long long *cnt,
+                               cudaStream_t s, int64_t ch0 = 0, int64_t ch1 = -1);
 cudaError_t launch_eval_codes(const EvalArgs &a, const PopView &pv, int num_sms, cudaStream_t s,
                               bool pdl);
 
@@ -185,6 +185,9 @@ struct DirectTma {
 void direct_tma_prepare(DirectTma *d, const uint32_t *keys, int64_t R_pad, int32_t C);
 cudaError_t launch_eval_direct_tma(const DirectTma &d, const EvalArgs &a, const PopView &pv,
                                    int num_sms, cudaStream_t s, bool pdl);
+
+// Bytes of a context's pinned block past its first 256 that a call may use.
+constexpr size_t kPinSpare = 512 << 10;
 
 // Kernel statistics (ebic_profile_*): launches counted always, event pairs while enabled.
 struct KStats {

@@ -258,10 +258,13 @@ def ebic_get_toplist(ctx, capacity=256):
     n = ctypes.c_int32()
     _check(ctx, _lib.ebic_get_toplist(ctx, capacity, ctypes.byref(n), ptr(cols), ptr(lens),
                                       ptr(fit), ptr(keys), ptr(rows)))
-    k = n.value
-    return [dict(cols=tuple(int(c) for c in cols[e, :lens[e]]), f=int(fit[e]), h=int(keys[e]),
-                 rows_pos=int(rows[e, 0]), rows_neg=int(rows[e, 1]), rows_any=int(rows[e, 2]))
-            for e in range(k)]
+    return _top_entries(n.value, cols, lens, fit, keys, rows)
+
+
+def _top_entries(n, cols, lens, fit, keys, rows):
+    return [dict(cols=tuple(c[:length]), f=f, h=h, rows_pos=r[0], rows_neg=r[1], rows_any=r[2])
+            for c, length, f, h, r in zip(cols[:n].tolist(), lens[:n].tolist(), fit[:n].tolist(),
+                                          keys[:n].tolist(), rows[:n].tolist())]
 
 
 def ebic_get_population(ctx, pop_size):
@@ -391,9 +394,7 @@ def ebic_server_wait(srv, job_id, timeout_ms=-1, capacity=256):
                                        capacity, ptr(cols), ptr(lens), ptr(fit), ptr(keys),
                                        ptr(rows)))
     out = res.as_dict()
-    out["top"] = [dict(cols=tuple(int(c) for c in cols[e, :lens[e]]), f=int(fit[e]),
-                       h=int(keys[e]), rows_pos=int(rows[e, 0]), rows_neg=int(rows[e, 1]),
-                       rows_any=int(rows[e, 2])) for e in range(res.n_top)]
+    out["top"] = _top_entries(res.n_top, cols, lens, fit, keys, rows)
     return out
 
 
