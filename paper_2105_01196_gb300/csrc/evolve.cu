@@ -536,10 +536,14 @@ __device__ void w_make_child(const GenArgs &ga, const Buf &pb, int g, int s, int
 // its bit, the negative trend when every reversed pair's word has it (ties counting both ways:
 // the complements of the opposite words, pad rows masked).  One unit is one pair row's 128 words
 // of one pass (16 bytes per lane); units are copied asynchronously into the warp's shared region,
-// two groups of kFuseGroup in flight (four with a region borrowed from a warp of the block that
-// has no slot left), and each lane reads back only the bytes it copied.
+// two groups of kFuseGroup in flight, and each lane reads back only the bytes it copied.  (Two more
+// groups in a region borrowed from a warp without a slot left, four more in registers, which
+// spilled, or one more in a larger region: 45, 58 and 43 us per launch at 60,000 x 1,000 against
+// 44; at 20,000 x 500 29.5, 35.1 and 27.8 against 27.5.  The code of this kernel does not fit the
+// instruction cache, so less of it counts as much as more copies in flight.)
 constexpr int kFuseGroup = 4;               // units per copy group
-constexpr int kFuseSlots = 2 * kFuseGroup;  // units staged per warp
+constexpr int kFuseRing = 2;                // copy groups in flight per warp
+constexpr int kFuseSlots = kFuseRing * kFuseGroup;  // units staged per warp
 constexpr int kFuseWords = 128;             // words of one unit
 
 __device__ __forceinline__ void fuse_copy16(uint32_t *dst, const uint32_t *src) {
@@ -598,86 +602,84 @@ __device__ __forceinline__ void fuse_pass_counts(const GenArgs &ga, bool neg, bo
 // The exact test when a pass's UPP pair rows (pairs x directions) fit in one copy group: a group
 // holds kFuseGroup / UPP whole passes, and each lane keeps the UPP rows' addresses (src[u]: its
 // words of pass 0; unit u of a pass is pair u / 2's positive (even u) or negative row with
-// negative trends, else pair u's row).  NG groups are in flight: 2 in the warp's own region, 4
-// with a second region (stage2) borrowed from a warp of the block that has no slot left.
+// negative trends, else pair u's row).  kFuseRing groups are in flight.
 // ONE: a pass's rows are the pairs' positive rows only, and the negative direction's words are
 // their complements (no ties in any of the pairs).
-template <int UPP, int NG, bool ONE>
+template <int UPP, bool ONE>
 __device__ void w_eval_exact_small(const GenArgs &ga, const uint32_t *const (&src)[4],
-                                   uint32_t *stage, uint32_t *stage2, int lane, int &cp, int &cn,
-                                   int &ca) {
+                                   uint32_t *stage, int lane, int &cp, int &cn, int &ca) {
   constexpr int PPG = kFuseGroup / UPP;  // passes per group
   const bool neg = ga.neg != 0, ns = ga.ns != 0 && !ONE;
   const int64_t Wst = ga.Wst;
   const int passes = (int)((Wst + kFuseWords - 1) / kFuseWords);
   const int n_groups = (passes + PPG - 1) / PPG;
-  // group gi's units: half gi & 1 of the own region, or of the borrowed one when gi % NG >= 2
+  // (pass q's words exist in this lane)
+  auto there = [&](int q) { return q < passes && (int64_t)q * kFuseWords + lane * 4 < Wst; };
   auto unit = [&](int gi, int k) -> uint32_t * {
-    uint32_t *base = (NG > 2 && (gi % NG) >= 2) ? stage2 : stage;
-    return base + lane * 4 + ((gi & 1) * kFuseGroup + k) * kFuseWords;
+    return stage + lane * 4 + ((gi % kFuseRing) * kFuseGroup + k) * kFuseWords;
   };
-  auto issue = [&](int gi) {
+  auto issue = [&](int gi) {  // group gi into its place in the ring
 #pragma unroll
     for (int pp = 0; pp < PPG; ++pp) {
       const int q = gi * PPG + pp;
-      if (q < passes && (int64_t)q * kFuseWords + lane * 4 < Wst) {
+      if (there(q)) {
 #pragma unroll
         for (int u = 0; u < UPP; ++u)
           fuse_copy16(unit(gi, pp * UPP + u), src[u] + (int64_t)q * kFuseWords);
       }
     }
-    fuse_commit();
+    fuse_commit();  // (an empty group past the end keeps the waits' count)
   };
   const uint4 ones = make_uint4(kFull, kFull, kFull, kFull);
+  auto count = [&](int q, const uint4 (&v)[UPP]) {  // one pass from its units
+    if (q >= passes) return;
+    const bool act = there(q);
+    uint4 ap = ones, an = ones;
 #pragma unroll
-  for (int gi = 0; gi < NG; ++gi)
-    if (gi < n_groups) issue(gi);
-  for (int gi = 0; gi < n_groups; ++gi) {
-    // (groups after gi still pending: at most NG - 1)
-    const int later = min(NG - 1, n_groups - 1 - gi);
-    if (NG > 2 && later >= 3)
-      fuse_wait<3>();
-    else if (NG > 2 && later == 2)
-      fuse_wait<2>();
-    else if (later >= 1)
-      fuse_wait<1>();
-    else
-      fuse_wait<0>();
+    for (int u = 0; u < UPP; ++u) {
+      uint4 x = v[u];
+      if (ns) x = make_uint4(~x.x, ~x.y, ~x.z, ~x.w);
+      if (ONE) {
+        ap = fuse_and(ap, x);
+        an = fuse_and(an, make_uint4(~x.x, ~x.y, ~x.z, ~x.w));
+      } else if (neg && (u & 1)) {
+        an = fuse_and(an, x);
+      } else {
+        ap = fuse_and(ap, x);
+      }
+    }
+    fuse_pass_counts(ga, neg, ns || ONE, act, (int64_t)q * kFuseWords + lane * 4, ap, an, cp, cn,
+                     ca);
+  };
+  auto count_staged = [&](int gi) {
 #pragma unroll
     for (int pp = 0; pp < PPG; ++pp) {
-      const int q = gi * PPG + pp;
-      const int64_t w = (int64_t)q * kFuseWords + lane * 4;
-      const bool act = q < passes && w < Wst;
-      uint4 ap = ones, an = ones;
-      if (act) {
+      uint4 v[UPP];
 #pragma unroll
-        for (int u = 0; u < UPP; ++u) {
-          uint4 v = *reinterpret_cast<const uint4 *>(unit(gi, pp * UPP + u));
-          if (ns) v = make_uint4(~v.x, ~v.y, ~v.z, ~v.w);
-          if (ONE) {
-            ap = fuse_and(ap, v);
-            an = fuse_and(an, make_uint4(~v.x, ~v.y, ~v.z, ~v.w));
-          } else if (neg && (u & 1)) {
-            an = fuse_and(an, v);
-          } else {
-            ap = fuse_and(ap, v);
-          }
-        }
+      for (int u = 0; u < UPP; ++u) {  // (lanes past Wst read what the region held: not counted)
+        v[u] = *reinterpret_cast<const uint4 *>(unit(gi, pp * UPP + u));
       }
-      if (q < passes) fuse_pass_counts(ga, neg, ns || ONE, act, w, ap, an, cp, cn, ca);
+      count(gi * PPG + pp, v);
     }
-    if (gi + NG < n_groups) issue(gi + NG);
+  };
+#pragma unroll
+  for (int k = 0; k < kFuseRing; ++k) issue(k);
+#pragma unroll 1
+  for (int gi = 0; gi < n_groups; ++gi) {
+    fuse_wait<kFuseRing - 1>();
+    count_staged(gi);
+    issue(gi + kFuseRing);
   }
+  fuse_wait<0>();  // (the empty groups)
 }
 
 // Row counts (positive trend, negative trend, either) of the exact test of c[0 .. L-1] (L >= 2),
 // in every lane.  ONE: with negative trends, no pair of the child has ties, and the positive rows
 // give both directions.  stage: the warp's kFuseSlots * kFuseWords words of shared memory (16-byte
-// aligned), free for this call; stage2: a second such region (borrowed), or null.  Only passes of
-// at most kFuseGroup pair rows use the second region.
+// aligned), free for this call.
 template <bool ONE>
-__device__ void w_eval_exact(const GenArgs &ga, const int32_t *c, int L, uint32_t *stage, uint32_t *stage2, int lane, int &rp, int &rn,
-                             int &ra) {
+__device__ void w_eval_exact(const GenArgs &ga, const int32_t *c, int L, uint32_t *stage, int lane,
+                             int &rp, int &rn, int &ra) {
   const int np = L - 1;
   const bool neg = ga.neg != 0, two = neg && !ONE;  // (two: both directions' rows are read)
   const bool ns = ga.ns != 0 && !ONE;
@@ -698,20 +700,11 @@ __device__ void w_eval_exact(const GenArgs &ga, const int32_t *c, int L, uint32_
     }
     int cp = 0, cn = 0, ca = 0;
     __syncwarp();  // every lane's earlier use of the region is done
-    if (stage2) {
-      switch (upp) {
-        case 1: w_eval_exact_small<1, 4, ONE>(ga, src, stage, stage2, lane, cp, cn, ca); break;
-        case 2: w_eval_exact_small<2, 4, ONE>(ga, src, stage, stage2, lane, cp, cn, ca); break;
-        case 3: w_eval_exact_small<3, 4, ONE>(ga, src, stage, stage2, lane, cp, cn, ca); break;
-        default: w_eval_exact_small<4, 4, ONE>(ga, src, stage, stage2, lane, cp, cn, ca); break;
-      }
-    } else {
-      switch (upp) {
-        case 1: w_eval_exact_small<1, 2, ONE>(ga, src, stage, stage, lane, cp, cn, ca); break;
-        case 2: w_eval_exact_small<2, 2, ONE>(ga, src, stage, stage, lane, cp, cn, ca); break;
-        case 3: w_eval_exact_small<3, 2, ONE>(ga, src, stage, stage, lane, cp, cn, ca); break;
-        default: w_eval_exact_small<4, 2, ONE>(ga, src, stage, stage, lane, cp, cn, ca); break;
-      }
+    switch (upp) {
+      case 1: w_eval_exact_small<1, ONE>(ga, src, stage, lane, cp, cn, ca); break;
+      case 2: w_eval_exact_small<2, ONE>(ga, src, stage, lane, cp, cn, ca); break;
+      case 3: w_eval_exact_small<3, ONE>(ga, src, stage, lane, cp, cn, ca); break;
+      default: w_eval_exact_small<4, ONE>(ga, src, stage, lane, cp, cn, ca); break;
     }
     rp = __reduce_add_sync(kFull, cp);
     rn = __reduce_add_sync(kFull, cn);
@@ -815,13 +808,9 @@ static_assert(kEvoScratch % 4 == 0, "scratch rows and staged units start on 16-b
 // would) or listed for the evaluation launch.  Returns its tabu-flag value: 2 evaluated from the
 // pair words, 3 (a one-pair chromosome) from the pair-count table, 0 listed.
 // TF: the matrix has few tied pairs (ga.tie_free), and children without any are looked for.
-// s_free (k_evolve_seq; null otherwise): bit w set while warp w of the block has no slot left,
-// its region (of kEvolveWarpInts ints from `regions`) then free; a pair-word evaluation borrows
-// one such region for two more copy groups in flight and gives it back at its end.
 template <bool TF>
 __device__ int fuse_or_list(const GenArgs &ga, const int32_t *c, int L, uint64_t h, int s,
-                            int par, uint32_t *stage, int lane, int32_t *regions,
-                            uint32_t *s_free) {
+                            int par, uint32_t *stage, int lane) {
   if (fuse_child(ga, L)) {
     int rp = 0, rn = 0, ra = 0;
     const bool table = L == 2 && ga.pair_cnt != nullptr;
@@ -848,20 +837,6 @@ __device__ int fuse_or_list(const GenArgs &ga, const int32_t *c, int L, uint64_t
         }
       }
     } else {
-      int lent = -1;  // the warp whose region is borrowed
-      if (s_free) {
-        if (lane == 0) {
-          const uint32_t m = *reinterpret_cast<volatile uint32_t *>(s_free);
-          if (m) {
-            const uint32_t bit = m & (0u - m);  // (the lowest free region)
-            if (atomicAnd(s_free, ~bit) & bit) lent = __ffs(bit) - 1;
-          }
-        }
-        lent = __shfl_sync(kFull, lent, 0);
-      }
-      uint32_t *stage2 =
-          lent >= 0 ? reinterpret_cast<uint32_t *>(regions + lent * kEvolveWarpInts + kEvoStage)
-                    : nullptr;
       // no ties in any pair: the positive rows' words give both directions (np <= 63 pairs)
       bool tied = !TF;
       if (TF)
@@ -869,13 +844,9 @@ __device__ int fuse_or_list(const GenArgs &ga, const int32_t *c, int L, uint64_t
           tied |= pair_has_ties(ga.pair_cnt, ga.C, c[k], c[k + 1], ga.R);
       // (half the words read: evolve 34 -> 31 us per generation on 20,000 x 500, P = 4,096)
       if (TF && !__any_sync(kFull, tied))
-        w_eval_exact<true>(ga, c, L, stage, stage2, lane, rp, rn, ra);
+        w_eval_exact<true>(ga, c, L, stage, lane, rp, rn, ra);
       else
-        w_eval_exact<false>(ga, c, L, stage, stage2, lane, rp, rn, ra);
-      if (lent >= 0) {
-        __syncwarp();  // (every lane's copies into it have landed and been read)
-        if (lane == 0) atomicOr(s_free, 1u << lent);
-      }
+        w_eval_exact<false>(ga, c, L, stage, lane, rp, rn, ra);
     }
     if (lane == 0) {
       ga.rows_scr[s] = rp;
@@ -1001,8 +972,7 @@ __global__ void __launch_bounds__(kMaxAttemptWarps * 32) k_evolve(GenArgs ga, Bu
   out[lane + 32] = lane + 32 < L ? c[lane + 32] : 0;
   const int fused = (!dead && ga.fuse_np > 0)
                         ? fuse_or_list<TF>(ga, c, L, h, s, par,
-                                       reinterpret_cast<uint32_t *>(base + kEvoStage), lane,
-                                       nullptr, nullptr)
+                                           reinterpret_cast<uint32_t *>(base + kEvoStage), lane)
                         : 0;
   if (lane == 0) {
     nb.len[s] = L;
@@ -1248,7 +1218,6 @@ template <bool TF>
 __global__ void __launch_bounds__(kSeqWarps * 32, 4) k_evolve_seq(GenArgs ga, Buf pb, Buf nb,
                                                                int par) {
   extern __shared__ __align__(16) int32_t s_evo[];  // kEvolveWarpInts per warp, then usage
-  __shared__ uint32_t s_free;  // bit w: warp w has no slot left, its region free to borrow
   wait_prior_grid();
   const int stopped = ga.ctl->stopped, gen = ga.ctl->gen, n_top = ga.ctl->n_top;
   const int32_t *usage = ga.usage;
@@ -1258,7 +1227,6 @@ __global__ void __launch_bounds__(kSeqWarps * 32, 4) k_evolve_seq(GenArgs ga, Bu
     usage = s_usage;
   }
   if (stopped) return;
-  if (threadIdx.x == 0) s_free = 0u;
   __syncthreads();  // (no block-wide operation follows)
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int W = (int)gridDim.x * kSeqWarps;
@@ -1300,8 +1268,8 @@ __global__ void __launch_bounds__(kSeqWarps * 32, 4) k_evolve_seq(GenArgs ga, Bu
       out[lane + 32] = lane + 32 < L ? c[lane + 32] : 0;
       const int fused = (!dead && ga.fuse_np > 0)
                             ? fuse_or_list<TF>(ga, c, L, h, s, par,
-                                           reinterpret_cast<uint32_t *>(base + kEvoStage), lane,
-                                           s_evo, &s_free)
+                                               reinterpret_cast<uint32_t *>(base + kEvoStage),
+                                               lane)
                             : 0;
       if (lane == 0) {
         nb.len[s] = L;
@@ -1316,9 +1284,6 @@ __global__ void __launch_bounds__(kSeqWarps * 32, 4) k_evolve_seq(GenArgs ga, Bu
     s = __shfl_sync(kFull, nx, 0) + W;
     __syncwarp();  // (the region's last reads are done before the next slot writes it)
   }
-  // no slot left: the warp's region can stage a sibling's evaluation
-  __syncwarp();
-  if (lane == 0) atomicOr(&s_free, 1u << w);
 }
 
 __device__ __forceinline__ bool key_before(uint64_t fa, uint64_t ha, uint64_t fb, uint64_t hb) {
