@@ -180,6 +180,15 @@ struct WarpStream {
     return __shfl_sync(0xFFFFFFFFu, mine, (int)(b - base));
   }
   __device__ uint32_t below(uint32_t n) { return __umulhi(next(), n); }
+  // Word i of the stream, i differing from lane to lane, among the words held now.
+  __device__ uint32_t at(uint32_t i) const {
+    const int from = (int)((i >> 2) - base);
+    uint32_t v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = __shfl_sync(0xFFFFFFFFu, w[k], from);
+    const uint32_t k = i & 3u;
+    return k == 0 ? v[0] : (k == 1 ? v[1] : (k == 2 ? v[2] : v[3]));
+  }
 };
 
 // ------------------------------------------------------------------ FNV-1a 64 chromosome key
@@ -319,9 +328,9 @@ __device__ __forceinline__ bool beats(uint64_t fa, int ua, int ia, uint64_t fb, 
   return c > 0 || (c == 0 && ia < ib);
 }
 
-// Both tournaments of a child when T <= 4: the first one's T candidates, the crossover word and
-// the second one's T candidates are drawn in stream order (the second set from a copy of the
-// stream, adopted only when the crossover happens).  The sets take candidate places 0..T-1 and
+// Both tournaments of a child when T <= 4, from a stream at its start: the first one's T candidates,
+// the crossover word and the second one's T candidates are its first words (the second set counts
+// as drawn only when the crossover happens).  The sets take candidate places 0..T-1 and
 // 4..4+T-1, four lanes each, so all candidates' data arrive in one round of loads and each set's
 // winner comes out of a two-step butterfly over its places.  The winner is the one w_tournament
 // picks (the maximum of one total order: penalised score, then the lower slot).  Returns whether
@@ -330,24 +339,16 @@ __device__ bool w_tournament_pair(WarpStream &st, const GenArgs &ga, const Buf &
                                   int32_t *scratch, int32_t *A, int *LA, int32_t *B, int *LB,
                                   int lane, const int32_t *usage) {
   const int T = ga.T;
-  int ids[8];
-#pragma unroll
-  for (int q = 0; q < 8; ++q) ids[q] = -1;
-#pragma unroll
-  for (int q = 0; q < 4; ++q)
-    if (q < T) ids[q] = (int)st.below((uint32_t)ga.P);
-  const bool cross = st.next() < (1u << 30);  // one-point crossover, probability 1/4
-  WarpStream st2 = st;
-#pragma unroll
-  for (int q = 0; q < 4; ++q)
-    if (q < T) ids[4 + q] = (int)st2.below((uint32_t)ga.P);
-  if (cross) st = st2;
   const int mine = lane >> 2, sub = lane & 3;
-  int my = -1;
-#pragma unroll
-  for (int q = 0; q < 8; ++q)
-    if (q == mine) my = ids[q];
-  if (!cross && mine >= 4) my = -1;  // the second set is not needed
+  // The stream starts with the first set's T words, the crossover word and the second set's T
+  // words (at most nine: all in the words the warp holds): each lane takes its candidate's.
+  const bool second = mine >= 4;
+  const uint32_t mine_w = st.at((uint32_t)(second ? T + 1 + (mine - 4) : mine));
+  const bool cross = st.at((uint32_t)T) < (1u << 30);  // one-point crossover, probability 1/4
+  st.pos = (uint32_t)(cross ? 2 * T + 1 : T + 1);
+  // (the second set is not needed without the crossover)
+  const bool drawn = second ? cross && mine - 4 < T : mine < T;
+  const int my = drawn ? (int)__umulhi(mine_w, (uint32_t)ga.P) : -1;
   uint64_t f = 0ull;
   int u = 0, L = 0;
   if (my >= 0) {
