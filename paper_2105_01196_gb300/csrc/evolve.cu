@@ -141,86 +141,85 @@ __device__ __forceinline__ void philox_block(uint32_t k0, uint32_t k1, uint32_t 
   w[3] = x3;
 }
 
-// The same as a call (for the rare refills of WarpStream, which would otherwise be inlined at
-// every draw).
-__device__ __noinline__ uint4 philox_block_call(uint32_t k0, uint32_t k1, uint32_t c0, uint32_t c1,
-                                                uint32_t c2, uint32_t c3) {
+// The 128 words of blocks `block` .. `block` + 31 of counter (c0, c1, c2), into shared memory by one
+// warp (lane j: block + j).  Not inlined: a stream's start and its rare refills share one copy.
+__device__ __noinline__ void philox_words(uint32_t k0, uint32_t k1, uint32_t c0, uint32_t c1,
+                                          uint32_t c2, uint32_t block, uint32_t *words, int lane) {
   uint32_t w[4];
-  philox_block(k0, k1, c0, c1, c2, c3, w);
-  return make_uint4(w[0], w[1], w[2], w[3]);
+  philox_block(k0, k1, c0, c1, c2, block + (uint32_t)lane, w);
+  __syncwarp();  // (the words held before have been read)
+  reinterpret_cast<uint4 *>(words)[lane] = make_uint4(w[0], w[1], w[2], w[3]);
+  __syncwarp();
 }
 
+constexpr int kStreamWords = 128;  // words of the stream a warp holds (a power of two)
+
 // The word stream of counter (g, s, a) - the words of Philox blocks 0, 1, 2, ... in order - for
-// a whole warp: lane j holds block base + j, so one round of Philox in all lanes yields 128
-// words, and word i comes from lane i / 4 - base by a shuffle (every lane calls next() together
-// and gets the same word).
+// a whole warp: one round of Philox in all lanes yields 128 words, kept in the warp's kStreamWords
+// words of shared memory (16-byte aligned), and a draw is one load (every lane calls next()
+// together and gets the same word).  (Words held in the lanes' registers and passed round by
+// shuffles took three times the instructions per draw; with that, the key's shorter chain and the
+// tournament's compared exponents: evolve launch 26.7 to 25.6 us at 20,000 x 500 with 4,096
+// individuals, 43.0 to 41.2 us at 60,000 x 1,000 with 8,192, 14.4 to 14.1 us per generation at
+// 10,000 x 100 with 800.  More warps per SM, at 48 registers, gained nothing: 25.8 and 42.0 us.)
 struct WarpStream {
   uint32_t k0, k1, c0, c1, c2;
-  uint32_t w[4];
-  uint32_t base, pos;  // first block held; next word index
+  uint32_t *words;
+  uint32_t pos, end;  // next word index; first word index after those held
   int lane;
-  __device__ WarpStream(uint64_t seed, uint32_t g, uint32_t s, uint32_t a, int lane_)
-      : k0((uint32_t)seed), k1((uint32_t)(seed >> 32)), c0(g), c1(s), c2(a), base(0), pos(0),
-        lane(lane_) {
-    philox_block(k0, k1, c0, c1, c2, base + (uint32_t)lane, w);
+  __device__ WarpStream(uint64_t seed, uint32_t g, uint32_t s, uint32_t a, uint32_t *words_,
+                        int lane_)
+      : k0((uint32_t)seed), k1((uint32_t)(seed >> 32)), c0(g), c1(s), c2(a), words(words_), pos(0),
+        end(kStreamWords), lane(lane_) {
+    philox_words(k0, k1, c0, c1, c2, 0u, words, lane);
   }
   __device__ uint32_t next() {
-    const uint32_t b = pos >> 2;
-    if (b >= base + 32u) {  // (warp-uniform) the next 32 blocks
-      base += 32u;
-      const uint4 v = philox_block_call(k0, k1, c0, c1, c2, base + (uint32_t)lane);
-      w[0] = v.x;
-      w[1] = v.y;
-      w[2] = v.z;
-      w[3] = v.w;
+    if (pos == end) {  // (warp-uniform) the next 32 blocks
+      philox_words(k0, k1, c0, c1, c2, end >> 2, words, lane);
+      end += kStreamWords;
     }
-    const uint32_t k = pos & 3u;
-    const uint32_t mine = k == 0 ? w[0] : (k == 1 ? w[1] : (k == 2 ? w[2] : w[3]));
-    ++pos;
-    return __shfl_sync(0xFFFFFFFFu, mine, (int)(b - base));
+    return words[pos++ & (kStreamWords - 1)];
   }
   __device__ uint32_t below(uint32_t n) { return __umulhi(next(), n); }
   // Word i of the stream, i differing from lane to lane, among the words held now.
-  __device__ uint32_t at(uint32_t i) const {
-    const int from = (int)((i >> 2) - base);
-    uint32_t v[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) v[k] = __shfl_sync(0xFFFFFFFFu, w[k], from);
-    const uint32_t k = i & 3u;
-    return k == 0 ? v[0] : (k == 1 ? v[1] : (k == 2 ? v[2] : v[3]));
-  }
+  __device__ uint32_t at(uint32_t i) const { return words[i & (kStreamWords - 1)]; }
 };
 
 // ------------------------------------------------------------------ FNV-1a 64 chromosome key
 
+// The key takes a column's four bytes in turn (h = (h ^ byte) * p modulo 2^64).  A matrix has at
+// most 65,535 columns, so the upper two are zero and their steps are one multiplication with the
+// second byte's: two dependent multiplications per column instead of four.
 __device__ uint64_t chromosome_key(const int32_t *c, int L) {
+  constexpr uint64_t p = 0x100000001B3ull, p3 = p * p * p;
   uint64_t h = 0xCBF29CE484222325ull;
   for (int k = 0; k < L; ++k) {
     const uint32_t v = (uint32_t)c[k];
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      h ^= (v >> (8 * b)) & 0xFFu;
-      h *= 0x100000001B3ull;
-    }
+    h = (h ^ (v & 0xFFu)) * p;
+    h = (h ^ (v >> 8)) * p3;
   }
   return h ? h : 0x9E3779B97F4A7C15ull;
 }
 
 // ------------------------------------------------------------------ selection
 
-// Sign of fa * 2^s - fb for s >= 0, exactly.
-__device__ __forceinline__ int cmp_shifted(uint64_t fa, int s, uint64_t fb) {
-  if (fa == 0ull) return fb == 0ull ? 0 : -1;
-  if (s >= 64) return 1;
-  const uint64_t q = fb >> s;  // fa * 2^s > fb  <=>  fa > floor(fb / 2^s)
-  if (fa > q) return 1;
-  if (fa < q) return -1;
-  return (fb & ((s ? (1ull << s) : 1ull) - 1ull)) ? -1 : 0;
+// A candidate's penalised score f * 2^-u in a form whose order is that of (e, m): m is f shifted
+// until its top bit is set, e the exponent that goes with it.  Zero comes below every other score,
+// a missing candidate (slot < 0) below zero.
+struct Score {
+  int e;
+  uint64_t m;
+};
+__device__ __forceinline__ Score penalised(uint64_t f, int u, int slot) {
+  if (f == 0ull || slot < 0) return {slot < 0 ? INT_MIN : INT_MIN + 1, 0ull};
+  const int z = __clzll((long long)f);
+  return {63 - z - u, f << z};
 }
-
-// Sign of fa * 2^-ua - fb * 2^-ub, exactly (ua, ub >= 0).
-__device__ __forceinline__ int cmp_penalised(uint64_t fa, int ua, uint64_t fb, int ub) {
-  return ub >= ua ? cmp_shifted(fa, ub - ua, fb) : -cmp_shifted(fb, ua - ub, fa);
+// Whether candidate a in slot ia beats b in slot ib: the higher score, then the lower slot.
+__device__ __forceinline__ bool beats(const Score &a, int ia, const Score &b, int ib) {
+  if (a.e != b.e) return a.e > b.e;
+  if (a.m != b.m) return a.m > b.m;
+  return ia < ib;
 }
 
 // ------------------------------------------------------------------ variation
@@ -257,8 +256,8 @@ __device__ int w_draw_free(WarpStream &st, int C, const int32_t *c, int L, int l
 // winner as the sequential rule (exact penalised comparison, ties to the lower slot).
 __device__ int w_tournament(WarpStream &st, const GenArgs &ga, const Buf &pb, int32_t *scratch,
                             int32_t *win, int *win_len, int lane, const int32_t *usage) {
-  int best = -1, ub = 0, bl = 0;
-  uint64_t fb = 0ull;
+  int best = -1, bl = 0;
+  Score sb = {INT_MIN, 0ull};
   const int mine = lane >> 2, sub = lane & 3;
   for (int t0 = 0; t0 < ga.T; t0 += 8) {
     int ids[8];
@@ -290,20 +289,20 @@ __device__ int w_tournament(WarpStream &st, const GenArgs &ga, const Buf &pb, in
     }
     u += __shfl_xor_sync(kFull, u, 1);
     u += __shfl_xor_sync(kFull, u, 2);
+    const Score mine_s = penalised(f, u, my);
     __syncwarp();
     int take = -1;
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-      const uint64_t fq = __shfl_sync(kFull, f, q * 4);
-      const int uq = __shfl_sync(kFull, u, q * 4);
+      Score sq;
+      sq.e = __shfl_sync(kFull, mine_s.e, q * 4);
+      sq.m = __shfl_sync(kFull, mine_s.m, q * 4);
       const int lq = __shfl_sync(kFull, L, q * 4);
       const int iq = ids[q];
       if (iq < 0) continue;
-      const int c = best < 0 ? 1 : cmp_penalised(fq, uq, fb, ub);
-      if (c > 0 || (c == 0 && iq < best)) {
+      if (beats(sq, iq, sb, best)) {
         best = iq;
-        fb = fq;
-        ub = uq;
+        sb = sq;
         bl = lq;
         take = q;
       }
@@ -317,15 +316,6 @@ __device__ int w_tournament(WarpStream &st, const GenArgs &ga, const Buf &pb, in
   }
   *win_len = bl;
   return best;
-}
-
-// Whether candidate (fa, ua, ia) beats (fb, ub, ib): exact penalised comparison, ties to the
-// lower slot; a missing candidate (slot < 0) never wins.
-__device__ __forceinline__ bool beats(uint64_t fa, int ua, int ia, uint64_t fb, int ub, int ib) {
-  if (ia < 0) return false;
-  if (ib < 0) return true;
-  const int c = cmp_penalised(fa, ua, fb, ub);
-  return c > 0 || (c == 0 && ia < ib);
 }
 
 // Both tournaments of a child when T <= 4, from a stream at its start: the first one's T candidates,
@@ -371,23 +361,22 @@ __device__ bool w_tournament_pair(WarpStream &st, const GenArgs &ga, const Buf &
   u += __shfl_xor_sync(kFull, u, 1);
   u += __shfl_xor_sync(kFull, u, 2);
   // butterfly over the places of each set (lanes 0-15: first set, 16-31: second set)
-  int wi = my, wq = mine, wl = L, wu = u;
-  uint64_t wf = f;
+  Score w = penalised(f, u, my);
+  int wi = my, wp = mine << 8 | L;  // (its place and length)
 #pragma unroll
   for (int off = 4; off <= 8; off <<= 1) {
-    const uint64_t of = __shfl_xor_sync(kFull, wf, off);
-    const int ou = __shfl_xor_sync(kFull, wu, off), oi = __shfl_xor_sync(kFull, wi, off);
-    const int ol = __shfl_xor_sync(kFull, wl, off), oq = __shfl_xor_sync(kFull, wq, off);
-    if (beats(of, ou, oi, wf, wu, wi)) {
-      wf = of;
-      wu = ou;
+    Score o;
+    o.e = __shfl_xor_sync(kFull, w.e, off);
+    o.m = __shfl_xor_sync(kFull, w.m, off);
+    const int oi = __shfl_xor_sync(kFull, wi, off), op = __shfl_xor_sync(kFull, wp, off);
+    if (beats(o, oi, w, wi)) {
+      w = o;
       wi = oi;
-      wl = ol;
-      wq = oq;
+      wp = op;
     }
   }
-  const int take0 = __shfl_sync(kFull, wq, 0), take1 = __shfl_sync(kFull, wq, 16);
-  const int bl0 = __shfl_sync(kFull, wl, 0), bl1 = __shfl_sync(kFull, wl, 16);
+  const int w0 = __shfl_sync(kFull, wp, 0), w1 = __shfl_sync(kFull, wp, 16);
+  const int take0 = w0 >> 8, take1 = w1 >> 8, bl0 = w0 & 0xFF, bl1 = w1 & 0xFF;
   __syncwarp();  // the scratch rows are written
   const int32_t *ra = scratch + take0 * kS;
   A[lane] = ra[lane];
@@ -467,10 +456,29 @@ __device__ void w_mutate(WarpStream &st, int32_t *c, int &L, int C, int max_len,
   w_swap(st, c, L, lane);
 }
 
-__device__ void w_make_child(const GenArgs &ga, const Buf &pb, int g, int s, int a, int32_t *c,
-                             int32_t *scratch, int32_t *A, int32_t *B, int &L, int lane,
-                             const int32_t *usage) {
-  WarpStream st(ga.seed, (uint32_t)g, (uint32_t)s, (uint32_t)a, lane);
+// The evaluation of short children (below) stages pair words in units of kFuseWords words.
+constexpr int kFuseGroup = 4;               // units per copy group
+constexpr int kFuseRing = 2;                // copy groups in flight per warp
+constexpr int kFuseSlots = kFuseRing * kFuseGroup;  // units staged per warp
+constexpr int kFuseWords = 128;             // words of one unit
+
+// Per-warp shared memory of the evolve kernels, in ints: the child (kS + 1 used), then 8 tournament
+// scratch rows, the two parents and the word stream; once the child is final, the region after it
+// stages the pair words of its evaluation (kFuseSlots units).  Every part starts on a 16-byte
+// boundary (the scratch rows and words are written with 16-byte stores, the staged units by
+// 16-byte copies), and the total is a multiple of 16 bytes.
+constexpr int kEvoChild = 0, kEvoScratch = kS + 4, kEvoA = kEvoScratch + 8 * kS,
+              kEvoB = kEvoA + kS, kEvoWords = kEvoB + kS, kEvoStage = kEvoScratch;
+constexpr int kEvoBuild = kEvoWords + kStreamWords, kEvoEval = kEvoStage + kFuseSlots * kFuseWords;
+constexpr int kEvolveWarpInts = kEvoBuild > kEvoEval ? kEvoBuild : kEvoEval;
+static_assert(kEvoScratch % 4 == 0 && kEvoWords % 4 == 0, "parts start on 16-byte boundaries");
+
+__device__ void w_make_child(const GenArgs &ga, const Buf &pb, int g, int s, int a, int32_t *base,
+                             int &L, int lane, const int32_t *usage) {
+  int32_t *c = base + kEvoChild, *scratch = base + kEvoScratch;
+  int32_t *A = base + kEvoA, *B = base + kEvoB;
+  WarpStream st(ga.seed, (uint32_t)g, (uint32_t)s, (uint32_t)a,
+                reinterpret_cast<uint32_t *>(base + kEvoWords), lane);
   int LA = 0, LB = 0;
   bool cross;
   if (ga.T <= 4) {
@@ -542,11 +550,6 @@ __device__ void w_make_child(const GenArgs &ga, const Buf &pb, int g, int s, int
 // spilled, or one more in a larger region: 45, 58 and 43 us per launch at 60,000 x 1,000 against
 // 44; at 20,000 x 500 29.5, 35.1 and 27.8 against 27.5.  The code of this kernel does not fit the
 // instruction cache, so less of it counts as much as more copies in flight.)
-constexpr int kFuseGroup = 4;               // units per copy group
-constexpr int kFuseRing = 2;                // copy groups in flight per warp
-constexpr int kFuseSlots = kFuseRing * kFuseGroup;  // units staged per warp
-constexpr int kFuseWords = 128;             // words of one unit
-
 __device__ __forceinline__ void fuse_copy16(uint32_t *dst, const uint32_t *src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
                    (uint32_t)__cvta_generic_to_shared(dst)),
@@ -793,17 +796,6 @@ __device__ void w_eval_exact(const GenArgs &ga, const int32_t *c, int L, uint32_
   ra = __reduce_add_sync(kFull, ca);
 }
 
-// Per-warp shared memory of k_evolve, in ints: the child (kS + 1 used), then 8 tournament scratch
-// rows and the two parents; once the child is final, the region after it stages the pair words
-// of its evaluation (kFuseSlots units).  Every part starts on a 16-byte boundary (the scratch
-// rows are written with 16-byte stores, the staged units by 16-byte copies), and the total is a
-// multiple of 16 bytes.
-constexpr int kEvoChild = 0, kEvoScratch = kS + 4, kEvoA = kEvoScratch + 8 * kS,
-              kEvoB = kEvoA + kS, kEvoStage = kEvoScratch;
-constexpr int kEvolveWarpInts =
-    kEvoScratch + (10 * kS > kFuseSlots * kFuseWords ? 10 * kS : kFuseSlots * kFuseWords);
-static_assert(kEvoScratch % 4 == 0, "scratch rows and staged units start on 16-byte boundaries");
-
 // The end of a live slot s's evolve step when fusion is on: the slot is evaluated here (its
 // counts stored, its key entered in generation g's duplicate table, as the evaluation launch
 // would) or listed for the evaluation launch.  Returns its tabu-flag value: 2 evaluated from the
@@ -868,11 +860,12 @@ __device__ int fuse_or_list(const GenArgs &ga, const int32_t *c, int L, uint64_t
 constexpr int kInitWarps = 8;
 __global__ void __launch_bounds__(kInitWarps * 32) k_init(GenArgs ga, Buf nb) {
   __shared__ int32_t s_c[kInitWarps][kS];
+  __shared__ __align__(16) uint32_t s_words[kInitWarps][kStreamWords];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int s = blockIdx.x * kInitWarps + warp;
   if (s >= ga.P) return;  // (whole warps)
   int32_t *c = s_c[warp];
-  WarpStream st(ga.seed, 0u, (uint32_t)s, 0u, lane);
+  WarpStream st(ga.seed, 0u, (uint32_t)s, 0u, s_words[warp], lane);
   const int want = ga.init_min + (int)st.below((uint32_t)(ga.init_max - ga.init_min + 1));
   int L = 0;
   for (int j = 0; j < want; ++j) {
@@ -945,13 +938,12 @@ __global__ void __launch_bounds__(kMaxAttemptWarps * 32) k_evolve(GenArgs ga, Bu
     return;
   }
   int32_t *base = s_evo + a * kEvolveWarpInts;
-  int32_t *scratch = base + kEvoScratch, *A = base + kEvoA, *B = base + kEvoB;
   int32_t *c = base + kEvoChild;
   int L = 0;
   uint64_t h = 0ull;
   int ok = 0;
   if (a < ga.A) {
-    w_make_child(ga, pb, g, s, a, c, scratch, A, B, L, lane, usage);
+    w_make_child(ga, pb, g, s, a, base, L, lane, usage);
     h = chromosome_key(c, L);
     // lane 0 probes the hashed tabu list, lane 1 generation g-1's live keys
     const bool hit = (lane == 0 && tabu_contains(ga.tabu, ga.tmask, h)) ||
@@ -1138,8 +1130,7 @@ __global__ void __launch_bounds__(kBlockWarps * 32, 8) k_evolve_block(GenArgs ga
   if (a < ga.A) {
     int L = 0;
     int32_t *c = base + kEvoChild;
-    w_make_child(ga, pb, g, s, a, c, base + kEvoScratch, base + kEvoA, base + kEvoB, L, lane,
-                 usage);
+    w_make_child(ga, pb, g, s, a, base, L, lane, usage);
     const uint64_t h = chromosome_key(c, L);
     // lane 0 probes the hashed tabu list, lane 1 generation g-1's live keys
     const bool hit = (lane == 0 && tabu_contains(ga.tabu, ga.tmask, h)) ||
@@ -1234,7 +1225,6 @@ __global__ void __launch_bounds__(kSeqWarps * 32, 4) k_evolve_seq(GenArgs ga, Bu
   const int g = gen + 1;
   const int n_el = min(ga.E, n_top);
   int32_t *base = s_evo + w * kEvolveWarpInts;
-  int32_t *scratch = base + kEvoScratch, *A = base + kEvoA, *B = base + kEvoB;
   int32_t *c = base + kEvoChild;
   for (int s = blockIdx.x * kSeqWarps + w; s < ga.P;) {
     int32_t *out = nb.cols + (size_t)s * kS;
@@ -1253,7 +1243,7 @@ __global__ void __launch_bounds__(kSeqWarps * 32, 4) k_evolve_seq(GenArgs ga, Bu
       int L = 0, win = -1;
       uint64_t h = 0ull;
       for (int a = 0; a < ga.A; ++a) {
-        w_make_child(ga, pb, g, s, a, c, scratch, A, B, L, lane, usage);
+        w_make_child(ga, pb, g, s, a, base, L, lane, usage);
         h = chromosome_key(c, L);
         // lane 0 probes the hashed tabu list, lane 1 generation g-1's live keys
         const bool hit = (lane == 0 && tabu_contains(ga.tabu, ga.tmask, h)) ||
