@@ -38,6 +38,8 @@ namespace {
 constexpr unsigned kFull = 0xFFFFFFFFu;
 constexpr int kNaWarps = 8;
 constexpr int kNaThreads = kNaWarps * 32;
+constexpr int kNaEvalWarps = 32;  // of the evaluation: one block per SM
+constexpr int kNaEvalThreads = kNaEvalWarps * 32;
 constexpr int kMaxDevices = 64;
 
 struct NoAllocScratch {
@@ -100,28 +102,35 @@ __global__ void __launch_bounds__(kNaThreads) k_na_prepare(const float *__restri
 }
 
 // Direct float32 comparisons (-0 equals +0; no FTZ in this file's compilation).  An item is an
-// individual and a segment of 128-row passes, segment-major, taken by the warps in turn; a lane
-// counts four rows of a pass: consecutive ones by one 16-byte load per column where every column
-// starts on a 16-byte boundary (VEC: x aligned, R a multiple of 4), else rows 32 apart by four
-// 4-byte loads (coalesced whatever the alignment).  NS / LK are the pair-test variants of
-// trend.cuh.  Bound: L2 (4 bytes per row and pair, about 8 TB/s): 43 us at 10,000 x 100, 800
-// individuals of 2-20 columns (214 us with a row per lane and the items of 32-row passes taken
-// from one counter), 0.96 ms at 30,000 x 300, 4,000 individuals of 2-40 (1.04 ms with three items
-// per warp instead of six, 1.22 ms with one).
+// individual and a segment of 128-row passes, segment-major.  A block (one per SM, up to every warp
+// the SM holds) owns a run of consecutive items, taken by its warps from a counter in shared
+// memory: its individuals read the same rows' pieces of the columns, largely from L1, and uneven
+// lengths even out within the block.  A lane counts four rows of a pass: consecutive ones by one
+// 16-byte load per column where every column starts on a 16-byte boundary (VEC: x aligned, R a
+// multiple of 4), else rows 32 apart by four 4-byte loads (coalesced whatever the alignment).
+// NS / LK are the pair-test variants of trend.cuh.
+// Bound: latency of an item's loads, then L1 / L2 (4 bytes per row and pair).  Whole calls: 108 us
+// at 10,000 x 100, 800 individuals of 2-20 columns (116 with the items dealt to all warps of the
+// grid in turn, 329 with a row per lane and 32-row items from one global counter), 0.90 ms at
+// 30,000 x 300, 4,000 individuals of 2-40 (1.05 dealt in turn).
 template <bool NEG, bool NS, bool LK, bool VEC>
-__global__ void __launch_bounds__(kNaThreads, 4) k_na_eval(const float *__restrict__ x, int64_t R,
-                                                           const int32_t *__restrict__ cols,
-                                                           const int32_t *__restrict__ off,
-                                                           int32_t n, int32_t n_seg,
-                                                           int32_t seg_passes, int32_t rnum,
-                                                           int32_t rden, NoAllocScratch *sc) {
-  __shared__ int64_t s_base[kNaWarps][EBIC_MAX_LEN];
+__global__ void __launch_bounds__(kNaEvalThreads, 1)
+    k_na_eval(const float *__restrict__ x, int64_t R, const int32_t *__restrict__ cols,
+              const int32_t *__restrict__ off, int32_t n, int32_t n_seg, int32_t seg_passes,
+              int32_t rnum, int32_t rden, NoAllocScratch *sc) {
+  __shared__ int64_t s_base[kNaEvalWarps][EBIC_MAX_LEN];
+  __shared__ unsigned long long s_next;  // items of the block taken so far
   wait_prior_grid();
   if (sc->err) return;  // (a bad population is never indexed with)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (threadIdx.x == 0) s_next = blockDim.x >> 5;
+  __syncthreads();
   const int64_t passes_total = (R + 127) / 128;
-  const int64_t n_items = (int64_t)n * n_seg, W = (int64_t)gridDim.x * kNaWarps;
-  for (int64_t q = (int64_t)blockIdx.x * kNaWarps + warp; q < n_items; q += W) {
+  const int64_t n_items = (int64_t)n * n_seg;
+  const int64_t q0 = n_items * blockIdx.x / gridDim.x;
+  const int64_t mine = n_items * (blockIdx.x + 1) / gridDim.x - q0;
+  for (int64_t d = warp; d < mine;) {
+    const int64_t q = q0 + d;
     const int seg = (int)(q / n), i = (int)(q - (int64_t)seg * n);
     const int st = off[i], L = off[i + 1] - st;
     __syncwarp();
@@ -177,6 +186,9 @@ __global__ void __launch_bounds__(kNaThreads, 4) k_na_eval(const float *__restri
       if (cn) atomicAdd(&sc->counts[n + i], cn);
       if (ca) atomicAdd(&sc->counts[2 * n + i], ca);
     }
+    unsigned long long nx = 0;
+    if (lane == 0) nx = atomicAdd(&s_next, 1ull);
+    d = (int64_t)__shfl_sync(kFull, nx, 0);
   }
 }
 
@@ -331,19 +343,20 @@ extern "C" int ebic_eval_population_noalloc(const float *x, int64_t rows, int32_
     k_na_prepare<<<(unsigned)std::min<int64_t>(pre, 8 * num_sms), kNaThreads, 0, s>>>(
         x, total, col_idx, offsets, n_ind, cols, sc);
     if ((e = cudaGetLastError()) != cudaSuccess) break;
-    // Segments: about six items per resident warp (four blocks per SM), so that the uneven
-    // lengths even out without a queue.
+    // Segments: about six items per warp, so that the uneven lengths even out.  10,000 x 100 and
+    // 30,000 x 300, as above: 108 us and 0.90 ms; with three items 109 and 0.98, with ten 116 and
+    // 0.85; segments of one pass 113 us and 0.91 ms.
     const int64_t passes_total = (rows + 127) / 128;
-    int64_t seg = ((int64_t)n_ind * passes_total) / (6 * 4 * num_sms * kNaWarps);
+    int64_t seg = ((int64_t)n_ind * passes_total) / (6 * num_sms * kNaEvalWarps);
     if (seg < 1) seg = 1;
     if (seg > passes_total) seg = passes_total;
-    int64_t n_seg = (passes_total + seg - 1) / seg;
-    const int64_t grid =
-        std::min<int64_t>(((int64_t)n_ind * n_seg + kNaWarps - 1) / kNaWarps, 4 * num_sms);
+    const int64_t n_seg = (passes_total + seg - 1) / seg;
+    const int64_t items = (int64_t)n_ind * n_seg, grid = std::min<int64_t>(items, num_sms);
+    const int64_t warps = std::min<int64_t>((items + grid - 1) / grid, kNaEvalWarps);
     const int aligned = rows % 4 == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0;
     const NaKernel kern = kNaEval[(p->neg_trends ? 8 : 0) + (p->non_strict ? 4 : 0) +
                                   (p->last_kept ? 2 : 0) + aligned];
-    if ((e = launch_next(kern, (unsigned)grid, kNaThreads, s, x, rows, col_idx, offsets, n_ind,
+    if ((e = launch_next(kern, (unsigned)grid, (unsigned)warps * 32u, s, x, rows, col_idx, offsets, n_ind,
                          (int32_t)n_seg, (int32_t)seg, p->ratio_num, p->ratio_den, sc)) !=
         cudaSuccess)
       break;

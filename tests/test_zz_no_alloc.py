@@ -235,3 +235,21 @@ def test_noalloc_any_alignment_and_row_count(ebic, R, C, offset):
         with pytest.raises(ebic.EbicError) as e:
             ebic.ebic_eval_population_noalloc(y, ci_d, off_d, p, *outs)
         assert e.value.code == ebic.EBIC_ENAN
+
+
+@pytest.mark.parametrize("R,n", [(100, 1), (90, 151), (128, 153), (300, 500), (20_000, 40),
+                                 (3_001, 2_000)])
+def test_noalloc_runs_of_items(ebic, R, n):
+    """Fewer individuals than SMs, one more, and several row segments: the runs of items that the
+    blocks own start and end anywhere.  Equal to the oracle."""
+    torch = pytest.importorskip("torch")
+    dev = torch.device("cuda:0")
+    x, ci, off = make_inputs(R + n, R, 12, n)
+    x_cm = torch.from_numpy(np.ascontiguousarray(x.T)).to(dev)
+    ci_d, off_d = torch.from_numpy(ci).to(dev), torch.from_numpy(off).to(dev)
+    p = ebic.Params.make(neg_trends=1, ratio_num=85, ratio_den=100)
+    op = OParams(neg_trends=1, ratio_num=85, ratio_den=100, min_rows=p.min_rows,
+                 col_cap=p.col_cap)
+    outs = _outs(torch, n, dev)
+    ebic.ebic_eval_population_noalloc(x_cm, ci_d, off_d, p, *outs)
+    assert _same([o.cpu().numpy() for o in outs], ocounts.eval_population(x, ci, off, op))
