@@ -121,8 +121,10 @@ typedef struct ebic_params {
                           column pairs whose pair test is exact (the ratio lets no pair fail,
                           ceil(ratio * pairs) = pairs) is evaluated by the warp that built it,
                           inside the evolve kernel; the other slots go to the evaluation
-                          launch.  0 (default) = the library's choice, -1 = never, 1-63 = this
-                          limit.  Results never depend on it                                */
+                          launch.  0 (default) = the library's choice (for a small population
+                          over a short matrix: every child, whatever its test, by the block that
+                          built it), -1 = never, 1-63 = this limit.  Results never depend
+                          on it                                                             */
 } ebic_params;
 
 /* Progress of a run (Sec. 2.4, steps 6 and 8). */

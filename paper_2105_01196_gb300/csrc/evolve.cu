@@ -2,8 +2,9 @@
 // elitism, tournament selection with an exponential penalty on overused columns, tabu list of
 // chromosome hashes, tabu-hit termination; parameters of Sec. 2.4's last paragraph).
 //
-// One generation is three kernels, captured as CUDA graphs (one per buffer parity, and one of
-// sixteen consecutive generations per starting parity) and replayed:
+// One generation is three kernels, or two (k_evolve_block, k_finish) where a small population's
+// blocks are all resident and evaluate their children whole.  They are captured as CUDA graphs (one
+// per buffer parity, and one of sixteen consecutive generations per starting parity) and replayed:
 //   k_evolve    one block per slot, one warp per tabu attempt: elites from the top list (step
 //               4), otherwise penalised tournament, optional one-point crossover and one
 //               mutation, tabu probe; the lowest attempt that misses the tabu list wins (step 5).
@@ -985,7 +986,8 @@ __global__ void __launch_bounds__(kMaxAttemptWarps * 32) k_evolve(GenArgs ga, Bu
 // evaluation launch's side task (the previous generation's keys into the tabu list).  Elites
 // take their row counts from the list.
 // Bound: latency, the slot's chain of dependent loads (tournament, tabu probe) and then one round
-// trip per four pairs.  10,000 x 100, P = 800: 17.3 us per generation with three launches.
+// trip per four pairs.  10,000 x 100, P = 800: 14.0 us per generation; 17.3 with three launches
+// (15.5 with these two, the rest by cheaper children).
 constexpr int kBlockWarps = 4;        // attempt warps at most
 constexpr int kBlockMaxSteps = 4;     // steps of four words per thread over a pair row, at most
 
