@@ -157,7 +157,7 @@ def eval_kernel_name(mode, cols):
 # carries a hash of them as they were when the capture ran; a row whose hash differs from the
 # files now describes an earlier kernel and is not reported.
 KERNEL_SOURCES = {
-    "k_evolve_seq": ["evolve.cu", "tables.cuh"],
+    "k_evolve_seq": ["evolve.cu", "trend.cuh", "tables.cuh"],
     "k_eval_bitmap": ["eval.cu", "items.cuh", "trend.cuh", "tables.cuh"],
 }
 
