@@ -40,6 +40,24 @@ __device__ __forceinline__ void wait_prior_grid() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+// Launches `kern` so that it may be scheduled while the previous kernel of the stream drains
+// (pdl; the kernel waits for that kernel's results before it reads them).
+template <class... Args>
+cudaError_t launch_pdl_opt(void (*kern)(Args...), unsigned grid, size_t smem, cudaStream_t s,
+                           bool pdl, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 // ------------------------------------------------------------------------------- rank codes
 
 // One warp ranks one row at a time.  Its C keys (padded with 0xFFFFFFFF, above every key of a
@@ -240,6 +258,7 @@ __global__ void __launch_bounds__(kThreads, EPL >= 32 ? 3 : 2)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t *srt = s_rank + warp * kSorted;
   uint32_t *tile = s_rank + kWarps * kSorted;  // [C][kTileStride]: keys, then codes in place
+  wait_prior_grid();
   // (tiles [t_begin, t_end) of the R_pad / kRankRows)
   for (int64_t t = t_begin + blockIdx.x; t < t_end; t += gridDim.x) {
     const int64_t r0 = t * kRankRows;
@@ -369,6 +388,7 @@ __global__ void __launch_bounds__(kThreads) k_code_planes(const uint8_t *__restr
                                                           int64_t ch0, int64_t ch1,
                                                           uint32_t *__restrict__ planes,
                                                           unsigned long long *__restrict__ cnt) {
+  wait_prior_grid();
   const int lane = threadIdx.x & 31;
   if (cnt)  // the pair counts, which the build accumulates, cleared beside
     for (int64_t q = (int64_t)blockIdx.x * kThreads + threadIdx.x; q < (int64_t)C * C;
@@ -547,21 +567,6 @@ __global__ void __launch_bounds__(kThreads, 4) k_eval_codes(EvalArgs a, PopView 
   }
 }
 
-template <class... Args>
-cudaError_t launch_pdl_opt(void (*kern)(Args...), dim3 grid, dim3 block, cudaStream_t s,
-                           bool pdl, Args... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = pdl ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kern, args...);
-}
-
 }  // namespace
 
 int code_bytes_for(int32_t C) { return C <= 128 ? 1 : (C <= 1024 ? 2 : 0); }
@@ -597,8 +602,8 @@ cudaError_t launch_code_planes(const void *codes, int code_bytes, int64_t S, int
   const uint8_t *cd = static_cast<const uint8_t *>(codes);
 #define EBIC_PLANES(W, NB)                                                               \
   case NB:                                                                               \
-    k_code_planes<W, NB><<<grid, kThreads, 0, s>>>(cd, S, C, chunks, ch0, ch1, planes, cnt); \
-    break
+    return launch_pdl_opt(k_code_planes<W, NB>, grid, 0, s, true, cd, S, C, chunks, ch0, ch1, \
+                          planes, cnt)
   switch (code_plane_bits(C)) {
     EBIC_PLANES(1, 1);
     EBIC_PLANES(1, 2);
@@ -613,7 +618,6 @@ cudaError_t launch_code_planes(const void *codes, int code_bytes, int64_t S, int
     default: return cudaErrorInvalidValue;
   }
 #undef EBIC_PLANES
-  return cudaGetLastError();
 }
 
 namespace {
@@ -645,9 +649,8 @@ cudaError_t launch_rank_epl(const uint32_t *keys, int64_t R_pad, int32_t C, T *c
   const int64_t t_begin = r_begin / kRankRows, t_end = r_end / kRankRows;
   const int64_t grid = std::min<int64_t>(
       t_end - t_begin, (int64_t)num_sms * resident_blocks((const void *)k_rank_codes<T, EPL>, kThreads, smem));
-  k_rank_codes<T, EPL><<<(unsigned)grid, kThreads, smem, s>>>(keys, R_pad, C, S, codes,
-                                                                t_begin, t_end);
-  return cudaGetLastError();
+  return launch_pdl_opt(k_rank_codes<T, EPL>, (unsigned)grid, smem, s, true, keys, R_pad, C, S,
+                        codes, t_begin, t_end);
 }
 
 }  // namespace
@@ -725,5 +728,5 @@ cudaError_t launch_eval_codes(const EvalArgs &a0, const PopView &pv, int num_sms
   int64_t grid = (int64_t)num_sms * bps;
   const int64_t need = (items + kWarps - 1) / kWarps;
   if (grid > need) grid = need;
-  return launch_pdl_opt(kern, dim3((unsigned)grid), dim3(kThreads), s, pdl, a, pv);
+  return launch_pdl_opt(kern, (unsigned)grid, 0, s, pdl, a, pv);
 }
