@@ -30,6 +30,8 @@
 #include <string.h>
 
 #include <algorithm>
+#include <memory>
+#include <new>
 #include <vector>
 
 #include "internal.h"
@@ -2305,12 +2307,14 @@ int gen_reset(ebic_ctx *ctx, GenState *g) {
   return EBIC_OK;
 }
 
+// The state becomes the context's only when it is complete: after a failure (an allocation, say) the
+// context has none, and the next call creates it anew.
 int gen_create(ebic_ctx *ctx, const ebic_params *p) {
   gen_state_free(ctx->gen);
   ctx->gen = nullptr;
-  GenState *g = new (std::nothrow) GenState();
+  std::unique_ptr<GenState> own(new (std::nothrow) GenState());
+  GenState *g = own.get();
   if (!g) return ebic_fail(ctx, EBIC_ENOMEM, "host allocation failed");
-  ctx->gen = g;
   g->p = *p;
   g->P = p->pop_size;
   g->K = p->n_biclusters;
@@ -2380,7 +2384,9 @@ int gen_create(ebic_ctx *ctx, const ebic_params *p) {
       1, std::min<int64_t>((g->P + kTopThreads - 1) / kTopThreads, ctx->num_sms));
   EBIC_CHECK_CUDA(ctx, cudaStreamCreateWithFlags(&g->cap_stream, cudaStreamNonBlocking));
   for (cudaEvent_t &e : g->cap_ev) EBIC_CHECK_CUDA(ctx, cudaEventCreate(&e));
-  return gen_reset(ctx, g);
+  EBIC_TRY(gen_reset(ctx, g));
+  ctx->gen = own.release();
+  return EBIC_OK;
 }
 
 // (through the context's pinned block: a copy to pageable memory is slower)

@@ -1,0 +1,76 @@
+"""Host paths of the library on a stand-in CUDA runtime (host_only.py): what the entry points
+allocate, launch and leave behind where a real device would have to fail or be probed."""
+
+import ctypes
+
+import numpy as np
+import pytest
+
+from tests.host_only import Library
+
+
+@pytest.fixture()
+def lib():
+    lib = Library()
+    yield lib
+    lib.hook(None)
+    lib.fake_fail_alloc(0)
+
+
+def words(address, n):
+    return [v or 0 for v in (ctypes.c_uint64 * n).from_address(address)]
+
+
+@pytest.mark.parametrize("first", ["run", "tune", "load_state"])
+@pytest.mark.parametrize("reload", [0, 1])
+def test_a_search_that_ran_out_of_memory_leaves_nothing_behind(lib, first, reload):
+    """Whichever allocation of a search fails, the call says EBIC_ENOMEM, and the same call (after a
+    reload of the matrix or not) allocates anew: no launch gets the buffers that are missing."""
+    ebic = lib.ebic
+    p = ebic.Params.make(pop_size=100, max_len=6, init_max_len=6, elite=2, n_biclusters=3, mode=1)
+    ci = np.tile(np.arange(2, dtype=np.int32), 10)
+    off = np.arange(0, 22, 2, dtype=np.int32)
+    null = []
+
+    def check(kernel, grid, args):
+        if "k_reset" in kernel:
+            seg = words(args[0], 28)
+            null.extend(k for k in range(14) if seg[14 + k] and not seg[k])
+        if "k_init" in kernel:
+            null.extend(k for k in range(8) if not words(args[1], 8)[k])
+
+    lib.hook(check)
+    blob = np.zeros(1 << 20, np.uint8)
+    ctx = lib.context()
+    assert lib.load(ctx, 300, 20) == 0
+    assert lib.run(ctx, p, 1)[0] == 0
+    size = lib.ebic_state_bytes(ctx)
+    assert 0 < size <= blob.size and lib.ebic_save_state(ctx, blob.ctypes.data, size) == 0
+    lib.ebic_destroy(ctx)
+
+    def begin(ctx):
+        if first == "run":
+            return lib.run(ctx, p, 1)[0]
+        if first == "load_state":
+            return lib.ebic_load_state(ctx, ctypes.byref(p), blob.ctypes.data, size)
+        return lib.ebic_autotune(ctx, ci.ctypes.data, off.ctypes.data, 10, ctypes.byref(p), 5, None)
+
+    failed = 0
+    for n in range(1, 200):
+        ctx = lib.context()
+        assert lib.load(ctx, 300, 20) == 0
+        lib.fake_fail_alloc(n)
+        st = begin(ctx)
+        lib.fake_fail_alloc(0)
+        if st == 0:
+            lib.ebic_destroy(ctx)
+            break
+        assert st == ebic.EBIC_ENOMEM
+        failed += 1
+        if reload:
+            assert lib.load(ctx, 300, 20) == 0
+        assert lib.run(ctx, p, 1)[0] == 0
+        lib.ebic_destroy(ctx)
+    assert failed > 25 and n < 199
+    assert not null
+    assert lib.fake_device_blocks() == 0
