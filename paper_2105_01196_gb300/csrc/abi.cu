@@ -779,6 +779,25 @@ static int eval_population_plain(ebic_ctx *ctx, const int32_t *col_idx, const in
   return EBIC_OK;
 }
 
+// Whether the device outputs of an evaluation of n individuals can be written as they are: each on its
+// type's boundary, and none over another or over the offsets (which the launch that writes them
+// reads).  A caller's arena may hold them otherwise.
+static bool outputs_apart(void *const outs[4], const bool dev_out[4], size_t n,
+                          const int32_t *offsets) {
+  const uintptr_t begin[5] = {(uintptr_t)outs[0], (uintptr_t)outs[1], (uintptr_t)outs[2],
+                              (uintptr_t)outs[3], (uintptr_t)offsets};
+  const size_t bytes[5] = {n * 4, n * 4, n * 4, n * 8, (n + 1) * 4};
+  for (int k = 0; k < 4; ++k) {
+    if (!outs[k] || !dev_out[k]) continue;
+    if (begin[k] % (k == 3 ? 8 : 4)) return false;
+    for (int j = k + 1; j < 5; ++j)
+      if (begin[j] && (j == 4 || dev_out[j]) && begin[j] < begin[k] + bytes[k] &&
+          begin[k] < begin[j] + bytes[j])
+        return false;
+  }
+  return true;
+}
+
 // One evaluation is three launches (check and clears, evaluation, fitness and outputs) and one
 // synchronisation; the evaluation and the output do nothing when the check failed.  Only where
 // AUTO's choice of the form depends on the mean length of a device population is there a second
@@ -913,26 +932,25 @@ int ebic_eval_population(ebic_ctx *ctx, const int32_t *col_idx, const int32_t *o
     prof_end(ctx, e0, EBIC_KERNEL_EVAL, eval_bytes(ctx, mode, total, n_ind, a.neg),
              pairs * (double)ctx->R * nd, (double)n_ind * (double)ctx->R);
     prof_count(ctx, EBIC_KERNEL_EVAL, 1);
-    // device outputs are written in place; host outputs come through the pinned block, or from
-    // the device buffers by copies once the call is known to be good
+    // device outputs are written in place where the last launch may write them in any order and by
+    // whole words (outputs_apart); host outputs come through the pinned block where they fit; the
+    // others by copies from the device buffers, once the call is known to be good
     SweepOut o{};
-    bool copy_out = false;
+    const bool in_place = outputs_apart(outs, dev_out, n, dev_off ? offsets : nullptr);
     const bool fits = n * 20 <= kPinOut;
-    for (int k = 0; k < 3; ++k) {
-      if (!outs[k]) continue;
-      if (dev_out[k])
-        o.rows[k] = static_cast<int32_t *>(outs[k]);
-      else if (fits)
-        o.rows[k] = reinterpret_cast<int32_t *>(pin_out + n * 8) + k * n;
-      else
-        copy_out = true;
+    bool copy[4], copies = false;
+    for (int k = 0; k < 4; ++k) {
+      copy[k] = outs[k] && !(dev_out[k] ? in_place : fits);
+      copies |= copy[k];
     }
-    if (fitness) {
-      copy_out |= !dev_out[3] && !fits;
-      o.fitness = dev_out[3] ? fitness
-                  : fits     ? reinterpret_cast<uint64_t *>(pin_out)
-                             : ctx->ev_fit.as<uint64_t>();
-    }
+    for (int k = 0; k < 3; ++k)
+      if (outs[k] && !copy[k])
+        o.rows[k] = dev_out[k] ? static_cast<int32_t *>(outs[k])
+                               : reinterpret_cast<int32_t *>(pin_out + n * 8) + k * n;
+    if (fitness)
+      o.fitness = copy[3]      ? ctx->ev_fit.as<uint64_t>()
+                  : dev_out[3] ? fitness
+                               : reinterpret_cast<uint64_t *>(pin_out);
     EBIC_CHECK_CUDA(ctx, launch_sweep_finish(a, pv, sw, o, status_d, s));
     prof_count(ctx, -1, 1);
     EBIC_CHECK_CUDA(ctx, cudaStreamSynchronize(s));
@@ -942,14 +960,13 @@ int ebic_eval_population(ebic_ctx *ctx, const int32_t *col_idx, const int32_t *o
       if (outs[k] && !dev_out[k] && fits)
         memcpy(outs[k], pin_out + n * 8 + (size_t)k * n * 4, n * 4);
     if (fitness && !dev_out[3] && fits) memcpy(fitness, pin_out, n * 8);
-    if (copy_out) {
+    if (copies) {
       for (int k = 0; k < 3; ++k)
-        if (outs[k] && !dev_out[k])
+        if (copy[k])
           EBIC_CHECK_CUDA(ctx, cudaMemcpyAsync(outs[k], counts + (size_t)k * n, n * 4,
-                                               cudaMemcpyDeviceToHost, s));
-      if (fitness && !dev_out[3])
-        EBIC_CHECK_CUDA(ctx, cudaMemcpyAsync(fitness, ctx->ev_fit.p, n * 8,
-                                             cudaMemcpyDeviceToHost, s));
+                                               cudaMemcpyDefault, s));
+      if (copy[3])
+        EBIC_CHECK_CUDA(ctx, cudaMemcpyAsync(fitness, ctx->ev_fit.p, n * 8, cudaMemcpyDefault, s));
       EBIC_CHECK_CUDA(ctx, cudaStreamSynchronize(s));
     }
     if (status[1]) {

@@ -74,3 +74,42 @@ def test_a_search_that_ran_out_of_memory_leaves_nothing_behind(lib, first, reloa
     assert failed > 25 and n < 199
     assert not null
     assert lib.fake_device_blocks() == 0
+
+
+@pytest.mark.parametrize("at,written", [
+    ((0, 1024, 2048, 4096), (1, 1, 1, 1)),            # apart, on their boundaries: all in place
+    ((0, 1024, 2048, 4100), (0, 0, 0, 0)),            # fitness between two boundaries
+    ((2, 1024, 2048, 4096), (0, 0, 0, 0)), ((0, 1024, 2049, 4096), (0, 0, 0, 0)),
+    ((0, 0, 2048, 4096), (0, 0, 0, 0)),               # one over another
+    ((0, 1024, 2048, 2176), (0, 0, 0, 0)),
+    ((8192, 1024, 2048, 4096), (0, 0, 0, 0)),         # over the offsets
+    ((8192 - 396, 1024, 2048, 4096), (0, 0, 0, 0)), ((8192 - 400, 1024, 2048, 4096), (1, 1, 1, 1)),
+    ((None, 1024, None, 4100), (0, 0, 0, 0)), ((None, 1024, None, 4104), (0, 1, 0, 1))])
+def test_device_outputs_are_written_in_place_only_where_they_can_be(lib, at, written):
+    """100 individuals; outputs at byte offsets of one device block, the population's offsets at
+    8,192.  What is not written in place is copied there, outputs in their order."""
+    n = 100
+    seen, copied = [], []
+
+    def look(kernel, grid, args):
+        if "k_sweep_finish" in kernel:
+            seen.extend(words(args[3], 4))
+            copied.append(lib.fake_calls(b"copy"))
+
+    ctx = lib.context()
+    assert lib.load(ctx, 300, 20) == 0
+    block = lib.device(1 << 14)
+    cols = lib.device(4 * 2 * n)
+    off = np.arange(0, 2 * n + 2, 2, dtype=np.int32)
+    ctypes.memmove(block + 8192, off.ctypes.data, off.nbytes)
+    outs = [None if o is None else block + o for o in at]
+    p = lib.ebic.Params.make(mode=1)
+    lib.hook(look)
+    lib.fake_clear_log()
+    assert lib.ebic_eval_population(ctx, cols, block + 8192, n, ctypes.byref(p), *outs) == 0
+    assert [int(s == o) for s, o in zip(seen, [o or 0 for o in outs])] == \
+        [1 if o is None and k < 3 else w for k, (o, w) in enumerate(zip(outs, written))]
+    assert all(s % (8 if k == 3 else 4) == 0 for k, s in enumerate(seen))
+    wanted = sum(o is not None for o in outs)
+    assert lib.fake_calls(b"copy") - copied[0] == wanted - sum(written)
+    lib.ebic_destroy(ctx)
