@@ -800,8 +800,9 @@ static bool outputs_apart(void *const outs[4], const bool dev_out[4], size_t n,
 
 // One evaluation is three launches (check and clears, evaluation, fitness and outputs) and one
 // synchronisation; the evaluation and the output do nothing when the check failed.  Only where
-// AUTO's choice of the form depends on the mean length of a device population is there a second
-// synchronisation, after the check.  A small host population goes through the context's pinned
+// AUTO's choice of the form depends on the mean length of a device population, or where the form
+// has its operand (bitmap, rank codes) built by this call, is there a second synchronisation, after
+// the check.  A small host population goes through the context's pinned
 // block, which the first launch reads and the last one writes, instead of through copies.
 // (With separate clears, copies and two to three synchronisations, a call took about 90 us more
 // than its kernels: 64 individuals on 200 x 20 from host arrays 110 us, now 31; 800 on
@@ -889,8 +890,16 @@ int ebic_eval_population(ebic_ctx *ctx, const int32_t *col_idx, const int32_t *o
   }
   const bool wait_len =
       !known && mode_needs_mean_len(ctx, p->mode, n_ind, 1, p->last_kept);
+  auto choose = [&]() {  // (2: any length will do)
+    return choose_mode(ctx, p->mode, n_ind, known ? (double)total / n_ind : 2.0, 1, p->last_kept);
+  };
+  int mode = wait_len ? EBIC_MODE_AUTO : choose();
+  // the form's first use on this matrix builds its operand: not for a population that is refused
+  const bool builds =
+      (mode == EBIC_MODE_BITMAP && !ctx->bitmap_ok) ||
+      (direct_form_used(ctx, mode, p) && ctx->code_bytes && !ctx->codes_ready);
   // (the algorithmic work, for the kernel statistics, needs the total too)
-  const bool want_ends = !known && (wait_len || ctx->prof);
+  const bool want_ends = wait_len || builds || (!known && ctx->prof);
   status[4] = 0;
   EBIC_CHECK_CUDA(ctx, launch_sweep_prepare(src_cols, src_off, n_ind, ctx->C, counts, sw,
                                             copy_cols, copy_off,
@@ -905,9 +914,8 @@ int ebic_eval_population(ebic_ctx *ctx, const int32_t *col_idx, const int32_t *o
     }
     total = (int64_t)status[3] - status[2];
     known = true;
+    if (wait_len) mode = choose();
   }
-  const double mean_len = known ? (double)total / n_ind : 2.0;  // (2: any length will do)
-  const int mode = choose_mode(ctx, p->mode, n_ind, mean_len, 1, p->last_kept);
   // from here on a failure leaves the check's word to be cleared
   auto evaluate = [&]() -> int {
     if (mode == EBIC_MODE_BITMAP && !ctx->bitmap_ok) EBIC_TRY(ebic_build_bitmap(ctx));

@@ -17,6 +17,10 @@ def lib():
     lib.fake_fail_alloc(0)
 
 
+def ints(address, n):
+    return (ctypes.c_int32 * n).from_address(address)
+
+
 def words(address, n):
     return [v or 0 for v in (ctypes.c_uint64 * n).from_address(address)]
 
@@ -112,4 +116,51 @@ def test_device_outputs_are_written_in_place_only_where_they_can_be(lib, at, wri
     assert all(s % (8 if k == 3 else 4) == 0 for k, s in enumerate(seen))
     wanted = sum(o is not None for o in outs)
     assert lib.fake_calls(b"copy") - copied[0] == wanted - sum(written)
+    lib.ebic_destroy(ctx)
+
+
+@pytest.mark.parametrize("mode", [0, 1, 2])
+@pytest.mark.parametrize("device", [0, 1])
+def test_a_refused_population_builds_nothing(lib, mode, device):
+    """A population that the check refuses is refused before the form's bitmap or rank codes are
+    built (there may be no memory for them), and the next good one is evaluated."""
+    n = 800                       # (AUTO: the bitmap pays for device and host populations alike)
+    ci = np.tile(np.arange(20, dtype=np.int32), n)
+    off = np.arange(0, 20 * n + 20, 20, dtype=np.int32)
+    bad = True
+
+    def check(kernel, grid, args):     # what the first and the last launch write of the check
+        if "k_sweep_prepare" in kernel:
+            ints(words(args[5], 1)[0], 3)[1] = 2 * bad
+            if words(args[8], 1)[0]:
+                ends = ints(words(args[8], 1)[0], 3)
+                ends[0], ends[1] = 0, 20 * n
+                if bad:
+                    ends[2] = 1
+        if "k_sweep_finish" in kernel:
+            ints(words(args[4], 1)[0], 1)[0] = ints(words(args[2], 1)[0], 3)[1]
+
+    lib.hook(check)
+    ctx = lib.context()
+    assert lib.load(ctx, 3000, 20) == 0
+    a, o = ci.ctypes.data, off.ctypes.data
+    if device:
+        a, o = lib.device(ci.nbytes), lib.device(off.nbytes)
+        ctypes.memmove(a, ci.ctypes.data, ci.nbytes)
+        ctypes.memmove(o, off.ctypes.data, off.nbytes)
+    out = np.zeros(n, np.int32)
+    p = lib.ebic.Params.make(mode=mode)
+
+    def call():
+        lib.fake_clear_log()
+        st = lib.ebic_eval_population(ctx, a, o, n, ctypes.byref(p), out.ctypes.data, None, None, None)
+        return st, [k for k, _ in lib.log()]
+
+    st, ran = call()
+    assert st == lib.ebic.EBIC_EINVAL
+    assert len(ran) == 1 and "k_sweep_prepare" in ran[0]
+    assert lib.ebic_copy_bitmap(ctx, out.ctypes.data, 1 << 30) == lib.ebic.EBIC_ESTATE
+    bad = False
+    st, ran = call()
+    assert st == 0 and any("k_rank_codes" in k for k in ran) and "k_sweep_finish" in ran[-1]
     lib.ebic_destroy(ctx)
