@@ -164,6 +164,20 @@ static int classify_ptr(ebic_ctx *ctx, const void *p, const char *name, bool *is
   return EBIC_OK;
 }
 
+// Keeps the word that uploads and population checks report in (ebic_ctx::d_err) zero between calls: a
+// call that ends without having read it as zero leaves it cleared.
+namespace {
+struct ErrWordGuard {
+  ebic_ctx *ctx;
+  bool clean = false;
+  ~ErrWordGuard() {
+    if (clean) return;
+    if (cudaMemsetAsync(ctx->d_err.p, 0, sizeof(int32_t), ctx->stream) != cudaSuccess)
+      cudaGetLastError();
+  }
+};
+}  // namespace
+
 static int check_device_ptr(ebic_ctx *ctx, const void *p, const char *name) {
   cudaPointerAttributes attr;
   if (cudaPointerGetAttributes(&attr, p) != cudaSuccess) {
@@ -305,21 +319,19 @@ int stage_population(ebic_ctx *ctx, const int32_t *col_idx, const int32_t *offse
                                          cudaMemcpyHostToDevice, s));
     d_cols = ctx->ev_cols.as<int32_t>();
     d_off = ctx->ev_off.as<int32_t>();
-    EBIC_CHECK_CUDA(ctx, cudaMemsetAsync(ctx->d_err.p, 0, sizeof(int32_t), s));
+    ErrWordGuard guard{ctx};
     EBIC_CHECK_CUDA(ctx, launch_validate_csr(d_cols, d_off, n_ind, ctx->C,
                                              ctx->d_err.as<int32_t>(), s));
     prof_count(ctx, -1, 1);
     int32_t herr = 0;
     EBIC_CHECK_CUDA(ctx, cudaMemcpyAsync(&herr, ctx->d_err.p, 4, cudaMemcpyDeviceToHost, s));
     EBIC_CHECK_CUDA(ctx, cudaStreamSynchronize(s));
-    if (herr) {
-      EBIC_CHECK_CUDA(ctx, cudaMemsetAsync(ctx->d_err.p, 0, sizeof(int32_t), s));
-      return ebic_fail(ctx, EBIC_EINVAL, "invalid chromosome in the population");
-    }
+    if (herr) return ebic_fail(ctx, EBIC_EINVAL, "invalid chromosome in the population");
+    guard.clean = true;
     if (want_host_offsets) h_off.assign(offsets, offsets + n_ind + 1);
   } else {
     // Device CSR: validate on the device before any kernel indexes the matrix with it.
-    EBIC_CHECK_CUDA(ctx, cudaMemsetAsync(ctx->d_err.p, 0, sizeof(int32_t), s));
+    ErrWordGuard guard{ctx};
     EBIC_CHECK_CUDA(ctx, launch_validate_csr(col_idx, offsets, n_ind, ctx->C,
                                              ctx->d_err.as<int32_t>(), s));
     prof_count(ctx, -1, 1);
@@ -334,10 +346,8 @@ int stage_population(ebic_ctx *ctx, const int32_t *col_idx, const int32_t *offse
                                            cudaMemcpyDeviceToHost, s));
     }
     EBIC_CHECK_CUDA(ctx, cudaStreamSynchronize(s));
-    if (herr) {
-      EBIC_CHECK_CUDA(ctx, cudaMemsetAsync(ctx->d_err.p, 0, sizeof(int32_t), s));
-      return ebic_fail(ctx, EBIC_EINVAL, "invalid chromosome in the population");
-    }
+    if (herr) return ebic_fail(ctx, EBIC_EINVAL, "invalid chromosome in the population");
+    guard.clean = true;
     total = (int64_t)ends[1] - ends[0];
     mean_len = (double)total / n_ind;
   }
@@ -509,16 +519,16 @@ void ctx_release_buffers(ebic_ctx *ctx) {
 
 namespace {
 
-// Waits for the uploads of a load and reads their error word, which is 0 between calls.
-int read_upload_error(ebic_ctx *ctx) {
+// Waits for the uploads of a load and reads their error word.
+int read_upload_error(ebic_ctx *ctx, ErrWordGuard *guard) {
   EBIC_CHECK_CUDA(ctx, cudaMemcpyAsync(ctx->pin, ctx->d_err.p, sizeof(int32_t),
                                        cudaMemcpyDeviceToHost, ctx->stream));
   EBIC_CHECK_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
   int32_t herr = 0;
   memcpy(&herr, ctx->pin, sizeof(herr));
-  if (!herr) return EBIC_OK;
-  EBIC_CHECK_CUDA(ctx, cudaMemsetAsync(ctx->d_err.p, 0, sizeof(int32_t), ctx->stream));
-  return ebic_fail(ctx, EBIC_ENAN, "matrix holds NaN or Inf");
+  if (herr) return ebic_fail(ctx, EBIC_ENAN, "matrix holds NaN or Inf");
+  guard->clean = true;
+  return EBIC_OK;
 }
 
 // The segmented load of a row-major host matrix (see ebic_load_matrix): kLoadSegments segments
@@ -557,6 +567,7 @@ int load_matrix_segmented(ebic_ctx *ctx, const float *x, int64_t rows, int32_t c
   EBIC_CHECK_CUDA(ctx, cudaEventRecord(ctx->seg_ev[n_seg], s));
   EBIC_CHECK_CUDA(ctx, cudaStreamWaitEvent(ctx->copy_stream, ctx->seg_ev[n_seg], 0));
   float *stage = ctx->stage_x.as<float>();
+  ErrWordGuard guard{ctx};
   for (int64_t i = 0; i < n_seg; ++i) {
     const int64_t r0 = i * seg, r1 = std::min(R_pad, r0 + seg);
     if (r0 < rows) {
@@ -588,7 +599,7 @@ int load_matrix_segmented(ebic_ctx *ctx, const float *x, int64_t rows, int32_t c
     prof_count(ctx, EBIC_KERNEL_BITMAP_BUILD, 1);
     ctx->tie_state = -1;
   }
-  EBIC_TRY(read_upload_error(ctx));
+  EBIC_TRY(read_upload_error(ctx, &guard));
   ctx->R = rows;
   ctx->C = cols;
   ctx->R_pad = R_pad;
@@ -649,10 +660,11 @@ int ebic_load_matrix(ebic_ctx *ctx, const float *x, int64_t rows, int32_t cols, 
                                          cudaMemcpyHostToDevice, ctx->stream));
     src = ctx->stage_x.as<float>();
   }
+  ErrWordGuard guard{ctx};
   EBIC_CHECK_CUDA(ctx, launch_upload(src, rows, cols, R_pad, layout, ctx->keys.as<uint32_t>(),
                                      ctx->d_err.as<int32_t>(), ctx->stream));
   prof_count(ctx, -1, 1);
-  EBIC_TRY(read_upload_error(ctx));
+  EBIC_TRY(read_upload_error(ctx, &guard));
   ctx->R = rows;
   ctx->C = cols;
   ctx->R_pad = R_pad;

@@ -2,7 +2,7 @@
 // the library are linked with this file instead of the CUDA runtime.  Device memory is host memory
 // (zeroed), streams run at once, and kernels do nothing but report their launch: the hook gets the
 // kernel's name, its grid and the addresses of its arguments, and may write what the kernel would
-// have written.  An allocation can be made to fail (fake_fail_alloc), and the times between events
+// have written.  An allocation or a copy can be made to fail (fake_fail_alloc, fake_fail_copy), and the times between events
 // are what the test says (fake_elapsed).
 #include <cuda_runtime_api.h>
 #include <string.h>
@@ -32,6 +32,7 @@ std::vector<Launch> g_log;                     // launches that ran, graph repla
 std::vector<std::string> g_calls;              // copies and synchronisations
 Hook g_hook = nullptr;
 int64_t g_fail_at = 0, g_allocs = 0;
+int64_t g_fail_copy = 0, g_copies = 0;
 size_t g_free = size_t(64) << 30;
 float g_elapsed = 1.f, g_elapsed_step = 0.f;
 cudaError_t g_last = cudaSuccess;
@@ -99,6 +100,10 @@ void fake_hook(Hook h) { g_hook = h; }
 void fake_fail_alloc(int64_t n) {  // the n-th allocation from now on fails (0: none)
   g_allocs = 0;
   g_fail_at = n;
+}
+void fake_fail_copy(int64_t n) {  // the same for copies
+  g_copies = 0;
+  g_fail_copy = n;
 }
 int64_t fake_allocs() { return g_allocs; }
 int64_t fake_device_blocks() { return (int64_t)g_device.size(); }
@@ -205,7 +210,7 @@ cudaError_t cudaPointerGetAttributes(cudaPointerAttributes *a, const void *p) {
 }
 cudaError_t cudaMemcpy(void *d, const void *s, size_t n, cudaMemcpyKind) {
   g_calls.push_back("copy");
-  if (n && (!d || !s)) return set(cudaErrorInvalidValue);
+  if (++g_copies == g_fail_copy || (n && (!d || !s))) return set(cudaErrorInvalidValue);
   memmove(d, s, n);
   return cudaSuccess;
 }

@@ -43,7 +43,8 @@ class Library:
             getattr(self.raw, name).restype = ctypes.c_int64
         self.raw.fake_log_kernel.restype = ctypes.c_char_p
         self.raw.fake_log_kernel.argtypes = self.raw.fake_log_grid.argtypes = [ctypes.c_int64]
-        self.raw.fake_fail_alloc.argtypes = self.raw.fake_set_free.argtypes = [ctypes.c_int64]
+        for name in ("fake_fail_alloc", "fake_fail_copy", "fake_set_free"):
+            getattr(self.raw, name).argtypes = [ctypes.c_int64]
         self.raw.fake_elapsed.argtypes = [ctypes.c_float, ctypes.c_float]
         self.raw.cudaMalloc.argtypes = [ctypes.c_void_p, ctypes.c_size_t]
         self._hook = None

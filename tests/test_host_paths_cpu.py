@@ -15,6 +15,7 @@ def lib():
     yield lib
     lib.hook(None)
     lib.fake_fail_alloc(0)
+    lib.fake_fail_copy(0)
 
 
 def ints(address, n):
@@ -163,4 +164,37 @@ def test_a_refused_population_builds_nothing(lib, mode, device):
     bad = False
     st, ran = call()
     assert st == 0 and any("k_rank_codes" in k for k in ran) and "k_sweep_finish" in ran[-1]
+    lib.ebic_destroy(ctx)
+
+
+@pytest.mark.parametrize("call,copy", [("load", 2), ("evaluate", 3), ("tune", 3)])
+def test_an_error_that_was_never_read_does_not_reach_the_next_load(lib, call, copy):
+    """A load (NaN in the matrix) or a population check (a bad chromosome) whose result could not be
+    read: the copy fails, and the next load of a good matrix is accepted."""
+    bad = True
+
+    def check(kernel, grid, args):
+        if bad and "k_upload" in kernel and call == "load":
+            ints(words(args[5], 1)[0], 1)[0] = 1
+        if bad and "k_validate_csr" in kernel:
+            ints(words(args[4], 1)[0], 1)[0] = 2
+
+    lib.hook(check)
+    ctx = lib.context()
+    ci, off = np.zeros(8, np.int32), np.arange(0, 10, 2, dtype=np.int32)
+    p = lib.ebic.Params.make(mode=3)                   # (the plain form)
+    if call != "load":
+        assert lib.load(ctx, 300, 20) == 0
+    lib.fake_fail_copy(copy)
+    if call == "load":
+        assert lib.load(ctx, 300, 20) == lib.ebic.EBIC_ECUDA
+    elif call == "evaluate":
+        assert lib.ebic_eval_population(ctx, ci.ctypes.data, off.ctypes.data, 4, ctypes.byref(p),
+                                        None, None, None, None) == lib.ebic.EBIC_ECUDA
+    else:
+        assert lib.ebic_autotune(ctx, ci.ctypes.data, off.ctypes.data, 4, ctypes.byref(p), 1,
+                                 None) == lib.ebic.EBIC_ECUDA
+    lib.fake_fail_copy(0)
+    bad = False
+    assert lib.load(ctx, 300, 20) == 0
     lib.ebic_destroy(ctx)
