@@ -590,6 +590,18 @@ def timed_steps(job, stream, flush, steps, dist=None, profile_range=False):
     return total_ms, units
 
 
+def loop_evaluates_in_evolve(ctx, ebic):
+    """Whether the steps since the counters were reset made fewer evaluation than evolve launches:
+    every child is then evaluated inside the evolve launch."""
+    return (ctx.profile_read(ebic.KERNEL_EVAL)["launches"]
+            < ctx.profile_read(ebic.KERNEL_EVOLVE)["launches"])
+
+
+SEPARATE_NOTE = ("the timed steps evaluate every child inside the evolve launch (k_evolve_block, two "
+                 "launches per generation); the kernel times and the roofline are of the pass with "
+                 "kernel statistics, which makes an evaluation launch of its own")
+
+
 def kernel_stats(job, stream, flush, steps):
     """A second pass of the same steps with CUDA events around every kernel of the path (event
     nodes inside the generation graphs): per-kernel durations, work and shares, and the pass's
@@ -656,7 +668,10 @@ def workload_summary(job, stream, flush, steps, warmup, peak, peak_kind):
     job.tune()
     for _ in range(warmup):
         job.step(False)
+    job.ctx.profile_enable(True)        # (resets the launch counters)
+    job.ctx.profile_enable(False)
     ms, units = timed_steps(job, stream, flush, steps)
+    separate = loop_evaluates_in_evolve(job.ctx, job.ebic)
     stats, passes = kernel_stats(job, stream, flush, steps)
     w = job.w
     out = {"value": units / (ms / 1e3), "unit": UNIT, "ms_per_step": ms / steps,
@@ -672,6 +687,8 @@ def workload_summary(job, stream, flush, steps, warmup, peak, peak_kind):
            "kernel_ms": {k: v["ms"] / steps for k, v in stats.items()}, **passes}
     if job.gens > 0:
         out["generations_per_s"] = job.gens * steps / (ms / 1e3)
+    if separate:
+        out["kernel_stats_note"] = SEPARATE_NOTE
     return out
 
 
@@ -793,6 +810,7 @@ def main():
     total_ms, units = timed_steps(job, stream, flush, args.steps,
                                   profile_range=args.profile_range)
     st_all = job.ctx.profile_read(ebic.KERNEL_ALL)
+    separate = loop_evaluates_in_evolve(job.ctx, ebic)
     clk = clocks.stop()
     stats, passes = kernel_stats(job, stream, flush, args.steps)
     if dist:
@@ -894,6 +912,8 @@ def main():
                                                           "fuse_loop",
                                                           "direct_ms", "bitmap_ms", "build_ms",
                                                           "staged_ms")}
+    if separate:
+        line["kernel_passes"]["note"] = SEPARATE_NOTE
     if gens > 0:
         line["generations_per_s"] = gens * args.steps / (total_ms / 1e3)
         line["quality"] = search_quality(job.ctx, job.truth, job.R, w.cols, gens)

@@ -279,7 +279,11 @@ EBIC_API int ebic_load_state(ebic_ctx *ctx, const ebic_params *p, const void *bl
  * Kernel statistics for roofline accounting (no counterpart in the paper).  While enabled, the
  * context records CUDA events on its stream around every launch of the evaluation kernel, the
  * bitmap build and the generation-loop kernels (inside replayed CUDA graphs too, through event
- * nodes re-pointed at fresh events before each replay), and it counts every kernel it launches.
+ * nodes re-pointed at fresh events before each replay); it counts every kernel it launches, enabled
+ * or not.  Where the loop evaluates every child inside the evolve launch (fuse_pairs 0, a small
+ * population over a short matrix: two launches per generation), it makes a separate evaluation
+ * launch per generation while this is enabled, so that the two can be timed apart: the times are
+ * then those of the three-launch form, the launch counts those of the launches made.
  *   kernel  EBIC_KERNEL_EVAL (direct or bitmap evaluation, single sweeps and generations),
  *           EBIC_KERNEL_BITMAP_BUILD, EBIC_KERNEL_EVOLVE (children of one generation),
  *           EBIC_KERNEL_FINISH (scoring, tabu list and top-list update of one generation),

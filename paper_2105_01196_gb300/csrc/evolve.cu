@@ -2616,7 +2616,7 @@ int ebic_run_generations(ebic_ctx *ctx, const ebic_params *p, int32_t n_gen,
         if (!g->multi[parity]) EBIC_TRY(capture_multi(ctx, g, parity));
         EBIC_CHECK_CUDA(ctx, cudaGraphLaunch(g->multi[parity], s));
         prof_count(ctx, EBIC_KERNEL_EVOLVE, kGraphGenerations);
-        prof_count(ctx, EBIC_KERNEL_EVAL, kGraphGenerations);
+        if (!g->block_eval) prof_count(ctx, EBIC_KERNEL_EVAL, kGraphGenerations);
         prof_count(ctx, EBIC_KERNEL_FINISH, kGraphGenerations);
         i += kGraphGenerations - 1;
         continue;
@@ -2638,7 +2638,7 @@ int ebic_run_generations(ebic_ctx *ctx, const ebic_params *p, int32_t n_gen,
       }
       if (timed) push_generation_timing(ctx, m, true);
       prof_count(ctx, EBIC_KERNEL_EVOLVE, 1);
-      prof_count(ctx, EBIC_KERNEL_EVAL, 1);
+      if (timed || !g->block_eval) prof_count(ctx, EBIC_KERNEL_EVAL, 1);
       prof_count(ctx, EBIC_KERNEL_FINISH, 1);
       if (!p->use_graph) {
         GenCtl cc{};

@@ -198,3 +198,41 @@ def test_an_error_that_was_never_read_does_not_reach_the_next_load(lib, call, co
     bad = False
     assert lib.load(ctx, 300, 20) == 0
     lib.ebic_destroy(ctx)
+
+
+@pytest.mark.parametrize("graph", [0, 1])
+@pytest.mark.parametrize("fuse,form", [(0, "k_evolve_block"), (-1, "k_evolve"), (2, "k_evolve")])
+def test_the_counters_count_the_launches_made(lib, fuse, form, graph):
+    """A search of 21 generations (a chunk of sixteen and singles in graph replays): the evaluation,
+    evolve and scoring counters are the launches made, with no evaluation launch per generation
+    where k_evolve_block evaluates; with statistics on (eager here) it does have one."""
+    ebic = lib.ebic
+    p = ebic.Params.make(pop_size=100, max_len=6, init_max_len=6, elite=2, n_biclusters=3, mode=2,
+                         fuse_pairs=fuse, use_graph=graph, tabu_hit_limit=0)
+    ctx = lib.context()
+    assert lib.load(ctx, 300, 20) == 0
+
+    def made(part):
+        return sum(part in k for k, _ in lib.log())
+
+    def counted(kernel):
+        st = ebic.KernelStats()
+        assert lib.ebic_profile_read(ctx, kernel, ctypes.byref(st)) == 0
+        return st.launches
+
+    for timed in (0, 1) if not graph else (0,):
+        assert lib.ebic_profile_enable(ctx, 1) == 0
+        assert lib.ebic_profile_enable(ctx, timed) == 0
+        lib.fake_clear_log()
+        st, rep = lib.run(ctx, p, 21)
+        assert st == 0
+        evals, evolves, ends = made("k_eval_bitmap"), made("k_evolve"), made("k_finish")
+        first = 1 - timed                            # (the initial population, scored once)
+        assert evolves == 21 and ends == 21 + first
+        assert evals == first + (0 if form == "k_evolve_block" and not timed else 21)
+        assert (made("k_evolve_block") > 0) == (form == "k_evolve_block" and not timed)
+        assert counted(ebic.KERNEL_EVAL) == evals
+        assert counted(ebic.KERNEL_EVOLVE) == evolves
+        assert counted(ebic.KERNEL_FINISH) == ends
+        assert counted(ebic.KERNEL_ALL) == len(lib.log())
+    lib.ebic_destroy(ctx)
