@@ -631,8 +631,8 @@ int ebic_load_matrix(ebic_ctx *ctx, const float *x, int64_t rows, int32_t cols, 
     return ebic_fail(ctx, EBIC_EINVAL, "rows must be < 2^31 - 128");
   DeviceGuard g(ctx->device);
   EBIC_TRY(check_device_ptr(ctx, x, "x"));
-  // (the autotuner's measurements depend on the matrix's shape only, not on its values: a
-  // matrix of the same shape keeps its decisions)
+  // (a matrix of the same shape keeps the autotuner's decisions; sizes that also depend on whether
+  // many of its column pairs are tied are set aside where they are used: tuned_sizes_hold)
   if (rows != ctx->R || cols != ctx->C) ctx->tuned = false;
   ctx->have_matrix = false;
   ctx->bitmap_ok = false;
@@ -936,11 +936,12 @@ int ebic_eval_population(ebic_ctx *ctx, const int32_t *col_idx, const int32_t *o
       EBIC_TRY(ensure_tie_state(ctx));
     if (direct_form_used(ctx, mode, p)) EBIC_TRY(ensure_codes(ctx));
     set_args();
-    a.seg_passes =
-        ctx->tuned ? (mode == EBIC_MODE_BITMAP ? ctx->seg_bitmap
-                                               : (mode == EBIC_MODE_DIRECT ? ctx->seg_direct : 0))
-                   : 0;
-    a.ipw = p->ipw > 0 ? p->ipw : (ctx->tuned && mode == EBIC_MODE_BITMAP ? ctx->ipw_bitmap : 1);
+    const bool tuned = tuned_sizes_hold(ctx, mode, p);
+    a.seg_passes = !tuned                      ? 0
+                   : mode == EBIC_MODE_BITMAP ? ctx->seg_bitmap
+                   : mode == EBIC_MODE_DIRECT ? ctx->seg_direct
+                                              : 0;
+    a.ipw = p->ipw > 0 ? p->ipw : (tuned && mode == EBIC_MODE_BITMAP ? ctx->ipw_bitmap : 1);
     PopView pv{};
     pv.cols = d_cols;
     pv.off = d_off;

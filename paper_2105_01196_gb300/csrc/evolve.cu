@@ -2098,7 +2098,7 @@ EvalArgs gen_eval_args(ebic_ctx *ctx, GenState *g, int k, bool has_prev) {
   a.fitness = nullptr;
   a.work = g->work.as<int32_t>();
   // (the autotuner's loop sizes were measured in the loop, with the form it chose)
-  const bool tuned = ctx->tuned && g->eval_mode == ctx->tuned_mode;
+  const bool tuned = g->eval_mode == ctx->tuned_mode && tuned_sizes_hold(ctx, g->eval_mode, &g->p);
   a.seg_passes = tuned ? ctx->seg_loop : 0;
   a.ipw = g->p.ipw > 0 ? g->p.ipw : (tuned ? ctx->ipw_loop : 1);
   return a;
@@ -2446,7 +2446,7 @@ int fuse_limit(const ebic_ctx *ctx, int mode, const ebic_params *p) {
   if (mode != EBIC_MODE_BITMAP || p->fuse_pairs < 0 || p->last_kept) return 0;
   if (p->fuse_pairs > 0) return p->fuse_pairs;
   // (the autotuner's limit, measured in the loop with this form)
-  if (ctx->tuned && ctx->tuned_mode == mode && ctx->fuse_loop != 0)
+  if (ctx->tuned_mode == mode && ctx->fuse_loop != 0 && tuned_sizes_hold(ctx, mode, p))
     return ctx->fuse_loop > 0 ? ctx->fuse_loop : 0;
   int G = 1;
   while (G < p->max_attempts) G <<= 1;
@@ -2481,13 +2481,16 @@ int ensure_eval_ready(ebic_ctx *ctx, GenState *g, const ebic_params *p, int n_ge
   // the captured graphs hold the evaluation kernel's data buffer: recapture when it changed
   const void *buf = mode == EBIC_MODE_BITMAP ? ctx->bitmap.p
                     : (direct && ctx->codes_ready ? ctx->codes.p : nullptr);
-  // (and the fusion limit, which the captured evolve launches hold)
-  const int fuse = fuse_limit(ctx, mode, p);
+  // (and the fusion limit, which the captured evolve launches hold; a tuned one may not hold once
+  // the ties are counted)
+  int fuse = fuse_limit(ctx, mode, p);
+  if (mode == EBIC_MODE_BITMAP && p->neg_trends &&
+      (fuse > 1 || (p->ratio_num < p->ratio_den && eval_args_for(ctx).stage_bitmap))) {
+    EBIC_TRY(ensure_tie_state(ctx));
+    fuse = fuse_limit(ctx, mode, p);
+  }
   const bool block = block_eval_fits(ctx, mode, p, fuse);
   const void *cnt = mode == EBIC_MODE_BITMAP && ctx->pair_cnt_ok ? ctx->pair_cnt.p : nullptr;
-  if (mode == EBIC_MODE_BITMAP && p->neg_trends &&
-      (fuse > 1 || (p->ratio_num < p->ratio_den && eval_args_for(ctx).stage_bitmap)))
-    EBIC_TRY(ensure_tie_state(ctx));
   if (mode != g->eval_mode || buf != g->graph_buf || fuse != g->fuse_np ||
       cnt != g->graph_cnt || ctx->tie_state != g->graph_tie || block != g->block_eval) {
     g->drop_graphs();

@@ -255,6 +255,7 @@ struct ebic_ctx {
   int seg_loop = 0;                    // the same for the generation loop's evaluations
   int ipw_bitmap = 1, ipw_loop = 1;    // individuals per work item (staged bitmap form)
   int fuse_loop = 0;  // pair limit of the evaluation inside the evolve kernel (-1: none, 0: untuned)
+  int tuned_tie = -1;  // tie_state that the bitmap form's sizes were measured with
 
   // generation loop state (evolve.cu)
   struct GenState *gen = nullptr;
@@ -284,6 +285,14 @@ int ebic_fail(ebic_ctx *ctx, int code, const std::string &msg);
 // Counts the tied pairs of the bitmap's matrix, once per build (a launch and a synchronisation):
 // called where a form that looks for individuals without ties may run.
 int ensure_tie_state(ebic_ctx *ctx);
+// Whether the autotuner's sizes for form `mode` are those of the loaded matrix.  Its decisions follow
+// the shape, but with negative trends the bitmap's kernels also depend on whether few pairs are
+// tied (tie_state, counted by then where a call's kernels depend on it): sizes measured on a matrix
+// of the other kind are left aside for the built-in ones.
+inline bool tuned_sizes_hold(const ebic_ctx *ctx, int mode, const ebic_params *p) {
+  return ctx->tuned && (mode != EBIC_MODE_BITMAP || !p->neg_trends || ctx->tie_state < 0 ||
+                        ctx->tuned_tie < 0 || ctx->tie_state == ctx->tuned_tie);
+}
 // Builds the rank codes of the loaded matrix if it has some and they are not built yet.
 int ensure_codes(ebic_ctx *ctx);
 // Whether evaluation form `mode` runs the direct kernel (the staged form falls back to it).

@@ -4,7 +4,8 @@
 // work-item size (passes of 128 rows or 128 words per item) that minimise the expected time of
 // `expected_sweeps` evaluations, the bitmap build included when the bitmap does not exist yet.
 // EBIC_MODE_AUTO then follows the recorded choice, both in ebic_eval_population and in the
-// generation loop, until a matrix of another shape is loaded.  When a run of generations is
+// generation loop, until a matrix of another shape is loaded (sizes of the bitmap form's kernels for
+// few or for many tied column pairs only on a matrix of the same kind).  When a run of generations is
 // expected, the loop's own work-item size is measured in a scratch run of the loop (selection
 // soon makes its population shorter than the one given here).
 #include <float.h>
@@ -264,6 +265,7 @@ extern "C" int ebic_autotune(ebic_ctx *ctx, const int32_t *col_idx, const int32_
   const double cost_bitmap = best_bitmap == DBL_MAX
                                  ? DBL_MAX
                                  : build_ms + (double)expected_sweeps * best_bitmap;
+  ctx->tuned_tie = ctx->tie_state;
   ctx->tuned = true;
   ctx->tuned_mode = cost_bitmap < cost_direct ? EBIC_MODE_BITMAP : direct_mode;
   ctx->seg_direct = seg_direct;

@@ -236,3 +236,50 @@ def test_the_counters_count_the_launches_made(lib, fuse, form, graph):
         assert counted(ebic.KERNEL_FINISH) == ends
         assert counted(ebic.KERNEL_ALL) == len(lib.log())
     lib.ebic_destroy(ctx)
+
+
+def test_tuned_sizes_are_for_matrices_of_the_same_kind_of_ties(lib):
+    """Tuned on a matrix with few tied pairs (later candidates time faster here, so the tuner picks
+    the last ones): a reload without many ties runs the same launches, one with many ties those
+    of a context that was never tuned, and after it one with few again the tuned ones."""
+    ebic = lib.ebic
+    R, C = 4500, 650                                  # (243 MB of pair words: larger than L2)
+    tied = 0
+
+    def count(kernel, grid, args):
+        if "k_count_tied" in kernel:
+            ints(words(args[3], 1)[0], 1)[0] = tied
+
+    lib.hook(count)
+    ci = np.arange(600, dtype=np.int32)
+    off = np.arange(0, 606, 6, dtype=np.int32)
+    p = ebic.Params.make(pop_size=2000, max_len=6, init_max_len=6, elite=2, n_biclusters=3, mode=0,
+                         tabu_hit_limit=0, neg_trends=1, ratio_num=85, ratio_den=100)
+
+    def launches(ctx, n_tied):
+        nonlocal tied
+        tied = n_tied
+        assert lib.load(ctx, R, C) == 0 and lib.ebic_build_bitmap(ctx) == 0
+        lib.fake_clear_log()
+        assert lib.ebic_eval_population(ctx, ci.ctypes.data, off.ctypes.data, 100, ctypes.byref(p),
+                                        None, None, None, None) == 0
+        st, rep = lib.run(ctx, p, 3)
+        assert st == 0
+        return [(k, g) for k, g in lib.log() if "k_eval" in k or "k_evolve" in k], rep.fuse_pairs
+
+    many = C * C
+    ctx, plain = lib.context(), lib.context()
+    untuned = {n: launches(plain, n) for n in (0, many)}
+    tied = 0
+    assert lib.load(ctx, R, C) == 0 and lib.ebic_build_bitmap(ctx) == 0
+    lib.fake_elapsed(1000.0, -0.01)
+    rep = ebic.TuneReport()
+    assert lib.ebic_autotune(ctx, ci.ctypes.data, off.ctypes.data, 100, ctypes.byref(p), 100,
+                             ctypes.byref(rep)) == 0
+    assert rep.mode == ebic.MODE_BITMAP and (rep.ipw_bitmap, rep.ipw_loop, rep.fuse_loop) == (4, 4, 63)
+    tuned = launches(ctx, 0)
+    assert tuned[1] == 63 and tuned != untuned[0]
+    assert launches(ctx, many) == untuned[many]
+    assert launches(ctx, 0) == tuned
+    for c in (ctx, plain):
+        lib.ebic_destroy(c)
