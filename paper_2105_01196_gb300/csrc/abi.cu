@@ -1074,7 +1074,7 @@ EvalArgs eval_args_for(const ebic_ctx *ctx) {
   a.codes = ctx->codes_ready ? ctx->codes.as<uint8_t>() : nullptr;
   a.code_bytes = ctx->codes_ready ? ctx->code_bytes : 0;
   a.S = ctx->codes_ready ? ctx->code_stride : 0;
-  a.stage_bitmap = ctx->bitmap_ok && (double)ebic_bitmap_bytes(ctx->R, ctx->C) > (double)ctx->l2_bytes;
+  a.stage_bitmap = ctx->bitmap_ok && bitmap_stored_bytes(ctx->R, ctx->C) > ctx->l2_bytes;
   a.ipw = 1;
   return a;
 }
@@ -1104,18 +1104,17 @@ int choose_mode(const ebic_ctx *ctx, int requested, int64_t n_ind, double mean_l
   }
   if (ctx->tuned) return ctx->tuned_mode;
   if (ctx->bitmap_ok) return EBIC_MODE_BITMAP;
-  const double Wst = (double)ctx->Wst, C = (double)ctx->C;
-  if (!cost_model_prefers_bitmap((double)ctx->R_pad, C, ctx->code_bytes, (double)n_ind, mean_len,
-                                 (double)expected_sweeps))
+  if (!cost_model_prefers_bitmap((double)ctx->R_pad, (double)ctx->C, ctx->code_bytes,
+                                 (double)n_ind, mean_len, (double)expected_sweeps))
     return EBIC_MODE_DIRECT;
   // (the query of the free memory is slow: only where a bitmap is wanted)
-  const double bitmap_bytes = C * C * Wst * 4.0;
   size_t free_b = 0, total_b = 0;
   if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
     cudaGetLastError();
     free_b = 0;
   }
-  return bitmap_bytes > 0.5 * (double)free_b ? EBIC_MODE_DIRECT : EBIC_MODE_BITMAP;
+  const double need = (double)bitmap_build_bytes(ctx->R, ctx->C);
+  return need > 0.5 * (double)free_b ? EBIC_MODE_DIRECT : EBIC_MODE_BITMAP;
 }
 
 bool mode_needs_mean_len(const ebic_ctx *ctx, int requested, int64_t n_ind, int expected_sweeps,

@@ -329,6 +329,17 @@ int ebic_check_run_params(ebic_ctx *ctx, const ebic_params *p);
 // (1.32 ms padded to sectors only), and the evaluations' reads touch a line more per piece.
 // Above 1,024 columns (the build from the keys) rows are not padded.
 int64_t bitmap_stride(int64_t rows, int32_t cols);
+// Bytes of the stored pair words, and of everything that building the bitmap allocates: the words,
+// the bit planes they are built from and the pair counts (rank codes apart).
+inline int64_t bitmap_stored_bytes(int64_t rows, int32_t cols) {
+  return (int64_t)cols * cols * bitmap_stride(rows, cols) * 4;
+}
+inline int64_t bitmap_build_bytes(int64_t rows, int32_t cols) {
+  int64_t b = bitmap_stored_bytes(rows, cols);
+  if (code_bytes_for(cols))
+    b += code_plane_words(cols, bitmap_stride(rows, cols)) * 4 + (int64_t)cols * cols * 8;
+  return b;
+}
 
 // matrix.cu
 cudaError_t launch_upload(const float *x, int64_t R, int32_t C, int64_t R_pad, int32_t layout,

@@ -208,7 +208,7 @@ extern "C" int ebic_autotune(ebic_ctx *ctx, const int32_t *col_idx, const int32_
       seg_direct = seg;
     }
   }
-  // the bitmap form, when its C^2 * R / 8 bytes fit comfortably
+  // the bitmap form, when what its build allocates (about C^2 * R / 8 bytes) fits comfortably
   double build_ms = 0.0;
   size_t free_b = 0, total_b = 0;
   if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
@@ -218,7 +218,7 @@ extern "C" int ebic_autotune(ebic_ctx *ctx, const int32_t *col_idx, const int32_
   const bool had_bitmap = ctx->bitmap_ok;
   // (the last-kept pair test has no bitmap form)
   if (!p->last_kept &&
-      (had_bitmap || (double)ebic_bitmap_bytes(ctx->R, ctx->C) < 0.5 * (double)free_b)) {
+      (had_bitmap || (double)bitmap_build_bytes(ctx->R, ctx->C) < 0.5 * (double)free_b)) {
     if (!had_bitmap) {
       cudaEvent_t e0, e1;
       EBIC_CHECK_CUDA(ctx, cudaEventCreate(&e0));

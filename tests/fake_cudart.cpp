@@ -107,6 +107,11 @@ void fake_fail_copy(int64_t n) {  // the same for copies
 }
 int64_t fake_allocs() { return g_allocs; }
 int64_t fake_device_blocks() { return (int64_t)g_device.size(); }
+int64_t fake_device_bytes() {
+  int64_t n = 0;
+  for (const auto &b : g_device) n += (int64_t)b.second;
+  return n;
+}
 int64_t fake_pinned_blocks() { return (int64_t)g_pinned.size(); }
 int fake_on_device(const void *p) { return inside(g_device, p); }
 void fake_set_free(int64_t n) { g_free = (size_t)n; }

@@ -38,7 +38,7 @@ class Library:
         self.raw = ctypes.CDLL(link())
         for name, (res, args) in ebic.SIGNATURES.items():
             getattr(self.raw, name).restype, getattr(self.raw, name).argtypes = res, args
-        for name in ("fake_allocs", "fake_device_blocks", "fake_pinned_blocks", "fake_log_size",
+        for name in ("fake_allocs", "fake_device_blocks", "fake_device_bytes", "fake_pinned_blocks", "fake_log_size",
                      "fake_calls"):
             getattr(self.raw, name).restype = ctypes.c_int64
         self.raw.fake_log_kernel.restype = ctypes.c_char_p

@@ -283,3 +283,53 @@ def test_tuned_sizes_are_for_matrices_of_the_same_kind_of_ties(lib):
     assert launches(ctx, 0) == tuned
     for c in (ctx, plain):
         lib.ebic_destroy(c)
+
+
+@pytest.mark.parametrize("rows,cols", [(4225, 300), (40_000, 100), (5000, 1100)])
+@pytest.mark.parametrize("call", ["evaluate", "tune"])
+def test_auto_takes_the_bitmap_where_what_it_allocates_is_half_of_the_free_memory(lib, rows, cols, call):
+    """AUTO and the autotuner weigh what the build really allocates (padded pair rows, bit planes,
+    pair counts): with one byte of free memory less than twice that, there is no bitmap."""
+    ebic = lib.ebic
+    n = 16_000                                        # (enough sweeps' work for the cost model)
+    ci = np.tile(np.arange(20, dtype=np.int32), n)
+    off = np.arange(0, 20 * n + 20, 20, dtype=np.int32)
+    p = ebic.Params.make(mode=0)
+
+    def look(kernel, grid, args):                     # (the population is good; its ends)
+        if "k_sweep_prepare" in kernel and words(args[8], 1)[0]:
+            ints(words(args[8], 1)[0], 3)[1] = 20 * n
+
+    lib.hook(look)
+
+    def build_bytes():
+        """What ebic_build_bitmap allocates over rank codes that are there already."""
+        ctx = lib.context()
+        q = ebic.Params.make(mode=1)
+        assert lib.load(ctx, rows, cols) == 0
+        assert lib.ebic_eval_population(ctx, ci.ctypes.data, off.ctypes.data, 1, ctypes.byref(q),
+                                        None, None, None, None) == 0
+        before = lib.fake_device_bytes()
+        assert lib.ebic_build_bitmap(ctx) == 0
+        got = lib.fake_device_bytes() - before
+        lib.ebic_destroy(ctx)
+        return got
+
+    def takes_bitmap(free):
+        lib.fake_set_free(free)
+        ctx = lib.context()
+        assert lib.load(ctx, rows, cols) == 0
+        if call == "tune":
+            assert lib.ebic_autotune(ctx, ci.ctypes.data, off.ctypes.data, n, ctypes.byref(p), 2,
+                                     None) == 0
+        else:
+            assert lib.ebic_eval_population(ctx, ci.ctypes.data, off.ctypes.data, n,
+                                            ctypes.byref(p), None, None, None, None) == 0
+        lib.fake_clear_log()
+        st = lib.ebic_copy_bitmap(ctx, None, 0)       # (EBIC_ESTATE: no bitmap)
+        lib.ebic_destroy(ctx)
+        return st != ebic.EBIC_ESTATE
+
+    need = build_bytes()
+    assert takes_bitmap(2 * need + 2)
+    assert not takes_bitmap(2 * need - 2)
