@@ -173,11 +173,9 @@ int64_t ebic_job_footprint(int64_t rows, int32_t cols, const ebic_params *p, int
   int64_t bytes = (int64_t)cols * R_pad * 4;              // order keys
   bytes += rows * (int64_t)cols * 4;                      // staged host matrix
   if (job_mode(rows, cols, *p, n_gen) == EBIC_MODE_BITMAP)
-    bytes += (int64_t)cols * cols * bitmap_stride(rows, cols) * 4;  // pair bitmap
+    bytes += bitmap_build_bytes(rows, cols);              // pair bitmap, bit planes, pair counts
   const int w = code_bytes_for(cols);
-  if (w)  // rank codes and (bitmap form) their bit planes
-    bytes += (int64_t)cols * code_stride_for(rows, w) * w +
-             code_plane_words(cols, bitmap_stride(rows, cols)) * 4;
+  if (w) bytes += (int64_t)cols * code_stride_for(rows, w) * w;  // rank codes (both forms)
   bytes += 2 * P * (EBIC_MAX_LEN * 4 + 4 + 4 + 12 + 1 + 1 + 8 + 8);  // population buffers
   bytes += P * 12 + 64;                                   // evaluation scratch
   bytes += (int64_t)tabu_capacity(P * ((int64_t)n_gen + 2)) * 8;  // tabu list

@@ -333,3 +333,19 @@ def test_auto_takes_the_bitmap_where_what_it_allocates_is_half_of_the_free_memor
     need = build_bytes()
     assert takes_bitmap(2 * need + 2)
     assert not takes_bitmap(2 * need - 2)
+
+
+@pytest.mark.parametrize("rows,cols", [(300, 20), (10_000, 100), (33_333, 777), (5000, 1100)])
+@pytest.mark.parametrize("mode", [1, 2])
+def test_a_jobs_footprint_is_what_it_allocates(lib, rows, cols, mode):
+    """The server reserves what a job's search allocates, and no more than its 1/16 slack and a few
+    small buffers beyond it: a job of the direct form reserves nothing for the bitmap's planes."""
+    p = lib.ebic.Params.make(pop_size=400, max_len=8, init_max_len=8, mode=mode, tabu_hit_limit=0)
+    foot = lib.ebic_job_footprint(rows, cols, ctypes.byref(p), 20)
+    before = lib.fake_device_bytes()
+    ctx = lib.context()
+    assert lib.load(ctx, rows, cols) == 0
+    assert lib.run(ctx, p, 20)[0] == 0
+    used = lib.fake_device_bytes() - before
+    lib.ebic_destroy(ctx)
+    assert used <= foot <= used * 17 / 16 + 16384
