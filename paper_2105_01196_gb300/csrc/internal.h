@@ -356,6 +356,9 @@ cudaError_t launch_build_bitmap(const uint32_t *keys, int64_t R_pad, int32_t C, 
 cudaError_t launch_build_bitmap_planes(const uint32_t *planes, int32_t C, int64_t Wst,
                                        uint32_t *bitmap, unsigned long long *cnt, int num_sms,
                                        cudaStream_t s);
+// n_rows stored pair rows (Gst words each) without their padding, to device memory: Wst words each.
+cudaError_t launch_copy_rows(const uint32_t *G, int64_t Gst, int64_t Wst, int64_t n_rows,
+                             uint32_t *out, cudaStream_t s);
 // *out (device) = the column pairs with equal values in some row, from the pair counts.
 cudaError_t launch_count_tied(const unsigned long long *cnt, int32_t C, int64_t R, int32_t *out,
                               cudaStream_t s);

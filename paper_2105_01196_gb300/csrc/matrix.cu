@@ -427,6 +427,41 @@ __global__ void __launch_bounds__(kBuildWarps * 32, 3) k_build_bitmap_planes(con
   }
 }
 
+// Copies `total` pieces of pair rows without their padding: n of the `stride` pieces of each row (16
+// bytes a piece, or 4 where the output starts between 16-byte boundaries), N pieces per thread, their
+// loads ahead of their stores.  Bound: HBM.  33,333 x 777 (2.53 GB out): 0.72 ms, 3.5 TB/s written;
+// the runtime's strided copy 1.29 ms, its plain copy of unpadded rows 0.75 ms.
+template <class T, int N>
+__global__ void __launch_bounds__(256) k_copy_rows(const T *__restrict__ G, int64_t stride,
+                                                   uint32_t n, int64_t total,
+                                                   T *__restrict__ out) {
+  const int64_t q0 = (int64_t)blockIdx.x * (256 * N), r0 = q0 / n;
+  const uint32_t c0 = (uint32_t)(q0 - r0 * n);
+  T v[N];
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    const uint32_t k = j * 256 + threadIdx.x, c = c0 + k, dr = c / n;
+    if (q0 + k < total) v[j] = __ldcs(G + (r0 + dr) * stride + (c - dr * n));
+  }
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    const int64_t q = q0 + j * 256 + threadIdx.x;
+    if (q < total) __stcs(out + q, v[j]);
+  }
+}
+
+template <class T, int N>
+cudaError_t copy_rows(const uint32_t *G, int64_t Gst, int64_t Wst, int64_t n_rows, uint32_t *out,
+                      cudaStream_t s) {
+  constexpr int kWords = sizeof(T) / 4, kBlock = 256 * N;
+  const int64_t total = n_rows * (Wst / kWords), blocks = (total + kBlock - 1) / kBlock;
+  if (blocks > 0x7FFFFFFF) return cudaErrorInvalidValue;
+  k_copy_rows<T, N><<<(unsigned)blocks, 256, 0, s>>>(reinterpret_cast<const T *>(G), Gst / kWords,
+                                                    (uint32_t)(Wst / kWords), total,
+                                                    reinterpret_cast<T *>(out));
+  return cudaGetLastError();
+}
+
 // Pairs of columns with equal values in some row: those whose two counts do not add up to R.
 __global__ void __launch_bounds__(256) k_count_tied(const unsigned long long *__restrict__ cnt,
                                                     int32_t C, int64_t R, int32_t *out) {
@@ -444,6 +479,13 @@ __global__ void __launch_bounds__(256) k_count_tied(const unsigned long long *__
 }
 
 }  // namespace
+
+cudaError_t launch_copy_rows(const uint32_t *G, int64_t Gst, int64_t Wst, int64_t n_rows,
+                             uint32_t *out, cudaStream_t s) {
+  return (reinterpret_cast<uintptr_t>(out) & 15) == 0
+             ? copy_rows<uint4, 4>(G, Gst, Wst, n_rows, out, s)
+             : copy_rows<uint32_t, 16>(G, Gst, Wst, n_rows, out, s);
+}
 
 cudaError_t launch_count_tied(const unsigned long long *cnt, int32_t C, int64_t R, int32_t *out,
                               cudaStream_t s) {

@@ -349,3 +349,22 @@ def test_a_jobs_footprint_is_what_it_allocates(lib, rows, cols, mode):
     used = lib.fake_device_bytes() - before
     lib.ebic_destroy(ctx)
     assert used <= foot <= used * 17 / 16 + 16384
+
+
+@pytest.mark.parametrize("rows,cols,device,packs,strided,plain", [
+    (4225, 300, 1, 1, 0, 0), (33_333, 200, 1, 1, 0, 0), (33_333, 50, 0, 1, 0, 1),
+    (4225, 300, 0, 2, 0, 2), (4225, 520, 0, 4, 0, 4), (33_333, 200, 0, 0, 1, 0),
+    (4096, 300, 1, 0, 0, 1), (4096, 300, 0, 0, 0, 1)])
+def test_padded_pair_rows_go_out_packed(lib, rows, cols, device, packs, strided, plain):
+    """ebic_copy_bitmap: packed by a kernel for the device and, whole or in pieces, for the host where
+    rows are short or the bitmap is small; unpadded rows as one copy."""
+    ctx = lib.context()
+    assert lib.load(ctx, rows, cols) == 0 and lib.ebic_build_bitmap(ctx) == 0
+    n = lib.ebic_bitmap_bytes(rows, cols) // 4
+    out = np.empty(n, np.uint32)
+    dst = lib.device(4 * n) if device else out.ctypes.data
+    lib.fake_clear_log()
+    assert lib.ebic_copy_bitmap(ctx, dst, n) == 0
+    assert sum("k_copy_rows" in k for k, _ in lib.log()) == packs
+    assert (lib.fake_calls(b"copy2d"), lib.fake_calls(b"copy")) == (strided, plain)
+    lib.ebic_destroy(ctx)
