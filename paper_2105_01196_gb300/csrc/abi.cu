@@ -115,10 +115,12 @@ bool ebic_is_device_ptr(const void *p) {
 }
 
 // The context's pinned block (see ebic_ctx::pin).  Pinning host memory takes a few hundred
-// microseconds, so blocks of closed contexts are kept for the next ones, up to kPinKeep of them.
+// microseconds, so blocks of closed contexts are kept for the next ones: up to kPinKeep of them (32
+// MB), as many as a job server has workers.  (With eight kept, the ninth context open at once and
+// those after it took about 100 us longer to make and 130 us longer to close, every time.)
 constexpr size_t kPinStatus = 256, kPinIn = 256 << 10, kPinOut = 256 << 10;
 static_assert(kPinIn + kPinOut == kPinSpare, "the pinned block's size");
-constexpr size_t kPinKeep = 8;
+constexpr size_t kPinKeep = 64;
 static std::mutex g_pin_mu;
 static unsigned char *g_pin_free[kPinKeep];
 static size_t g_pin_n = 0;
@@ -448,17 +450,19 @@ int ebic_create(ebic_ctx **out, int32_t device, void *cuda_stream) {
     }
     ctx->own_stream = true;
   }
-  if (ctx->d_err.ensure(64, ctx->stream) != cudaSuccess ||
-      ctx->d_ties.ensure(64, ctx->stream) != cudaSuccess ||
-      ctx->d_work.ensure(64, ctx->stream) != cudaSuccess ||
-      ctx->d_kerr.ensure(64, ctx->stream) != cudaSuccess ||
-      cudaMemsetAsync(ctx->d_kerr.p, 0, 64, ctx->stream) != cudaSuccess ||
-      cudaMemsetAsync(ctx->d_work.p, 0, 64, ctx->stream) != cudaSuccess ||
-      cudaMemsetAsync(ctx->d_err.p, 0, 64, ctx->stream) != cudaSuccess ||
+  DevWords *const words[] = {&ctx->d_err, &ctx->d_work, &ctx->d_kerr, &ctx->d_ties};
+  constexpr size_t kWordsBytes = 64 * sizeof(words) / sizeof(words[0]);
+  if (ctx->d_words.ensure(kWordsBytes, ctx->stream) != cudaSuccess ||
+      cudaMemsetAsync(ctx->d_words.p, 0, kWordsBytes, ctx->stream) != cudaSuccess ||
       !(ctx->pin = take_pin())) {
     cudaGetLastError();
     ebic_destroy(ctx);
     return EBIC_ENOMEM;
+  }
+  unsigned char *at = ctx->d_words.as<unsigned char>();
+  for (DevWords *w : words) {
+    w->p = at;
+    at += 64;
   }
   *out = ctx;
   return EBIC_OK;
@@ -471,9 +475,9 @@ int ebic_destroy(ebic_ctx *ctx) {
   cudaGetLastError();
   gen_state_free(ctx->gen);
   ctx->gen = nullptr;
-  DevBuf *bufs[] = {&ctx->keys, &ctx->bitmap, &ctx->stage_x, &ctx->d_err, &ctx->d_work,
-                    &ctx->ev_cols, &ctx->ev_off, &ctx->ev_out, &ctx->ev_fit, &ctx->d_kerr,
-                    &ctx->codes, &ctx->planes, &ctx->pair_cnt, &ctx->d_ties};
+  DevBuf *bufs[] = {&ctx->keys, &ctx->bitmap, &ctx->stage_x, &ctx->d_words, &ctx->ev_cols,
+                    &ctx->ev_off, &ctx->ev_out, &ctx->ev_fit, &ctx->codes, &ctx->planes,
+                    &ctx->pair_cnt};
   for (DevBuf *b : bufs) b->release();
   give_pin(ctx->pin);
   prof_collect(ctx);

@@ -75,6 +75,13 @@ struct DevBuf {
   T *as() const { return reinterpret_cast<T *>(p); }
 };
 
+// Part of a context's block of words on the device (ebic_ctx::d_words).
+struct DevWords {
+  void *p = nullptr;
+  template <class T>
+  T *as() const { return reinterpret_cast<T *>(p); }
+};
+
 // Population as the kernels see it: CSR (off != nullptr, len derived) or fixed-stride storage
 // with explicit lengths (off == nullptr).  dead (optional) marks slots that are not scored.  In
 // the generation loop, a slot whose key a lower slot also produced is not scored either (dkeys,
@@ -228,18 +235,22 @@ struct ebic_ctx {
   bool pair_cnt_ok = false;
   // tied column pairs of the bitmap's matrix (d_ties), and what follows: 1 few pairs are tied, so
   // the evaluations look for individuals without ties; 0 many; -1 not counted yet
-  DevBuf d_ties;
+  DevWords d_ties;
   int tie_state = -1;
 
   // scratch for single evaluations
-  DevBuf d_err, d_work, ev_cols, ev_off, ev_out, ev_fit;
+  DevBuf ev_cols, ev_off, ev_out, ev_fit;
+  // error, work, kernel-error and tie words of 64 bytes each: one allocation, cleared when the
+  // context is made
+  DevBuf d_words;
+  DevWords d_err, d_work;
   // pinned host memory the device reads and writes: the state of a call (kPinStatus words), then
   // kPinIn bytes of a small host population and kPinOut bytes of its results (abi.cu)
   unsigned char *pin = nullptr;
 
   // staged direct form of the loaded matrix, and the kernels' error word
   DirectTma dtma;
-  DevBuf d_kerr;
+  DevWords d_kerr;
 
   // per-row rank codes of the loaded matrix (code_bytes 0: none), built on first use, and their
   // bit planes (the pair-bitmap build's operand), built with the bitmap

@@ -44,6 +44,7 @@ def test_a_search_that_ran_out_of_memory_leaves_nothing_behind(lib, first, reloa
         if "k_init" in kernel:
             null.extend(k for k in range(8) if not words(args[1], 8)[k])
 
+    before = lib.fake_device_blocks()
     lib.hook(check)
     blob = np.zeros(1 << 20, np.uint8)
     ctx = lib.context()
@@ -78,7 +79,7 @@ def test_a_search_that_ran_out_of_memory_leaves_nothing_behind(lib, first, reloa
         lib.ebic_destroy(ctx)
     assert failed > 25 and n < 199
     assert not null
-    assert lib.fake_device_blocks() == 0
+    assert lib.fake_device_blocks() == before
 
 
 @pytest.mark.parametrize("at,written", [
@@ -368,3 +369,24 @@ def test_padded_pair_rows_go_out_packed(lib, rows, cols, device, packs, strided,
     assert sum("k_copy_rows" in k for k, _ in lib.log()) == packs
     assert (lib.fake_calls(b"copy2d"), lib.fake_calls(b"copy")) == (strided, plain)
     lib.ebic_destroy(ctx)
+
+
+def test_contexts_are_made_of_kept_blocks(lib):
+    """A context takes one device allocation; its pinned block goes back for the next one, up to as
+    many as a job server has workers (64), and no further."""
+    def several(n):
+        lib.fake_fail_alloc(0)
+        ctxs = [lib.context() for _ in range(n)]
+        made = lib.fake_allocs()
+        for c in ctxs:
+            lib.ebic_destroy(c)
+        return made
+
+    before = lib.fake_device_blocks()
+    several(64)
+    kept = lib.fake_pinned_blocks()
+    assert kept == 64
+    assert several(64) == 64                          # (no pinned block anew)
+    assert several(70) == 76
+    assert lib.fake_pinned_blocks() == kept
+    assert lib.fake_device_blocks() == before
