@@ -2457,14 +2457,30 @@ int fuse_limit(const ebic_ctx *ctx, int mode, const ebic_params *p) {
 
 // Whether the loop evaluates every child in k_evolve_block: the bitmap form in the block-per-slot
 // regime (every slot's block resident at once, at most kBlockWarps attempts), no pair limit set
-// (the caller's -1 keeps the evaluation launch), and pair rows short enough that a block's threads
-// cover one in kBlockMaxSteps steps of four words.
+// (the caller's -1 keeps the evaluation launch), and little to count for a child.
+// A block counts its own child alone, in steps over a pair row (four words per thread in an exact
+// test, two in a counting one) of a round trip per four pairs, where the evaluation launch spreads
+// a child's rows over the GPU.  So the launch it saves has to outweigh the longest children's steps.
+// Times of three launches per generation over times of two, at 64-1,200 slots of 1-4 attempts,
+// 1,000-60,000 rows, 64-500 columns, lengths up to 12-64:
+//   ratio below 85/100 (chromosomes grow to ten columns and more): one step 1.0-1.5, two steps
+//   0.8-1.2, four 0.6-0.9, eight 0.4-0.9;
+//   from 85/100 on (they shrink to a few columns), up to 12 attempt warps per SM: four steps (an
+//   exact test: three) of at most 32 round trips in all 1.0-1.2, more round trips 0.9-1.1, eight
+//   steps 0.7-1.1; with more warps per SM: up to 80 round trips 1.0-1.7, 128 0.9-1.3.
 bool block_eval_fits(const ebic_ctx *ctx, int mode, const ebic_params *p, int fuse) {
   int G = 1;
   while (G < p->max_attempts) G <<= 1;
+  const bool exact = p->ratio_num == p->ratio_den;
+  const int64_t words = (exact ? 4 : 2) * 32 * G;
+  const int64_t steps = (ctx->Gst + words - 1) / words;
+  const int64_t trips = steps * ((p->max_len - 1 + 3) / 4);
+  const int64_t warps = (int64_t)p->pop_size * G;
+  const bool little = 100 * (int64_t)p->ratio_num < 85 * (int64_t)p->ratio_den ? steps <= 1
+                      : warps > 12 * (int64_t)ctx->num_sms ? trips <= 80
+                                                           : steps <= (exact ? 3 : 4) && trips <= 32;
   return mode == EBIC_MODE_BITMAP && fuse == 0 && p->fuse_pairs >= 0 && !p->last_kept &&
-         G <= kBlockWarps &&
-         (int64_t)p->pop_size * G <= (int64_t)ctx->num_sms * kEvolveResidentWarps &&
+         G <= kBlockWarps && little && warps <= (int64_t)ctx->num_sms * kEvolveResidentWarps &&
          (int64_t)p->pop_size <= (int64_t)ctx->num_sms *
                                      resident_blocks((const void *)k_evolve_block, G * 32,
                                                      evolve_smem(G, ctx->C)) &&

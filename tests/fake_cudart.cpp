@@ -249,14 +249,13 @@ cudaError_t cudaFuncGetAttributes(cudaFuncAttributes *a, const void *) {
   memset(a, 0, sizeof(*a));
   return cudaSuccess;
 }
-cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int *n, const void *, int, size_t,
-                                                                   unsigned) {
-  *n = 2;
-  return cudaSuccess;
-}
 cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessor(int *n, const void *, int, size_t) {
   *n = 8;
   return cudaSuccess;
+}
+cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int *n, const void *f, int t,
+                                                                   size_t s, unsigned) {
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, f, t, s);
 }
 cudaError_t cudaGetDriverEntryPointByVersion(const char *, void **, unsigned, unsigned long long,
                                              cudaDriverEntryPointQueryResult *) {

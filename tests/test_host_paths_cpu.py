@@ -390,3 +390,36 @@ def test_contexts_are_made_of_kept_blocks(lib):
     assert several(70) == 76
     assert lib.fake_pinned_blocks() == kept
     assert lib.fake_device_blocks() == before
+
+
+def generation(lib, rows, cols, **kw):
+    """The launches of the second of two generations of a bitmap search."""
+    base = dict(pop_size=100, max_len=20, init_max_len=20, elite=2, n_biclusters=3, mode=2,
+                tabu_hit_limit=0, neg_trends=1, ratio_num=85, ratio_den=100, use_graph=0)
+    base.update(kw)
+    p = lib.ebic.Params.make(**base)
+    ctx = lib.context()
+    assert lib.load(ctx, rows, cols) == 0 and lib.run(ctx, p, 1)[0] == 0
+    lib.fake_clear_log()
+    assert lib.run(ctx, p, 1)[0] == 0
+    lib.ebic_destroy(ctx)
+    return [k for k, _ in lib.log()]
+
+
+@pytest.mark.parametrize("rows,pop,attempts,ratio,max_len,block", [
+    (10_000, 800, 4, (85, 100), 20, 1), (13_579, 800, 4, (85, 100), 20, 1),   # the usual searches
+    (8192, 100, 4, (1, 2), 64, 1), (8193, 100, 4, (1, 2), 12, 0),              # long children
+    (8192, 1200, 4, (3, 4), 20, 1), (16_000, 1200, 4, (4, 5), 20, 0),
+    (32_768, 100, 4, (85, 100), 20, 1), (32_768, 100, 4, (85, 100), 64, 0),    # few warps
+    (33_000, 100, 4, (85, 100), 20, 0), (50_000, 456, 4, (9, 10), 20, 0),
+    (60_000, 800, 4, (85, 100), 20, 1), (60_000, 800, 4, (85, 100), 64, 0),    # many warps
+    (40_000, 800, 4, (85, 100), 64, 1), (65_536, 1200, 4, (85, 100), 41, 1),
+    (65_537, 1200, 4, (85, 100), 20, 0), (16_384, 1200, 4, (1, 1), 64, 1),
+    (49_152, 100, 4, (1, 1), 20, 1), (50_000, 100, 4, (1, 1), 20, 0),
+    (16_384, 100, 1, (85, 100), 20, 0), (8192, 100, 1, (85, 100), 20, 1)])
+def test_small_searches_evaluate_in_the_evolve_launch_where_it_pays(lib, rows, pop, attempts, ratio,
+                                                                     max_len, block):
+    ran = generation(lib, rows, 30 if max_len < 30 else 64, pop_size=pop, max_attempts=attempts,
+                     ratio_num=ratio[0], ratio_den=ratio[1], max_len=max_len, init_max_len=max_len)
+    assert any("k_evolve_block" in k for k in ran) == bool(block)
+    assert sum("k_eval" in k for k in ran) == 1 - block
