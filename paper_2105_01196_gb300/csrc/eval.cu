@@ -1280,7 +1280,16 @@ cudaError_t launch_eval_kernel(int mode, const EvalArgs &a0, const PopView &pv, 
   // k_eval_bitmap_one); with ties, both directions' words beside each other, which then keep HBM
   // busy with 16 warps per SM (a kernel counting the directions in turn took 0.67 ms at
   // 60,000 x 1,000, against 0.55 ms).
-  const bool one = stage && a.neg && a.tie_free && a.pair_cnt && a.ipw == 1;
+  // Not where a generation's launch over every slot has few items and short children (a ratio from
+  // 85/100 on): the look at the pair counts then costs more than the bytes it saves.  Generations
+  // of 64-4,096 slots on 3,000 x 1,000 to 60,000 x 400, against both directions: 0.88-1.03 times as
+  // fast below eight passes per resident warp of the launch, 1.13-1.48 from there on; with the
+  // list of the longer slots, which an evolve kernel that evaluates short ones leaves, 0.96-1.1,
+  // and at a ratio of 1/2 1.05-1.54, whatever the size.
+  const bool short_few = a.mv_table && !pv.list &&
+                         100 * (int64_t)a.rnum >= 85 * (int64_t)a.rden &&
+                         pv.n * passes_total < 8 * 2 * kWarps * (int64_t)num_sms;
+  const bool one = stage && a.neg && a.tie_free && a.pair_cnt && a.ipw == 1 && !short_few;
   const EvalKernel kern =
       one ? (a.non_strict ? k_eval_bitmap_one<true> : k_eval_bitmap_one<false>)
       : bitmap ? bitmap_kernel(a.neg, a.non_strict, stage, a.ipw > 1)

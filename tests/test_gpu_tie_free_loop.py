@@ -25,7 +25,8 @@ def test_loop_reads_one_direction(pop, fuse, ns):
         x[g.choice(R, size=1 + R * k // 12, replace=False), c] = -1.0
         x[:, c - 1] = np.where(x[:, c] < 0, -1.0, x[:, c - 1])
     assert C * C * R / 8 > 180e6
-    base = dict(neg_trends=1, ratio_num=85, ratio_den=100, max_len=20, init_min_len=2,
+    num, den = (1, 2) if fuse < 0 else (85, 100)
+    base = dict(neg_trends=1, ratio_num=num, ratio_den=den, max_len=20, init_min_len=2,
                 init_max_len=20, pop_size=pop, elite=6, n_biclusters=6, tabu_hit_limit=0, seed=23,
                 non_strict=ns)
     op = OParams(**base)

@@ -423,3 +423,22 @@ def test_small_searches_evaluate_in_the_evolve_launch_where_it_pays(lib, rows, p
                      ratio_num=ratio[0], ratio_den=ratio[1], max_len=max_len, init_max_len=max_len)
     assert any("k_evolve_block" in k for k in ran) == bool(block)
     assert sum("k_eval" in k for k in ran) == 1 - block
+
+
+@pytest.mark.parametrize("rows,pop,ratio,fuse,one", [
+    (4500, 96, (85, 100), -1, 0), (4500, 96, (1, 2), -1, 1), (4500, 96, (85, 100), 2, 1),
+    (4500, 1400, (9, 10), -1, 0), (60_000, 1200, (85, 100), -1, 0), (60_000, 1300, (85, 100), -1, 1),
+    (20_000, 4096, (85, 100), -1, 1), (16_000, 4096, (1, 1), -1, 0)])
+def test_generations_read_one_direction_where_it_pays(lib, rows, pop, ratio, fuse, one):
+    """No tied pairs: a generation's evaluation over every slot takes the one-direction form from
+    19,456 passes on, over a list or at a low ratio always (an exact ratio has no staged form)."""
+    def count(kernel, grid, args):
+        if "k_count_tied" in kernel:
+            ints(words(args[3], 1)[0], 1)[0] = 0
+
+    lib.hook(count)
+    ran = generation(lib, rows, 700, pop_size=pop, ratio_num=ratio[0], ratio_den=ratio[1],
+                     fuse_pairs=fuse)
+    used = [k for k in ran if "k_eval_bitmap" in k]
+    assert len(used) == 1
+    assert ("k_eval_bitmap_one" in used[0]) == bool(one)
