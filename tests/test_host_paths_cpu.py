@@ -442,3 +442,21 @@ def test_generations_read_one_direction_where_it_pays(lib, rows, pop, ratio, fus
     used = [k for k in ran if "k_eval_bitmap" in k]
     assert len(used) == 1
     assert ("k_eval_bitmap_one" in used[0]) == bool(one)
+
+
+@pytest.mark.parametrize("rows,entries,waits", [(10_000, 20, 1), (10_000, 100, 1), (10_000, 256, 2),
+                                                (33_333, 100, 2)])
+def test_large_masks_are_not_copied_twice(lib, rows, entries, waits):
+    """Masks of up to 160 KB for the whole list come with the counters in one wait; larger ones, of the
+    entries there are, straight to the caller after the count."""
+    p = lib.ebic.Params.make(pop_size=300, max_len=6, init_max_len=6, elite=2, n_biclusters=entries,
+                             mode=1)
+    ctx = lib.context()
+    assert lib.load(ctx, rows, 20) == 0 and lib.run(ctx, p, 1)[0] == 0
+    out = np.zeros((256, (rows + 127) // 128 * 4), np.uint32)
+    n = ctypes.c_int32()
+    for _ in range(2):                                # (the first call makes the buffer)
+        lib.fake_clear_log()
+        assert lib.ebic_extract_biclusters(ctx, 256, out.ctypes.data, ctypes.byref(n)) == 0
+    assert lib.fake_calls(b"synchronise") == waits
+    lib.ebic_destroy(ctx)
