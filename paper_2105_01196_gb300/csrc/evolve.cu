@@ -990,7 +990,7 @@ __global__ void __launch_bounds__(kMaxAttemptWarps * 32) k_evolve(GenArgs ga, Bu
 // Bound: latency, the slot's chain of dependent loads (tournament, tabu probe) and then one round
 // trip per four pairs.  10,000 x 100, P = 800: 14.0 us per generation; 17.3 with three launches
 // (15.5 with these two, the rest by cheaper children).
-constexpr int kWorkStopped = 1;       // word of GenArgs::work: the stop flag this launch found
+constexpr int kWorkStopped = 1;       // word of GenArgs::work: this launch found the run stopped
 constexpr int kBlockWarps = 4;        // attempt warps at most
 constexpr int kBlockMaxSteps = 4;     // steps of four words per thread over a pair row, at most
 
@@ -1106,9 +1106,10 @@ __global__ void __launch_bounds__(kBlockWarps * 32, 8) k_evolve_block(GenArgs ga
     for (int c = threadIdx.x; c < ga.C; c += blockDim.x) s_usage[c] = ga.usage[c];
     usage = s_usage;
   }
-  // (k_finish's side task goes by what this launch saw, not by the flag that k_finish may set)
-  if (blockIdx.x == 0 && threadIdx.x == 0) ga.work[kWorkStopped] = stopped;
-  if (stopped) return;
+  if (stopped) {  // (k_finish's side task goes by what this launch found, see there)
+    if (blockIdx.x == 0 && threadIdx.x == 0) ga.work[kWorkStopped] = 1;
+    return;
+  }
   if (threadIdx.x < 3) s_cnt[threadIdx.x] = 0;
   __syncthreads();
   const int lane = threadIdx.x & 31, a = threadIdx.x >> 5;
@@ -1605,9 +1606,10 @@ __device__ __forceinline__ SlotIn load_slot(const GenArgs &ga, const Buf &nb, in
 // scores a share of the slots; the last block to finish then runs the single-block part.
 // Blocks n_fin and on (the loop without an evaluation launch: mv.mv_table set) do its side task
 // instead: the previous generation's keys join the tabu list, its duplicate table is cleared.  They
-// do so in the generation that the tabu-hit limit ends, too: the stop flag they test is the one
-// that k_evolve_block found (the last scoring block of this launch may be setting ctl->stopped, and
-// a table cleared by some warps while others leave their keys unmoved would lose keys).
+// do so in the generation that the tabu-hit limit ends, too, and in none after it: they test whether
+// k_evolve_block found the run stopped (the last scoring block of this launch may be setting
+// ctl->stopped, and a table cleared by some warps while others leave their keys unmoved would
+// lose keys).
 __global__ void __launch_bounds__(kTopThreads, 1) k_finish(GenArgs ga, Buf nb, int par, int n_fin,
                                                            EvalArgs mv) {
   extern __shared__ __align__(16) unsigned char smem[];
