@@ -122,9 +122,9 @@ typedef struct ebic_params {
                           ceil(ratio * pairs) = pairs) is evaluated by the warp that built it,
                           inside the evolve kernel; the other slots go to the evaluation
                           launch.  0 (default) = the library's choice (for a small population
-                          over a short matrix: every child, whatever its test, by the block that
-                          built it), -1 = never, 1-63 = this limit.  Results never depend
-                          on it                                                             */
+                          whose children take a block little counting: every child, whatever
+                          its test, by the block that built it), -1 = never, 1-63 = this limit.
+                          Results never depend on it                                        */
 } ebic_params;
 
 /* Progress of a run (Sec. 2.4, steps 6 and 8). */

@@ -548,7 +548,7 @@ int ensure_copy_stream(ebic_ctx *ctx, int64_t n) {
 }
 
 // The segmented load of a row-major host matrix (see ebic_load_matrix): kLoadSegments segments
-// of a multiple of 8,192 rows (whole 1,024-row chunks of the bitmap, whole tiles of every
+// of a multiple of 8,192 rows (whole 2,048-row chunks of the planes, whole tiles of every
 // kernel), the last one with the padded tail.
 constexpr int64_t kLoadSegments = 4;
 

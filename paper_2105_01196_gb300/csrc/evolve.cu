@@ -3,7 +3,7 @@
 // chromosome hashes, tabu-hit termination; parameters of Sec. 2.4's last paragraph).
 //
 // One generation is three kernels, or two (k_evolve_block, k_finish) where a small population's
-// blocks are all resident and evaluate their children whole.  They are captured as CUDA graphs (one
+// blocks are all resident and have little to count for a child (block_eval_fits).  They are captured as CUDA graphs (one
 // per buffer parity, and one of sixteen consecutive generations per starting parity) and replayed:
 //   k_evolve    one block per slot, one warp per tabu attempt: elites from the top list (step
 //               4), otherwise penalised tournament, optional one-point crossover and one
@@ -224,11 +224,6 @@ __device__ __forceinline__ bool beats(const Score &a, int ia, const Score &b, in
   if (a.m != b.m) return a.m > b.m;
   return ia < ib;
 }
-
-// ------------------------------------------------------------------ variation
-
-// ------------------------------------------------------------------ kernels
-
 
 // ------------------------------------------------------------------ warp-cooperative children
 // One warp builds one child.  The word stream and every decision are uniform across the warp (all
