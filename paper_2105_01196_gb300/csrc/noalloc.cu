@@ -109,7 +109,8 @@ __global__ void __launch_bounds__(kNaThreads) k_na_prepare(const float *__restri
 // 16-byte load per column where every column starts on a 16-byte boundary (VEC: x aligned, R a
 // multiple of 4), else rows 32 apart by four 4-byte loads (coalesced whatever the alignment).
 // NS / LK are the pair-test variants of trend.cuh.
-// Bound: latency of an item's loads, then L1 / L2 (4 bytes per row and pair).  Whole calls: 108 us
+// Bound: instruction issue (83% of cycles at 10,000 x 100, the ALU pipe 75%; the values come from L1,
+// 93% hits): comparisons and additions per row, pair and direction.  Whole calls: 108 us
 // at 10,000 x 100, 800 individuals of 2-20 columns (116 with the items dealt to all warps of the
 // grid in turn, 329 with a row per lane and 32-row items from one global counter), 0.90 ms at
 // 30,000 x 300, 4,000 individuals of 2-40 (1.05 dealt in turn).
