@@ -1612,6 +1612,9 @@ __global__ void __launch_bounds__(kTopThreads, 1) k_finish(GenArgs ga, Buf nb, i
       s_nc;
   GenCtl *ctl = ga.ctl;
   wait_prior_grid();
+  // The counters, the list's last entry and this thread's first slot are loaded in one round,
+  // ahead of the stop test (which must still come before any store).
+  const int stopped = ctl->stopped, n0 = ctl->n_top, gen0 = ctl->gen;
   if ((int)blockIdx.x >= n_fin) {
     if (ga.work[kWorkStopped]) return;
     const int n = items::move_chunks(mv), step = ((int)gridDim.x - n_fin) * (kTopThreads / 32);
@@ -1620,9 +1623,6 @@ __global__ void __launch_bounds__(kTopThreads, 1) k_finish(GenArgs ga, Buf nb, i
       items::move_chunk(mv, m, threadIdx.x & 31);
     return;
   }
-  // The counters, the list's last entry and this thread's first slot are loaded in one round,
-  // ahead of the stop test (which must still come before any store).
-  const int stopped = ctl->stopped, n0 = ctl->n_top, gen0 = ctl->gen;
   const uint64_t last_f = ga.top[ga.K - 1].f, last_h = ga.top[ga.K - 1].h;
   const int tid = blockIdx.x * blockDim.x + threadIdx.x, stride = n_fin * blockDim.x;
   SlotIn first;
