@@ -240,8 +240,7 @@ struct ebic_ctx {
 
   // scratch for single evaluations
   DevBuf ev_cols, ev_off, ev_out, ev_fit;
-  // error, work, kernel-error and tie words of 64 bytes each: one allocation, cleared when the
-  // context is made
+  // error, work, kernel-error and tie words: one allocation, cleared when the context is made
   DevBuf d_words;
   DevWords d_err, d_work;
   // pinned host memory the device reads and writes: the state of a call (kPinStatus words), then
